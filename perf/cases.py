@@ -121,24 +121,33 @@ class State:
     pass
 
 
-def prepare(case, seed):
-    T, H, I, E, K = (case[k] for k in "THIEK")
+def _inputs(case, seed):
+    """Router logits, tokens, weights and (training) the gradient of the output."""
+    T, H, I, E = (case[k] for k in "THIE")
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
-    s = State()
-    s.case, s.d = case, B.dims(T, H, I, E, K)
 
     def normal(shape, std):
         return torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, std, generator=gen)
 
+    s = State()
     s.logits = _logits(case, gen, seed)
     s.x = normal((T, H), 1.0)
     s.w_gate, s.w_up, s.w_down = normal((E, H, I), 0.02), normal((E, H, I), 0.02), normal((E, I, H), 0.02)
+    if case["kind"] not in ("forward", "fp8_forward"):
+        s.dy = normal((T, H), 1.0)
+    return s
+
+
+def prepare(case, seed):
+    T, H, I, E, K = (case[k] for k in "THIEK")
+    s = _inputs(case, seed)
+    s.case, s.d = case, B.dims(T, H, I, E, K)
     s.topk_idx = torch.empty((T, K), dtype=torch.int32, device="cuda")
     s.topk_w = torch.empty((T, K), dtype=torch.float32, device="cuda")
     kind = case["kind"]
     if kind == "host":
-        _prepare_host(s, normal)
+        _prepare_host(s)
         return s
     if kind in ("forward", "fp8_forward"):
         s.b = State()
@@ -154,7 +163,6 @@ def prepare(case, seed):
             s.b.gu = torch.empty((R, 2 * I), **bf)
     else:
         s.b = B.alloc_layer_buffers(T, H, I, E, K)
-        s.dy = normal((T, H), 1.0)
         s.dlogits = torch.empty((T, E), dtype=torch.float32, device="cuda")
     if kind in FP8_KINDS:
         _prepare_fp8(s)
@@ -188,12 +196,12 @@ def _quantise_weights(s):
         B.moe_mxfp8_quantize_w_gateup_dgrad(s.d, s.w_gate, s.w_up, *s.w_gateup_dgrad_q)
 
 
-def _prepare_host(s, normal):
-    T, H, E, K = (s.case[k] for k in "THEK")
+def _prepare_host(s):
+    T, K = (s.case[k] for k in "TK")
     B.moe_router_topk(s.d, s.logits, s.topk_idx, s.topk_w)
     s.dw_gate, s.dw_up, s.dw_down = torch.empty_like(s.w_gate), torch.empty_like(s.w_up), torch.empty_like(s.w_down)
     s.arena = _bytes(B.moe_layer_arena_bytes(s.d))
-    s.x_host, s.dy_host = s.x.cpu().pin_memory(), normal((T, H), 1.0).cpu().pin_memory()
+    s.x_host, s.dy_host = s.x.cpu().pin_memory(), s.dy.cpu().pin_memory()
     s.idx_host, s.w_host = s.topk_idx.cpu().pin_memory(), s.topk_w.cpu().pin_memory()
     s.y_host, s.dx_host = torch.empty_like(s.x_host, pin_memory=True), torch.empty_like(s.x_host, pin_memory=True)
     s.dw_host = torch.empty((T, K), dtype=torch.float32, pin_memory=True)
@@ -318,3 +326,70 @@ def tolerance(case):
     if case["kind"] in FP8_KINDS:
         return {"rel": 2e-3, "max": 0.15}
     return {"rel": 1e-2, "max": 0.3}
+
+
+# ---------------------------------------------------------------------------------------------------------------------
+# the same pass in 64 bits
+# ---------------------------------------------------------------------------------------------------------------------
+def _mx(v, axis):
+    """`v` after quantisation to E4M3 with one power-of-two scale per 32 values along `axis` (a short last block is
+    filled with zeros): scale 2^(floor(log2 of the largest magnitude) - 8), to nearest even, saturating at 448."""
+    v = v.transpose(axis, -1)
+    n = v.shape[-1]
+    b = torch.nn.functional.pad(v, (0, -n % 32)).unflatten(-1, (-1, 32))
+    top = b.abs().amax(-1, keepdim=True)
+    scale = torch.ldexp(torch.ones_like(top), torch.frexp(top)[1] - 9)   # frexp: top = m * 2^e with m in [0.5, 1)
+    scale = torch.where(top > 0, scale, torch.ones_like(scale))
+    q = (b / scale).clamp(-448.0, 448.0).float().to(torch.float8_e4m3fn).double() * scale
+    return q.flatten(-2)[..., :n].transpose(axis, -1)
+
+
+def exact(case, seed):
+    """What `run` returns, every product, sum and intermediate in 64 bits; the FP8 passes with their operands quantised
+    (from the 64-bit intermediates)."""
+    T, H, I, E, K = (case[k] for k in "THIEK")
+    s, kind = _inputs(case, seed), case["kind"]
+    training = kind not in ("forward", "fp8_forward")
+    fp8_wgrad = kind == "fp8_step" and case["fp8_wgrad"]
+
+    def q(v, axis, on=kind in FP8_KINDS):
+        return _mx(v, axis) if on else v
+
+    def tok(v):
+        return q(v, 0, fp8_wgrad)
+
+    z, idx = torch.sort(s.logits, dim=1, descending=True, stable=True)
+    idx, w = idx[:, :K], torch.softmax(z[:, :K].double(), dim=1)
+    f64 = dict(dtype=torch.float64, device="cuda")
+    y = torch.zeros((T, H), **f64)
+    if training:
+        dx, dw = torch.zeros((T, H), **f64), torch.zeros((T, K), **f64)
+        dw_gate, dw_up, dw_down = torch.zeros((E, H, I), **f64), torch.zeros((E, H, I), **f64), torch.zeros((E, I, H), **f64)
+    for e in range(E):
+        t, k = torch.nonzero(idx == e, as_tuple=True)
+        if t.numel() == 0:
+            continue
+        x, wk = s.x[t].double(), w[t, k].unsqueeze(1)
+        w_gate, w_up, w_down = s.w_gate[e].double(), s.w_up[e].double(), s.w_down[e].double()
+        xq = q(x, 1)
+        g, u = xq @ q(w_gate, 0), xq @ q(w_up, 0)
+        sg = torch.sigmoid(g)
+        h = g * sg * u
+        out = q(h, 1) @ q(w_down, 0)
+        y.index_add_(0, t, wk * out)
+        if not training:
+            continue
+        dy = s.dy[t].double()
+        dw[t, k] = (dy * out).sum(1)
+        dy = wk * dy
+        dh = q(dy, 1) @ q(w_down, 1).T
+        dg, du = dh * u * sg * (1.0 + g * (1.0 - sg)), dh * g * sg
+        dx.index_add_(0, t, q(dg, 1) @ q(w_gate, 1).T + q(du, 1) @ q(w_up, 1).T)
+        dw_down[e] = tok(h).T @ tok(dy)
+        dw_gate[e], dw_up[e] = tok(x).T @ tok(dg), tok(x).T @ tok(du)
+    if not training:
+        return dict(idx=idx.int(), y=y)
+    if kind == "host":
+        return dict(y=y, dx=dx, dtopk_w=dw, dw_gate=dw_gate, dw_up=dw_up, dw_down=dw_down)
+    dlogits = torch.zeros((T, E), **f64).scatter_(1, idx, w * (dw - (w * dw).sum(1, keepdim=True)))
+    return dict(idx=idx.int(), y=y, dx=dx, dlogits=dlogits, dw_gate=dw_gate, dw_up=dw_up, dw_down=dw_down)
