@@ -832,74 +832,88 @@ __device__ __forceinline__ uint32_t mx_e4m3x2(float lo, float hi) {
     return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(lo, hi), __NV_SATFINITE, __NV_E4M3);
 }
 
-// rows x n bf16 -> codes (same layout) and scales.  A warp takes two (row, 128-wide slice) units per load: lane l holds
-// the 8 elements 8l..8l+7 of the 256 contiguous ones (one 16-byte load), the 4 lanes of a block of 32 agree on its scale
-// through two shuffles; four such loads are in flight per lane.  The 4 scale bytes of a (row, slice) are one 32-bit word:
-//   WEIGHTS = false (activations): word [slice][row];
+// Largest magnitude of the 8 bf16 values of a 16-byte piece, kept packed (two running maxima, one per half word).  The
+// maximum of bf16 values is exact, so the packed form decides the same scale as the fp32 one; a NaN loses against any number.
+__device__ __forceinline__ __nv_bfloat162 mx_max2(uint32_t a, uint32_t b) {
+    return __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+}
+__device__ __forceinline__ uint32_t mx_abs_max4(const uint4& v) {
+    const __nv_bfloat162 m = __hmax2(mx_max2(v.x & 0x7fff7fffu, v.y & 0x7fff7fffu), mx_max2(v.z & 0x7fff7fffu, v.w & 0x7fff7fffu));
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+__device__ __forceinline__ uint32_t mx_abs_max(uint32_t a, uint32_t b) {   // of packed magnitudes
+    const __nv_bfloat162 m = mx_max2(a, b);
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+__device__ __forceinline__ float mx_lo(uint32_t w) { return __uint_as_float(w << 16); }          // bf16 -> fp32 is a shift
+__device__ __forceinline__ float mx_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ uint2 mx_codes8(const uint4& v, float inv) {   // 8 consecutive values -> 8 code bytes
+    return make_uint2(mx_e4m3x2(mx_lo(v.x) * inv, mx_hi(v.x) * inv) | (mx_e4m3x2(mx_lo(v.y) * inv, mx_hi(v.y) * inv) << 16),
+                      mx_e4m3x2(mx_lo(v.z) * inv, mx_hi(v.z) * inv) | (mx_e4m3x2(mx_lo(v.w) * inv, mx_hi(v.w) * inv) << 16));
+}
+// Where the scale word of feature `f` (4 scale bytes of one K slice) sits inside a 128-feature block of 512 bytes, in words.
+__device__ __forceinline__ int mx_sf_word(int f) { return (f % 32) * 4 + (f % 128) / 32; }
+// The scale words of 128 features f0 .. f0 + 127 (f0 a multiple of 128) of one K slice, in shared memory, into both
+// weight-scale tilings; `block` is the slice's 512-byte block of the first, `pair` the slice's place in the second
+// (which the column tile's index times `pair_stride` is added to).  Threads 0..127.
+__device__ __forceinline__ void mx_store_weight_scales(const uint32_t* words, int f0, uint32_t* block, uint8_t* pair, long long pair_stride,
+                                                       int i) {
+    if (block != nullptr) block[i] = words[(i % 4) * 32 + i / 4];   // consecutive threads, consecutive words
+    const int nt = (f0 + i) / MXP_NT, c = (f0 + i) % MXP_NT;
+    *reinterpret_cast<uint32_t*>(pair + nt * pair_stride + (c >> 7) * 512 + mx_sf_word(c) * 4) = words[i];
+}
+
+// rows x n bf16 -> codes (same layout) and scales.  A block takes 128 rows x one 128-wide slice; a half-warp holds a row
+// (8 elements per lane, one 16-byte load), eight rows one after the other with their loads all in flight; the 4 lanes of a
+// block of 32 agree on its scale through two shuffles.  The scale bytes meet in shared memory and leave as one 32-bit word
+// per (row, slice):
+//   WEIGHTS = false (activations): word [slice][row], 512 contiguous bytes per block of threads;
 //   WEIGHTS = true  (weights whose contraction axis is contiguous, rows = E * n_feat, e.g. W_down read as [I, H] for the
 //                    data gradient): the word's place in each of the two weight-scale tilings.  The output may be a
 //                    column range of a wider operand (out_k_tiles slices per row, this input filling slices
 //                    out_kt0 .. out_kt0 + n/128): W_gate and W_up side by side along the contraction of the gate/up
 //                    data gradient.
+// 3 bytes of HBM traffic per element, so bound by HBM only if few instructions and few partial sectors go into one.  Inside
+// an FP8 step, 201 M weights (128 x 2048 x 768): 242 -> 122 us (4.9 TB/s); activations 131072 x 2048: 184 -> 130 us
+// (6.2 TB/s).  Before, a warp walked along a row: every (row, slice) took a 64-bit division, eight shuffles and, for
+// weights, two 4-byte stores into a sector each.
 template <bool WEIGHTS>
 __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n, int n_feat,
                                                                int out_k_tiles, int out_kt0, uint2* __restrict__ codes,
                                                                uint8_t* __restrict__ scales, uint8_t* __restrict__ scales_pair) {
-    constexpr int U = 4;
-    const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const int k_tiles = n / 128;
-    const long long total = rows * k_tiles;            // units of 128 elements, contiguous in memory
-    const long long pairs = (total + 1) / 2;
-    const int n_tiles_p = WEIGHTS ? (n_feat + MXP_NT - 1) / MXP_NT : 0;
-    for (long long p0 = warp * U; p0 < pairs; p0 += n_warps * U) {
-        uint4 raw[U];
+    __shared__ __align__(16) uint8_t sf[128 * 4];
+    const int k_tiles = n >> 7;
+    const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
+    const long long row0 = 128ll * row_tile;
+    const int sub = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+    const int n_rows = (int)min(128ll, rows - row0);
+    const uint4* src = x + (row0 + sub) * (n >> 3) + kt * 16 + l16;
+    uint2* dst = codes + ((row0 + sub) * out_k_tiles + out_kt0 + kt) * 16 + l16;
+    const long long src_step = 16ll * (n >> 3), dst_step = 16ll * out_k_tiles * 16;
+    uint4 v[8];
 #pragma unroll
-        for (int i = 0; i < U; ++i) {
-            const long long u = 2 * (p0 + i) + (lane >> 4);
-            raw[i] = (u < total) ? __ldg(x + (p0 + i) * 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
-        }
+    for (int i = 0; i < 8; ++i) v[i] = sub + 16 * i < n_rows ? __ldg(src + i * src_step) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int i = 0; i < U; ++i) {
-            if (p0 + i >= pairs) break;
-            const long long u = 2 * (p0 + i) + (lane >> 4);   // this half-warp's unit
-            const uint32_t* rw = reinterpret_cast<const uint32_t*>(&raw[i]);
-            float v[8];
-            float amax = 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&rw[j]));
-                v[2 * j] = f.x; v[2 * j + 1] = f.y;
-                amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-            }
-            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
-            const int se = mx_scale_exp(amax);
-            const float inv = mx_inv_scale(se);
-            uint2 out;
-            out.x = mx_e4m3x2(v[0] * inv, v[1] * inv) | (mx_e4m3x2(v[2] * inv, v[3] * inv) << 16);
-            out.y = mx_e4m3x2(v[4] * inv, v[5] * inv) | (mx_e4m3x2(v[6] * inv, v[7] * inv) << 16);
-            const long long r = (total >> 32) == 0 ? (long long)((uint32_t)u / (uint32_t)k_tiles) : u / k_tiles;
-            const int kt = (int)(u - r * k_tiles) + out_kt0;
-            if (u < total) codes[(r * out_k_tiles + kt) * 16 + (lane & 15)] = out;
-            const uint32_t sbyte = (uint32_t)(se + 127);
-            const int base = lane & 16;                       // first lane of this half-warp
-            const uint32_t word = __shfl_sync(0xffffffffu, sbyte, base) | (__shfl_sync(0xffffffffu, sbyte, base + 4) << 8) |
-                                  (__shfl_sync(0xffffffffu, sbyte, base + 8) << 16) | (__shfl_sync(0xffffffffu, sbyte, base + 12) << 24);
-            if ((lane & 15) == 0 && u < total) {
-                if (!WEIGHTS) {
-                    reinterpret_cast<uint32_t*>(scales)[(long long)kt * rows + r] = word;
-                } else {
-                    const int e = (int)(r / n_feat), f = (int)(r - (long long)e * n_feat);
-                    *reinterpret_cast<uint32_t*>(scales + (((long long)e * (n_feat / 128) + f / 128) * out_k_tiles + kt) * 512 +
-                                                 (f % 32) * 16 + ((f % 128) / 32) * 4) = word;
-                    const int nt = f / MXP_NT, c = f % MXP_NT;
-                    *reinterpret_cast<uint32_t*>(scales_pair + (((long long)e * n_tiles_p + nt) * out_k_tiles + kt) * 1024 +
-                                                 (c >> 7) * 512 + (c % 32) * 16 + ((c % 128) / 32) * 4) = word;
-                }
-            }
-        }
+    for (int i = 0; i < 8; ++i) {
+        uint32_t m = mx_abs_max4(v[i]);
+        m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        const int se = mx_scale_exp(fmaxf(mx_lo(m), mx_hi(m)));
+        if (sub + 16 * i < n_rows) dst[i * dst_step] = mx_codes8(v[i], mx_inv_scale(se));
+        if ((l16 & 3) == 0) sf[(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se + 127);
+    }
+    __syncthreads();
+    const int i = threadIdx.x;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(sf);
+    if (!WEIGHTS) {
+        if (i < n_rows) reinterpret_cast<uint32_t*>(scales)[(long long)(out_kt0 + kt) * rows + row0 + i] = words[i];
+    } else if (i < 128) {   // n_feat is a multiple of 128: the 128 rows are 128 features of one expert
+        const long long e = row0 / n_feat;
+        const int f0 = (int)(row0 - e * n_feat);
+        const int n_tiles_p = (n_feat + MXP_NT - 1) / MXP_NT;
+        mx_store_weight_scales(words, f0,
+                               reinterpret_cast<uint32_t*>(scales + ((e * (n_feat / 128) + f0 / 128) * out_k_tiles + out_kt0 + kt) * 512),
+                               scales_pair + (e * n_tiles_p * out_k_tiles + out_kt0 + kt) * 1024, (long long)out_k_tiles * 1024, i);
     }
 }
 
@@ -1019,48 +1033,77 @@ __global__ void __launch_bounds__(256) mx_swiglu_bwd_quantize_kernel(const uint4
     }
 }
 
+// ---- quantisers along the rows of a row-major operand (codes stored transposed) ----
+// 128 rows x 128 features of a row-major bf16 matrix -> 128 code bytes per feature, contiguous, and a scale byte per (feature,
+// block of 32 rows).  Shared by the weight quantiser (weights whose output-feature axis is contiguous) and the token-axis
+// quantiser.  The tile comes in with 16-byte asynchronous copies (rows from `n_rows` on as zeros); a thread then owns a
+// pair of features over one block of 32 rows: 32 words from shared memory (blocks of rows are set 8 words apart so that
+// the 4 x 8 lanes of a warp hit 32 banks), both maxima in packed arithmetic, 2 x 32 code bytes.  The 4 lanes that share a
+// feature write its 128 contiguous bytes.
+constexpr int MXT_BLOCK_WORDS = 32 * 64 + 8;   // shared-memory words of 32 rows x 128 features, with the bank offset
+__device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long long ld, int n_rows, uint8_t* dst, long long dst_ld,
+                                                           uint32_t* tile, uint8_t* sf) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int row = i * 16 + (tid >> 4), piece = tid & 15;
+        const bool in = row < n_rows;
+        const bf16* from = src + (in ? row * ld : 0) + piece * 8;
+        const uint32_t to = smem_u32(tile + (row >> 5) * MXT_BLOCK_WORDS + (row & 31) * 64 + piece * 4);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(in ? 16 : 0) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const int lane = tid & 31, block = lane >> 3, pair = (tid >> 5) * 8 + (lane & 7);   // features 2 * pair, 2 * pair + 1
+    const uint32_t* col = tile + block * MXT_BLOCK_WORDS + pair;
+    uint32_t v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = col[j * 64];
+    uint32_t m = 0u;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) m = mx_abs_max(m, v[j] & 0x7fff7fffu);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int se = mx_scale_exp(h ? mx_hi(m) : mx_lo(m));
+        const float inv = mx_inv_scale(se);
+        uint32_t out[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            float f[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) f[t] = (h ? mx_hi(v[4 * g + t]) : mx_lo(v[4 * g + t])) * inv;
+            out[g] = mx_e4m3x2(f[0], f[1]) | (mx_e4m3x2(f[2], f[3]) << 16);
+        }
+        uint4* to = reinterpret_cast<uint4*>(dst + (2 * pair + h) * dst_ld + block * 32);
+        to[0] = make_uint4(out[0], out[1], out[2], out[3]);
+        to[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        sf[(2 * pair + h) * 4 + block] = (uint8_t)(se + 127);
+    }
+    __syncthreads();
+}
+
 // Weights whose OUTPUT-feature axis is contiguous: w [E, k, n] bf16 (W_down [E, I, H]; W_gate, W_up [E, H, I]) -> codes
 // transposed, contraction contiguous, as rows n_off .. n_off + n of [E, n_total, k] (W_gate and W_up stacked along the 2I
-// output features of the gate/up projection), and the scale bytes in both tilings.  One thread per (expert, block of
-// 32 along k, feature): consecutive lanes take consecutive features, so the 32 loads of a thread are coalesced across
-// the warp; the thread keeps the 32 values, picks the scale and writes 32 contiguous code bytes.
-__global__ void __launch_bounds__(256) mx_quantize_w_transposed_kernel(const bf16* __restrict__ w, int E, int k, int n,
-                                                                       int n_total, int n_off, uint8_t* __restrict__ codes,
+// output features of the gate/up projection), and the scale bytes in both tilings.  One block per (expert, K slice of
+// 128, 128 features), features fastest.
+// 201 M weights (128 x 768 x 2048): 165 -> 113 us (5.3 TB/s) inside an FP8 step.  Before, a thread loaded its 32 x 1 values
+// two bytes at a time and stored its scale bytes one by one into both tilings.
+__global__ void __launch_bounds__(256) mx_quantize_w_transposed_kernel(const bf16* __restrict__ w, int k, int n, int n_total,
+                                                                       int n_off, uint8_t* __restrict__ codes,
                                                                        uint8_t* __restrict__ scales,
                                                                        uint8_t* __restrict__ scales_pair) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int blocks_k = k / 32;
-    const long long total = (long long)E * blocks_k * n;
-    if (idx >= total) return;
-    const int h = (int)(idx % n);
-    const int ib = (int)((idx / n) % blocks_k);
-    const int e = (int)(idx / ((long long)n * blocks_k));
-    const bf16* src = w + ((long long)e * k + (long long)ib * 32) * n + h;
-    float v[32];
-    float amax = 0.f;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        v[j] = __bfloat162float(src[(long long)j * n]);
-        amax = fmaxf(amax, fabsf(v[j]));
-    }
-    const int se = mx_scale_exp(amax);
-    const float inv = mx_inv_scale(se);
-    uint32_t out[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-        out[q] = mx_e4m3x2(v[4 * q] * inv, v[4 * q + 1] * inv) | (mx_e4m3x2(v[4 * q + 2] * inv, v[4 * q + 3] * inv) << 16);
-    const int f = n_off + h;   // output feature of the GEMM
-    uint4* dst = reinterpret_cast<uint4*>(codes + ((long long)e * n_total + f) * k + (long long)ib * 32);
-    dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-    dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
-    const int k_tiles = k / 128;
-    scales[(((long long)e * (n_total / 128) + f / 128) * k_tiles + ib / 4) * 512 + (f % 32) * 16 + ((f % 128) / 32) * 4 + (ib % 4)] =
-        (uint8_t)(se + 127);
-    // the same byte in the tiling of the CTA-pair kernel: per (208-column tile, K slice) two 512-byte blocks
-    const int nt = f / MXP_NT, c = f % MXP_NT;
+    __shared__ __align__(16) uint32_t tile[4 * MXT_BLOCK_WORDS];
+    __shared__ __align__(16) uint8_t sf[128 * 4];
+    const int f_tiles = n >> 7, k_tiles = k >> 7;
+    const int ft = blockIdx.x % f_tiles, rest = blockIdx.x / f_tiles, kt = rest % k_tiles;
+    const long long e = rest / k_tiles;
+    const int f0 = n_off + ft * 128;   // first output feature of the GEMM
+    mx_transpose_quantize_tile(w + (e * k + kt * 128ll) * n + ft * 128, n, 128, codes + (e * n_total + f0) * k + kt * 128, k, tile, sf);
     const int n_tiles_p = (n_total + MXP_NT - 1) / MXP_NT;
-    scales_pair[(((long long)e * n_tiles_p + nt) * k_tiles + ib / 4) * 1024 + (c >> 7) * 512 + (c % 32) * 16 + ((c % 128) / 32) * 4 +
-                (ib % 4)] = (uint8_t)(se + 127);
+    if (threadIdx.x < 128)
+        mx_store_weight_scales(reinterpret_cast<const uint32_t*>(sf), f0,
+                               reinterpret_cast<uint32_t*>(scales + ((e * (n_total / 128) + f0 / 128) * k_tiles + kt) * 512),
+                               scales_pair + (e * n_tiles_p * k_tiles + kt) * 1024, (long long)k_tiles * 1024, threadIdx.x);
 }
 
 
@@ -1072,110 +1115,67 @@ __global__ void __launch_bounds__(256) mx_quantize_w_transposed_kernel(const bf1
 // K-major like everywhere else in this file, and the ragged contraction needs no clearing of foreign rows in shared
 // memory.  The tile list is fixed (every expert x M tiles x N tiles); an expert's K slices are
 // [slice_prefix[e], slice_prefix[e+1]); a tile of an expert without rows skips the pipeline and its epilogue writes zeros.
-// slice_prefix[e] = number of 128-row slices of the experts before e, every expert's rows rounded up to whole slices
-__global__ void __launch_bounds__(1024) mx_slice_prefix_kernel(const int32_t* __restrict__ offsets, int E, int32_t* __restrict__ sp) {
-    __shared__ int32_t part[32];
-    const int e = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int v = (e < E) ? (offsets[e + 1] - offsets[e] + 127) >> 7 : 0;
-    int incl = v;
+// x [R, ld] bf16, columns [col0, col0 + n) -> codes_t [n, pitch] (transposed, zero-padded per expert), scale words
+// [pitch/128][n] (the operand as the M side) and scale blocks in the pair tiling [ceil(n/208)][pitch/128][1024] (the
+// operand as the N side).  One block per (slice of 128 columns of the output, 128 features), features fastest.  Every block
+// derives slice_prefix (slice_prefix[e] = number of 128-row slices of the experts before e, every expert's rows rounded
+// up to whole slices) from the offsets by itself -- a scan over at most 1024 experts that overlaps the copies of the other
+// blocks on the SM -- and the first one stores it for the GEMM.
+// Inside an FP8 step, 16384 x 14336: 240 + 3 -> 196 us, 16384 x 4096: 98 + 3 -> 59 us (a kernel of its own wrote
+// slice_prefix before); alone on the chip 150 us and 49 us.  What is left inside the step is instruction issue at the clock
+// that the power cap leaves.  Taking several slices before the next 128 features (4 to 32: longer runs of code bytes per
+// feature) changed nothing.
+__global__ void __launch_bounds__(256) mx_quantize_tokens_kernel(const bf16* __restrict__ x, long long ld, int col0, int n,
+                                                                 const int32_t* __restrict__ offsets, int32_t* __restrict__ sp,
+                                                                 int E, long long pitch, uint8_t* __restrict__ codes_t,
+                                                                 uint32_t* __restrict__ sa_words, uint8_t* __restrict__ sb_atoms) {
+    __shared__ __align__(16) uint32_t tile[4 * MXT_BLOCK_WORDS];
+    __shared__ __align__(16) uint8_t sf[128 * 4];
+    __shared__ int32_t part[8];
+    __shared__ int32_t mine[3];   // first row, rows and existence of this block's slice
+    const int f_tiles = n >> 7;
+    const int f0 = (int)(blockIdx.x % (unsigned)f_tiles) * 128, slice = (int)(blockIdx.x / (unsigned)f_tiles);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // thread t scans the experts 4t .. 4t + 3
+    int32_t off[5], before[4], sum = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) off[i] = __ldg(offsets + min(4 * tid + i, E));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        before[i] = sum;
+        sum += (off[i + 1] - off[i] + 127) >> 7;
+    }
+    int incl = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, incl, d);
         if (lane >= d) incl += t;
     }
     if (lane == 31) part[warp] = incl;
+    if (tid == 0) mine[2] = 0;
     __syncthreads();
-    if (warp == 0) {
-        int w = part[lane];
+    int base = incl - sum;
+    for (int w = 0; w < warp; ++w) base += part[w];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, w, d);
-            if (lane >= d) w += t;
+    for (int i = 0; i < 4; ++i) {
+        const int first = base + before[i], local = slice - first;
+        const int rows = off[i + 1] - off[i];
+        if (local >= 0 && local * 128 < rows) {   // at most one (thread, i) of the block: the expert that holds the slice
+            mine[0] = off[i] + local * 128;
+            mine[1] = min(128, rows - local * 128);
+            mine[2] = 1;
         }
-        part[lane] = w;
+        if (blockIdx.x == 0 && 4 * tid + i <= E) sp[4 * tid + i] = first;
     }
+    if (blockIdx.x == 0 && E == 1024 && tid == 255) sp[E] = base + sum;
     __syncthreads();
-    const int before = incl - v + (warp > 0 ? part[warp - 1] : 0);
-    if (e < E) sp[e] = before;
-    if (e == E - 1) sp[E] = before + v;
-}
-
-// x [R, ld] bf16, columns [col0, col0 + n) -> codes_t [n, pitch] (transposed, zero-padded per expert), scale words
-// [pitch/128][n] (the operand as the M side) and scale blocks in the pair tiling [ceil(n/208)][pitch/128][1024] (the
-// operand as the N side).  One thread per (128-column slice, group of 8 features): the slice's four blocks of 32 rows one
-// after the other -- a 16-byte load per row, 512 contiguous bytes per warp; the thread keeps the 32 x 8 values as
-// loaded, finds the 8 block maxima, writes 32 code bytes per feature -- then the four scale bytes of each feature as
-// one word into each of the two scale layouts.
-__global__ void __launch_bounds__(128) mx_quantize_tokens_kernel(const bf16* __restrict__ x, long long ld, int col0, int n,
-                                                                 const int32_t* __restrict__ offsets, const int32_t* __restrict__ sp,
-                                                                 int E, long long pitch, uint8_t* __restrict__ codes_t,
-                                                                 uint8_t* __restrict__ sa_words, uint8_t* __restrict__ sb_atoms) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int groups = n >> 3;
-    const int f0 = (int)(idx % groups) * 8;
-    const int slice = (int)(idx / groups);
-    if (slice >= sp[E]) return;
-    int lo = 0, hi = E;                                 // the expert whose slices hold `slice`: largest e with sp[e] <= slice
-    while (hi - lo > 1) {                               // (experts without rows share their successor's prefix)
-        const int mid = (lo + hi) >> 1;
-        if (sp[mid] <= slice) lo = mid; else hi = mid;
-    }
-    const int e = lo;
-    const int n_e = offsets[e + 1] - offsets[e];
-    const long long ld16 = ld >> 3;
-    uint32_t words[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) words[q] = 0u;
-#pragma unroll 1
-    for (int blk = 0; blk < 4; ++blk) {
-        const int local_block = 4 * (slice - sp[e]) + blk;
-        const long long pb = 4ll * slice + blk;         // padded block of 32 rows
-        const int valid = max(0, min(32, n_e - 32 * local_block));
-        const uint4* src = reinterpret_cast<const uint4*>(x + ((long long)offsets[e] + 32ll * local_block) * ld + col0 + f0);
-        uint4 raw[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) raw[j] = j < valid ? __ldg(src + (long long)j * ld16) : make_uint4(0u, 0u, 0u, 0u);
-        float amax[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) amax[q] = 0.f;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw[j]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[q]));
-                amax[2 * q] = fmaxf(amax[2 * q], fabsf(v.x));
-                amax[2 * q + 1] = fmaxf(amax[2 * q + 1], fabsf(v.y));
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int se = mx_scale_exp(amax[q]);
-            const float inv = mx_inv_scale(se);
-            uint32_t out[8];
-#pragma unroll
-            for (int g = 0; g < 8; ++g) {      // rows 4g .. 4g+3 of feature f0 + q
-                float v[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const uint32_t w = reinterpret_cast<const uint32_t*>(&raw[4 * g + t])[q >> 1];
-                    v[t] = __uint_as_float((q & 1) ? (w & 0xffff0000u) : (w << 16));      // bf16 -> fp32 is a shift
-                }
-                out[g] = mx_e4m3x2(v[0] * inv, v[1] * inv) | (mx_e4m3x2(v[2] * inv, v[3] * inv) << 16);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(codes_t + (long long)(f0 + q) * pitch + pb * 32);
-            dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-            dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
-            words[q] |= (uint32_t)(se + 127) << (8 * blk);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int f = f0 + q;
-        *reinterpret_cast<uint32_t*>(sa_words + ((long long)slice * n + f) * 4) = words[q];
-        const int nt = f / MXP_NT, c = f % MXP_NT;
-        *reinterpret_cast<uint32_t*>(sb_atoms + ((long long)nt * (pitch >> 7) + slice) * 1024 + (c >> 7) * 512 + (c % 32) * 16 +
-                                     ((c % 128) / 32) * 4) = words[q];
+    if (mine[2] == 0) return;   // past the last slice
+    mx_transpose_quantize_tile(x + (long long)mine[0] * ld + col0 + f0, ld, mine[1], codes_t + (long long)f0 * pitch + slice * 128ll, pitch,
+                               tile, sf);
+    if (tid < 128) {
+        const uint32_t* words = reinterpret_cast<const uint32_t*>(sf);
+        sa_words[(long long)slice * n + f0 + tid] = words[tid];
+        mx_store_weight_scales(words, f0, nullptr, sb_atoms + slice * 1024ll, (pitch >> 7) * 1024, tid);
     }
 }
 
@@ -1188,15 +1188,10 @@ size_t mx_w_scale_bytes(int E, int n_feat, int k) {
     return mx_w_scale_single_bytes(E, n_feat, k) + (size_t)E * ((n_feat + MXP_NT - 1) / MXP_NT) * (k / 128) * 1024;
 }
 
-static unsigned mx_row_quantiser_blocks(long long units) {
-    long long blocks = (units + 63) / 64;   // 8 warps x 8 units per block and pass
-    const long long cap = (long long)sm_count() * 16;
-    if (blocks > cap) blocks = cap;
-    return (unsigned)(blocks < 1 ? 1 : blocks);
-}
+static unsigned mx_row_quantiser_blocks(long long rows, int k) { return (unsigned)((rows + 127) / 128 * (k / 128)); }
 
 int launch_mx_quantize_rows(long long rows, int n, const bf16* x, uint8_t* codes, uint8_t* scales, cudaStream_t s) {
-    mx_quantize_rows_kernel<false><<<mx_row_quantiser_blocks(rows * (n / 128)), 256, 0, s>>>(
+    mx_quantize_rows_kernel<false><<<mx_row_quantiser_blocks(rows, n), 256, 0, s>>>(
         reinterpret_cast<const uint4*>(x), rows, n, 0, n / 128, 0, reinterpret_cast<uint2*>(codes), scales, nullptr);
     return check_launch();
 }
@@ -1204,9 +1199,9 @@ int launch_mx_quantize_rows(long long rows, int n, const bf16* x, uint8_t* codes
 // w [E, k, n] -> rows [n_off, n_off + n) of the transposed codes [E, n_total, k] and the matching scale bytes
 int launch_mx_quantize_w_transposed(int E, int k, int n, int n_total, int n_off, const bf16* w, uint8_t* codes_t, uint8_t* scales,
                                     cudaStream_t s) {
-    const long long total = (long long)E * (k / 32) * n;
-    mx_quantize_w_transposed_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-        w, E, k, n, n_total, n_off, codes_t, scales, scales + mx_w_scale_single_bytes(E, n_total, k));
+    const long long blocks = (long long)E * (k / 128) * (n / 128);
+    mx_quantize_w_transposed_kernel<<<(unsigned)blocks, 256, 0, s>>>(w, k, n, n_total, n_off, codes_t, scales,
+                                                                     scales + mx_w_scale_single_bytes(E, n_total, k));
     return check_launch();
 }
 
@@ -1235,7 +1230,7 @@ int launch_mx_swiglu_bwd_quantize(long long rows, int I, const bf16* dh_act, con
 int launch_mx_quantize_w_rows(int E, int n_feat, int k, int k_total, int k_off, const bf16* w, uint8_t* codes, uint8_t* scales,
                               cudaStream_t s) {
     const long long rows = (long long)E * n_feat;
-    mx_quantize_rows_kernel<true><<<mx_row_quantiser_blocks(rows * (k / 128)), 256, 0, s>>>(
+    mx_quantize_rows_kernel<true><<<mx_row_quantiser_blocks(rows, k), 256, 0, s>>>(
         reinterpret_cast<const uint4*>(w), rows, k, n_feat, k_total / 128, k_off / 128, reinterpret_cast<uint2*>(codes), scales,
         scales + mx_w_scale_single_bytes(E, n_feat, k_total));
     return check_launch();
@@ -1255,11 +1250,9 @@ int launch_mx_quantize_tokens(long long R, int E, const bf16* x, long long ld, i
     int32_t* sp = reinterpret_cast<int32_t*>(scales);
     uint8_t* sa = scales + MX_TOKENS_HEADER_BYTES;
     uint8_t* sb = sa + (size_t)(pitch / 128) * n * 4;
-    mx_slice_prefix_kernel<<<1, 1024, 0, s>>>(offsets, E, sp);
-    int st_ = check_launch();
-    if (st_ != MOE_OK) return st_;
-    const long long total = (pitch / 128) * (n / 8);
-    mx_quantize_tokens_kernel<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(x, ld, col0, n, offsets, sp, E, pitch, codes_t, sa, sb);
+    const long long blocks = (pitch / 128) * (n / 128);
+    mx_quantize_tokens_kernel<<<(unsigned)blocks, 256, 0, s>>>(x, ld, col0, n, offsets, sp, E, pitch, codes_t,
+                                                               reinterpret_cast<uint32_t*>(sa), sb);
     return check_launch();
 }
 

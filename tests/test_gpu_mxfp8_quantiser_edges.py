@@ -1,0 +1,68 @@
+"""Edges of the block-scaled FP8 quantisers that the layer's own values do not reach: infinities, NaN, subnormals and signed
+zeros, and the token-axis quantiser's scan over the experts at its smallest and largest expert counts.  Codes and scale
+bytes are whole numbers and compared bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import moe_oracle as O
+from paper_2606_26453_b200 import workloads as W
+from tests import helpers as Hh
+from tests.test_gpu_mxfp8 import _act_scales_from_layout, _oracle_tokens_layout
+
+pytestmark = pytest.mark.gpu
+
+
+def _u8(n):
+    return torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("rows", [1, 127, 129])
+def test_special_values(rows):
+    """A NaN takes no part in its block's scale and keeps a NaN code; an infinity gives the largest scale and saturates."""
+    from paper_2606_26453_b200 import binding as B
+    n, r = 256, rows - 1
+    x = W.round_to_bf16(np.random.default_rng(rows).standard_normal((rows, n)).astype(np.float32))
+    x[r, 0:32] = -0.0
+    x[r, 32:64] = np.linspace(-31, 31, 32, dtype=np.float32) * 2.0 ** -133       # subnormal bf16 values
+    finite = x.copy()
+    x[r, 70] = np.nan                                                           # one NaN among numbers
+    x[r, 96:128] = np.nan                                                       # nothing but NaN
+    x[r, 130], x[r, 131] = np.inf, -np.inf
+    finite[r, 70], finite[r, 96:128], finite[r, 128:160] = 0.0, 0.0, 0.0
+    codes, scales, _ = O.mxfp8_quantize(finite)
+    codes[r, 70], codes[r, 96:128] = 0x7F, 0x7F
+    codes[r, 128:160] = np.where(np.signbit(x[r, 128:160]), 0x80, 0)            # any finite value over 2^120
+    codes[r, 130], codes[r, 131] = 0x7E, 0xFE
+    scales[r, 4] = 120 + 127
+    d = B.dims(rows, 128, n, 1, 1)
+    c, s = _u8(rows * n), _u8(B.moe_mxfp8_act_scale_bytes(d))
+    B.moe_mxfp8_quantize_h_act(d, Hh.to_dev_bf16(x), c, s)
+    torch.cuda.synchronize()
+    got = c.cpu().numpy().reshape(rows, n)
+    nan = np.isnan(x)
+    assert np.array_equal(np.where(nan, got & 0x7F, got), codes)                # the sign of a NaN is nobody's
+    assert np.array_equal(_act_scales_from_layout(s.cpu().numpy(), rows, n), scales)
+
+
+@pytest.mark.parametrize("E", [1, 2, 127, 1023, 1024])
+def test_token_quantiser_expert_scan(E):
+    from paper_2606_26453_b200 import binding as B
+    rng = np.random.default_rng(E)
+    counts = rng.integers(0, 3, size=E)
+    counts[rng.integers(0, E)] = 129
+    counts[-1] = 31
+    offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    R, ld, col0, n = int(offsets[-1]), 384, 8, 256
+    x = W.round_to_bf16(rng.standard_normal((R, ld)).astype(np.float32))
+    d = B.dims(R, 128, 128, E, 1)
+    P = ((R + 127) // 128) * 128 + 128 * E
+    codes, scales = _u8(B.moe_mxfp8_tokens_codes_bytes(d, n)), _u8(B.moe_mxfp8_tokens_scale_bytes(d, n))
+    B.moe_mxfp8_quantize_tokens(d, Hh.to_dev_bf16(x), ld, col0, n, torch.from_numpy(offsets).cuda(), codes, scales)
+    torch.cuda.synchronize()
+    want_codes, want_scales, sp = _oracle_tokens_layout(x[:, col0:col0 + n], offsets)
+    n_sl = int(sp[-1])
+    assert np.array_equal(scales[:4 * (E + 1)].cpu().numpy().view(np.int32), sp.astype(np.int32))
+    assert np.array_equal(codes.view(n, P)[:, :n_sl * 128].cpu().numpy(), want_codes)
+    words = scales[8192: 8192 + (P // 128) * n * 4].view(P // 128, n, 4)[:n_sl].cpu().numpy()
+    assert np.array_equal(words, want_scales)
