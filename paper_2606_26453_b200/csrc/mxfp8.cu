@@ -23,15 +23,16 @@
 //                      column = (f % 128) / 32, byte = block); then the same bytes in the tiling of the CTA-pair kernel
 //                      (see there)
 //
-// Single-CTA kernel: one CTA per SM, persistent over the same row-ragged tile list as the bf16 kernels (tiles of 128 rows x
-// 128 output features), K slices of 128 (= 128 bytes per row: the same swizzled stage geometry as 64 bf16).
+// Single-CTA kernel: one or two CTAs per SM, persistent over the same row-ragged tile list as the bf16 kernels (tiles of 128 or
+// 64 rows x 128 output features), K slices of 128 (= 128 bytes per row: the same swizzled stage geometry as 64 bf16).
 //   warp 0      TMA producer: A and B code tiles, bulk copy of the weight-scale block
-//   warp 1      one thread: tcgen05.cp of both scale blocks into tensor memory, four tcgen05.mma (K = 32 each, scale
-//               byte k selected through the instruction descriptor), commit
+//   warp 1      one thread: four tcgen05.mma (K = 32 each, scale byte k selected through the instruction descriptor), commit
 //   warp 2      activation scales: gathers the tile's 128 words of the K slice and writes them in the copy's pattern
 //   warps 3..6  epilogue: tcgen05.ld, round to bf16, staged bulk tensor stores
-// Accumulator double buffered (2 x 128 columns); the scale blocks of a stage use 8 tensor-memory columns, two such
-// slots alternate (copies and MMAs of one thread execute in issue order).
+//   warp 7      one thread: tcgen05.cp of both scale blocks of a stage into tensor memory (with them the MMA thread took ~750
+//               cycles per K slice, without ~580 of which it waits 110; that is fast enough for the weights to come at HBM rate)
+// Accumulator double buffered; the scale blocks of a ring stage have 8 tensor-memory columns of their own.  Two forms of
+// the kernel, see MxGeo.
 #include <cuda_fp8.h>
 
 #include "tc_ptx.cuh"
@@ -59,36 +60,53 @@ int mx_read_and_clear_status(int* status_out) {
 
 namespace {
 
-constexpr int MX_BM = 128, MX_BN = 128, MX_BK = 128;   // tile rows, tile columns, contraction elements per stage
-constexpr int MX_STAGES = 6;
-constexpr int MX_A_BYTES = MX_BM * MX_BK, MX_B_BYTES = MX_BN * MX_BK, MX_SF_BYTES = 512;
-constexpr int MX_STAGE_BYTES = MX_A_BYTES + MX_B_BYTES + 2 * MX_SF_BYTES;   // 33 KB
+constexpr int MX_BM = 128, MX_BN = 128, MX_BK = 128;   // rows of a pair CTA's tile, features of a single-CTA tile, contraction elements per stage
+constexpr int MX_MAX_STAGES = 6;
+constexpr int MX_W_BYTES = MX_BN * MX_BK, MX_SF_BYTES = 512;
 constexpr int MX_EPI_WARPS = 4;
-constexpr int MX_THREADS = 32 * (3 + MX_EPI_WARPS);
+constexpr int MX_COPY_WARP = 3 + MX_EPI_WARPS;   // the scale-copy warp comes after the epilogue warps
+constexpr int MX_THREADS = 32 * (4 + MX_EPI_WARPS);
 constexpr int MX_STAGING_BYTES = MX_EPI_WARPS * 2048;
 constexpr int MX_MAX_E = 1024;
 constexpr int MX_TMEM_COLS = 512;
 constexpr int MX_SCALE_AHEAD = 4;   // K slices whose activation-scale words the scale warp keeps in flight
-constexpr int MX_SF_COL0 = 2 * MX_BN;   // first tensor-memory column of the scale slots (after the two accumulators)
-
 struct MxCtl {
-    unsigned long long full[MX_STAGES];
-    unsigned long long empty[MX_STAGES];
+    unsigned long long full[MX_MAX_STAGES];
+    unsigned long long sf_full[MX_MAX_STAGES];   // the stage's scales are in tensor memory (and its operands landed)
+    unsigned long long empty[MX_MAX_STAGES];
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     unsigned long long drain;
+    unsigned long long drain_copy;
     uint32_t tmem_base;
     int abort_flag;
-    int32_t offs[MX_MAX_E + 1];
-    int32_t tile_prefix[MX_MAX_E + 1];
+    // followed by int32_t offs[E + 1], tile_prefix[E + 1]
 };
-constexpr int MX_SMEM_BYTES = MX_STAGES * MX_STAGE_BYTES + MX_STAGING_BYTES + 1024 + (int)sizeof(MxCtl);
-static_assert(MX_SMEM_BYTES <= 232448, "exceeds the shared memory a CTA can opt in to");
+// The two forms of the single-CTA kernel, by the most rows of a tile (which of them runs: launch_mx_gemm).
+//   128  rows on the M side of the MMA, 128 output features on the N side; one CTA per SM.
+//   64   operand roles swapped: 128 output features on the M side, 64 rows on the N side, so that no stage carries rows of
+//        other experts and both accumulators take 128 tensor-memory columns together; two CTAs per SM.
+template <int ROWS>
+struct MxGeo {
+    static constexpr bool SWAPPED = ROWS < MX_BM;
+    static constexpr int CTAS = SWAPPED ? 2 : 1;                // per SM
+    static constexpr int STAGES = SWAPPED ? 4 : 6;
+    static constexpr int TMEM_COLS = 512 / CTAS;
+    static constexpr int SF_COL0 = 2 * ROWS;                    // scale slots after the two accumulators, 8 columns per stage
+    static constexpr int X_BYTES = ROWS * MX_BK;
+    static constexpr int SFX_OFF = MX_W_BYTES + X_BYTES, SFW_OFF = SFX_OFF + MX_SF_BYTES;
+    static constexpr int STAGE_BYTES = SFW_OFF + MX_SF_BYTES;   // 25 KB, 33 KB
+    static int smem_bytes(int E) {
+        return STAGES * STAGE_BYTES + MX_STAGING_BYTES + 1024 + (int)sizeof(MxCtl) + 2 * (E + 1) * (int)sizeof(int32_t);
+    }
+    static_assert(STAGES <= MX_MAX_STAGES && STAGE_BYTES % 1024 == 0 && SF_COL0 + STAGES * 8 <= TMEM_COLS, "stage layout");
+};
 
 struct MxParams {
     const int32_t* offsets;
     int E, k_tiles, n_tiles, n_cols;
     long long R;
+    uint32_t x_bytes;     // that one load of activation codes delivers
     const uint32_t* sa;   // activation scale words [k_tiles][R]
     const uint8_t* sb;    // weight scale blocks [E][n_tiles][k_tiles][512]
     bf16* out;
@@ -111,8 +129,9 @@ __device__ __forceinline__ uint64_t mx_scale_desc(uint32_t addr) {
 }
 // Instruction descriptor of the block-scaled kind: E4M3 x E4M3, both K-major, E8M0 scales, scale byte `sf` of the
 // scale columns for both operands.
-__device__ __forceinline__ uint32_t mx_idesc(uint32_t sf) {
-    return (sf << 4) | ((uint32_t)(MX_BN >> 3) << 17) | (1u << 23) | ((uint32_t)(MX_BM >> 4) << 24) | (sf << 29);
+template <int ROWS>
+__device__ __forceinline__ uint32_t mx_idesc(uint32_t sf) {   // M = 128, N = ROWS (128 features are as many as 128 rows)
+    return (sf << 4) | ((uint32_t)(ROWS >> 3) << 17) | (1u << 23) | ((uint32_t)(MX_BN >> 4) << 24) | (sf << 29);
 }
 __device__ __forceinline__ void mx_copy_scales(uint32_t taddr, uint64_t sdesc) {
     asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
@@ -129,38 +148,45 @@ __device__ __forceinline__ void mx_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
 struct MxTile {
     int e, row0, row_end, n0;
 };
-__device__ __forceinline__ MxTile mx_decode(const MxParams& p, const MxCtl* ctl, long long t) {
+template <int ROWS>
+__device__ __forceinline__ MxTile mx_decode(const MxParams& p, const int32_t* offs, const int32_t* tile_prefix, long long t) {
     int lo = 0, hi = p.E;   // largest e with tile_prefix[e] * n_tiles <= t
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if ((long long)ctl->tile_prefix[mid] * p.n_tiles <= t) lo = mid; else hi = mid;
+        if ((long long)tile_prefix[mid] * p.n_tiles <= t) lo = mid; else hi = mid;
     }
-    const int local = (int)(t - (long long)ctl->tile_prefix[lo] * p.n_tiles);
-    const int m_tiles_e = ctl->tile_prefix[lo + 1] - ctl->tile_prefix[lo];
+    const int local = (int)(t - (long long)tile_prefix[lo] * p.n_tiles);
+    const int m_tiles_e = tile_prefix[lo + 1] - tile_prefix[lo];
     MxTile tl;
     tl.e = lo;
     // column tile major inside an expert: the CTAs that run at the same time share the expert's weight tiles in L2
     const int nt = local / m_tiles_e, mt = local - nt * m_tiles_e;
-    tl.row0 = ctl->offs[lo] + mt * MX_BM;
-    tl.row_end = ctl->offs[lo + 1];
+    tl.row0 = offs[lo] + mt * ROWS;
+    tl.row_end = min(offs[lo + 1], tl.row0 + ROWS);
     tl.n0 = nt * MX_BN;
     return tl;
 }
 
-__global__ void __launch_bounds__(MX_THREADS, 1)
+template <int ROWS>
+__global__ void __launch_bounds__(MX_THREADS, MxGeo<ROWS>::CTAS)
 mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_o, const MxParams p) {
+    using G = MxGeo<ROWS>;
+    constexpr int MX_STAGES = G::STAGES, MX_STAGE_BYTES = G::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* tiles_ptr = smem_raw + (tiles_base - smem_u32(smem_raw));
     MxCtl* ctl = reinterpret_cast<MxCtl*>(tiles_ptr + MX_STAGES * MX_STAGE_BYTES + MX_STAGING_BYTES);
+    int32_t* offs = reinterpret_cast<int32_t*>(ctl + 1);   // sized by E: two CTAs have to fit an SM
+    int32_t* tile_prefix = offs + p.E + 1;
     volatile int* abort_flag = &ctl->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    for (int e = threadIdx.x; e <= p.E; e += MX_THREADS) ctl->offs[e] = p.offsets[e];
+    for (int e = threadIdx.x; e <= p.E; e += MX_THREADS) offs[e] = p.offsets[e];
     if (threadIdx.x == 0) {
         for (int s = 0; s < MX_STAGES; ++s) {
             mbar_init(smem_u32(&ctl->full[s]), 2);    // the producer's arrive (with the byte count) + the scale warp's
+            mbar_init(smem_u32(&ctl->sf_full[s]), 1);
             mbar_init(smem_u32(&ctl->empty[s]), 1);
         }
         for (int a = 0; a < 2; ++a) {
@@ -168,6 +194,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             mbar_init(smem_u32(&ctl->tmem_empty[a]), MX_EPI_WARPS);
         }
         mbar_init(smem_u32(&ctl->drain), 1);
+        mbar_init(smem_u32(&ctl->drain_copy), 1);
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tmap(&map_a);
@@ -178,14 +205,14 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (threadIdx.x == 0) {
         int run = 0;
         for (int e = 0; e < p.E; ++e) {
-            ctl->tile_prefix[e] = run;
-            run += (ctl->offs[e + 1] - ctl->offs[e] + MX_BM - 1) / MX_BM;
+            tile_prefix[e] = run;
+            run += (offs[e + 1] - offs[e] + ROWS - 1) / ROWS;
         }
-        ctl->tile_prefix[p.E] = run;
+        tile_prefix[p.E] = run;
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
-                     "r"((uint32_t)MX_TMEM_COLS)
+                     "r"((uint32_t)G::TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -193,7 +220,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    const long long n_tiles_total = (long long)ctl->tile_prefix[p.E] * p.n_tiles;
+    const long long n_tiles_total = (long long)tile_prefix[p.E] * p.n_tiles;
     auto stage_base = [&](uint32_t s) { return tiles_base + s * MX_STAGE_BYTES; };
 
     if (warp == 0) {
@@ -202,7 +229,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             uint32_t stage = 0, phase = 0, issued = 0;
             bool ok = true;
             for (long long t = blockIdx.x; ok && t < n_tiles_total; t += gridDim.x) {
-                const MxTile tl = mx_decode(p, ctl, t);
+                const MxTile tl = mx_decode<ROWS>(p, offs, tile_prefix, t);
                 const uint8_t* sb_tile = p.sb + ((long long)tl.e * p.n_tiles + tl.n0 / MX_BN) * p.k_tiles * MX_SF_BYTES;
                 for (int kt = 0; kt < p.k_tiles; ++kt) {
                     if (!mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -215,11 +242,11 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #endif
                     const uint32_t full = smem_u32(&ctl->full[stage]);
                     const uint32_t a_dst = stage_base(stage);
-                    mbar_arrive_expect_tx(full, MX_A_BYTES + MX_B_BYTES + MX_SF_BYTES);
-                    tma_load_2d(a_dst, &map_a, kt * MX_BK, tl.row0, full);
-                    tma_load_2d(a_dst + MX_A_BYTES, &map_b, kt * MX_BK, tl.e * p.n_cols + tl.n0, full);
+                    mbar_arrive_expect_tx(full, MX_W_BYTES + p.x_bytes + MX_SF_BYTES);
+                    tma_load_2d(a_dst, &map_b, kt * MX_BK, tl.e * p.n_cols + tl.n0, full);
+                    tma_load_2d(a_dst + MX_W_BYTES, &map_a, kt * MX_BK, tl.row0, full);
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                     a_dst + MX_A_BYTES + MX_B_BYTES + MX_SF_BYTES),
+                                     a_dst + G::SFW_OFF),
                                  "l"(sb_tile + (long long)kt * MX_SF_BYTES), "r"(MX_SF_BYTES), "r"(full)
                                  : "memory");
                     ++issued;
@@ -239,33 +266,31 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     } else if (warp == 1) {
         // ================= MMA issuer: one thread =================
         if (lane == 0) {
-            uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0, slot = 0;
+            uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
             for (long long t = blockIdx.x; ok && t < n_tiles_total; t += gridDim.x) {
                 if (!mx_wait(smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag)) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * MX_BN;
+                const uint32_t d_tmem = tmem_base + acc * ROWS;
                 for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    if (!mx_wait(smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
+                    if (!mx_wait(smem_u32(&ctl->sf_full[stage]), phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a_base = stage_base(stage);
-                    const uint32_t sfa_t = tmem_base + MX_SF_COL0 + slot * 8, sfb_t = sfa_t + 4;
-                    mx_copy_scales(sfa_t, mx_scale_desc(a_base + MX_A_BYTES + MX_B_BYTES));
-                    mx_copy_scales(sfb_t, mx_scale_desc(a_base + MX_A_BYTES + MX_B_BYTES + MX_SF_BYTES));
-                    const uint64_t a_desc = mx_operand_desc(a_base), b_desc = mx_operand_desc(a_base + MX_A_BYTES);
+                    const uint32_t sfw_t = tmem_base + G::SF_COL0 + stage * 8, sfx_t = sfw_t + 4;
+                    const uint64_t w_desc = mx_operand_desc(a_base), x_desc = mx_operand_desc(a_base + MX_W_BYTES);
 #pragma unroll
                     for (int k = 0; k < MX_BK / 32; ++k)
-                        mx_mma(d_tmem, a_desc + (uint64_t)((k * 32) >> 4), b_desc + (uint64_t)((k * 32) >> 4), mx_idesc(k), sfa_t,
-                               sfb_t, (kt != 0 || k != 0) ? 1u : 0u);
+                        mx_mma(d_tmem, (G::SWAPPED ? w_desc : x_desc) + (uint64_t)((k * 32) >> 4),
+                               (G::SWAPPED ? x_desc : w_desc) + (uint64_t)((k * 32) >> 4), mx_idesc<ROWS>(k), G::SWAPPED ? sfw_t : sfx_t,
+                               G::SWAPPED ? sfx_t : sfw_t, (kt != 0 || k != 0) ? 1u : 0u);
                     tc_commit<false>(smem_u32(&ctl->empty[stage]));
-                    slot ^= 1u;
                     if (++stage == MX_STAGES) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
                 tc_commit<false>(smem_u32(&ctl->tmem_full[acc]));
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            // all issued copies and MMAs must have retired before tensor memory is released
+            // all issued MMAs must have retired before tensor memory is released
             tc_commit_local<false>(smem_u32(&ctl->drain));
             const unsigned long long t0 = global_timer_ns();
             while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < WAIT_LIMIT_NS) {}
@@ -277,7 +302,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t stage = 0, phase = 0;
         bool ok = true;
         for (long long t = blockIdx.x; ok && t < n_tiles_total; t += gridDim.x) {
-            const MxTile tl = mx_decode(p, ctl, t);
+            const MxTile tl = mx_decode<ROWS>(p, offs, tile_prefix, t);
             long long rows[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -288,7 +313,10 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             // bound the whole pipeline (the loads wait behind the operand traffic)
             auto load_slice = [&](int kt) {
                 const uint32_t* s = p.sa + (long long)kt * p.R;
-                return make_uint4(__ldg(s + rows[0]), __ldg(s + rows[1]), __ldg(s + rows[2]), __ldg(s + rows[3]));
+                uint4 w = make_uint4(__ldg(s + rows[0]), 0u, 0u, 0u);
+                if (ROWS > 32) w.y = __ldg(s + rows[1]);
+                if (ROWS > 64) { w.z = __ldg(s + rows[2]); w.w = __ldg(s + rows[3]); }
+                return w;
             };
             uint4 q[MX_SCALE_AHEAD];
 #pragma unroll
@@ -301,7 +329,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     const uint4 cur = q[i];
                     if (kt + MX_SCALE_AHEAD < p.k_tiles) q[i] = load_slice(kt + MX_SCALE_AHEAD);
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag))) { ok = false; break; }
-                    *reinterpret_cast<uint4*>(tiles_ptr + stage * MX_STAGE_BYTES + MX_A_BYTES + MX_B_BYTES + lane * 16) = cur;
+                    *reinterpret_cast<uint4*>(tiles_ptr + stage * MX_STAGE_BYTES + G::SFX_OFF + lane * 16) = cur;
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&ctl->full[stage]));
@@ -309,48 +337,94 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 }
             }
         }
+    } else if (warp == MX_COPY_WARP) {
+        // ================= scale copies: one thread =================
+        // Every ring stage has its own scale slot in tensor memory (as in the pair kernel): full[stage] can only complete
+        // after the MMAs that read the slot's previous contents have.
+        if (lane == 0) {
+            uint32_t stage = 0, phase = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; ok && t < n_tiles_total; t += gridDim.x) {
+                for (int kt = 0; kt < p.k_tiles; ++kt) {
+                    if (!mx_wait(smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t sfw_t = tmem_base + G::SF_COL0 + stage * 8;
+                    mx_copy_scales(sfw_t, mx_scale_desc(stage_base(stage) + G::SFW_OFF));
+                    mx_copy_scales(sfw_t + 4, mx_scale_desc(stage_base(stage) + G::SFX_OFF));
+                    tc_commit_local<false>(smem_u32(&ctl->sf_full[stage]));
+                    if (++stage == MX_STAGES) { stage = 0; phase ^= 1u; }
+                }
+            }
+            // all issued copies must have retired before tensor memory is released
+            tc_commit_local<false>(smem_u32(&ctl->drain_copy));
+            const unsigned long long t0 = global_timer_ns();
+            while (!mbar_try_wait(smem_u32(&ctl->drain_copy), 0) && global_timer_ns() - t0 < WAIT_LIMIT_NS) {}
+        }
+        __syncwarp();
     } else {
         // ================= epilogue (warps 3..6) =================
+        // A full block of 32 rows x 32 features goes through the warp's staging buffer and leaves as a bulk tensor store; of a
+        // block that the expert only partly fills the rows are stored directly.
+        //   not swapped  lane = row, tensor-memory column = feature: the warp has one slab of 32 rows and all features
+        //   swapped      lane = feature, column = row: the warp has 32 features and all rows; the block is transposed on its
+        //                way into the staging buffer (2-byte stores, 64 contiguous bytes per warp instruction)
         const int quarter = warp & 3;   // tensor-memory lanes [32 * quarter, 32 * quarter + 32)
-        uint8_t* stage_ptr = tiles_ptr + MX_STAGES * MX_STAGE_BYTES + (warp - 3) * 2048;
-        const int sw = (lane >> 1) & 3;
+        uint8_t* stage_ptr = tiles_ptr + MX_STAGES * MX_STAGE_BYTES + quarter * 2048;
+        const int sw = (lane >> 1) & 3, piece = lane >> 3, within = (lane & 7) * 2;
         uint32_t n_stores = 0, acc = 0, acc_phase = 0;
         for (long long t = blockIdx.x; t < n_tiles_total; t += gridDim.x) {
-            const MxTile tl = mx_decode(p, ctl, t);
+            const MxTile tl = mx_decode<ROWS>(p, offs, tile_prefix, t);
             if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag))) break;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + acc * MX_BN + ((uint32_t)(quarter * 32) << 16);
-            const int slab0 = tl.row0 + quarter * 32;
-            const int rows_valid = max(0, min(32, tl.row_end - slab0));
+            const uint32_t taddr = tmem_base + acc * ROWS + ((uint32_t)(quarter * 32) << 16);
+            const int n_rows = tl.row_end - tl.row0;
 #pragma unroll 1
-            for (int c = 0; c < MX_BN / 32; ++c) {
+            for (int c = 0; c < ROWS / 32; ++c) {   // the warp's blocks
+                const int r = (G::SWAPPED ? c : quarter) * 32, f = tl.n0 + (G::SWAPPED ? quarter : c) * 32;
+                const int rv = min(32, n_rows - r);
+                if (rv <= 0) break;
                 uint32_t v[32];
                 tc_ld32(taddr + c * 32, v);
                 tc_wait_ld();
-                const int n = tl.n0 + c * 32;
-                if (rows_valid == 0 || n >= p.n_cols) continue;
-                uint32_t w[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) w[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-                if (rows_valid == 32) {
+                if (rv == 32) {
                     if (n_stores != 0) {
                         if (lane == 0) bulk_wait_read0();
                         __syncwarp();
                     }
+                    if (G::SWAPPED) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        *reinterpret_cast<uint4*>(stage_ptr + lane * 64 + ((j ^ sw) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+                        for (int j = 0; j < 32; ++j)
+                            *reinterpret_cast<__nv_bfloat16*>(stage_ptr + j * 64 + (((piece ^ ((j >> 1) & 3)) << 4) + within)) =
+                                __float2bfloat16_rn(__uint_as_float(v[j]));
+                    } else {
+                        uint32_t w[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) w[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            *reinterpret_cast<uint4*>(stage_ptr + lane * 64 + ((j ^ sw) << 4)) =
+                                make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+                    }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) {
-                        tma_store_2d(&map_o, n, slab0, smem_u32(stage_ptr));
+                        tma_store_2d(&map_o, f, tl.row0 + r, smem_u32(stage_ptr));
                         bulk_commit();
                     }
                     ++n_stores;
-                } else if (lane < rows_valid) {
-                    uint4* d4 = reinterpret_cast<uint4*>(p.out + ((long long)slab0 + lane) * p.ldo + n);
+                } else if (G::SWAPPED) {
+                    bf16* dst = p.out + ((long long)tl.row0 + r) * p.ldo + f + lane;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) d4[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+                    for (int j = 0; j < 32; ++j)
+                        if (j < rv) dst[(long long)j * p.ldo] = __float2bfloat16_rn(__uint_as_float(v[j]));
+                } else if (lane < rv) {
+                    uint4* d4 = reinterpret_cast<uint4*>(p.out + ((long long)tl.row0 + r + lane) * p.ldo + f);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        d4[j] = make_uint4(pack_bf16(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1])),
+                                           pack_bf16(__uint_as_float(v[8 * j + 2]), __uint_as_float(v[8 * j + 3])),
+                                           pack_bf16(__uint_as_float(v[8 * j + 4]), __uint_as_float(v[8 * j + 5])),
+                                           pack_bf16(__uint_as_float(v[8 * j + 6]), __uint_as_float(v[8 * j + 7])));
                 }
             }
             tc_fence_before();
@@ -366,7 +440,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)MX_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)G::TMEM_COLS) : "memory");
     }
 }
 
@@ -1134,7 +1208,7 @@ __global__ void __launch_bounds__(256) mx_quantize_tokens_kernel(const bf16* __r
     __shared__ int32_t part[8];
     __shared__ int32_t mine[3];   // first row, rows and existence of this block's slice
     const int f_tiles = n >> 7;
-    const int f0 = (int)(blockIdx.x % (unsigned)f_tiles) * 128, slice = (int)(blockIdx.x / (unsigned)f_tiles);
+        const int f0 = (int)(blockIdx.x % (unsigned)f_tiles) * 128, slice = (int)(blockIdx.x / (unsigned)f_tiles);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // thread t scans the experts 4t .. 4t + 3
     int32_t off[5], before[4], sum = 0;
@@ -1305,6 +1379,14 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
 
 // CTA pairs from this many rows per expert on average (below it the 256-row tiles are mostly padding)
 constexpr long long kMxPairRows = 256;
+// The swapped form of the single-CTA kernel up to this many rows per expert on average.  There the time is the weights'
+// way from HBM, and what counts is bytes in flight and an even spread over the SMs: two CTAs with four stages of weights
+// and at most 64 rows each, against one with six stages that also hold 128 rows.  Down projection of 8 experts,
+// 14336 x 4096, 25 rows each (event times, cold L2): 92 -> 80 us, gate/up 162 -> 152 us; 37 such experts 351 -> 328 and
+// 715 -> 650 us (6.9 TB/s).  128 experts, 768 x 2048, down projection, rows per expert 32: 47 -> 44 us, 64: 51 -> 47 us,
+// 94: 51 -> 55 us -- a second tile per expert reads the expert's weights again, from L2.  Tiles of 32 rows lost to
+// tiles of 64 everywhere but below 4 rows per expert (N = 32 makes the MMAs no cheaper to issue).
+constexpr long long kMxSwappedRows = 64;
 
 static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
                                const uint8_t* b_codes, const uint8_t* b_scales_pair, const int32_t* offsets, bf16* out,
@@ -1349,6 +1431,42 @@ static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint
     return check_launch();
 }
 
+struct MxSingleArgs {
+    long long R;
+    int E, n_feat, k;
+    const uint8_t *a_codes, *a_scales, *b_codes, *b_scales;
+    const int32_t* offsets;
+    bf16* out;
+};
+template <int ROWS>
+static int launch_mx_gemm_single(const MxSingleArgs& g, cudaStream_t s) {
+    // never a box of more rows than there are: a load that is mostly out of bounds is slow (8 rows of
+    // 14336 against 8 large experts, in boxes of 128 rows: 113 us, of 8 rows: 82 us)
+    const uint32_t box = g.R < ROWS ? (uint32_t)g.R : (uint32_t)ROWS;
+    CUtensorMap a, b, o;
+    if (!make_map_typed(&a, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.a_codes, g.k, (uint64_t)g.R, MX_BK, box, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&b, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.b_codes, g.k, (uint64_t)g.E * g.n_feat, MX_BK, MX_BN,
+                        CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_out_map(&o, g.out, g.n_feat, (uint64_t)g.R))
+        return MOE_ERR_CUDA;
+    MxParams p = {};
+    p.offsets = g.offsets; p.E = g.E; p.k_tiles = g.k / MX_BK; p.n_tiles = g.n_feat / MX_BN; p.n_cols = g.n_feat; p.R = g.R; p.x_bytes = box * MX_BK;
+    p.sa = reinterpret_cast<const uint32_t*>(g.a_scales); p.sb = g.b_scales; p.out = g.out; p.ldo = g.n_feat;
+    static bool attr_set[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
+    if (!attr_set[dev]) {
+        if (cudaFuncSetAttribute(mx_gemm_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, MxGeo<ROWS>::smem_bytes(MX_MAX_E)) !=
+            cudaSuccess)
+            return MOE_ERR_CUDA;
+        attr_set[dev] = true;
+    }
+    const int sms = sm_count();
+    if (sms <= 0) return MOE_ERR_CUDA;
+    mx_gemm_kernel<ROWS><<<MxGeo<ROWS>::CTAS * sms, MX_THREADS, MxGeo<ROWS>::smem_bytes(g.E), s>>>(a, b, o, p);
+    return check_launch();
+}
+
 // out[r, :] = dequant(a row r) . dequant(b[e])^T for the rows r of expert e: a [R, k] codes with scale words
 // [k/128][R], b [E, n_feat, k] codes with both scale tilings, out [R, n_feat] bf16.
 int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* b_codes,
@@ -1356,27 +1474,9 @@ int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes
     if (R >= kMxPairRows * E)
         return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales + mx_w_scale_single_bytes(E, n_feat, k),
                                    offsets, out, s);
-    CUtensorMap a, b, o;
-    if (!make_map_typed(&a, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a_codes, k, (uint64_t)R, MX_BK, MX_BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_typed(&b, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, b_codes, k, (uint64_t)E * n_feat, MX_BK, MX_BN,
-                        CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_out_map(&o, out, n_feat, (uint64_t)R))
-        return MOE_ERR_CUDA;
-    MxParams p = {};
-    p.offsets = offsets; p.E = E; p.k_tiles = k / MX_BK; p.n_tiles = n_feat / MX_BN; p.n_cols = n_feat; p.R = R;
-    p.sa = reinterpret_cast<const uint32_t*>(a_scales); p.sb = b_scales; p.out = out; p.ldo = n_feat;
-    static bool attr_set[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
-    if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(mx_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MX_SMEM_BYTES) != cudaSuccess)
-            return MOE_ERR_CUDA;
-        attr_set[dev] = true;
-    }
-    const int sms = sm_count();
-    if (sms <= 0) return MOE_ERR_CUDA;
-    mx_gemm_kernel<<<sms, MX_THREADS, MX_SMEM_BYTES, s>>>(a, b, o, p);
-    return check_launch();
+    const MxSingleArgs args = {R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out};
+    if (R <= kMxSwappedRows * E) return launch_mx_gemm_single<64>(args, s);
+    return launch_mx_gemm_single<128>(args, s);
 }
 
 }  // namespace moe
