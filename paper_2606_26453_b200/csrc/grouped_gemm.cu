@@ -4,7 +4,7 @@
 // (no host round trip, no extra launch).  Per CTA:
 //   warp 0      TMA producer: cp.async.bulk.tensor loads of 64-wide K blocks of A and B into a
 //               ring of 128-byte-swizzled shared-memory stages, completion on mbarriers
-//   warp 1      MMA issuer: one lane issues tcgen05.mma (bf16 -> fp32) with the accumulator in
+//   warp 1      MMA issuer: one elected lane issues tcgen05.mma (bf16 -> fp32) with the accumulator in
 //               tensor memory; tcgen05.commit releases ring stages and publishes finished
 //               accumulators
 //   warps 2..9  epilogue: tcgen05.ld the accumulator (32-lane quarter x half of the columns), apply
@@ -163,11 +163,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 //   MN-major tile [chunk][64 k-rows][64 mn]: 8-k-row groups 1024 B apart (stride byte offset),
 //                 64-wide mn chunks CHUNK_BYTES apart (leading byte offset)
 template <bool MN_MAJOR>
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr) {
-    const uint64_t lbo = MN_MAJOR ? (uint64_t)(CHUNK_BYTES >> 4) : 1ull;
-    const uint64_t sbo = 1024 >> 4;
-    return (uint64_t)((addr >> 4) & 0x3FFF) | (lbo << 16) | (sbo << 32) | (1ull << 46) | (2ull << 61);
+__device__ __forceinline__ uint32_t make_smem_desc(uint32_t addr) {   // the low word; the high word is SMEM_DESC_HI
+    return ((addr >> 4) & 0x3FFF) | ((MN_MAJOR ? (uint32_t)(CHUNK_BYTES >> 4) : 1u) << 16);
 }
+constexpr uint32_t SMEM_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 // Instruction descriptor: fp32 accumulate, bf16 x bf16, given M (128, or 256 over a CTA pair), N and
 // operand major-ness.
 __host__ __device__ constexpr uint32_t make_idesc(int m, int n, bool a_mn, bool b_mn) {
@@ -224,6 +223,13 @@ template <int KIND>
 __device__ __forceinline__ long long total_tiles(const Params& p, const SharedCtl* ctl) {
     if (wgrad(KIND)) return (long long)p.E * p.m_tiles * p.n_tiles;
     return (long long)ctl->tile_prefix[p.E] * p.n_tiles;
+}
+
+// every field the same in all lanes, and known to the compiler to be
+__device__ __forceinline__ void make_uniform(Tile& tl) {
+    auto uni = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };
+    tl.e = uni(tl.e); tl.row0 = uni(tl.row0); tl.n0 = uni(tl.n0); tl.k_blocks = uni(tl.k_blocks);
+    tl.k_row0 = uni(tl.k_row0); tl.k_rows = uni(tl.k_rows); tl.rows = uni(tl.rows); tl.half = uni(tl.half);
 }
 
 template <int KIND, int TILE_M>
@@ -411,7 +417,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     SharedCtl* ctl = reinterpret_cast<SharedCtl*>(tiles_ptr + G::RING_BYTES + G::STAGING_BYTES);
     volatile int* abort_flag = &ctl->abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;          // 0 = the CTA that issues the MMAs
     const long long first_tile = PAIR ? (long long)(blockIdx.x >> 1) : (long long)blockIdx.x;
     const long long tile_stride = PAIR ? (long long)(gridDim.x >> 1) : (long long)gridDim.x;
@@ -479,8 +485,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     __syncthreads();
     if (PAIR) cluster_sync_all();   // the other CTA's barriers and tensor memory exist from here on
     tc_fence_after();
-    const uint32_t tmem_base = ctl->tmem_base;
-    const long long n_tiles_total = total_tiles<KIND>(p, ctl);
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, ctl->tmem_base, 0);
+    const long long n_tiles_total = __shfl_sync(0xffffffffu, total_tiles<KIND>(p, ctl), 0);
 
     if (warp == 0) {
         // ================= TMA producer (both CTAs of a pair; each fills its own ring) =================
@@ -489,7 +495,13 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         // a stage travels producer -> loads -> MMA with no relay hop.  Only a weight-gradient stage whose ragged last
         // K block needs surplus rows cleared reports to this CTA's landed[stage]; the tail-fix / relay warp clears the
         // rows and makes the arrival on full[stage] in the producer's place.
-        if (lane == 0) {
+        //
+        // The whole warp runs the loop on warp-uniform values and one elected lane issues: the compiler then keeps the
+        // operands of the copies in uniform registers.  Against a loop under `if (lane == 0)` that is worth 3-10 % on the
+        // kernels with short stages (384 rows per expert, gate/up dgrad 230 -> 207 us).  Not for single-CTA weight gradients:
+        // their tiles are one or two stages long, and making a tile's fields uniform costs more than it gives (434 -> 469 us).
+        constexpr bool UNIFORM = PAIR || !wgrad(KIND);
+        if (UNIFORM || lane == 0) {
             uint32_t stage = 0, phase = 0;
             uint32_t issued = 0;
             bool ok = true;
@@ -497,18 +509,19 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             for (long long it = 0; ok; ++it) {
                 const long long t = tile_of<KIND>(it, first_tile, tile_stride, n_tiles_total);
                 if (t < 0) break;
-                const Tile tl = decode_tile<KIND, G::TILE_M>(p, ctl, t);
+                Tile tl = decode_tile<KIND, G::TILE_M>(p, ctl, t);
+                if (UNIFORM) make_uniform(tl);
                 for (int kb = 0; kb < tl.k_blocks; ++kb) {
-                    if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
+                    bool free = mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag);
+                    if (UNIFORM) free = __all_sync(0xffffffffu, free);
+                    if (!free) { ok = false; break; }
                     const bool fix = wgrad(KIND) && kb == tl.k_blocks - 1 && (tl.k_rows & 15) != 0;
                     uint32_t bytes = STAGE_BYTES;
                     if (SWAP) {
-                        ctl->stage_n[stage] = (tl.rows + 15) & ~15;   // read by the MMA thread after its wait on full[stage]
                         const int my_n = PAIR ? (((tl.rows + 15) & ~15) >> 1) : tl.rows;
                         constexpr int BOX = PAIR ? 32 : 64;
                         bytes = G::A_BYTES + min(4, (my_n + BOX - 1) / BOX) * (BOX * BK * 2);
                     } else if (HALF_TILES) {
-                        ctl->stage_half[stage] = tl.half;   // read by the MMA thread after its wait on full[stage]
                         if (tl.half) bytes = STAGE_BYTES - G::A_BYTES / 2;
                     }
                     const uint32_t a_dst = tiles_base + stage * STAGE_BYTES;
@@ -519,17 +532,23 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                         continue;
                     }
 #endif
-                    if (fix) {
-                        const uint32_t land = smem_u32(&ctl->landed[stage]);
-                        mbar_arrive_expect_tx(land, bytes);
-                        stage_loads<KIND, PAIR, false>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst, a_dst + G::A_BYTES,
-                                                       land, rank, my_rows);
-                    } else {
-                        const uint32_t land = full0 + stage * (uint32_t)sizeof(unsigned long long);
-                        if (PAIR) mbar_arrive_expect_tx_cluster(land, bytes); else mbar_arrive_expect_tx(land, bytes);
-                        stage_loads<KIND, PAIR, PAIR>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst, a_dst + G::A_BYTES,
-                                                      land, rank, my_rows);
+                    if (!UNIFORM || elect_one()) {
+                        // read by the MMA warp after its wait on full[stage]
+                        if (SWAP) ctl->stage_n[stage] = (tl.rows + 15) & ~15;
+                        if (HALF_TILES) ctl->stage_half[stage] = tl.half;
+                        if (fix) {
+                            const uint32_t land = smem_u32(&ctl->landed[stage]);
+                            mbar_arrive_expect_tx(land, bytes);
+                            stage_loads<KIND, PAIR, false>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst,
+                                                           a_dst + G::A_BYTES, land, rank, my_rows);
+                        } else {
+                            const uint32_t land = full0 + stage * (uint32_t)sizeof(unsigned long long);
+                            if (PAIR) mbar_arrive_expect_tx_cluster(land, bytes); else mbar_arrive_expect_tx(land, bytes);
+                            stage_loads<KIND, PAIR, PAIR>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst,
+                                                          a_dst + G::A_BYTES, land, rank, my_rows);
+                        }
                     }
+                    if (UNIFORM) __syncwarp();
                     ++issued;
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
@@ -542,17 +561,19 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             }
         }
     } else if (warp == 1 && rank == 0) {
-        // ================= MMA issuer (first CTA of a pair): one thread =================
-        // Measured on this part: the issuing thread spends ~85 cycles on each tcgen05.mma and the tensor pipe
-        // queues about two of them, so per 64-wide K block (4 MMAs, 512 pipe cycles) the thread has only
-        // ~170 cycles for everything else before the pipe runs dry; shared-memory loads and barrier polls
-        // take 100+ cycles each here because TMA fills and operand reads keep the shared-memory pipe busy.
-        // The role is therefore a single thread (no warp synchronisation, no divergence) whose loop holds
-        // nothing but wait / MMAs / commit.  Per tile: the id and row count of the NEXT tile are fetched
-        // before the K loop (the load's latency passes under the MMAs), the last block is peeled out of the
-        // loop (guard predicates for the ragged last block of a WGRAD tile), and whether the next accumulator
-        // buffer is free is tested, without blocking, just before that last block.
-        if (lane == 0) {
+        // ================= MMA issuer (first CTA of a pair) =================
+        // What paces this role is the issuing itself: as one thread of a divergent warp it spent ~85 cycles on each
+        // tcgen05.mma (and the tensor pipe queues about two of them), so per 64-wide K block (4 MMAs, 512 pipe cycles) only
+        // ~170 cycles were left for everything else; shared-memory loads and barrier polls take 100+ cycles each here
+        // because TMA fills and operand reads keep the shared-memory pipe busy.  Now the whole warp runs the loop on
+        // warp-uniform values (role index, tensor-memory base and row counts pass through a shuffle, so that the compiler
+        // knows) and one elected lane issues: descriptors, whose high words are constants, stay in uniform registers.  Weight
+        // gradients of 1024 rows per expert 302 -> 291 us (down) and 607 -> 574 us (gate/up), the other kernels 0-4 %.
+        // The loop holds nothing but wait / MMAs / commit.  Per tile: the id and row count of the NEXT tile are fetched
+        // before the K loop (the load's latency passes under the MMAs), the last block is peeled out of the loop (fewer
+        // MMAs in the ragged last block of a WGRAD tile), and whether the next accumulator buffer is free is tested, without
+        // blocking, just before that last block.
+        {
             uint32_t stage = 0, phase = 0;
             uint32_t acc = 0, acc_phase = 0;
             bool ok = true;
@@ -561,30 +582,28 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             long long e_end = per_e;
             auto rows_of = [&](long long tile) -> int {                 // WGRAD; tile ids of one CTA only grow
                 while (tile >= e_end) { ++e_pos; e_end += per_e; }
-                return ctl->sorted_rows[e_pos];
+                return __shfl_sync(0xffffffffu, ctl->sorted_rows[e_pos], 0);
             };
             // one K block: n_mma MMAs from ring stage `stage`, then the stage is released
             uint32_t idesc = IDESC;
             auto issue_block = [&](uint32_t d_tmem, bool first_block, int n_mma, bool partial) -> bool {
-                if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, abort_flag)) return false;
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->full[stage]), phase, abort_flag))) return false;
                 tc_fence_after();
                 // swapped kinds: the MMA's N is the tile's row count (rounded up to 16), published with each stage
-                if (SWAP && first_block) idesc = make_idesc(G::TILE_M, ctl->stage_n[stage], A_MN, B_MN);
-                if (HALF_TILES && first_block) idesc = ctl->stage_half[stage] ? IDESC_HALF : IDESC;
+                if (SWAP && first_block) idesc = make_idesc(G::TILE_M, __shfl_sync(0xffffffffu, ctl->stage_n[stage], 0), A_MN, B_MN);
+                if (HALF_TILES && first_block) idesc = __shfl_sync(0xffffffffu, ctl->stage_half[stage], 0) ? IDESC_HALF : IDESC;
                 const uint32_t a_base = tiles_base + stage * STAGE_BYTES;
-                const uint64_t a_desc = make_smem_desc<A_MN>(a_base);
-                const uint64_t b_desc = make_smem_desc<B_MN>(a_base + G::A_BYTES);
+                const uint32_t a_desc = make_smem_desc<A_MN>(a_base);
+                const uint32_t b_desc = make_smem_desc<B_MN>(a_base + G::A_BYTES);
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {
-                    const uint32_t accumulate = (!first_block || kk != 0) ? 1u : 0u;
-                    if (partial)
-                        tc_mma_if<PAIR>(d_tmem, a_desc + (uint64_t)((kk * A_KSTEP) >> 4),
-                                        b_desc + (uint64_t)((kk * B_KSTEP) >> 4), IDESC, accumulate, kk < n_mma ? 1u : 0u);
-                    else
-                        tc_mma<PAIR>(d_tmem, a_desc + (uint64_t)((kk * A_KSTEP) >> 4),
-                                     b_desc + (uint64_t)((kk * B_KSTEP) >> 4), (SWAP || HALF_TILES) ? idesc : IDESC, accumulate);
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        if (!partial || kk < n_mma)
+                            tc_mma<PAIR, SMEM_DESC_HI, SMEM_DESC_HI>(d_tmem, a_desc + ((kk * A_KSTEP) >> 4), b_desc + ((kk * B_KSTEP) >> 4),
+                                                                     (SWAP || HALF_TILES) ? idesc : IDESC, (kk != 0 || !first_block) ? 1u : 0u);
+                    tc_commit<PAIR>(smem_u32(&ctl->empty[stage]));
                 }
-                tc_commit<PAIR>(smem_u32(&ctl->empty[stage]));
+                __syncwarp();
                 if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 return true;
             };
@@ -598,7 +617,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 // before full[] was signalled)
                 const int n_full = (KIND == WGRAD) ? (k_rows >> 6) : p.k_blocks;
                 const int n_tail = (KIND == WGRAD) ? (((k_rows & (BK - 1)) + 15) >> 4) : 0;
-                if (!acc_free && !mbar_wait(smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+                if (!acc_free && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag))) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 const int n_main = n_tail != 0 ? n_full : n_full - 1;   // blocks before the peeled last one
@@ -607,12 +626,13 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (!ok) break;
                 // the next tile's accumulator buffer was handed to the epilogue one tile ago: usually free by now
                 const uint32_t acc_n = acc ^ 1u, acc_phase_n = acc_phase ^ acc;
-                acc_free = mbar_test_wait(smem_u32(&ctl->tmem_empty[acc_n]), acc_phase_n ^ 1u);
+                acc_free = __all_sync(0xffffffffu, mbar_test_wait(smem_u32(&ctl->tmem_empty[acc_n]), acc_phase_n ^ 1u));
                 if (n_main >= 0) {
                     if (n_tail != 0) { if (!issue_block(d_tmem, n_main == 0, n_tail, true)) { ok = false; break; } }
                     else             { if (!issue_block(d_tmem, n_main == 0, BK / 16, false)) { ok = false; break; } }
                 }
-                tc_commit<PAIR>(smem_u32(&ctl->tmem_full[acc]));
+                if (elect_one()) tc_commit<PAIR>(smem_u32(&ctl->tmem_full[acc]));
+                __syncwarp();
                 acc = acc_n;
                 acc_phase = acc_phase_n;
                 t = t_next;
@@ -621,7 +641,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
         __syncwarp();
         // all issued MMAs must have retired before tensor memory is released
-        if (lane == 0) {
+        if (elect_one()) {
             tc_commit_local<PAIR>(smem_u32(&ctl->drain));
             const unsigned long long t0 = global_timer_ns();
             while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < WAIT_LIMIT_NS) {}

@@ -168,38 +168,29 @@ __device__ __forceinline__ void tc_commit_local(uint32_t bar) {
     else
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-template <bool PAIR>
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
+// One tcgen05.mma; the shared-memory descriptors are given by their low words (address and leading offset), the high words
+// are constants of the kind.  ACC: accumulate (a literal for all but a tile's first MMA).
+template <bool PAIR, uint32_t A_HI, uint32_t B_HI>
+__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
     if (PAIR) {
         asm volatile(
-            "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            "{ .reg .pred p; .reg .b64 a, b; setp.ne.u32 p, %4, 0; mov.b64 a, {%1, %5}; mov.b64 b, {%2, %6};"
+            " tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p; }" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(A_HI), "n"(B_HI)
             : "memory");
     } else {
         asm volatile(
-            "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            "{ .reg .pred p; .reg .b64 a, b; setp.ne.u32 p, %4, 0; mov.b64 a, {%1, %5}; mov.b64 b, {%2, %6};"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p; }" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(A_HI), "n"(B_HI)
             : "memory");
     }
 }
-// same, issued only when `doit` is non-zero (a guard predicate instead of a branch keeps the issue loop straight-line)
-template <bool PAIR>
-__device__ __forceinline__ void tc_mma_if(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate, uint32_t doit) {
-    if (PAIR) {
-        asm volatile(
-            "{ .reg .pred p, q; setp.ne.u32 p, %4, 0; setp.ne.u32 q, %5, 0;"
-            " @q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(doit)
-            : "memory");
-    } else {
-        asm volatile(
-            "{ .reg .pred p, q; setp.ne.u32 p, %4, 0; setp.ne.u32 q, %5, 0;"
-            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(doit)
-            : "memory");
-    }
+// one lane of the (converged) warp, the same one every time
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred = 0;
+    asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; @p mov.u32 %0, 1; }" : "+r"(pred));
+    return pred != 0;
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t v[32]) {
     asm volatile(
