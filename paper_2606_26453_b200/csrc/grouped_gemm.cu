@@ -134,7 +134,7 @@ struct SharedCtl {
     int stage_half[MAX_STAGES];   // FWD_SWIGLU pair: the stage belongs to a half-height tile (published by the producer)
     int stage_n[MAX_STAGES];   // swapped kinds: MMA N (rows of the tile rounded up to 16) of the tile a stage belongs to
     int32_t offs[MAX_E + 1];
-    int32_t tile_prefix[MAX_E + 1];
+    alignas(16) int32_t tile_prefix[MAX_E + 1];
     int32_t sorted_rows[MAX_E];   // WGRAD: row count of the expert at each position of the largest-first order
 };
 
@@ -424,7 +424,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int my_rows = rank * BM;                                 // this CTA's row offset inside the tile
 
     // ---- set-up: barriers, schedule tables, TMEM ----
-    for (int e = threadIdx.x; e <= p.E; e += NUM_THREADS) ctl->offs[e] = p.offsets[e];
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             // pair mode, first CTA: own producer's (WGRAD: own tail-fix warp's) arrive + the relay's remote arrive
@@ -447,26 +446,36 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         prefetch_tmap(&map_o1);
         prefetch_tmap(&map_x);
     }
+    // everything above may run while the kernel before is still finishing; the schedule is derived from its output
+    grid_dependency_wait();
+    for (int e = threadIdx.x; e <= p.E; e += NUM_THREADS) ctl->offs[e] = p.offsets[e];
     __syncthreads();
     if (wgrad(KIND)) {
         // experts by row count, largest first (ties: lower id first): rank by counting, O(E^2 / threads)
-        for (int e = threadIdx.x; e < p.E; e += NUM_THREADS) {
-            const int n_e = ctl->offs[e + 1] - ctl->offs[e];
-            int rank = 0;
-            for (int f = 0; f < p.E; ++f) {
-                const int n_f = ctl->offs[f + 1] - ctl->offs[f];
-                rank += (n_f > n_e || (n_f == n_e && f < e)) ? 1 : 0;
+        int32_t* n_of = ctl->tile_prefix;   // row counts in expert order (padded to whole int4), until the order is known
+        for (int e = threadIdx.x; e < ((p.E + 3) & ~3); e += NUM_THREADS) n_of[e] = e < p.E ? ctl->offs[e + 1] - ctl->offs[e] : -1;
+        __syncthreads();
+        constexpr int PER_THREAD = (MAX_E + NUM_THREADS - 1) / NUM_THREADS;
+        int my_rank[PER_THREAD];
+#pragma unroll
+        for (int i = 0; i < PER_THREAD; ++i) {
+            const int e = threadIdx.x + i * NUM_THREADS;
+            my_rank[i] = 0;
+            if (e >= p.E) continue;
+            const int n_e = n_of[e];
+            for (int f = 0; f < p.E; f += 4) {
+                const int4 n_f = *reinterpret_cast<const int4*>(n_of + f);
+                my_rank[i] += (n_f.x > n_e || (n_f.x == n_e && f < e)) + (n_f.y > n_e || (n_f.y == n_e && f + 1 < e)) +
+                              (n_f.z > n_e || (n_f.z == n_e && f + 2 < e)) + (n_f.w > n_e || (n_f.w == n_e && f + 3 < e));
             }
-            ctl->tile_prefix[rank] = e;
-            ctl->sorted_rows[rank] = n_e;
+            ctl->sorted_rows[my_rank[i]] = n_e;
         }
-    } else if (threadIdx.x == 0) {
-        int run = 0;
-        for (int e = 0; e < p.E; ++e) {
-            ctl->tile_prefix[e] = run;
-            run += (ctl->offs[e + 1] - ctl->offs[e] + ROW_TILE - 1) / ROW_TILE;
-        }
-        ctl->tile_prefix[p.E] = run;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < PER_THREAD; ++i)
+            if (threadIdx.x + i * NUM_THREADS < p.E) ctl->tile_prefix[my_rank[i]] = threadIdx.x + i * NUM_THREADS;
+    } else if (warp == 0) {
+        exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, ROW_TILE, lane);
     }
     if (warp == 1) {
         if (PAIR) {
@@ -1013,6 +1022,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
 
     // ---- teardown ----
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync_all();   // neither CTA's shared memory / barriers may go away while the other still uses them
@@ -1078,19 +1088,8 @@ int launch(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, c
             grid_of_device[dev] = sms;
         }
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3(grid_of_device[dev]);
-    cfg.blockDim = dim3(NUM_THREADS);
-    cfg.dynamicSmemBytes = Geo<PAIR, fused_sb(KIND)>::SMEM_BYTES;
-    cfg.stream = s;
-    if (PAIR) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-    }
-    if (cudaLaunchKernelEx(&cfg, kernel, a, b0, b1, o0, o1, x, p) != cudaSuccess) return MOE_ERR_CUDA;
-    return check_launch();
+    return launch_dependent(kernel, grid_of_device[dev], NUM_THREADS, Geo<PAIR, fused_sb(KIND)>::SMEM_BYTES, PAIR ? 2 : 1, s, a, b0, b1, o0,
+                            o1, x, p);
 }
 
 // The plain row-ragged GEMMs (down forward, down dgrad, gate/up dgrad) run with swapped operand roles -- always as

@@ -13,7 +13,8 @@ namespace {
 
 constexpr int kWorkspacePairsPerRow = 256;   // the workspace holds one histogram row per 256 pairs (an upper bound on what is used)
 constexpr int kWarpsPerBlock = 8;
-constexpr int kThreads = kWarpsPerBlock * 32;
+constexpr int kThreads = kWarpsPerBlock * 32;   // also what launch_streaming launches
+static_assert(kThreads == 256, "launch_streaming");
 
 __device__ __forceinline__ uint4 ldg16(const uint4* p) { return __ldg(p); }
 
@@ -56,11 +57,6 @@ __device__ __forceinline__ uint4 pack8(const float f[8]) {
 // A pair whose expert id lies outside [0, E) is dropped (it gets no row; the rows past offsets[E] stay
 // unwritten) and MOE_ERR_BAD_INDEX is recorded in the device status word.
 // ------------------------------------------------------------------------------------------------
-// Programmatic dependent launch: rank_rows may start (and run step 1) while hist is still finishing;
-// grid_dependency_wait() then blocks until everything hist wrote is visible.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 constexpr int kIdxGroup = 8;   // index loads in flight per thread in the permute index kernels
 __device__ int g_movement_status = 0;
 
@@ -68,6 +64,8 @@ __global__ void __launch_bounds__(kThreads) permute_hist_kernel(const int32_t* _
                                                                 int chunk, int32_t* __restrict__ ws) {
     extern __shared__ int32_t smem_i[];
     int32_t* hist = smem_i;   // [E]
+    if (!grid_dependency_wait_tested()) return;
+    // rank_rows reads the routing indices and token rows before its own wait: it may start from here on, not earlier
     grid_launch_dependents();
     for (int e = threadIdx.x; e < E; e += kThreads) hist[e] = 0;
     __syncthreads();
@@ -221,7 +219,8 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     int32_t* mine = whist + warp * E;
     if (own >= 0) atomicAdd(&mine[own], 1);   // counts only: order-free
     // ---- (2) the chunk histograms are complete and visible from here on ----
-    grid_dependency_wait();
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     for (int i = threadIdx.x; i < n_chunks * E; i += kPermThreads) {
         const int v = ws[i];
         if (v != 0) {
@@ -336,6 +335,8 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
                                                               uint4* __restrict__ dst, long long total, int hv,
                                                               int K) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (i >= total) return;
     const int t = (int)(i / hv);
     const int c = (int)(i - (long long)t * hv);
@@ -395,6 +396,8 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
     float dot[KA];
 #pragma unroll
     for (int k = 0; k < KA; ++k) dot[k] = 0.f;
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     for (int c = threadIdx.x; c < hv; c += kThreads) {
         const uint4 dv = ldg16(dy + (long long)t * hv + c);
         float d[8];
@@ -455,6 +458,8 @@ __global__ void __launch_bounds__(kThreads) swiglu_bwd_kernel(const uint4* __res
                                                               const uint4* __restrict__ gu,
                                                               uint4* __restrict__ dgu, long long total, int iv) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (i >= total) return;
     const long long r = i / iv;
     const int c = (int)(i - r * iv);
@@ -511,7 +516,8 @@ int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, 
     const int chunk = permute_chunk(R);
     const int n_chunks = (R + chunk - 1) / chunk;
     int32_t* ws = static_cast<int32_t*>(workspace);
-    permute_hist_kernel<<<n_chunks, kThreads, E * sizeof(int32_t), s>>>(topk_idx, R, E, chunk, ws);
+    int st_ = launch_dependent(permute_hist_kernel, n_chunks, kThreads, E * sizeof(int32_t), 1, s, topk_idx, R, E, chunk, ws);
+    if (st_ != MOE_OK) return st_;
 
     const bool rows = x_perm != nullptr;
     const int row_bytes = d.H * 2;
@@ -529,37 +535,24 @@ int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, 
         attr_set[dev] = true;
     }
     const unsigned grid = (unsigned)((d.T + kTokPerBlock - 1) / kTokPerBlock);
-    // launched as a programmatic dependent of the histogram kernel: its blocks start, prefetch rows and count from
-    // the routing indices while the histogram kernel is still running
-    cudaLaunchAttribute pdl[1];
-    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kPermThreads); cfg.dynamicSmemBytes = lay.total_bytes; cfg.stream = s;
-    cfg.attrs = pdl; cfg.numAttrs = 1;
-    const int32_t* ws_c = ws;
-    if (cudaLaunchKernelEx(&cfg, permute_rank_rows_kernel, topk_idx, R, E, (int)d.K, (int)d.T, chunk,
-                           n_chunks, ws_c, counts, offsets, row_to_pair, pair_to_row,
-                           reinterpret_cast<const uint8_t*>(x), reinterpret_cast<uint8_t*>(x_perm), row_bytes,
-                           seg_bytes, n_seg) != cudaSuccess)
-        return MOE_ERR_CUDA;
-    return check_launch();
+    // its blocks start, prefetch rows and count from the routing indices while the histogram kernel is still running
+    return launch_dependent(permute_rank_rows_kernel, grid, kPermThreads, lay.total_bytes, 1, s, topk_idx, R, E, d.K, d.T, chunk,
+                            n_chunks, ws, counts, offsets, row_to_pair, pair_to_row, reinterpret_cast<const uint8_t*>(x),
+                            reinterpret_cast<uint8_t*>(x_perm), row_bytes, seg_bytes, n_seg);
 }
 
 template <bool WEIGHTED>
-static void gather_sum_dispatch(const moe_dims_t& d, const uint4* src, const float* w, const int32_t* p2r,
+static int gather_sum_dispatch(const moe_dims_t& d, const uint4* src, const float* w, const int32_t* p2r,
                                 uint4* dst, cudaStream_t s) {
     const int hv = d.H / 8;
     const long long total = (long long)d.T * hv;
-#define MOE_GS_CASE(KT)                                                                                          \
-    case KT:                                                                                                     \
-        gather_sum_kernel<KT, WEIGHTED><<<blocks_for(total), kThreads, 0, s>>>(src, w, p2r, dst, total, hv, d.K); \
-        break;
+#define MOE_GS_CASE(KT) \
+    case KT: return launch_streaming(gather_sum_kernel<KT, WEIGHTED>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
     switch (d.K) {
         MOE_GS_CASE(1) MOE_GS_CASE(2) MOE_GS_CASE(3) MOE_GS_CASE(4) MOE_GS_CASE(5) MOE_GS_CASE(6) MOE_GS_CASE(7)
         MOE_GS_CASE(8)
         default:
-            gather_sum_kernel<0, WEIGHTED><<<blocks_for(total), kThreads, 0, s>>>(src, w, p2r, dst, total, hv, d.K);
+            return launch_streaming(gather_sum_kernel<0, WEIGHTED>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
     }
 #undef MOE_GS_CASE
 }
@@ -568,27 +561,22 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
                       bf16* dst, cudaStream_t s) {
     const uint4* src = reinterpret_cast<const uint4*>(src_perm);
     uint4* out = reinterpret_cast<uint4*>(dst);
-    if (topk_w != nullptr)
-        gather_sum_dispatch<true>(d, src, topk_w, pair_to_row, out, s);
-    else
-        gather_sum_dispatch<false>(d, src, nullptr, pair_to_row, out, s);
-    return check_launch();
+    return topk_w != nullptr ? gather_sum_dispatch<true>(d, src, topk_w, pair_to_row, out, s)
+                             : gather_sum_dispatch<false>(d, src, nullptr, pair_to_row, out, s);
 }
 
 template <bool WITH_DW>
-static void combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w,
+static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w,
                                  const int32_t* p2r, uint4* dyp, float* dw, cudaStream_t s) {
     const int hv = d.H / 8;
     const unsigned blocks = (unsigned)d.T;
-#define MOE_CB_CASE(KT)                                                                                     \
-    case KT:                                                                                                \
-        combine_bwd_kernel<KT, WITH_DW><<<blocks, kThreads, 0, s>>>(dy, yp, w, p2r, dyp, dw, d.T, hv, d.K); \
-        break;
+#define MOE_CB_CASE(KT) \
+    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     switch (d.K) {
         MOE_CB_CASE(1) MOE_CB_CASE(2) MOE_CB_CASE(3) MOE_CB_CASE(4) MOE_CB_CASE(5) MOE_CB_CASE(6) MOE_CB_CASE(7)
         MOE_CB_CASE(8)
         default:
-            combine_bwd_kernel<0, WITH_DW><<<blocks, kThreads, 0, s>>>(dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+            return launch_streaming(combine_bwd_kernel<0, WITH_DW>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     }
 #undef MOE_CB_CASE
 }
@@ -598,11 +586,8 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    if (dtopk_w != nullptr)
-        combine_bwd_dispatch<true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s);
-    else
-        combine_bwd_dispatch<false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
-    return check_launch();
+    return dtopk_w != nullptr ? combine_bwd_dispatch<true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
+                              : combine_bwd_dispatch<false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -633,10 +618,8 @@ int launch_permute_static_scratch(const moe_dims_t& d, const bf16* x, const int3
 int launch_swiglu_bwd(const moe_dims_t& d, const bf16* dh_act, const bf16* gu, bf16* dgu, cudaStream_t s) {
     const int iv = d.I / 8;
     const long long total = (long long)d.T * d.K * iv;
-    swiglu_bwd_kernel<<<blocks_for(total), kThreads, 0, s>>>(reinterpret_cast<const uint4*>(dh_act),
-                                                            reinterpret_cast<const uint4*>(gu),
-                                                            reinterpret_cast<uint4*>(dgu), total, iv);
-    return check_launch();
+    return launch_streaming(swiglu_bwd_kernel, blocks_for(total), s, reinterpret_cast<const uint4*>(dh_act),
+                            reinterpret_cast<const uint4*>(gu), reinterpret_cast<uint4*>(dgu), total, iv);
 }
 
 }  // namespace moe

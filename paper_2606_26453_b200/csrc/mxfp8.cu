@@ -182,7 +182,6 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     volatile int* abort_flag = &ctl->abort_flag;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, and known to be)
 
-    for (int e = threadIdx.x; e <= p.E; e += MX_THREADS) offs[e] = p.offsets[e];
     if (threadIdx.x == 0) {
         for (int s = 0; s < MX_STAGES; ++s) {
             mbar_init(smem_u32(&ctl->full[s]), 2);    // the producer's arrive (with the byte count) + the scale warp's
@@ -201,15 +200,11 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         prefetch_tmap(&map_b);
         prefetch_tmap(&map_o);
     }
+    // everything above may run while the kernel before is still finishing; the schedule is derived from its output
+    grid_dependency_wait();
+    for (int e = threadIdx.x; e <= p.E; e += MX_THREADS) offs[e] = p.offsets[e];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int e = 0; e < p.E; ++e) {
-            tile_prefix[e] = run;
-            run += (offs[e + 1] - offs[e] + ROWS - 1) / ROWS;
-        }
-        tile_prefix[p.E] = run;
-    }
+    if (warp == 0) exclusive_tile_prefix(offs, tile_prefix, p.E, ROWS, lane);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                      "r"((uint32_t)G::TMEM_COLS)
@@ -451,6 +446,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         __syncwarp();
     }
 
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -623,7 +619,6 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t rank = cluster_ctarank();   // 0 = the CTA that issues the MMAs
     const long long first_tile = blockIdx.x >> 1, tile_stride = gridDim.x >> 1;
 
-    for (int e = threadIdx.x; e <= p.E; e += MXP_THREADS) ctl->offs[e] = p.prefix[e];
     if (threadIdx.x == 0) {
         for (int s = 0; s < MXP_STAGES; ++s) {
             mbar_init(smem_u32(&ctl->full[s]), 4);   // per CTA: the producer's arrive (with its byte count) + the scale warp's
@@ -643,15 +638,11 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         prefetch_tmap(&map_sfb);
         prefetch_tmap(&map_o);
     }
+    // everything above may run while the kernel before is still finishing; the schedule is derived from its output
+    grid_dependency_wait();
+    for (int e = threadIdx.x; e <= p.E; e += MXP_THREADS) ctl->offs[e] = p.prefix[e];
     __syncthreads();
-    if (!WGRAD && threadIdx.x == 0) {   // row-ragged form: tiles of 256 rows per expert
-        int run = 0;
-        for (int e = 0; e < p.E; ++e) {
-            ctl->tile_prefix[e] = run;
-            run += (ctl->offs[e + 1] - ctl->offs[e] + MXP_ROWS - 1) / MXP_ROWS;
-        }
-        ctl->tile_prefix[p.E] = run;
-    }
+    if (!WGRAD && warp == 0) exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, MXP_ROWS, lane);   // row-ragged form
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                      "r"((uint32_t)MX_TMEM_COLS)
@@ -900,6 +891,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         __syncwarp();
     }
 
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();   // neither CTA's shared memory / barriers may go away while the other still uses them
@@ -976,6 +968,8 @@ __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __re
                                                                int out_k_tiles, int out_kt0, uint2* __restrict__ codes,
                                                                uint8_t* __restrict__ scales, uint8_t* __restrict__ scales_pair) {
     __shared__ __align__(16) uint8_t sf[128 * 4];
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int k_tiles = n >> 7;
     const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
     const long long row0 = 128ll * row_tile;
@@ -1024,6 +1018,8 @@ __global__ void __launch_bounds__(256) mx_swiglu_quantize_kernel(const uint4* __
     const int k_tiles = I / 128;
     const long long total = rows * k_tiles;
     const long long pairs = (total + 1) / 2;
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     for (long long p0 = warp; p0 < pairs; p0 += n_warps) {
         const long long u = 2 * p0 + (lane >> 4);
         if (u >= total) continue;   // only the last pair can be half empty; no warp-wide operation below needs those lanes
@@ -1075,6 +1071,8 @@ __global__ void __launch_bounds__(256) mx_swiglu_bwd_quantize_kernel(const uint4
     const int lane = threadIdx.x & 31;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int iv = I >> 3;                       // 16-byte pieces per half row (a multiple of 16)
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (i >= rows * iv) return;                  // whole half-warps leave together
     const long long r = (rows * iv >> 32) == 0 ? (long long)((uint32_t)i / (uint32_t)iv) : i / iv;
     const int c = (int)(i - r * iv);
@@ -1188,6 +1186,8 @@ __global__ void __launch_bounds__(256) mx_quantize_w_transposed_kernel(const bf1
                                                                        uint8_t* __restrict__ scales_pair) {
     __shared__ __align__(16) uint32_t tile[4 * MXT_BLOCK_WORDS];
     __shared__ __align__(16) uint8_t sf[128 * 4];
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int f_tiles = n >> 7, k_tiles = k >> 7;
     const int ft = blockIdx.x % f_tiles, rest = blockIdx.x / f_tiles, kt = rest % k_tiles;
     const long long e = rest / k_tiles;
@@ -1227,6 +1227,8 @@ __global__ void __launch_bounds__(256) mx_quantize_tokens_kernel(const bf16* __r
     __shared__ __align__(16) uint8_t sf[128 * 4];
     __shared__ int32_t part[8];
     __shared__ int32_t mine[3];   // first row, rows and existence of this block's slice
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int f_tiles = n >> 7;
         const int f0 = (int)(blockIdx.x % (unsigned)f_tiles) * 128, slice = (int)(blockIdx.x / (unsigned)f_tiles);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1285,18 +1287,16 @@ size_t mx_w_scale_bytes(int E, int n_feat, int k) {
 static unsigned mx_row_quantiser_blocks(long long rows, int k) { return (unsigned)((rows + 127) / 128 * (k / 128)); }
 
 int launch_mx_quantize_rows(long long rows, int n, const bf16* x, uint8_t* codes, uint8_t* scales, cudaStream_t s) {
-    mx_quantize_rows_kernel<false><<<mx_row_quantiser_blocks(rows, n), 256, 0, s>>>(
-        reinterpret_cast<const uint4*>(x), rows, n, 0, n / 128, 0, reinterpret_cast<uint2*>(codes), scales, nullptr);
-    return check_launch();
+    return launch_streaming(mx_quantize_rows_kernel<false>, mx_row_quantiser_blocks(rows, n), s, reinterpret_cast<const uint4*>(x), rows, n, 0, n / 128, 0, reinterpret_cast<uint2*>(codes), scales,
+                            static_cast<uint8_t*>(nullptr));
 }
 
 // w [E, k, n] -> rows [n_off, n_off + n) of the transposed codes [E, n_total, k] and the matching scale bytes
 int launch_mx_quantize_w_transposed(int E, int k, int n, int n_total, int n_off, const bf16* w, uint8_t* codes_t, uint8_t* scales,
                                     cudaStream_t s) {
     const long long blocks = (long long)E * (k / 128) * (n / 128);
-    mx_quantize_w_transposed_kernel<<<(unsigned)blocks, 256, 0, s>>>(w, k, n, n_total, n_off, codes_t, scales,
-                                                                     scales + mx_w_scale_single_bytes(E, n_total, k));
-    return check_launch();
+    return launch_streaming(mx_quantize_w_transposed_kernel, (unsigned)blocks, s, w, k, n, n_total, n_off, codes_t, scales,
+                            scales + mx_w_scale_single_bytes(E, n_total, k));
 }
 
 int launch_mx_swiglu_quantize(long long rows, int I, const bf16* gu, bf16* h_act, uint8_t* codes, uint8_t* scales, cudaStream_t s) {
@@ -1305,29 +1305,26 @@ int launch_mx_swiglu_quantize(long long rows, int I, const bf16* gu, bf16* h_act
     const long long cap = (long long)sm_count() * 32;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    mx_swiglu_quantize_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const uint4*>(gu), rows, I,
-                                                             reinterpret_cast<uint4*>(h_act), reinterpret_cast<uint2*>(codes),
-                                                             reinterpret_cast<uint32_t*>(scales));
-    return check_launch();
+    return launch_streaming(mx_swiglu_quantize_kernel, (unsigned)blocks, s, reinterpret_cast<const uint4*>(gu), rows, I,
+                            reinterpret_cast<uint4*>(h_act), reinterpret_cast<uint2*>(codes),
+                            reinterpret_cast<uint32_t*>(scales));
 }
 
 int launch_mx_swiglu_bwd_quantize(long long rows, int I, const bf16* dh_act, const bf16* gu, bf16* dgu, uint8_t* codes,
                                   uint8_t* scales, cudaStream_t s) {
     const long long total = rows * (I / 8);
-    mx_swiglu_bwd_quantize_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-        reinterpret_cast<const uint4*>(dh_act), reinterpret_cast<const uint4*>(gu), rows, I, reinterpret_cast<uint4*>(dgu),
-        reinterpret_cast<uint2*>(codes), reinterpret_cast<uint32_t*>(scales));
-    return check_launch();
+    return launch_streaming(mx_swiglu_bwd_quantize_kernel, (unsigned)((total + 255) / 256), s,
+                            reinterpret_cast<const uint4*>(dh_act), reinterpret_cast<const uint4*>(gu), rows, I,
+                            reinterpret_cast<uint4*>(dgu), reinterpret_cast<uint2*>(codes), reinterpret_cast<uint32_t*>(scales));
 }
 
 // w [E * n_feat, k] -> columns [k_off, k_off + k) of the codes [E * n_feat, k_total] and the matching scale slices
 int launch_mx_quantize_w_rows(int E, int n_feat, int k, int k_total, int k_off, const bf16* w, uint8_t* codes, uint8_t* scales,
                               cudaStream_t s) {
     const long long rows = (long long)E * n_feat;
-    mx_quantize_rows_kernel<true><<<mx_row_quantiser_blocks(rows, k), 256, 0, s>>>(
-        reinterpret_cast<const uint4*>(w), rows, k, n_feat, k_total / 128, k_off / 128, reinterpret_cast<uint2*>(codes), scales,
-        scales + mx_w_scale_single_bytes(E, n_feat, k_total));
-    return check_launch();
+    return launch_streaming(mx_quantize_rows_kernel<true>, mx_row_quantiser_blocks(rows, k), s, reinterpret_cast<const uint4*>(w), rows, k, n_feat,
+                            k_total / 128, k_off / 128, reinterpret_cast<uint2*>(codes), scales,
+                            scales + mx_w_scale_single_bytes(E, n_feat, k_total));
 }
 
 // ---- weight-gradient operands and GEMM ----
@@ -1345,9 +1342,8 @@ int launch_mx_quantize_tokens(long long R, int E, const bf16* x, long long ld, i
     uint8_t* sa = scales + MX_TOKENS_HEADER_BYTES;
     uint8_t* sb = sa + (size_t)(pitch / 128) * n * 4;
     const long long blocks = (pitch / 128) * (n / 128);
-    mx_quantize_tokens_kernel<<<(unsigned)blocks, 256, 0, s>>>(x, ld, col0, n, offsets, sp, E, pitch, codes_t,
-                                                               reinterpret_cast<uint32_t*>(sa), sb);
-    return check_launch();
+    return launch_streaming(mx_quantize_tokens_kernel, (unsigned)blocks, s, x, ld, col0, n, offsets, sp, E,
+                            pitch, codes_t, reinterpret_cast<uint32_t*>(sa), sb);
 }
 
 // dW [E, M, N] = Q(A)^T Q(B) per expert: a_* the M-side operand ([M, pitch] codes, scales with header and words),
@@ -1391,10 +1387,7 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
         if (clusters > sms / 2) clusters = sms / 2;
         grid_of_device[dev] = 2 * clusters;
     }
-    cfg.gridDim = dim3(grid_of_device[dev]);
-    cfg.stream = s;
-    if (cudaLaunchKernelEx(&cfg, mx_pair_kernel<true>, a, b, sfb, o, p) != cudaSuccess) return MOE_ERR_CUDA;
-    return check_launch();
+    return launch_dependent(mx_pair_kernel<true>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
 }
 
 // CTA pairs from this many rows per expert on average (below it the 256-row tiles are mostly padding)
@@ -1445,10 +1438,7 @@ static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint
         if (clusters > sms / 2) clusters = sms / 2;
         grid_of_device[dev] = 2 * clusters;
     }
-    cfg.gridDim = dim3(grid_of_device[dev]);
-    cfg.stream = s;
-    if (cudaLaunchKernelEx(&cfg, mx_pair_kernel<false>, a, b, sfb, o, p) != cudaSuccess) return MOE_ERR_CUDA;
-    return check_launch();
+    return launch_dependent(mx_pair_kernel<false>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
 }
 
 struct MxSingleArgs {
@@ -1483,8 +1473,7 @@ static int launch_mx_gemm_single(const MxSingleArgs& g, cudaStream_t s) {
     }
     const int sms = sm_count();
     if (sms <= 0) return MOE_ERR_CUDA;
-    mx_gemm_kernel<ROWS><<<MxGeo<ROWS>::CTAS * sms, MX_THREADS, MxGeo<ROWS>::smem_bytes(g.E), s>>>(a, b, o, p);
-    return check_launch();
+    return launch_dependent(mx_gemm_kernel<ROWS>, MxGeo<ROWS>::CTAS * sms, MX_THREADS, MxGeo<ROWS>::smem_bytes(g.E), 1, s, a, b, o, p);
 }
 
 // out[r, :] = dequant(a row r) . dequant(b[e])^T for the rows r of expert e: a [R, k] codes with scale words

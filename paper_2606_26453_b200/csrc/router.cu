@@ -34,6 +34,8 @@ router_topk_kernel(const float* __restrict__ logits, int T, int E, int K, int32_
                    float* __restrict__ topk_w) {
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (t >= T) return;
     const float* row = logits + (size_t)t * E;
     uint32_t key[VPL];
@@ -80,6 +82,8 @@ router_topk_bwd_kernel(const int32_t* __restrict__ topk_idx, const float* __rest
                        const float* __restrict__ dtopk_w, int T, int E, int K, float* __restrict__ dlogits) {
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (t >= T) return;
     float w = 0.f, dw = 0.f;
     int idx = -1;
@@ -103,10 +107,7 @@ int launch_router_topk(const moe_dims_t& d, const float* logits, int32_t* topk_i
     const int blocks = (d.T + kWarpsPerBlock - 1) / kWarpsPerBlock;
     const int vpl = (d.E + 31) / 32;
 #define MOE_ROUTER_CASE(V)                                                                                     \
-    if (vpl <= V) {                                                                                            \
-        router_topk_kernel<V><<<blocks, kWarpsPerBlock * 32, 0, s>>>(logits, d.T, d.E, d.K, topk_idx, topk_w); \
-        return check_launch();                                                                                 \
-    }
+    if (vpl <= V) return launch_dependent(router_topk_kernel<V>, blocks, kWarpsPerBlock * 32, 0, 1, s, logits, d.T, d.E, d.K, topk_idx, topk_w);
     MOE_ROUTER_CASE(1)
     MOE_ROUTER_CASE(2)
     MOE_ROUTER_CASE(4)
@@ -120,8 +121,7 @@ int launch_router_topk(const moe_dims_t& d, const float* logits, int32_t* topk_i
 int launch_router_topk_bwd(const moe_dims_t& d, const int32_t* topk_idx, const float* topk_w, const float* dtopk_w,
                            float* dlogits, cudaStream_t s) {
     const int blocks = (d.T + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    router_topk_bwd_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(topk_idx, topk_w, dtopk_w, d.T, d.E, d.K, dlogits);
-    return check_launch();
+    return launch_dependent(router_topk_bwd_kernel, blocks, kWarpsPerBlock * 32, 0, 1, s, topk_idx, topk_w, dtopk_w, d.T, d.E, d.K, dlogits);
 }
 
 }  // namespace moe

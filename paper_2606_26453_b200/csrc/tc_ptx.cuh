@@ -211,6 +211,24 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 
+// prefix[e] = number of tiles of `rows_per_tile` rows of the experts before e, prefix[E] = all of them.  One warp.
+__device__ __forceinline__ void exclusive_tile_prefix(const int32_t* offs, int32_t* prefix, int E, int rows_per_tile, int lane) {
+    int run = 0;
+    for (int e0 = 0; e0 < E; e0 += 32) {
+        const int e = e0 + lane;
+        const int tiles = e < E ? (offs[e + 1] - offs[e] + rows_per_tile - 1) / rows_per_tile : 0;
+        int incl = tiles;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        if (e < E) prefix[e] = run + incl - tiles;
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) prefix[E] = run;
+}
+
 // ---- host side: tensor maps -------------------------------------------------------------------------
 inline PFN_cuTensorMapEncodeTiled_v12000 get_encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
