@@ -1092,12 +1092,20 @@ int launch(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, c
                             o1, x, p);
 }
 
+constexpr long long kSwappedFusedRows = 512;
 // The plain row-ragged GEMMs (down forward, down dgrad, gate/up dgrad) run with swapped operand roles -- always as
-// CTA pairs: 256 output features x up to 256 rows per tile -- when experts hold fewer than 512 rows on average:
-// there the fixed 128-row tiles lose 10-15 % of the tensor work to padding (measured: +2-5 % per kernel on the
-// 384- and 451-rows-per-expert workloads).  With larger experts the padding is small and the fixed-height tiles
-// are as fast or faster (the swapped kernels' issue thread, not the tensor pipe, bounds tiles of fewer than 256 rows).
-bool use_swapped(const moe_dims_t& d) { return (long long)d.T * d.K < 512ll * d.E; }
+// CTA pairs: 256 output features x up to 256 rows per tile -- when experts hold fewer than 1600 rows on average: there the
+// fixed 256-row tiles lose half a tile per expert to padding (12 % of the tensor work at 1024 rows).  Down / down dgrad /
+// gate/up dgrad, fixed tiles against swapped, by rows per expert:
+//   768   (32 experts, 2048 x 1408)   101 / 112 / 206 against  97 / 103 / 187 us
+//   1024  (16 experts, 4096 x 4096)   385 / 386 / 810 against 358 / 357 / 759 us
+//   1536  (64 experts, 2048 x 1408)   384 / 418 / 780 against 374 / 403 / 751 us
+//   2048  (8 experts, 4096 x 14336)  1332 / 1250 / 2731 against 1328 / 1226 / 2956 us
+// With larger experts the padding is small and the fixed-height tiles have fewer MMAs to issue.
+bool use_swapped(const moe_dims_t& d) { return (long long)d.T * d.K < 1600ll * d.E; }
+// The down dgrad with the SwiGLU backward in its epilogue: there the swapped form also transposes the two blocks it fetches,
+// and that outlasts short contractions, so the line lies lower.
+bool use_swapped_fused(const moe_dims_t& d) { return (long long)d.T * d.K < kSwappedFusedRows * d.E; }
 // The SwiGLU forward has no swapped form (measured slower: two accumulators per tile).  Its pair kernel runs an
 // expert's last <= 128 rows as a half-height tile, which makes pairs worthwhile from 320 rows per expert on average.
 constexpr long long kSwigluPairRows = 320;
@@ -1205,7 +1213,7 @@ int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const
     Params p = {};
     p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
     p.n_cols = d.I; p.b_rows_per_e = d.I; p.out0 = dgu; p.ldo = 2ll * d.I; p.n_split = d.I; p.I = d.I;
-    if (use_swapped(d)) {
+    if (use_swapped_fused(d)) {
         const int feats = 2 * SWAP_FEATS;   // a CTA pair's tile
         const uint32_t box = 32;            // row boxes of 32 / 64 / 128 rows per CTA
         CUtensorMap a, a2, a1, b0;
