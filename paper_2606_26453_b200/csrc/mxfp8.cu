@@ -933,9 +933,25 @@ __device__ __forceinline__ uint32_t mx_abs_max(uint32_t a, uint32_t b) {   // of
 }
 __device__ __forceinline__ float mx_lo(uint32_t w) { return __uint_as_float(w << 16); }          // bf16 -> fp32 is a shift
 __device__ __forceinline__ float mx_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-__device__ __forceinline__ uint2 mx_codes8(const uint4& v, float inv) {   // 8 consecutive values -> 8 code bytes
-    return make_uint2(mx_e4m3x2(mx_lo(v.x) * inv, mx_hi(v.x) * inv) | (mx_e4m3x2(mx_lo(v.y) * inv, mx_hi(v.y) * inv) << 16),
-                      mx_e4m3x2(mx_lo(v.z) * inv, mx_hi(v.z) * inv) | (mx_e4m3x2(mx_lo(v.w) * inv, mx_hi(v.w) * inv) << 16));
+// 2^-s as bf16 bits (exact: it is a power of two), and its product with two packed values: exact but for results so small
+// that their code is zero, so the codes are those of the fp32 product at half the multiplications.
+__device__ __forceinline__ uint32_t mx_inv_bits(int s) { return (uint32_t)__float_as_int(mx_inv_scale(s)) >> 16; }
+__device__ __forceinline__ uint32_t mx_scale2(uint32_t v, uint32_t inv2) {
+    const __nv_bfloat162 m = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&v), *reinterpret_cast<const __nv_bfloat162*>(&inv2));
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+__device__ __forceinline__ uint2 mx_codes8(const uint4& v, int se) {   // 8 consecutive values -> 8 code bytes
+    const uint32_t inv = mx_inv_bits(se), inv2 = inv | (inv << 16);
+    const uint32_t x = mx_scale2(v.x, inv2), y = mx_scale2(v.y, inv2), z = mx_scale2(v.z, inv2), w = mx_scale2(v.w, inv2);
+    return make_uint2(mx_e4m3x2(mx_lo(x), mx_hi(x)) | (mx_e4m3x2(mx_lo(y), mx_hi(y)) << 16),
+                      mx_e4m3x2(mx_lo(z), mx_hi(z)) | (mx_e4m3x2(mx_lo(w), mx_hi(w)) << 16));
+}
+// Scale exponent of a block of 32 values held by 4 consecutive lanes, 8 each.
+__device__ __forceinline__ int mx_block_exp(const uint4& v) {
+    uint32_t m = mx_abs_max4(v);
+    m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    return mx_scale_exp(fmaxf(mx_lo(m), mx_hi(m)));
 }
 // Where the scale word of feature `f` (4 scale bytes of one K slice) sits inside a 128-feature block of 512 bytes, in words.
 __device__ __forceinline__ int mx_sf_word(int f) { return (f % 32) * 4 + (f % 128) / 32; }
@@ -960,8 +976,8 @@ __device__ __forceinline__ void mx_store_weight_scales(const uint32_t* words, in
 //                    out_kt0 .. out_kt0 + n/128): W_gate and W_up side by side along the contraction of the gate/up
 //                    data gradient.
 // 3 bytes of HBM traffic per element, so bound by HBM only if few instructions and few partial sectors go into one.  Inside
-// an FP8 step, 201 M weights (128 x 2048 x 768): 242 -> 122 us (4.9 TB/s); activations 131072 x 2048: 184 -> 130 us
-// (6.2 TB/s).  Before, a warp walked along a row: every (row, slice) took a 64-bit division, eight shuffles and, for
+// an FP8 step, 201 M weights (128 x 2048 x 768): 242 -> 122 us (4.9 TB/s); activations 131072 x 2048: 184 -> 119 us
+// (6.8 TB/s).  Before, a warp walked along a row: every (row, slice) took a 64-bit division, eight shuffles and, for
 // weights, two 4-byte stores into a sector each.
 template <bool WEIGHTS>
 __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n, int n_feat,
@@ -983,11 +999,8 @@ __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __re
     for (int i = 0; i < 8; ++i) v[i] = sub + 16 * i < n_rows ? __ldg(src + i * src_step) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        uint32_t m = mx_abs_max4(v[i]);
-        m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-        m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        const int se = mx_scale_exp(fmaxf(mx_lo(m), mx_hi(m)));
-        if (sub + 16 * i < n_rows) dst[i * dst_step] = mx_codes8(v[i], mx_inv_scale(se));
+        const int se = mx_block_exp(v[i]);
+        if (sub + 16 * i < n_rows) dst[i * dst_step] = mx_codes8(v[i], se);
         if ((l16 & 3) == 0) sf[(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se + 127);
     }
     __syncthreads();
@@ -1007,122 +1020,115 @@ __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __re
 
 // The SwiGLU activation of saved pre-activations with the activation quantiser fused in: GU [rows, 2I] bf16 ->
 // H_act [rows, I] bf16 (silu(g) * u in fp32, rounded once) and the block-scaled FP8 codes and scale words of exactly those
-// bf16 values, in the layouts of the activation quantiser.  Same lane mapping as mx_quantize_rows_kernel: a half-warp per
-// (row, 128-wide slice of I), 8 elements per lane.
+// bf16 values, in the layouts of the activation quantiser.  Same mapping as mx_quantize_rows_kernel, on 64 rows: a half-warp
+// per (row, 128-wide slice of I), four rows one after the other with all eight loads in flight.
+// 16384 x 14336 inside an FP8 step 320 -> 248 us, alone 289 -> 242 us (6.8 TB/s); 131072 x 768 138 -> 110 us.  Before, a thread
+// had two loads in flight, and every row took a division and four more shuffles.
+constexpr int MX_SWIGLU_ROWS = 64;
 __global__ void __launch_bounds__(256) mx_swiglu_quantize_kernel(const uint4* __restrict__ gu, long long rows, int I,
                                                                  uint4* __restrict__ h_act, uint2* __restrict__ codes,
                                                                  uint32_t* __restrict__ scales) {
-    const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const int k_tiles = I / 128;
-    const long long total = rows * k_tiles;
-    const long long pairs = (total + 1) / 2;
+    __shared__ __align__(16) uint8_t sf[MX_SWIGLU_ROWS * 4];
     if (!grid_dependency_wait_tested()) return;
     grid_launch_dependents();
-    for (long long p0 = warp; p0 < pairs; p0 += n_warps) {
-        const long long u = 2 * p0 + (lane >> 4);
-        if (u >= total) continue;   // only the last pair can be half empty; no warp-wide operation below needs those lanes
-        const long long r = (total >> 32) == 0 ? (long long)((uint32_t)u / (uint32_t)k_tiles) : u / k_tiles;
-        const int kt = (int)(u - r * k_tiles);
-        const long long g_idx = (r * 2 * I + kt * 128) / 8 + (lane & 15);
-        const uint4 graw = __ldg(gu + g_idx), uraw = __ldg(gu + g_idx + I / 8);
-        const uint32_t* gw = reinterpret_cast<const uint32_t*>(&graw);
-        const uint32_t* uw = reinterpret_cast<const uint32_t*>(&uraw);
+    constexpr int N = MX_SWIGLU_ROWS / 16;
+    const int k_tiles = I >> 7, iv = I >> 3;
+    const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
+    const long long row0 = (long long)MX_SWIGLU_ROWS * row_tile;
+    const int sub = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+    const int n_rows = (int)min((long long)MX_SWIGLU_ROWS, rows - row0);
+    const uint4* src = gu + (row0 + sub) * (2 * iv) + kt * 16 + l16;
+    const long long dst0 = (row0 + sub) * iv + kt * 16 + l16;
+    uint4 g[N], u[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const bool in = sub + 16 * i < n_rows;
+        g[i] = in ? __ldg(src + 32ll * i * iv) : make_uint4(0u, 0u, 0u, 0u);
+        u[i] = in ? __ldg(src + 32ll * i * iv + iv) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t* gw = reinterpret_cast<const uint32_t*>(&g[i]);
+        const uint32_t* uw = reinterpret_cast<const uint32_t*>(&u[i]);
         uint32_t hw[4];
-        float v[8];
-        float amax = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float2 g2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw[j]));
-            const float2 u2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&uw[j]));
-            const float h0 = __fdividef(g2.x, 1.f + __expf(-g2.x)) * u2.x;
-            const float h1 = __fdividef(g2.y, 1.f + __expf(-g2.y)) * u2.y;
-            hw[j] = pack_bf16(h0, h1);
-            const float2 hr = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[j]));   // what H_act holds
-            v[2 * j] = hr.x; v[2 * j + 1] = hr.y;
-            amax = fmaxf(amax, fmaxf(fabsf(hr.x), fabsf(hr.y)));
+            const float g0 = mx_lo(gw[j]), g1 = mx_hi(gw[j]);
+            hw[j] = pack_bf16(__fdividef(g0, 1.f + __expf(-g0)) * mx_lo(uw[j]), __fdividef(g1, 1.f + __expf(-g1)) * mx_hi(uw[j]));
         }
-        const uint32_t half_mask = (lane & 16) ? 0xffff0000u : 0x0000ffffu;
-        amax = fmaxf(amax, __shfl_xor_sync(half_mask, amax, 1));
-        amax = fmaxf(amax, __shfl_xor_sync(half_mask, amax, 2));
-        const int se = mx_scale_exp(amax);
-        const float inv = mx_inv_scale(se);
-        uint2 out;
-        out.x = mx_e4m3x2(v[0] * inv, v[1] * inv) | (mx_e4m3x2(v[2] * inv, v[3] * inv) << 16);
-        out.y = mx_e4m3x2(v[4] * inv, v[5] * inv) | (mx_e4m3x2(v[6] * inv, v[7] * inv) << 16);
-        h_act[u * 16 + (lane & 15)] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        codes[u * 16 + (lane & 15)] = out;
-        const uint32_t sbyte = (uint32_t)(se + 127);
-        const int base = lane & 16;
-        const uint32_t word = __shfl_sync(half_mask, sbyte, base) | (__shfl_sync(half_mask, sbyte, base + 4) << 8) |
-                              (__shfl_sync(half_mask, sbyte, base + 8) << 16) | (__shfl_sync(half_mask, sbyte, base + 12) << 24);
-        if ((lane & 15) == 0) scales[(long long)kt * rows + r] = word;
+        const uint4 h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        const int se = mx_block_exp(h);
+        if (sub + 16 * i < n_rows) {
+            h_act[dst0 + 16ll * i * iv] = h;
+            codes[dst0 + 16ll * i * iv] = mx_codes8(h, se);
+        }
+        if ((l16 & 3) == 0) sf[(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se + 127);
     }
+    __syncthreads();
+    if ((int)threadIdx.x < n_rows) scales[(long long)kt * rows + row0 + threadIdx.x] = reinterpret_cast<const uint32_t*>(sf)[threadIdx.x];
 }
 
 // The SwiGLU backward (elementwise part of the gate/up backward) with the row quantiser of its result fused in:
 // dGU = [dg | du] [rows, 2I] bf16 exactly as moe_swiglu_bwd computes it, and the block-scaled FP8 codes and scale words of
-// those bf16 values along the 2I columns (the A operand of the FP8 gate/up dgrad).  One thread per 8 columns of a row
-// (its 8 gate and its 8 up columns), a half-warp per 128-wide slice of each half.
+// those bf16 values along the 2I columns (the A operand of the FP8 gate/up dgrad).  The same mapping on 32 rows: a half-warp
+// per (row, 128-wide slice of each half), two rows one after the other with all six loads in flight.
+// 16384 x 14336 inside an FP8 step 494 -> 478 us (5.9 TB/s), 131072 x 768 222 -> 205 us; alone 442 and 451 us.
+constexpr int MX_SWIGLU_BWD_ROWS = 32;
 __global__ void __launch_bounds__(256) mx_swiglu_bwd_quantize_kernel(const uint4* __restrict__ dh_act, const uint4* __restrict__ gu,
                                                                      long long rows, int I, uint4* __restrict__ dgu,
                                                                      uint2* __restrict__ codes, uint32_t* __restrict__ scales) {
-    const int lane = threadIdx.x & 31;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int iv = I >> 3;                       // 16-byte pieces per half row (a multiple of 16)
+    __shared__ __align__(16) uint8_t sf[2][MX_SWIGLU_BWD_ROWS * 4];
     if (!grid_dependency_wait_tested()) return;
     grid_launch_dependents();
-    if (i >= rows * iv) return;                  // whole half-warps leave together
-    const long long r = (rows * iv >> 32) == 0 ? (long long)((uint32_t)i / (uint32_t)iv) : i / iv;
-    const int c = (int)(i - r * iv);
-    const uint4 dhv = __ldg(dh_act + i), gv = __ldg(gu + r * (2 * iv) + c), uv = __ldg(gu + r * (2 * iv) + iv + c);
-    const uint32_t* dw = reinterpret_cast<const uint32_t*>(&dhv);
-    const uint32_t* gw = reinterpret_cast<const uint32_t*>(&gv);
-    const uint32_t* uw = reinterpret_cast<const uint32_t*>(&uv);
-    uint32_t og[4], ou[4];
-    float vg[8], vu[8], amax_g = 0.f, amax_u = 0.f;
+    constexpr int N = MX_SWIGLU_BWD_ROWS / 16;
+    const int k_tiles = I >> 7, iv = I >> 3;
+    const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
+    const long long row0 = (long long)MX_SWIGLU_BWD_ROWS * row_tile;
+    const int sub = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+    const int n_rows = (int)min((long long)MX_SWIGLU_BWD_ROWS, rows - row0);
+    const long long at = (row0 + sub) * (2 * iv) + kt * 16 + l16;   // in GU and dGU; dH_act has half the pitch
+    const uint4* dh_src = dh_act + (row0 + sub) * iv + kt * 16 + l16;
+    uint4 d[N], g[N], u[N];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 d2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&dw[j]));
-        const float2 g2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw[j]));
-        const float2 u2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&uw[j]));
-        const float s0 = __fdividef(1.f, 1.f + __expf(-g2.x)), s1 = __fdividef(1.f, 1.f + __expf(-g2.y));
-        og[j] = pack_bf16(d2.x * u2.x * s0 * (1.f + g2.x * (1.f - s0)), d2.y * u2.y * s1 * (1.f + g2.y * (1.f - s1)));
-        ou[j] = pack_bf16(d2.x * g2.x * s0, d2.y * g2.y * s1);
-        const float2 rg = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&og[j]));   // what dGU holds
-        const float2 ru = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ou[j]));
-        vg[2 * j] = rg.x; vg[2 * j + 1] = rg.y; vu[2 * j] = ru.x; vu[2 * j + 1] = ru.y;
-        amax_g = fmaxf(amax_g, fmaxf(fabsf(rg.x), fabsf(rg.y)));
-        amax_u = fmaxf(amax_u, fmaxf(fabsf(ru.x), fabsf(ru.y)));
+    for (int i = 0; i < N; ++i) {
+        const bool in = sub + 16 * i < n_rows;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        d[i] = in ? __ldg(dh_src + 16ll * i * iv) : zero;
+        g[i] = in ? __ldg(gu + at + 32ll * i * iv) : zero;
+        u[i] = in ? __ldg(gu + at + 32ll * i * iv + iv) : zero;
     }
-    dgu[r * (2 * iv) + c] = make_uint4(og[0], og[1], og[2], og[3]);
-    dgu[r * (2 * iv) + iv + c] = make_uint4(ou[0], ou[1], ou[2], ou[3]);
-    const uint32_t half_mask = (lane & 16) ? 0xffff0000u : 0x0000ffffu;
-    amax_g = fmaxf(amax_g, __shfl_xor_sync(half_mask, amax_g, 1));
-    amax_g = fmaxf(amax_g, __shfl_xor_sync(half_mask, amax_g, 2));
-    amax_u = fmaxf(amax_u, __shfl_xor_sync(half_mask, amax_u, 1));
-    amax_u = fmaxf(amax_u, __shfl_xor_sync(half_mask, amax_u, 2));
-    const int se_g = mx_scale_exp(amax_g), se_u = mx_scale_exp(amax_u);
-    const float inv_g = mx_inv_scale(se_g), inv_u = mx_inv_scale(se_u);
-    uint2 cg, cu;
-    cg.x = mx_e4m3x2(vg[0] * inv_g, vg[1] * inv_g) | (mx_e4m3x2(vg[2] * inv_g, vg[3] * inv_g) << 16);
-    cg.y = mx_e4m3x2(vg[4] * inv_g, vg[5] * inv_g) | (mx_e4m3x2(vg[6] * inv_g, vg[7] * inv_g) << 16);
-    cu.x = mx_e4m3x2(vu[0] * inv_u, vu[1] * inv_u) | (mx_e4m3x2(vu[2] * inv_u, vu[3] * inv_u) << 16);
-    cu.y = mx_e4m3x2(vu[4] * inv_u, vu[5] * inv_u) | (mx_e4m3x2(vu[6] * inv_u, vu[7] * inv_u) << 16);
-    codes[r * (2 * iv) + c] = cg;
-    codes[r * (2 * iv) + iv + c] = cu;
-    const int base = lane & 16;
-    const uint32_t bg = (uint32_t)(se_g + 127), bu = (uint32_t)(se_u + 127);
-    const uint32_t word_g = __shfl_sync(half_mask, bg, base) | (__shfl_sync(half_mask, bg, base + 4) << 8) |
-                            (__shfl_sync(half_mask, bg, base + 8) << 16) | (__shfl_sync(half_mask, bg, base + 12) << 24);
-    const uint32_t word_u = __shfl_sync(half_mask, bu, base) | (__shfl_sync(half_mask, bu, base + 4) << 8) |
-                            (__shfl_sync(half_mask, bu, base + 8) << 16) | (__shfl_sync(half_mask, bu, base + 12) << 24);
-    if ((lane & 15) == 0) {
-        const int kt = c >> 4;                   // 128-wide slice inside the half
-        scales[(long long)kt * rows + r] = word_g;
-        scales[(long long)((I >> 7) + kt) * rows + r] = word_u;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t* dw = reinterpret_cast<const uint32_t*>(&d[i]);
+        const uint32_t* gw = reinterpret_cast<const uint32_t*>(&g[i]);
+        const uint32_t* uw = reinterpret_cast<const uint32_t*>(&u[i]);
+        uint32_t og[4], ou[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 d2 = make_float2(mx_lo(dw[j]), mx_hi(dw[j])), g2 = make_float2(mx_lo(gw[j]), mx_hi(gw[j]));
+            const float2 u2 = make_float2(mx_lo(uw[j]), mx_hi(uw[j]));
+            const float s0 = __fdividef(1.f, 1.f + __expf(-g2.x)), s1 = __fdividef(1.f, 1.f + __expf(-g2.y));
+            og[j] = pack_bf16(d2.x * u2.x * s0 * (1.f + g2.x * (1.f - s0)), d2.y * u2.y * s1 * (1.f + g2.y * (1.f - s1)));
+            ou[j] = pack_bf16(d2.x * g2.x * s0, d2.y * g2.y * s1);
+        }
+        const uint4 vg = make_uint4(og[0], og[1], og[2], og[3]), vu = make_uint4(ou[0], ou[1], ou[2], ou[3]);
+        const int se_g = mx_block_exp(vg), se_u = mx_block_exp(vu);
+        if (sub + 16 * i < n_rows) {
+            const long long to = at + 32ll * i * iv;
+            dgu[to] = vg;
+            dgu[to + iv] = vu;
+            codes[to] = mx_codes8(vg, se_g);
+            codes[to + iv] = mx_codes8(vu, se_u);
+        }
+        if ((l16 & 3) == 0) {
+            sf[0][(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se_g + 127);
+            sf[1][(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se_u + 127);
+        }
     }
+    __syncthreads();
+    const int half = threadIdx.x >> 5, r = threadIdx.x & 31;   // a warp per half of the columns
+    if (half < 2 && r < n_rows)
+        scales[(long long)(half * k_tiles + kt) * rows + row0 + r] = reinterpret_cast<const uint32_t*>(sf[half])[r];
 }
 
 // ---- quantisers along the rows of a row-major operand (codes stored transposed) ----
@@ -1154,10 +1160,10 @@ __device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long
     uint32_t m = 0u;
 #pragma unroll
     for (int j = 0; j < 32; ++j) m = mx_abs_max(m, v[j] & 0x7fff7fffu);
+    const int exps[2] = {mx_scale_exp(mx_lo(m)), mx_scale_exp(mx_hi(m))};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int se = mx_scale_exp(h ? mx_hi(m) : mx_lo(m));
-        const float inv = mx_inv_scale(se);
+        const float inv = mx_inv_scale(exps[h]);
         uint32_t out[8];
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
@@ -1169,7 +1175,7 @@ __device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long
         uint4* to = reinterpret_cast<uint4*>(dst + (2 * pair + h) * dst_ld + block * 32);
         to[0] = make_uint4(out[0], out[1], out[2], out[3]);
         to[1] = make_uint4(out[4], out[5], out[6], out[7]);
-        sf[(2 * pair + h) * 4 + block] = (uint8_t)(se + 127);
+        sf[(2 * pair + h) * 4 + block] = (uint8_t)(exps[h] + 127);
     }
     __syncthreads();
 }
@@ -1300,22 +1306,17 @@ int launch_mx_quantize_w_transposed(int E, int k, int n, int n_total, int n_off,
 }
 
 int launch_mx_swiglu_quantize(long long rows, int I, const bf16* gu, bf16* h_act, uint8_t* codes, uint8_t* scales, cudaStream_t s) {
-    const long long units = rows * (I / 128);
-    long long blocks = (units + 15) / 16;   // 8 warps x 2 units per block and pass
-    const long long cap = (long long)sm_count() * 32;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
+    const long long blocks = (rows + MX_SWIGLU_ROWS - 1) / MX_SWIGLU_ROWS * (I / 128);
     return launch_streaming(mx_swiglu_quantize_kernel, (unsigned)blocks, s, reinterpret_cast<const uint4*>(gu), rows, I,
-                            reinterpret_cast<uint4*>(h_act), reinterpret_cast<uint2*>(codes),
-                            reinterpret_cast<uint32_t*>(scales));
+                            reinterpret_cast<uint4*>(h_act), reinterpret_cast<uint2*>(codes), reinterpret_cast<uint32_t*>(scales));
 }
 
 int launch_mx_swiglu_bwd_quantize(long long rows, int I, const bf16* dh_act, const bf16* gu, bf16* dgu, uint8_t* codes,
                                   uint8_t* scales, cudaStream_t s) {
-    const long long total = rows * (I / 8);
-    return launch_streaming(mx_swiglu_bwd_quantize_kernel, (unsigned)((total + 255) / 256), s,
-                            reinterpret_cast<const uint4*>(dh_act), reinterpret_cast<const uint4*>(gu), rows, I,
-                            reinterpret_cast<uint4*>(dgu), reinterpret_cast<uint2*>(codes), reinterpret_cast<uint32_t*>(scales));
+    const long long blocks = (rows + MX_SWIGLU_BWD_ROWS - 1) / MX_SWIGLU_BWD_ROWS * (I / 128);
+    return launch_streaming(mx_swiglu_bwd_quantize_kernel, (unsigned)blocks, s, reinterpret_cast<const uint4*>(dh_act),
+                            reinterpret_cast<const uint4*>(gu), rows, I, reinterpret_cast<uint4*>(dgu), reinterpret_cast<uint2*>(codes),
+                            reinterpret_cast<uint32_t*>(scales));
 }
 
 // w [E * n_feat, k] -> columns [k_off, k_off + k) of the codes [E * n_feat, k_total] and the matching scale slices
