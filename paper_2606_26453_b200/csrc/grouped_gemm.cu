@@ -37,7 +37,7 @@
 //     side of the MMA, the expert's rows on the N side, any tile height that is a multiple of 16)
 //     and, for the SwiGLU forward, half-height last tiles (FWD_SWIGLU_H: M = 128 over the pair).
 //   contraction-ragged (wgrad; the paper's dW1_e = X_e^T G_e): the expert's rows are the
-//     contraction.  The last K block issues only ceil(rem/16) MMAs (guard predicates) and the < 16
+//     contraction.  The last K block issues only ceil(rem/16) MMAs and the < 16
 //     surplus rows are zeroed in shared memory first, by the tail-fix warp of each CTA (warp 10 in the
 //     first, warp 1 in the second); an expert without rows gets a zero tile.
 //
@@ -1121,10 +1121,10 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
                       const int32_t* offsets, bf16* h_act, bf16* gu, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     const bool pair = use_pairs_for_swiglu(d);
-    // pair mode with small experts (fewer than 512 rows on average): an expert's last <= 128 rows run as a half-height
+    // pair mode with small experts (use_swapped: fewer than 1600 rows on average): an expert's last <= 128 rows run as a half-height
     // tile; that takes one-chunk weight boxes (a half-height tile mixes gate and up chunks per CTA) and a second A map
     // with a 64-row box.  With larger experts the padding is small and the two-chunk boxes (one load less per stage)
-    // are 2-4 % faster.
+    // were 2-4 % faster (at 768 / 1024 / 1536 rows the half-height tiles are 3 / 3 / 1 % faster).
     const bool half_tiles = pair && use_swapped(d);
     CUtensorMap a, ah, b0, b1, o0, o1;
     if (!make_map(&a, x_perm, d.H, R, BK, BM) || !make_map(&ah, x_perm, d.H, R, BK, BM / 2) ||

@@ -471,12 +471,13 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 //   warp 2      activation scales of this CTA's 128 rows
 //   warps 3..10 epilogue: 32-row slab x every other 32-column block (a 16-column remainder: plain stores)
 //   warp 11     first CTA: issues the scale copies (smem -> tensor memory) of each stage
-// What bounds it (cycle counters, throw-away builds): every tcgen05 instruction costs its issuing thread 60-85 cycles
-// whatever its size, so a K slice (wait, four MMAs, commit) takes the MMA warp ~470 cycles -- more than the ~420 the
-// tensor pipe needs for four N = 208 MMAs.  With the three scale copies in the same thread it was ~770; with two or four
-// scale slots the chain MMA -> stage released -> copies -> MMA set the pace instead (~510).  In the full kernel a slice
-// takes ~590 cycles: operand reads by the tensor core and fills by the TMA unit together ask shared memory for ~140 bytes
-// per cycle at this tile width (halving the waits and commits per slice changed nothing).
+// What bounds it (cycle counters, throw-away builds, before the issuing roles ran on uniform values): every tcgen05
+// instruction cost its issuing thread 60-85 cycles whatever its size, so a K slice (wait, four MMAs, commit) took the MMA
+// warp ~470 cycles -- more than the ~420 the tensor pipe needs for four N = 208 MMAs.  With the three scale copies in the
+// same thread it was ~770; with two or four scale slots the chain MMA -> stage released -> copies -> MMA set the pace
+// instead (~510).  In the full kernel a slice took ~590 cycles: operand reads by the tensor core and fills by the TMA unit
+// together ask shared memory for ~140 bytes per cycle at this tile width (halving the waits and commits per slice changed
+// nothing).  Uniform issuing took 6-9 % off (see the MMA issuer); the largest shapes now run into the power cap.
 constexpr int MXP_NT = 208;                 // tile columns over the pair
 constexpr int MXP_ROWS = 2 * MX_BM;         // tile rows over the pair
 constexpr int MXP_STAGES = 6;
