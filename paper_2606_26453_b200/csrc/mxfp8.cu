@@ -99,6 +99,8 @@ struct MxGeo {
     static int smem_bytes(int E) {
         return STAGES * STAGE_BYTES + MX_STAGING_BYTES + 1024 + (int)sizeof(MxCtl) + 2 * (E + 1) * (int)sizeof(int32_t);
     }
+    // an SM has 228 KB of shared memory, of which every CTA costs 1 KB more than it asks for
+    static bool all_ctas_fit(int E) { return CTAS * (smem_bytes(E) + 1024) <= 228 * 1024; }
     static_assert(STAGES <= MX_MAX_STAGES && STAGE_BYTES % 1024 == 0 && SF_COL0 + STAGES * 8 <= TMEM_COLS, "stage layout");
 };
 
@@ -177,7 +179,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* tiles_ptr = smem_raw + (tiles_base - smem_u32(smem_raw));
     MxCtl* ctl = reinterpret_cast<MxCtl*>(tiles_ptr + MX_STAGES * MX_STAGE_BYTES + MX_STAGING_BYTES);
-    int32_t* offs = reinterpret_cast<int32_t*>(ctl + 1);   // sized by E: two CTAs have to fit an SM
+    int32_t* offs = reinterpret_cast<int32_t*>(ctl + 1);   // sized by E: up to 486 experts two CTAs fit an SM
     int32_t* tile_prefix = offs + p.E + 1;
     volatile int* abort_flag = &ctl->abort_flag;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, and known to be)
@@ -1401,7 +1403,12 @@ constexpr long long kMxPairRows = 256;
 // 715 -> 650 us (6.9 TB/s).  128 experts, 768 x 2048, down projection, rows per expert 32: 47 -> 44 us, 64: 51 -> 47 us,
 // 94: 51 -> 55 us -- a second tile per expert reads the expert's weights again, from L2.  Tiles of 32 rows lost to
 // tiles of 64 everywhere but below 4 rows per expert (N = 32 makes the MMAs no cheaper to issue).
+// Not with so many experts (487 and more) that two CTAs and their tables no longer fit an SM: the second half of the grid
+// would wait for the first, and one CTA with four stages keeps less in flight than one with six.  Down projection, 1024 x 512,
+// swapped with one CTA per SM against this kernel unswapped: 512 experts of 4 rows 76 against 55 us, of 64 rows 108 against
+// 68 us, 1024 experts of 64 rows under a Zipf load 237 against 154 us; 480 experts of 64 rows, two CTAs per SM, 62 against 69 us.
 constexpr long long kMxSwappedRows = 64;
+static bool mx_single_swapped(long long R, int E) { return R <= kMxSwappedRows * E && MxGeo<64>::all_ctas_fit(E); }
 
 static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
                                const uint8_t* b_codes, const uint8_t* b_scales_pair, const int32_t* offsets, bf16* out,
@@ -1486,8 +1493,17 @@ int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes
         return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales + mx_w_scale_single_bytes(E, n_feat, k),
                                    offsets, out, s);
     const MxSingleArgs args = {R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out};
-    if (R <= kMxSwappedRows * E) return launch_mx_gemm_single<64>(args, s);
-    return launch_mx_gemm_single<128>(args, s);
+    return mx_single_swapped(R, E) ? launch_mx_gemm_single<64>(args, s) : launch_mx_gemm_single<128>(args, s);
 }
+
+#ifdef MOE_TEST_HOOKS
+// Test-only build: CTAs per SM that the single-CTA kernel is launched with for R rows of E experts, and the shared memory of one.
+// (The occupancy query is no help: it reports one CTA per SM for any kernel that allocates tensor memory.)
+extern "C" void moe_test_mx_single_ctas(int R, int E, int* ctas, int* smem) {
+    const bool swapped = mx_single_swapped(R, E);
+    *ctas = swapped ? MxGeo<64>::CTAS : MxGeo<128>::CTAS;
+    *smem = swapped ? MxGeo<64>::smem_bytes(E) : MxGeo<128>::smem_bytes(E);
+}
+#endif
 
 }  // namespace moe

@@ -3,12 +3,14 @@
 
 Tolerance: the per-call bound of the other FP8 GEMM tests (exact products of the dequantised operands, fp32 accumulation,
 one rounding to bf16)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 from oracle import moe_oracle as O
-from paper_2606_26453_b200 import workloads as W
+from paper_2606_26453_b200 import build, workloads as W
 from tests import helpers as Hh
 
 pytestmark = pytest.mark.gpu
@@ -21,6 +23,8 @@ CASES = {
     "at_the_border": [64, 60, 68],                                     # 64 rows per expert: the last of the swapped form
     "past_the_border": [64, 60, 69],                                   # the first of the other
     "unswapped_edges": [128, 127, 129, 31, 255, 1],
+    "most_experts_of_the_swapped_form": [1] * 450 + [0] * 35 + [70],
+    "more_experts": [1] * 450 + [0] * 36 + [70],                       # unswapped from here on
     "most_experts": [1] * 1000 + [0] * 23 + [70],
 }
 
@@ -48,3 +52,16 @@ def test_small_batches(name):
     assert B.moe_device_status() == 0
     assert bool(torch.isnan(out[R:]).all())
     Hh.assert_close(Hh.to_np64(out[:R]), O.down_mxfp8(h, w, offsets), name, rel_fro=Hh.PER_CALL_FROBENIUS)
+
+
+@pytest.mark.parametrize("E", [1, 8, 486, 487, 512, 1024])
+@pytest.mark.parametrize("rows", [1, 64, 100])
+def test_every_launched_cta_fits_its_sm(E, rows):
+    """The kernel runs over a tile list that is dealt out by CTA: a CTA that had to wait for another one's SM would double the
+    duration.  The tables grow with the experts, so the form with two CTAs per SM has a largest expert count."""
+    lib = ctypes.CDLL(build.build_library(waittest=True))
+    ctas, smem = ctypes.c_int(), ctypes.c_int()
+    lib.moe_test_mx_single_ctas(rows * E, E, ctypes.byref(ctas), ctypes.byref(smem))
+    per_sm = torch.cuda.get_device_properties(0).shared_memory_per_multiprocessor
+    assert ctas.value * (smem.value + 1024) <= per_sm                  # 1 KB of every CTA is the system's
+    assert ctas.value == (2 if rows <= 64 and E <= 486 else 1)
