@@ -45,13 +45,22 @@ def test_special_values(rows):
     assert np.array_equal(_act_scales_from_layout(s.cpu().numpy(), rows, n), scales)
 
 
-@pytest.mark.parametrize("E", [1, 2, 127, 1023, 1024])
-def test_token_quantiser_expert_scan(E):
-    from paper_2606_26453_b200 import binding as B
+def _mixed_counts(E):
     rng = np.random.default_rng(E)
     counts = rng.integers(0, 3, size=E)
     counts[rng.integers(0, E)] = 129
     counts[-1] = 31
+    return counts
+
+
+# ... and rows that need as many slices as there are rows, the most there can be: one row per expert, one row in all
+@pytest.mark.parametrize("counts", [_mixed_counts(E) for E in (1, 2, 127, 1023, 1024)] +
+                         [np.ones(130, int), np.ones(1024, int), np.eye(1, 300, 299, dtype=int)[0], np.eye(1, 1024, 0, dtype=int)[0]],
+                         ids=["E1", "E2", "E127", "E1023", "E1024", "one_each", "one_each_of_1024", "last_only", "first_only"])
+def test_token_quantiser_expert_scan(counts):
+    from paper_2606_26453_b200 import binding as B
+    E = counts.size
+    rng = np.random.default_rng(E)
     offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
     R, ld, col0, n = int(offsets[-1]), 384, 8, 256
     x = W.round_to_bf16(rng.standard_normal((R, ld)).astype(np.float32))
