@@ -1092,7 +1092,7 @@ int launch(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, c
                             o1, x, p);
 }
 
-constexpr long long kSwappedFusedRows = 512;
+bool rows_per_expert_below(const moe_dims_t& d, long long rows) { return (long long)d.T * d.K < rows * d.E; }
 // The plain row-ragged GEMMs (down forward, down dgrad, gate/up dgrad) run with swapped operand roles -- always as
 // CTA pairs: 256 output features x up to 256 rows per tile -- when experts hold fewer than 1600 rows on average: there the
 // fixed 256-row tiles lose half a tile per expert to padding (12 % of the tensor work at 1024 rows).  Down / down dgrad /
@@ -1101,11 +1101,23 @@ constexpr long long kSwappedFusedRows = 512;
 //   1024  (16 experts, 4096 x 4096)   385 / 386 / 810 against 358 / 357 / 759 us
 //   1536  (64 experts, 2048 x 1408)   384 / 418 / 780 against 374 / 403 / 751 us
 //   2048  (8 experts, 4096 x 14336)  1332 / 1250 / 2731 against 1328 / 1226 / 2956 us
-// With larger experts the padding is small and the fixed-height tiles have fewer MMAs to issue.
-bool use_swapped(const moe_dims_t& d) { return (long long)d.T * d.K < 1600ll * d.E; }
+// With larger experts the padding is small and the fixed-height tiles have fewer MMAs to issue.  The line holds for Zipf and
+// Dirichlet loads with the same averages: at 768 of them (64 experts, 2048 x 1408) 285 / 308 / 552 against 269 / 290 / 521 us
+// under the first, 1500 (16 experts, 4096 x 4096) 697 / 692 / 1515 against 689 / 694 / 1437 us under the second.
+// A contraction of fewer than 512 elements is over before the swapped form's transposed epilogue, and the line lies at 512
+// rows: down dgrad of 16 experts to 8192 features, fixed against swapped, contraction 256 at 768 / 1100 / 1500 rows
+// 75 / 104 / 130 against 85 / 115 / 143 us, 384 at 768 / 1500 rows 98 / 162 against 106 / 174 us; 512 at 768 / 1100 rows
+// 113 / 157 against 120 / 153 us and, of 32 experts to 2048 features, 60 / 83 against 62 / 84 us.
+bool use_swapped(const moe_dims_t& d, int contraction) { return rows_per_expert_below(d, contraction < 512 ? 512 : 1600); }
 // The down dgrad with the SwiGLU backward in its epilogue: there the swapped form also transposes the two blocks it fetches,
-// and that outlasts short contractions, so the line lies lower.
-bool use_swapped_fused(const moe_dims_t& d) { return (long long)d.T * d.K < kSwappedFusedRows * d.E; }
+// and that outlasts contractions of 2048, so the line lies at 512 rows.  Fixed against swapped at 512 / 768 / 1024 / 1536 rows:
+//   64 experts, 2048 x 1408   249 / 312 / 443 /  621 against 240 / 343 / 450 /  639 us
+//   16 experts, 4096 x 4096   324 / 456 / 564 /  776 against 304 / 411 / 520 /  756 us
+//   8 experts, 4096 x 14336   588 / 794 / 946 / 1099 against 502 / 712 / 885 / 1074 us
+// (a contraction of 4096 would bear a higher line).
+bool use_swapped_fused(const moe_dims_t& d) { return rows_per_expert_below(d, 512); }
+// Half-height last tiles of the SwiGLU forward, see launch_gateup_fwd.
+bool use_half_tiles(const moe_dims_t& d) { return rows_per_expert_below(d, 1600); }
 // The SwiGLU forward has no swapped form (measured slower: two accumulators per tile).  Its pair kernel runs an
 // expert's last <= 128 rows as a half-height tile, which makes pairs worthwhile from 320 rows per expert on average.
 constexpr long long kSwigluPairRows = 320;
@@ -1121,11 +1133,13 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
                       const int32_t* offsets, bf16* h_act, bf16* gu, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     const bool pair = use_pairs_for_swiglu(d);
-    // pair mode with small experts (use_swapped: fewer than 1600 rows on average): an expert's last <= 128 rows run as a half-height
+    // pair mode with small experts (fewer than 1600 rows on average): an expert's last <= 128 rows run as a half-height
     // tile; that takes one-chunk weight boxes (a half-height tile mixes gate and up chunks per CTA) and a second A map
     // with a 64-row box.  With larger experts the padding is small and the two-chunk boxes (one load less per stage)
-    // were 2-4 % faster (at 768 / 1024 / 1536 rows the half-height tiles are 3 / 3 / 1 % faster).
-    const bool half_tiles = pair && use_swapped(d);
+    // were 2-4 % faster (at 768 / 1024 / 1536 rows the half-height tiles are 3 / 3 / 1 %
+    // faster under even loads; under Zipf and Dirichlet loads with averages of 512 to 1500 rows 0-4 % slower: 16 experts,
+    // 4096 x 4096, 768 rows 795 -> 820 us).
+    const bool half_tiles = pair && use_half_tiles(d);
     CUtensorMap a, ah, b0, b1, o0, o1;
     if (!make_map(&a, x_perm, d.H, R, BK, BM) || !make_map(&ah, x_perm, d.H, R, BK, BM / 2) ||
         !make_map_mn(&b0, w_gate, d.I, (uint64_t)d.E * d.H, half_tiles ? 1 : 2) ||
@@ -1144,7 +1158,7 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
 int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, const int32_t* offsets,
                     bf16* y_perm, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
-    if (use_swapped(d)) {
+    if (use_swapped(d, d.I)) {
         // swapped roles: M side = w_down tile (128 features of H, MN-major), N side = rows of h_act (64-row boxes)
         const int feats = 2 * SWAP_FEATS;   // a CTA pair's tile
         const uint32_t box = 32;            // row boxes of 32 / 64 / 128 rows per CTA
@@ -1176,7 +1190,7 @@ int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, 
 int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const int32_t* offsets,
                       bf16* dh_act, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
-    if (use_swapped(d)) {
+    if (use_swapped(d, d.H)) {
         // swapped roles: M side = w_down tile (128 features of I, K-major), N side = rows of dy_perm
         const int feats = 2 * SWAP_FEATS;   // a CTA pair's tile
         const uint32_t box = 32;            // row boxes of 32 / 64 / 128 rows per CTA
@@ -1235,7 +1249,7 @@ int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const
 int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate, const bf16* w_up,
                         const int32_t* offsets, bf16* dx_perm, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
-    if (use_swapped(d)) {
+    if (use_swapped(d, 2 * d.I)) {
         const int feats = 2 * SWAP_FEATS;   // a CTA pair's tile
         const uint32_t box = 32;            // row boxes of 32 / 64 / 128 rows per CTA
         CUtensorMap a, a2, a1, b0, b1, o0;
