@@ -3,7 +3,8 @@
 The fixed parity cases pin the tile edges one knows about; these draw dimensions (multiples of 64), expert counts,
 top-k and per-expert row counts (with empty experts, single rows, tile-boundary sizes and one large expert mixed in)
 so that every launch-shape decision of the library -- single-CTA tiles, CTA pairs, half-height last tiles, swapped
-operand roles, weight-gradient pairs -- is crossed at sizes nobody picked by hand."""
+operand roles, weight-gradient pairs and, in the draws of large experts, fixed-height tiles -- is crossed at sizes nobody
+picked by hand."""
 import numpy as np
 import pytest
 
@@ -43,13 +44,38 @@ def draw_case(seed):
     return counts, K, H, I
 
 
+def draw_large_case(seed):
+    """Averages on both sides of 1600 rows per expert, where the fixed-height tiles of the plain GEMMs take over (widths of 512
+    and more; below, they do from 512 rows): one expert without rows, one with a single row, the rest around the level."""
+    rng = np.random.default_rng(2000 + seed)
+    H, I = 64 * int(rng.integers(4, 11)), 64 * int(rng.integers(4, 11))
+    E = int(rng.integers(4, 7))
+    average = [1500, 1620, 1700, 2200][seed % 4]
+    counts = np.maximum(1, rng.normal(1.0, 0.2, size=E))
+    empty, single = rng.choice(E, size=2, replace=False)
+    counts[[empty, single]] = 0
+    counts = (counts / counts.sum() * (average * E - 1)).astype(np.int64)
+    counts[single] = 1
+    total = int(counts.sum())
+    return counts, 2 if total % 2 == 0 and int(counts.max()) <= total // 2 else 1, H, I
+
+
 @pytest.mark.parametrize("seed", list(range(48)))
 def test_random_layer_against_oracle(seed):
-    from paper_2606_26453_b200 import binding as B
-    B.load_library()
     counts, K, H, I = draw_case(seed)
     if int(counts.sum()) % K or int(counts.max()) > int(counts.sum()) // K:
         pytest.skip("drawn counts cannot be routed without repeating an expert in a token")
+    check_layer(counts, K, H, I, seed)
+
+
+@pytest.mark.parametrize("seed", list(range(12)))
+def test_random_layer_of_large_experts_against_oracle(seed):
+    check_layer(*draw_large_case(seed), seed)
+
+
+def check_layer(counts, K, H, I, seed):
+    from paper_2606_26453_b200 import binding as B
+    B.load_library()
     cfg, host = Hh.ragged_workload(list(counts), K=K, H=H, I=I, seed=100 + seed)
     ref = O.layer_fwd_bwd(host["X"], host["topk_idx"], host["topk_w"], host["W_gate"], host["W_up"], host["W_down"],
                           host["dY"])
@@ -69,7 +95,7 @@ def test_random_layer_against_oracle(seed):
 @pytest.mark.parametrize("H,I,counts,K", [
     (1408, 2880, [300, 1, 129, 430, 0], 2),          # the real widths: 1408 = 5.5 x 256, 2880 = 45 x 64 (partial column tiles)
     (2880, 1408, [40, 700, 1, 0, 259], 1),
-    (2880, 2880, [520, 528, 8], 2),               # rows per expert above the pair / fixed-tile thresholds
+    (2880, 2880, [520, 528, 8], 2),               # rows per expert above the pair threshold of the SwiGLU forward
     (1408, 1408, [255, 257, 0, 600, 88], 2),
 ])
 def test_real_widths_at_small_row_counts(H, I, counts, K):

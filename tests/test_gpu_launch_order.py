@@ -1,7 +1,8 @@
 """The kernels of one stream start before their predecessors have finished (programmatic dependent launch).  Back to back
 without any synchronisation, and replayed from a CUDA graph, a step has to give bit for bit what it gives when the
 device is idle before every call; every buffer is reused from step to step, so that a kernel which read too early or
-wrote too early would meet the other step's values."""
+wrote too early would meet the other step's values.  The first test looks at the results of every step, with plain copies
+that then stand between the steps; the second one has nothing between them and every call of the library in them."""
 import pytest
 import torch
 
@@ -92,4 +93,90 @@ def test_back_to_back_and_replayed_steps_equal_synchronised_ones(shape):
         got = step.results()
         for a, b in zip(got, want[i % 2]):
             assert torch.equal(a, b)
+    assert B.moe_device_status() == 0
+
+
+class _EveryCall(_Step):
+    """The whole of the library's calls on one routing: the layer with the fused down dgrad, a second route-permute that takes
+    the layer's own output (the combine writes it right ahead of the permute), and the FP8 training step with both kinds of
+    weight gradients.  Nothing but these calls runs between one step and the next."""
+
+    def __init__(self, B, T, H, I, E, K):
+        super().__init__(B, T, H, I, E, K)
+        R, d = T * K, self.d
+        u8 = lambda n: torch.zeros(n, dtype=torch.uint8, device="cuda")
+        bf = lambda *s: torch.zeros(s, dtype=torch.bfloat16, device="cuda")
+        i32 = lambda n: torch.zeros(n, dtype=torch.int32, device="cuda")
+        self.again = [bf(R, H), i32(E), i32(E + 1), i32(R), i32(R)]     # x_perm, counts, offsets, row_to_pair, pair_to_row
+        self.static = [torch.zeros_like(t) for t in self.again]
+        self.dyq = u8(R * H), u8(B.moe_mxfp8_dy_scale_bytes(d))
+        self.dguq = u8(R * 2 * I), u8(B.moe_mxfp8_dgu_scale_bytes(d))
+        self.ddq = u8(E * I * H), u8(B.moe_mxfp8_w_down_dgrad_scale_bytes(d))
+        self.gdq = u8(E * H * 2 * I), u8(B.moe_mxfp8_w_gateup_dgrad_scale_bytes(d))
+        tok = lambda n: (u8(B.moe_mxfp8_tokens_codes_bytes(d, n)), u8(B.moe_mxfp8_tokens_scale_bytes(d, n)))
+        self.h_tok, self.dy_tok, self.x_tok, self.dg_tok, self.du_tok = tok(I), tok(H), tok(H), tok(I), tok(I)
+        self.dh8, self.dgu8, self.dx8, self.dgu_fused = bf(R, I), bf(R, 2 * I), bf(R, H), bf(R, 2 * I)
+        self.dw8 = bf(E, I, H), bf(E, H, I), bf(E, H, I)
+
+    def calls(self, v):
+        B, b, d, H, I = self.B, self.b, self.d, self.d.H, self.d.I
+        forward = super().calls(v)
+        return forward[:5] + [
+            lambda: B.moe_permute(d, b.y, self.idx, *self.again, b.workspace),
+            lambda: B.moe_permute_static_scratch(d, b.y, self.idx, *self.static)] + forward[5:7] + [
+            lambda: B.moe_grouped_gemm_down_dgrad_swiglu_bwd(d, b.dy_perm, v["wd"], b.gu, b.offsets, self.dgu_fused)] + forward[7:] + [
+            lambda: B.moe_mxfp8_quantize_w_down_dgrad(d, v["wd"], *self.ddq),
+            lambda: B.moe_mxfp8_quantize_w_gateup_dgrad(d, v["wg"], v["wu"], *self.gdq),
+            lambda: B.moe_mxfp8_quantize_dy_perm(d, b.dy_perm, *self.dyq),
+            lambda: B.moe_grouped_gemm_down_dgrad_mxfp8(d, *self.dyq, *self.ddq, b.offsets, self.dh8),
+            lambda: B.moe_swiglu_bwd_mxfp8(d, self.dh8, self.gu8, self.dgu8, *self.dguq),
+            lambda: B.moe_grouped_gemm_gateup_dgrad_mxfp8(d, *self.dguq, *self.gdq, b.offsets, self.dx8),
+            lambda: B.moe_mxfp8_quantize_tokens(d, self.h8, I, 0, I, b.offsets, *self.h_tok),
+            lambda: B.moe_mxfp8_quantize_tokens(d, b.dy_perm, H, 0, H, b.offsets, *self.dy_tok),
+            lambda: B.moe_grouped_gemm_down_wgrad_mxfp8(d, *self.h_tok, *self.dy_tok, self.dw8[0]),
+            lambda: B.moe_mxfp8_quantize_tokens(d, b.x_perm, H, 0, H, b.offsets, *self.x_tok),
+            lambda: B.moe_mxfp8_quantize_tokens(d, self.dgu8, 2 * I, 0, I, b.offsets, *self.dg_tok),
+            lambda: B.moe_mxfp8_quantize_tokens(d, self.dgu8, 2 * I, I, I, b.offsets, *self.du_tok),
+            lambda: B.moe_grouped_gemm_gateup_wgrad_mxfp8(d, *self.x_tok, *self.dg_tok, *self.du_tok, self.dw8[1], self.dw8[2]),
+        ]
+
+    def results(self):
+        return super().results() + [t.clone() for t in (*self.again, *self.static, self.dgu_fused, self.dh8, self.dgu8, self.dx8,
+                                                        *self.dw8)]
+
+
+# the last one: 2000 rows per expert, where the plain GEMMs run fixed-height tiles; the one before: the fused call swapped
+@pytest.mark.parametrize("shape", SHAPES + [(1000, 256, 128, 8, 2), (4000, 128, 256, 4, 2)])
+def test_steps_that_follow_one_another_directly(shape):
+    from paper_2606_26453_b200 import binding as B
+    B.load_library()
+    step = _EveryCall(B, *shape)
+    sets = [_inputs(B, *shape, seed) for seed in (1, 2)]
+    want = []
+    for v in sets:
+        for call in step.calls(v):
+            call()
+            torch.cuda.synchronize()
+        want.append(step.results())
+    assert all(torch.equal(a, b) for a, b in zip(want[0][13:18], want[0][18:23]))   # the two route-permutes agree
+    for last in range(2, 8):                              # steps of alternating inputs, then a look at the last one's results
+        for i in range(last + 1):
+            for call in step.calls(sets[i % 2]):
+                call()
+        for k, (a, b) in enumerate(zip(step.results(), want[last % 2])):
+            assert torch.equal(a, b), (last, k)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graphs = []
+    for first in (0, 1):                                  # two steps per graph
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1], stream=stream):
+            for v in (sets[first], sets[1 - first]):
+                for call in step.calls(v):
+                    call()
+    for first in (0, 1, 1, 0):
+        graphs[first].replay()
+        graphs[first].replay()
+        for k, (a, b) in enumerate(zip(step.results(), want[1 - first])):
+            assert torch.equal(a, b), ("graph", first, k)
     assert B.moe_device_status() == 0

@@ -32,9 +32,12 @@ CASES = {
     # H and I multiples of 64 only (the paper's 2880 = 45 * 64): partial column tiles everywhere
     "ragged_64": lambda: Hh.ragged_workload([200, 0, 31, 290, 1], K=2, H=192, I=320, seed=4),
     "pair_64": lambda: Hh.ragged_workload([600, 540, 0, 700], K=2, H=320, I=192, seed=6),
-    # CTA-pair kernels whose last 256-row tile per expert holds 100, exactly 128, 65 and 129 rows (the second CTA's
-    # half of the tile partly or wholly past the expert's end), plus one expert of several full tiles
+    # a last 256-row tile that holds 100, exactly 128, 65 and 129 rows (the second CTA's half of the tile partly or wholly past
+    # the expert's end), plus one expert of several full tiles: here in the SwiGLU forward's half-height form and, of the plain
+    # GEMMs, in the fixed-height form of the two with a contraction below 512 ...
     "pair_half": lambda: Hh.ragged_workload([356, 640, 321, 900, 385], K=2, H=256, I=320, seed=8),
+    # ... and at 1620 rows per expert in the fixed-height form of all of them, with an expert without rows
+    "pair_full": lambda: Hh.ragged_workload([2148, 1920, 1857, 0, 2177], K=2, H=256, I=320, seed=9),
 }
 
 
@@ -476,22 +479,25 @@ def test_degenerate_shapes_end_to_end(B, T, H, I, E, K):
     Hh.assert_close(b.dtopk_w.cpu().numpy().astype(np.float64), ref["dtopk_w"], "dtopk_w")
 
 
-def test_pair_and_single_tile_shapes_agree(B):
-    """The same experts' rows run through the CTA-pair kernels (>= 512 rows per expert on average) and, split
-    over twice as many experts with duplicated weights, through the single-CTA kernels: equal outputs."""
-    counts = [700, 650, 520, 690]
-    cfg, host = Hh.ragged_workload(counts, K=2, H=256, I=256, seed=5)
+@pytest.mark.parametrize("counts,pad,width", [
+    ([700, 650, 520, 690], 4, 256),        # 640 / 320 rows per expert: fixed-height against swapped, short contractions
+    ([2000, 1500, 1700, 1600], 4, 512),    # 1700 / 850: fixed-height against swapped and half-height tiles
+    ([420, 390, 350, 440], 12, 256),       # 400 / 100: the SwiGLU forward as CTA pairs against single CTAs
+])
+def test_pair_and_single_tile_shapes_agree(B, counts, pad, width):
+    """The same experts' rows among `pad` more experts without rows: fewer rows per expert on average, so other forms of the
+    kernels; equal outputs (same arithmetic order per element)."""
+    cfg, host = Hh.ragged_workload(counts, K=2, H=width, I=width, seed=5)
     ref = O.layer_fwd_bwd(host["X"], host["topk_idx"], host["topk_w"], host["W_gate"], host["W_up"],
                           host["W_down"], host["dY"])
-    b = Hh.run_cuda_layer(Hh.device_workload(host), cfg.E)            # 640 rows per expert: pair kernels
+    b = Hh.run_cuda_layer(Hh.device_workload(host), cfg.E)
     for attr, key in FLOAT_OUTPUTS:
         Hh.assert_close(Hh.to_np64(getattr(b, attr)), ref[key], key)
-    # pad with 4 experts that get no rows: 320 rows per expert on average -> single-CTA kernels
-    pad = lambda w: np.concatenate([w, np.zeros_like(w)], axis=0)
-    host2 = dict(host, W_gate=pad(host["W_gate"]), W_up=pad(host["W_up"]), W_down=pad(host["W_down"]))
-    b2 = Hh.run_cuda_layer(Hh.device_workload(host2), 2 * cfg.E)
+    more = lambda w: np.concatenate([w, np.zeros((pad, *w.shape[1:]), w.dtype)], axis=0)
+    host2 = dict(host, W_gate=more(host["W_gate"]), W_up=more(host["W_up"]), W_down=more(host["W_down"]))
+    b2 = Hh.run_cuda_layer(Hh.device_workload(host2), cfg.E + pad)
     for attr in ("y", "dx", "h_act", "gu", "y_perm", "dh_act", "dgu", "dx_perm"):
-        assert torch.equal(getattr(b, attr), getattr(b2, attr)), attr   # same arithmetic order per element
+        assert torch.equal(getattr(b, attr), getattr(b2, attr)), attr
     for attr in ("dw_gate", "dw_up", "dw_down"):
         assert torch.equal(getattr(b, attr), getattr(b2, attr)[:cfg.E]), attr
         assert not bool(getattr(b2, attr)[cfg.E:].any())

@@ -65,10 +65,12 @@ def test_a_wait_that_runs_out_reports_and_leaves_the_context_usable():
                     rel_fro=Hh.PER_CALL_FROBENIUS)
 
 
-@pytest.mark.parametrize("counts", [[60, 70, 0, 62], [700, 513, 64]], ids=["single_cta", "cta_pair"])
+@pytest.mark.parametrize("counts", [[60, 70, 0, 62], [150, 130, 0, 212], [700, 513, 64]],
+                         ids=["single_cta_swapped", "single_cta", "cta_pair"])
 def test_block_scaled_kernels_give_up_the_same_way(counts):
-    """The same for the two block-scaled FP8 GEMM kernels (more roles wait there: the scale-gather warps, the scale-copy
-    warp of the pair kernel): every wait runs out, the status word reads MOE_ERR_TIMEOUT, the next call is correct."""
+    """The same for the block-scaled FP8 GEMM kernels (more roles wait there: the scale-gather and scale-copy warps), both
+    forms of the single-CTA kernel among them: every wait runs out, the status word reads MOE_ERR_TIMEOUT, the next call
+    is correct."""
     from paper_2606_26453_b200 import binding as B
     B.load_library()
     lib = ctypes.CDLL(build.build_library(waittest=True))
