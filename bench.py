@@ -8,11 +8,12 @@ unpermute-combine, and the four backward calls) over one batch of seeded synthet
 headline workload is the largest of the five configurations ("imbalanced"); it is timed for at
 least one second (the number of timed steps is raised above --steps when needed, and the line says
 how many were timed).  The metric is whole-layer throughput in TFLOP/s on the algorithmic work
-18*R*H*I; the JSON line also carries the grouped-GEMM-only throughput, the permute bandwidth, a
-roofline object for the dominant kernel, an end-to-end number through the host-buffer entry point,
-the same step run back to back for two seconds, and the fp64 oracle timed on the host cores -- all
-on that workload.  The other workloads follow in `other_configs`, each timed for at least half a
-second with its own roofline object.  With N > 1 (torchrun) every rank runs an independent replica of the
+18*R*H*I; the JSON line on stdout also carries the grouped-GEMM-only throughput, the permute bandwidth, a
+roofline object for the dominant kernel, an end-to-end number through the host-buffer entry point and the
+fp64 oracle timed on the host cores -- all on that workload -- and step time and throughput of the other
+workloads in `other_configs`.  A second, long JSON line goes to stderr: per-call times of every workload, the same
+step run back to back for two seconds, the fused and the block-scaled FP8 forms, router, permute alone and the
+calibration runs.  With N > 1 (torchrun) every rank runs an independent replica of the
 same workload: the layer is single-GPU by design, there is no collective on the data path.
 `--impl reference` times the CPU oracle alone on a bounded sample of the same workload.
 """
@@ -873,6 +874,27 @@ def aggregate_tflops(world, flops_per_replica, ms_per_step):
     return world * flops_per_replica / (ms_per_step * 1e-3) / 1e12
 
 
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "steps_requested", "warmup", "ms_per_step", "higher_is_better",
+                 "scaling", "vs_baseline", "dtype", "data", "config", "clocks", "e2e", "gpu_launches", "gemm_tflops",
+                 "permute_gbs", "pct_of_dense_bf16_peak_nominal", "peaks")
+HEADLINE_ROOFLINE_KEYS = ("bound", "kernel", "achieved", "peak", "peak_kind", "unit", "frac", "frac_of_sustained",
+                          "flops_per_launch", "avg_launch_ms", "traffic")
+
+
+def headline(line):
+    """The one line for stdout: the headline workload's figures and a pair of numbers for each other workload, short enough to
+    survive a log that keeps the last few thousand characters.  Everything, per call and per workload, goes to stderr."""
+    out = {k: line[k] for k in HEADLINE_KEYS if k in line}
+    out["e2e"] = {k: v for k, v in line["e2e"].items() if k != "note"}
+    out["roofline"] = {k: line["roofline"][k] for k in HEADLINE_ROOFLINE_KEYS}
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = line["cpu_baseline"]
+    if "other_configs" in line:
+        out["other_configs"] = {c["workload"]: {"ms_per_step": round(c["ms_per_step"], 4), "layer_tflops": round(c["layer_tflops"], 1)}
+                                for c in line["other_configs"]}
+    return out
+
+
 def run_ours(args):
     world = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
@@ -981,7 +1003,8 @@ def run_ours(args):
         if wl_host is not None:
             line["cpu_baseline"] = cpu_baseline(cfg, wl_host, min(args.ref_tokens, cfg.T))
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
