@@ -34,11 +34,8 @@ int sm_count();
 //     set-up, and the blocks of a streaming kernel then settle beside the running GEMM: down dgrad and SwiGLU backward of
 //     24576 x 1408 together (contraction of 256) take 103 us that way, 91 us with the call behind the barrier, 95 us in plain
 //     stream order.  (Presumably such SMs keep the GEMM's split of their memory, with little L1 for loads in flight.)
-//   - Streaming kernels leave it out: a block that exits has triggered, and the explicit calls of a grid go through one at a
-//     time, about 1 ns each.  Combine backward of 40000 tokens of 256, a block per token: 42.7 us with the call, 37.0 without,
-//     38.9 in plain stream order; combine of 8000 tokens of 2048 from one expert each 9.5, 8.5 and 10.3 us.
 // Hides launch latency and set-up, 1.5-3 us at a kernel boundary: GEMM, streaming kernel, GEMM, streaming kernel on 1400 rows
-// of 1024 44 -> 35 us.
+// of 1024 44 -> 36 us, combine of 8000 tokens of 2048 from one expert each 10.3 -> 9.6 us.
 // Kernels that read through read-only loads, which the compiler takes to be invariant, use the form whose result must be
 // tested: the branch keeps such loads behind the wait.  (The GEMMs load their offsets through a plain pointer and everything
 // else with bulk copies or behind a barrier; they take the plain form.)

@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
                                                               int K) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (i >= total) return;
     const int t = (int)(i / hv);
     const int c = (int)(i - (long long)t * hv);
@@ -396,6 +397,7 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
 #pragma unroll
     for (int k = 0; k < KA; ++k) dot[k] = 0.f;
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     for (int c = threadIdx.x; c < hv; c += kThreads) {
         const uint4 dv = ldg16(dy + (long long)t * hv + c);
         float d[8];
@@ -457,6 +459,7 @@ __global__ void __launch_bounds__(kThreads) swiglu_bwd_kernel(const uint4* __res
                                                               uint4* __restrict__ dgu, long long total, int iv) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (i >= total) return;
     const long long r = i / iv;
     const int c = (int)(i - r * iv);

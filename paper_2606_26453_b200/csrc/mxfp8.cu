@@ -988,6 +988,7 @@ __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __re
                                                                uint8_t* __restrict__ scales, uint8_t* __restrict__ scales_pair) {
     __shared__ __align__(16) uint8_t sf[128 * 4];
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int k_tiles = n >> 7;
     const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
     const long long row0 = 128ll * row_tile;
@@ -1032,6 +1033,7 @@ __global__ void __launch_bounds__(256) mx_swiglu_quantize_kernel(const uint4* __
                                                                  uint32_t* __restrict__ scales) {
     __shared__ __align__(16) uint8_t sf[MX_SWIGLU_ROWS * 4];
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     constexpr int N = MX_SWIGLU_ROWS / 16;
     const int k_tiles = I >> 7, iv = I >> 3;
     const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
@@ -1080,6 +1082,7 @@ __global__ void __launch_bounds__(256) mx_swiglu_bwd_quantize_kernel(const uint4
                                                                      uint2* __restrict__ codes, uint32_t* __restrict__ scales) {
     __shared__ __align__(16) uint8_t sf[2][MX_SWIGLU_BWD_ROWS * 4];
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     constexpr int N = MX_SWIGLU_BWD_ROWS / 16;
     const int k_tiles = I >> 7, iv = I >> 3;
     const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
@@ -1193,6 +1196,7 @@ __global__ void __launch_bounds__(256) mx_quantize_w_transposed_kernel(const bf1
     __shared__ __align__(16) uint32_t tile[4 * MXT_BLOCK_WORDS];
     __shared__ __align__(16) uint8_t sf[128 * 4];
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int f_tiles = n >> 7, k_tiles = k >> 7;
     const int ft = blockIdx.x % f_tiles, rest = blockIdx.x / f_tiles, kt = rest % k_tiles;
     const long long e = rest / k_tiles;
@@ -1233,6 +1237,7 @@ __global__ void __launch_bounds__(256) mx_quantize_tokens_kernel(const bf16* __r
     __shared__ int32_t part[8];
     __shared__ int32_t mine[3];   // first row, rows and existence of this block's slice
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     const int f_tiles = n >> 7;
     const int f0 = (int)(blockIdx.x % (unsigned)f_tiles) * 128, slice = (int)(blockIdx.x / (unsigned)f_tiles);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -35,6 +35,7 @@ router_topk_kernel(const float* __restrict__ logits, int T, int E, int K, int32_
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (t >= T) return;
     const float* row = logits + (size_t)t * E;
     uint32_t key[VPL];
@@ -82,6 +83,7 @@ router_topk_bwd_kernel(const int32_t* __restrict__ topk_idx, const float* __rest
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
     if (t >= T) return;
     float w = 0.f, dw = 0.f;
     int idx = -1;
