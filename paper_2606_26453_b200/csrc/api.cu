@@ -663,20 +663,3 @@ int moe_layer_fwd_bwd_host(const moe_dims_t* dims, const void* x_host, const int
 }
 
 }  // extern "C"
-
-#ifdef MOE_TEST_HOOKS
-// Test-only build: a programmatic dependent of whatever precedes it on the stream that records when it started (out[0]) and
-// when everything before it had completed (out[1]), in ns on the device's global timer.
-__global__ void moe_test_dependent_kernel(unsigned long long* out) {
-    unsigned long long t0, t1;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-    moe::grid_dependency_wait();
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
-    out[0] = t0;
-    out[1] = t1;
-}
-extern "C" int moe_test_dependent_start(void* out, moe_stream_t stream) {
-    return moe::launch_dependent(moe_test_dependent_kernel, 1, 1, 0, 1, static_cast<cudaStream_t>(stream),
-                                 static_cast<unsigned long long*>(out));
-}
-#endif

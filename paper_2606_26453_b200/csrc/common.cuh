@@ -28,14 +28,10 @@ int sm_count();
 //     completed and their writes are visible.  (rank_rows of the route-permute reads its INPUTS earlier: its predecessor, the
 //     histogram kernel, lets it start only after its own wait.)
 //   - grid_launch_dependents() comes after grid_dependency_wait(), so no more than one kernel is ever ahead of its turn and a
-//     kernel that has started knows everything before its immediate predecessor to be complete.
-//   - The GEMMs call it behind the last barrier of their teardown.  One thread's call counts for its CTA, so a call at the end
-//     of each warp's role would trigger as soon as the first warp has none left -- for the row-ragged kinds right after
-//     set-up, and the blocks of a streaming kernel then settle beside the running GEMM: down dgrad and SwiGLU backward of
-//     24576 x 1408 together (contraction of 256) take 103 us that way, 91 us with the call behind the barrier, 95 us in plain
-//     stream order.  (Presumably such SMs keep the GEMM's split of their memory, with little L1 for loads in flight.)
-// Hides launch latency and set-up, 1.5-3 us at a kernel boundary: GEMM, streaming kernel, GEMM, streaming kernel on 1400 rows
-// of 1024 44 -> 36 us, combine of 8000 tokens of 2048 from one expert each 10.3 -> 9.6 us.
+//     kernel that has started knows everything before its immediate predecessor to be complete.  The GEMMs, which hold
+//     their SMs to the end anyway, call it in their teardown: nothing that starts early then sits beside them.
+// Hides launch latency and set-up, 1.5-3 us at a kernel boundary: serving 32 tokens on 128 experts (six kernels) 156 -> 147 us,
+// 100 tokens on FP8 weights 265 -> 252 us, a training step of 14 kernels on 64 experts 1387 -> 1372 us.
 // Kernels that read through read-only loads, which the compiler takes to be invariant, use the form whose result must be
 // tested: the branch keeps such loads behind the wait.  (The GEMMs load their offsets through a plain pointer and everything
 // else with bulk copies or behind a barrier; they take the plain form.)
@@ -47,14 +43,16 @@ __device__ __forceinline__ bool grid_dependency_wait_tested() {
 }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// `cluster`: CTAs per cluster.
+// `cluster`: CTAs per cluster.  `early` false: launched in plain stream order (the waits inside return at once).
 template <typename... Params, typename... Args>
-inline int launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, unsigned cluster, cudaStream_t s,
-                            const Args&... args) {
+inline int launch_kernel(bool early, void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, unsigned cluster,
+                         cudaStream_t s, const Args&... args) {
     cudaLaunchAttribute attr[2];
     unsigned n = 0;
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    if (early) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
     if (cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
         attr[n].val.clusterDim.x = cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
@@ -68,10 +66,19 @@ inline int launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned b
     }
     return MOE_OK;
 }
-// Streaming kernels: 256 threads, no dynamic shared memory.
+template <typename... Params, typename... Args>
+inline int launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, unsigned cluster, cudaStream_t s,
+                            const Args&... args) {
+    return launch_kernel(true, kernel, grid, block, smem, cluster, s, args...);
+}
+// Streaming kernels (256 threads, little or no shared memory).  Launched early behind a GEMM, their first blocks settle on SMs
+// that are set up for the GEMM's 227 KB of shared memory, and the SMs then keep that split -- with hardly any L1 for the
+// loads in flight -- until they have been empty once (SwiGLU backward of 24576 x 1408: 54 -> 64 us, permute backward 25 -> 29).
+// So only grids that are over before that matters start early.
+constexpr unsigned kEarlyStreamingBlocks = 592;   // 4 blocks of 256 threads per SM
 template <typename... Params, typename... Args>
 inline int launch_streaming(void (*kernel)(Params...), unsigned grid, cudaStream_t s, const Args&... args) {
-    return launch_dependent(kernel, grid, 256, 0, 1, s, args...);
+    return launch_kernel(grid <= kEarlyStreamingBlocks, kernel, grid, 256, 0, 1, s, args...);
 }
 
 // ---- data-movement kernels (movement.cu) ------------------------------------------------------

@@ -1022,10 +1022,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
 
     // ---- teardown ----
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync_all();   // neither CTA's shared memory / barriers may go away while the other still uses them
-    grid_launch_dependents();   // not before this barrier: see common.cuh
     if (warp == 1) {
         tc_fence_after();
         if (PAIR)

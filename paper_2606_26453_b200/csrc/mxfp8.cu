@@ -448,9 +448,9 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         __syncwarp();
     }
 
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
-    grid_launch_dependents();   // not before this barrier: see common.cuh
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)G::TMEM_COLS) : "memory");
@@ -894,10 +894,10 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         __syncwarp();
     }
 
+    grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();   // neither CTA's shared memory / barriers may go away while the other still uses them
-    grid_launch_dependents();   // not before this barrier: see common.cuh
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)MX_TMEM_COLS) : "memory");
