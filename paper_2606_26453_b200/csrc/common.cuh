@@ -34,14 +34,16 @@ int sm_count();
 //     free.  With the call behind the last barrier of the teardown steps of long GEMMs take longer, chip idle between steps:
 //     8 experts of 4096 x 14336 11.78 -> 11.89 ms, 64 experts of 4096 x 1536 under a Zipf load 22.41 -> 22.73 ms, 128 of
 //     2048 x 768 3.440 -> 3.448 ms.  (Presumably SMs that finish late get the CTAs with the fewest tiles.)
-//   - Streaming kernels call it right behind their wait, except where blocks are short: the calls of a grid go through one at
-//     a time, about 1 ns each, and a block that exits has triggered anyway (gather_sum_kernel, combine_bwd_kernel).
+//   - Streaming kernels call it right behind their wait, except where there are many short blocks: the calls of a grid go
+//     through one at a time, about 1 ns each, and a block that exits has triggered anyway (gather_sum_kernel, combine_bwd_kernel).
 // Hides launch latency and set-up, 1.5-3 us at a kernel boundary: serving 32 tokens on 128 experts (six kernels) 167 -> 148 us,
 // 100 tokens on FP8 weights 337 -> 261 us (both with what else changed since plain stream order); GEMM, streaming kernel,
 // GEMM, streaming kernel on 1400 rows of 1024 44 -> 37 us.
 // Kernels that read through read-only loads, which the compiler takes to be invariant, use the form whose result must be
 // tested: the branch keeps such loads behind the wait.  (The GEMMs load their offsets through a plain pointer and everything
 // else with bulk copies or behind a barrier; they take the plain form.)
+// A small grid of 256-thread blocks: four on each of the chip's SMs.  (Asking the device for its SMs on every launch costs 0.1 us.)
+constexpr unsigned kSmallGrid = 4 * 148;
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ bool grid_dependency_wait_tested() {
     uint32_t done;
@@ -81,10 +83,10 @@ inline int launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned b
 // Streaming kernels (256 threads, little or no shared memory).  Started early behind a GEMM their first blocks settle beside
 // it, and that slows both: down dgrad and SwiGLU backward of 24576 x 1408 together (contraction of 256) 93 -> 102 us, of
 // 131072 x 768 (contraction of 2048) 436 -> 463 us.  (Presumably such SMs keep the GEMM's split of their memory, with little
-// L1 for loads in flight.)  So only grids of at most four blocks per SM start early, which are over before that matters.
+// L1 for loads in flight.)  So only small grids start early, which are over before that matters.
 template <typename... Params, typename... Args>
 inline int launch_streaming(void (*kernel)(Params...), unsigned grid, cudaStream_t s, const Args&... args) {
-    return launch_kernel((int)grid <= 4 * sm_count(), kernel, grid, 256, 0, 1, s, args...);
+    return launch_kernel(grid <= kSmallGrid, kernel, grid, 256, 0, 1, s, args...);
 }
 
 // ---- data-movement kernels (movement.cu) ------------------------------------------------------

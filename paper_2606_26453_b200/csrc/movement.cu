@@ -326,8 +326,9 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
 
 // ------------------------------------------------------------------------------------------------
 // a4 / a8: dst[t,:] = sum_k w[t,k] * src[pair_to_row[t*K+k], :]  (w == NULL: unit weights).
-// fp32 accumulation in slot order, one rounding to bf16.  No grid_launch_dependents(): a block moves (K + 1) x 4 KB, and with
-// small K that outlasts the call by too little (8000 tokens of 2048 from one expert each 12.3 us with it, 10.3 us without).
+// fp32 accumulation in slot order, one rounding to bf16.  grid_launch_dependents() in small grids only: a block moves
+// (K + 1) x 4 KB, and with small K that outlasts the call by too little (8000 tokens of 2048 from one expert each 12.3 us with
+// it, 10.3 us without; a step of 256 tokens, 14 kernels, 58.8 us with it, 59.5 us without).
 // ------------------------------------------------------------------------------------------------
 template <int KT, bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __restrict__ src,
@@ -337,6 +338,7 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
                                                               int K) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (!grid_dependency_wait_tested()) return;
+    if (gridDim.x <= kSmallGrid) grid_launch_dependents();
     if (i >= total) return;
     const int t = (int)(i / hv);
     const int c = (int)(i - (long long)t * hv);
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
 // fixed-order sum over the block's warps: deterministic).  y_perm pieces are fetched four slots at a time
 // (three blocks per SM: with the 80 registers that allows nothing spills; at five blocks per SM the K = 8 kernel
 // spilled and ran 16 % slower inside a step; the instance for a run-time K keeps 32 accumulators and takes two blocks).
-// grid_launch_dependents() only in blocks of some length: 40000 tokens of 256 from one expert each 45.1 us with it, 38.9 us
+// grid_launch_dependents() only in small grids and in blocks of some length: 40000 tokens of 256 from one expert each 45.1 us with it, 38.9 us
 // without, but a step of 14442 tokens of 2880 takes 40 us more (of 8.5 ms) when no streaming kernel lets a GEMM in early.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTriggerPieces = 1024;   // 16-byte pieces that a block moves, 3 ns of the chip's bandwidth
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
 #pragma unroll
     for (int k = 0; k < KA; ++k) dot[k] = 0.f;
     if (!grid_dependency_wait_tested()) return;
-    if ((2 * kk + 1) * hv >= kTriggerPieces) grid_launch_dependents();
+    if (gridDim.x <= kSmallGrid || (2 * kk + 1) * hv >= kTriggerPieces) grid_launch_dependents();
     for (int c = threadIdx.x; c < hv; c += kThreads) {
         const uint4 dv = ldg16(dy + (long long)t * hv + c);
         float d[8];
