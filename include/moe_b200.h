@@ -332,7 +332,8 @@ int moe_swiglu_mxfp8(const moe_dims_t* dims, const void* gu, void* h_act, void* 
  *                              zero codes to a multiple of 128 (columns after the last expert's are not written);
  *                              scales (moe_mxfp8_tokens_scale_bytes): slice_prefix[E+1] as int32 in the first 8192
  *                              bytes, then the scale bytes as [P/128][n_features][4], then again tiled per 208 features
- *                              [ceil(n/208)][P/128][1024] for use as the N-side operand.  Two launches.
+ *                              [ceil(n/208)][P/128][1024] for use as the N-side operand.  One launch: every
+ *                              block derives the prefix from the offsets, the first one stores it.
  *   moe_grouped_gemm_down_wgrad_mxfp8    dw_down [E,I,H] bf16 = Q(h_act)^T Q(dy_perm) per expert, from the token-
  *                              quantised h_act (n_features = I) and dy_perm (n_features = H).
  *   moe_grouped_gemm_gateup_wgrad_mxfp8  dw_gate, dw_up [E,H,I] bf16 from the token-quantised x_perm (n_features = H)

@@ -1353,6 +1353,34 @@ int launch_mx_quantize_tokens(long long R, int E, const bf16* x, long long ld, i
                             pitch, codes_t, reinterpret_cast<uint32_t*>(sa), sb);
 }
 
+template <bool WGRAD>
+static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& sfb, const CUtensorMap& o, const MxPairParams& p,
+                          cudaStream_t s) {
+    static int grid_of_device[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(MXP_THREADS);
+    cfg.dynamicSmemBytes = MXP_SMEM_BYTES;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (grid_of_device[dev] == 0) {
+        if (cudaFuncSetAttribute(mx_pair_kernel<WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MXP_SMEM_BYTES) != cudaSuccess)
+            return MOE_ERR_CUDA;
+        const int sms = sm_count();
+        if (sms <= 0) return MOE_ERR_CUDA;
+        // as many pairs as can be resident at once: a pair that had to wait for a free SM pair would double the duration
+        cfg.gridDim = dim3(2 * (sms / 2));
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, mx_pair_kernel<WGRAD>, &cfg) != cudaSuccess || clusters <= 0) return MOE_ERR_CUDA;
+        if (clusters > sms / 2) clusters = sms / 2;
+        grid_of_device[dev] = 2 * clusters;
+    }
+    return launch_dependent(mx_pair_kernel<WGRAD>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
+}
+
 // dW [E, M, N] = Q(A)^T Q(B) per expert: a_* the M-side operand ([M, pitch] codes, scales with header and words),
 // b_* the N-side operand ([N, pitch] codes, its scales' pair-tiled blocks are used)
 int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, const uint8_t* a_scales, const uint8_t* b_codes_t,
@@ -1373,28 +1401,7 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
     p.prefix = reinterpret_cast<const int32_t*>(a_scales); p.E = E; p.M = M; p.m_tiles = m_tiles; p.n_tiles = n_tiles;
     p.n_cols = N; p.n_slices = n_slices; p.sa_rows = M;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales + MX_TOKENS_HEADER_BYTES); p.out = dw; p.ldo = N;
-    static int grid_of_device[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(MXP_THREADS);
-    cfg.dynamicSmemBytes = MXP_SMEM_BYTES;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (grid_of_device[dev] == 0) {
-        if (cudaFuncSetAttribute(mx_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MXP_SMEM_BYTES) != cudaSuccess)
-            return MOE_ERR_CUDA;
-        const int sms = sm_count();
-        if (sms <= 0) return MOE_ERR_CUDA;
-        cfg.gridDim = dim3(2 * (sms / 2));
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, mx_pair_kernel<true>, &cfg) != cudaSuccess || clusters <= 0) return MOE_ERR_CUDA;
-        if (clusters > sms / 2) clusters = sms / 2;
-        grid_of_device[dev] = 2 * clusters;
-    }
-    return launch_dependent(mx_pair_kernel<true>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
+    return launch_mx_pair<true>(a, b, sfb, o, p, s);
 }
 
 // CTA pairs from this many rows per expert on average (below it the 256-row tiles are mostly padding)
@@ -1406,6 +1413,9 @@ constexpr long long kMxPairRows = 256;
 // 715 -> 650 us (6.9 TB/s).  128 experts, 768 x 2048, down projection, rows per expert 32: 47 -> 44 us, 64: 51 -> 47 us,
 // 94: 51 -> 55 us -- a second tile per expert reads the expert's weights again, from L2.  Tiles of 32 rows lost to
 // tiles of 64 everywhere but below 4 rows per expert (N = 32 makes the MMAs no cheaper to issue).
+// Under Zipf and Dirichlet loads, where one expert runs many 64-row tiles, the form holds: 128 experts, 64 rows on average, at most
+// 973 / 756, down 54 -> 48 / 49 -> 44 us, gate/up 89 -> 83 / 78 -> 78 us (unswapped -> swapped); 64 experts of 2048 x 1408 40-43 -> 37-40 us.
+// Not so few large experts just below the line: 8 experts of 64 rows, 14336 x 4096, down 87 -> 108 us (gate/up 168 -> 173 us).
 // Not with so many experts (487 and more) that two CTAs and their tables no longer fit an SM: the second half of the grid
 // would wait for the first, and one CTA with four stages keeps less in flight than one with six.  Down projection, 1024 x 512,
 // swapped with one CTA per SM against this kernel unswapped: 512 experts of 4 rows 76 against 55 us, of 64 rows 108 against
@@ -1428,29 +1438,7 @@ static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint
     MxPairParams p = {};
     p.prefix = offsets; p.E = E; p.k_tiles = k_tiles; p.n_tiles = n_tiles; p.n_cols = n_feat; p.sa_rows = R;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales); p.out = out; p.ldo = n_feat;
-    static int grid_of_device[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(MXP_THREADS);
-    cfg.dynamicSmemBytes = MXP_SMEM_BYTES;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (grid_of_device[dev] == 0) {
-        if (cudaFuncSetAttribute(mx_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MXP_SMEM_BYTES) != cudaSuccess)
-            return MOE_ERR_CUDA;
-        const int sms = sm_count();
-        if (sms <= 0) return MOE_ERR_CUDA;
-        // as many pairs as can be resident at once: a pair that had to wait for a free SM pair would double the duration
-        cfg.gridDim = dim3(2 * (sms / 2));
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, mx_pair_kernel<false>, &cfg) != cudaSuccess || clusters <= 0) return MOE_ERR_CUDA;
-        if (clusters > sms / 2) clusters = sms / 2;
-        grid_of_device[dev] = 2 * clusters;
-    }
-    return launch_dependent(mx_pair_kernel<false>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
+    return launch_mx_pair<false>(a, b, sfb, o, p, s);
 }
 
 struct MxSingleArgs {
