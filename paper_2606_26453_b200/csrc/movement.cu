@@ -326,11 +326,11 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
 
 // ------------------------------------------------------------------------------------------------
 // a4 / a8: dst[t,:] = sum_k w[t,k] * src[pair_to_row[t*K+k], :]  (w == NULL: unit weights).
-// fp32 accumulation in slot order, one rounding to bf16.  grid_launch_dependents() in small grids only: a block moves
+// fp32 accumulation in slot order, one rounding to bf16.  TRIGGER (grid_launch_dependents) in small grids only: a block moves
 // (K + 1) x 4 KB, and with small K that outlasts the call by too little (8000 tokens of 2048 from one expert each 12.3 us with
-// it, 10.3 us without; a step of 256 tokens, 14 kernels, 58.8 us with it, 59.5 us without).
+// it, 10.3 us without; a branch in the kernel costs nearly as much, 12915 tokens of 1024 8.7 us without, 9.7 with the branch).
 // ------------------------------------------------------------------------------------------------
-template <int KT, bool WEIGHTED>
+template <int KT, bool WEIGHTED, bool TRIGGER>
 __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __restrict__ src,
                                                               const float* __restrict__ topk_w,
                                                               const int32_t* __restrict__ pair_to_row,
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
                                                               int K) {
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (!grid_dependency_wait_tested()) return;
-    if (gridDim.x <= kSmallGrid) grid_launch_dependents();
+    if (TRIGGER) grid_launch_dependents();
     if (i >= total) return;
     const int t = (int)(i / hv);
     const int c = (int)(i - (long long)t * hv);
@@ -380,11 +380,12 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
 // fixed-order sum over the block's warps: deterministic).  y_perm pieces are fetched four slots at a time
 // (three blocks per SM: with the 80 registers that allows nothing spills; at five blocks per SM the K = 8 kernel
 // spilled and ran 16 % slower inside a step; the instance for a run-time K keeps 32 accumulators and takes two blocks).
-// grid_launch_dependents() only in small grids and in blocks of some length: 40000 tokens of 256 from one expert each 45.1 us with it, 38.9 us
-// without, but a step of 14442 tokens of 2880 takes 40 us more (of 8.5 ms) when no streaming kernel lets a GEMM in early.
+// TRIGGER (grid_launch_dependents) only in small grids and blocks of some length: 40000 tokens of 256 from one expert each
+// 45.1 us with it, 38.9 us without, but a step of 14442 tokens of 2880 takes 40 us more (of 8.5 ms) when no streaming kernel
+// lets a GEMM in early.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTriggerPieces = 1024;   // 16-byte pieces that a block moves, 3 ns of the chip's bandwidth
-template <int KT, bool WITH_DW>
+template <int KT, bool WITH_DW, bool TRIGGER>
 __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(const uint4* __restrict__ dy,
                                                                   const uint4* __restrict__ y_perm,
                                                                   const float* __restrict__ topk_w,
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
 #pragma unroll
     for (int k = 0; k < KA; ++k) dot[k] = 0.f;
     if (!grid_dependency_wait_tested()) return;
-    if (gridDim.x <= kSmallGrid || (2 * kk + 1) * hv >= kTriggerPieces) grid_launch_dependents();
+    if (TRIGGER) grid_launch_dependents();
     for (int c = threadIdx.x; c < hv; c += kThreads) {
         const uint4 dv = ldg16(dy + (long long)t * hv + c);
         float d[8];
@@ -546,18 +547,18 @@ int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, 
                             reinterpret_cast<uint8_t*>(x_perm), row_bytes, seg_bytes, n_seg);
 }
 
-template <bool WEIGHTED>
+template <bool WEIGHTED, bool TRIGGER>
 static int gather_sum_dispatch(const moe_dims_t& d, const uint4* src, const float* w, const int32_t* p2r,
                                 uint4* dst, cudaStream_t s) {
     const int hv = d.H / 8;
     const long long total = (long long)d.T * hv;
 #define MOE_GS_CASE(KT) \
-    case KT: return launch_streaming(gather_sum_kernel<KT, WEIGHTED>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
+    case KT: return launch_streaming(gather_sum_kernel<KT, WEIGHTED, TRIGGER>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
     switch (d.K) {
         MOE_GS_CASE(1) MOE_GS_CASE(2) MOE_GS_CASE(3) MOE_GS_CASE(4) MOE_GS_CASE(5) MOE_GS_CASE(6) MOE_GS_CASE(7)
         MOE_GS_CASE(8)
         default:
-            return launch_streaming(gather_sum_kernel<0, WEIGHTED>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
+            return launch_streaming(gather_sum_kernel<0, WEIGHTED, TRIGGER>, blocks_for(total), s, src, w, p2r, dst, total, hv, d.K);
     }
 #undef MOE_GS_CASE
 }
@@ -566,22 +567,26 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
                       bf16* dst, cudaStream_t s) {
     const uint4* src = reinterpret_cast<const uint4*>(src_perm);
     uint4* out = reinterpret_cast<uint4*>(dst);
-    return topk_w != nullptr ? gather_sum_dispatch<true>(d, src, topk_w, pair_to_row, out, s)
-                             : gather_sum_dispatch<false>(d, src, nullptr, pair_to_row, out, s);
+    const bool trigger = blocks_for((long long)d.T * (d.H / 8)) <= kSmallGrid;
+    if (topk_w != nullptr)
+        return trigger ? gather_sum_dispatch<true, true>(d, src, topk_w, pair_to_row, out, s)
+                       : gather_sum_dispatch<true, false>(d, src, topk_w, pair_to_row, out, s);
+    return trigger ? gather_sum_dispatch<false, true>(d, src, nullptr, pair_to_row, out, s)
+                   : gather_sum_dispatch<false, false>(d, src, nullptr, pair_to_row, out, s);
 }
 
-template <bool WITH_DW>
+template <bool WITH_DW, bool TRIGGER>
 static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w,
                                  const int32_t* p2r, uint4* dyp, float* dw, cudaStream_t s) {
     const int hv = d.H / 8;
     const unsigned blocks = (unsigned)d.T;
 #define MOE_CB_CASE(KT) \
-    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW, TRIGGER>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     switch (d.K) {
         MOE_CB_CASE(1) MOE_CB_CASE(2) MOE_CB_CASE(3) MOE_CB_CASE(4) MOE_CB_CASE(5) MOE_CB_CASE(6) MOE_CB_CASE(7)
         MOE_CB_CASE(8)
         default:
-            return launch_streaming(combine_bwd_kernel<0, WITH_DW>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+            return launch_streaming(combine_bwd_kernel<0, WITH_DW, TRIGGER>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     }
 #undef MOE_CB_CASE
 }
@@ -591,8 +596,12 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    return dtopk_w != nullptr ? combine_bwd_dispatch<true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
-                              : combine_bwd_dispatch<false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
+    const bool trigger = d.T <= (int)kSmallGrid || (2ll * d.K + 1) * (d.H / 8) >= kTriggerPieces;
+    if (dtopk_w != nullptr)
+        return trigger ? combine_bwd_dispatch<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
+                       : combine_bwd_dispatch<true, false>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s);
+    return trigger ? combine_bwd_dispatch<false, true>(d, a, b, topk_w, pair_to_row, o, nullptr, s)
+                   : combine_bwd_dispatch<false, false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
 }
 
 // ------------------------------------------------------------------------------------------------
