@@ -1140,7 +1140,9 @@ __global__ void __launch_bounds__(256) mx_swiglu_bwd_quantize_kernel(const uint4
 // quantiser.  The tile comes in with 16-byte asynchronous copies (rows from `n_rows` on as zeros); a thread then owns a
 // pair of features over one block of 32 rows: 32 words from shared memory (blocks of rows are set 8 words apart so that
 // the 4 x 8 lanes of a warp hit 32 banks), both maxima in packed arithmetic, 2 x 32 code bytes.  The 4 lanes that share a
-// feature write its 128 contiguous bytes.
+// feature write its 128 contiguous bytes, 32 each with one store: two 16-byte stores write every 32-byte sector by halves, and
+// that costs the L2 as much as twice the bytes.  Token axis 131072 x 2048 186 -> 154 us, 16384 x 14336 166 -> 135 us; weights
+// 128 x 768 x 2048 113 -> 100 us.  Callers' buffers need only 16-byte alignment, hence the other branch.
 constexpr int MXT_BLOCK_WORDS = 32 * 64 + 8;   // shared-memory words of 32 rows x 128 features, with the bank offset
 __device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long long ld, int n_rows, uint8_t* dst, long long dst_ld,
                                                            uint32_t* tile, uint8_t* sf) {
@@ -1164,6 +1166,7 @@ __device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long
 #pragma unroll
     for (int j = 0; j < 32; ++j) m = mx_abs_max(m, v[j] & 0x7fff7fffu);
     const int exps[2] = {mx_scale_exp(mx_lo(m)), mx_scale_exp(mx_hi(m))};
+    const bool whole_sectors = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;   // for the whole grid: all but the buffer is a multiple of 32
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const float inv = mx_inv_scale(exps[h]);
@@ -1175,9 +1178,15 @@ __device__ __forceinline__ void mx_transpose_quantize_tile(const bf16* src, long
             for (int t = 0; t < 4; ++t) f[t] = (h ? mx_hi(v[4 * g + t]) : mx_lo(v[4 * g + t])) * inv;
             out[g] = mx_e4m3x2(f[0], f[1]) | (mx_e4m3x2(f[2], f[3]) << 16);
         }
-        uint4* to = reinterpret_cast<uint4*>(dst + (2 * pair + h) * dst_ld + block * 32);
-        to[0] = make_uint4(out[0], out[1], out[2], out[3]);
-        to[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        uint8_t* to = dst + (2 * pair + h) * dst_ld + block * 32;
+        if (whole_sectors) {
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(out[0]), "r"(out[1]), "r"(out[2]),
+                         "r"(out[3]), "r"(out[4]), "r"(out[5]), "r"(out[6]), "r"(out[7])
+                         : "memory");
+        } else {
+            reinterpret_cast<uint4*>(to)[0] = make_uint4(out[0], out[1], out[2], out[3]);
+            reinterpret_cast<uint4*>(to)[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        }
         sf[(2 * pair + h) * 4 + block] = (uint8_t)(exps[h] + 127);
     }
     __syncthreads();

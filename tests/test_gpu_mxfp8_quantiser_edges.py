@@ -75,3 +75,23 @@ def test_token_quantiser_expert_scan(counts):
     assert np.array_equal(codes.view(n, P)[:, :n_sl * 128].cpu().numpy(), want_codes)
     words = scales[8192: 8192 + (P // 128) * n * 4].view(P // 128, n, 4)[:n_sl].cpu().numpy()
     assert np.array_equal(words, want_scales)
+
+
+@pytest.mark.parametrize("shift", [16, 32])
+def test_transposing_quantisers_take_any_16_byte_alignment(shift):
+    from paper_2606_26453_b200 import binding as B
+    E, H, I = 3, 256, 384
+    rng = np.random.default_rng(shift)
+    w = W.round_to_bf16(rng.standard_normal((E, I, H)).astype(np.float32))
+    d = B.dims(40, H, I, E, 1)
+    out = []
+    for s in (0, shift):
+        room, scales = _u8(E * H * I + 64), _u8(B.moe_mxfp8_w_down_scale_bytes(d))
+        codes = room[s:s + E * H * I]
+        B.moe_mxfp8_quantize_w_down(d, Hh.to_dev_bf16(w), codes, scales)
+        torch.cuda.synchronize()
+        assert bool((room[s + E * H * I:] == 0xFF).all()) and bool((room[:s] == 0xFF).all())
+        out.append((codes.clone(), scales))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    want = np.stack([O.mxfp8_quantize(w[e].T)[0] for e in range(E)])               # [E, H, I]
+    assert np.array_equal(out[0][0].cpu().numpy().reshape(E, H, I), want)
