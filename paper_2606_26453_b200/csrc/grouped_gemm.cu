@@ -728,17 +728,20 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
             for (int j = 0; j < 4; ++j) d4[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
         };
-        // swapped kinds: this lane holds one output feature for 32 consecutive rows; the block is transposed on its
-        // way into the staging buffer (row j of the block, feature `lane`: 2-byte stores, 64 contiguous bytes per
-        // warp instruction) and then stored like any other 32 x 32 block
-        auto stage_transposed_and_store = [&](const float (&v)[32], const CUtensorMap* map, int x, int y) {
+        // swapped kinds: a block in fragment order, transposed through the staging buffer; of a block that the tile only partly
+        // fills the rows leave in 16-byte pieces.  Where most blocks are such, against 2-byte stores: 8 experts of 512 x 512 with
+        // 150 rows, down 7.7 -> 7.0 us, fused down dgrad 11.4 -> 10.4 us; with full blocks no difference.
+        const uint32_t frag_at = smem_u32(stage_ptr) + frag_offset(lane);
+        auto put_block = [&](const uint32_t (&w)[16], bf16* out, const CUtensorMap* map, long long ld, int x, int r0, int rv) {
             staging_free();
-            const int piece = lane >> 3, within = (lane & 7) * 2;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                *reinterpret_cast<__nv_bfloat16*>(stage_ptr + j * 64 + (((piece ^ ((j >> 1) & 3)) << 4) + within)) =
-                    __float2bfloat16_rn(v[j]);
-            send_block(map, x, y);
+            store_frag(frag_at, w);
+            if (rv == 32) {
+                send_block(map, x, r0);
+            } else {
+                __syncwarp();
+                copy_block_rows(stage_ptr, out + (long long)r0 * ld + x, ld, rv, lane);
+                __syncwarp();
+            }
         };
         // fused SwiGLU backward: the warp's g and u input blocks (behind its staging block), fetched with two bulk
         // tensor loads from the saved pre-activations [R, 2I] (map_b1: 32 x 32 boxes, 64-byte swizzle)
@@ -837,7 +840,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const long long t = tile_of<KIND>(it, first_tile, tile_stride, n_tiles_total);
             if (t < 0) break;
             const Tile tl = decode_tile<KIND, G::TILE_M>(p, ctl, t);
-            if (!mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag)) break;
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag))) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16);
             // first row of this warp's slab.  Half-height pair tile (FWD_SWIGLU, M = 128 over two CTAs): this CTA holds
@@ -858,51 +861,41 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (fused_sb(KIND) && feats_owed && half < n_row_blocks) fetch_gu(feat0, tl.row0 + half * 32);
 #pragma unroll 1
                 for (int i = half; i < n_row_blocks; i += 2) {
-                    uint32_t vr[32];
-                    tc_ld32(taddr + i * 32, vr);
+                    uint32_t v[32], w[16];
+                    tc_ld_frag32(taddr + i * 32, v);
                     tc_wait_ld();
                     if (!feats_owed) continue;
-                    float v[32];
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(vr[j]);
                     const int r0 = tl.row0 + i * 32;
                     const int rv = min(32, tl.rows - i * 32);
                     if (fused_sb(KIND)) {
-                        // element (row j, feature `lane`) of the g and u blocks; then the next block's fetch may start
-                        if (!mbar_wait(gu_bar, gu_phase, abort_flag)) break;
+                        // the g and u blocks in the same fragment order; then the next block's fetch may start
+                        if (!__all_sync(0xffffffffu, mbar_wait(gu_bar, gu_phase, abort_flag))) break;
                         gu_phase ^= 1u;
-                        const int piece = lane >> 3, within = (lane & 7) * 2;
-                        float du[32];
-                        uint32_t seen = 0;
+                        uint32_t gw[16], uw[16], dup[16], seen = 0;
+                        load_frag(smem_u32(g_blk) + frag_offset(lane), gw);
+                        load_frag(smem_u32(u_blk) + frag_offset(lane), uw);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const int off = j * 64 + (((piece ^ ((j >> 1) & 3)) << 4) + within);
-                            const uint32_t gr = *reinterpret_cast<const uint16_t*>(g_blk + off);
-                            const uint32_t ur = *reinterpret_cast<const uint16_t*>(u_blk + off);
-                            seen ^= gr ^ (ur << 16);
-                            swiglu_grad(v[j], __uint_as_float(gr << 16), __uint_as_float(ur << 16), v[j], du[j]);
-                        }
+                        for (int i8 = 0; i8 < 4; ++i8)
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                const uint32_t gr = gw[4 * i8 + m], ur = uw[4 * i8 + m];
+                                const uint32_t* d2 = v + 16 * (m >> 1) + 4 * i8 + 2 * (m & 1);
+                                seen ^= gr ^ ur;
+                                float dg0, du0, dg1, du1;
+                                swiglu_grad(__uint_as_float(d2[0]), __uint_as_float(gr << 16), __uint_as_float(ur << 16), dg0, du0);
+                                swiglu_grad(__uint_as_float(d2[1]), __uint_as_float(gr & 0xffff0000u), __uint_as_float(ur & 0xffff0000u), dg1, du1);
+                                w[4 * i8 + m] = pack_bf16(dg0, dg1);
+                                dup[4 * i8 + m] = pack_bf16(du0, du1);
+                            }
                         if (i + 2 < n_row_blocks) {
                             inputs_consumed(seen);   // all reads of the two input blocks have returned
                             fetch_gu(feat0, tl.row0 + (i + 2) * 32);
                         }
-                        if (rv == 32) {
-                            stage_transposed_and_store(v, &map_o0, feat0, r0);
-                            stage_transposed_and_store(du, &map_o0, p.I + feat0, r0);
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (j < rv) {
-                                    p.out0[(long long)(r0 + j) * p.ldo + feat0 + lane] = __float2bfloat16_rn(v[j]);
-                                    p.out0[(long long)(r0 + j) * p.ldo + p.I + feat0 + lane] = __float2bfloat16_rn(du[j]);
-                                }
-                        }
-                    } else if (rv == 32) {
-                        stage_transposed_and_store(v, &map_o0, feat0, r0);
+                        put_block(w, p.out0, &map_o0, p.ldo, feat0, r0, rv);
+                        put_block(dup, p.out0, &map_o0, p.ldo, p.I + feat0, r0, rv);
                     } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)   // rows past the tile belong to the expert's next tile, or to nobody
-                            if (j < rv) p.out0[(long long)(r0 + j) * p.ldo + feat0 + lane] = __float2bfloat16_rn(v[j]);
+                        pack_frag(v, w);
+                        put_block(w, p.out0, &map_o0, p.ldo, feat0, r0, rv);
                     }
                 }
             } else if (swiglu(KIND)) {

@@ -458,37 +458,42 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 }
 
 // ---- the CTA-pair form ----------------------------------------------------------------------------------
-// Two CTAs of a cluster share one 256-row x 208-column tile (tcgen05.mma.cta_group::2, M = 256): each keeps its own 128
-// rows of A and 104 of the tile's weight rows in shared memory, so a K slice of 128 costs each SM 29 KB of operand
-// loads against 58 KB per two 128 x 128 tiles of the single-CTA form, which the L2 -> SM path bounds.  208 columns, not
-// 256: the two accumulators (tensor-memory columns 0 and 256) leave 48 columns behind each for three 16-column scale
-// slots, one slot per ring stage.  A tile at the right edge is narrower (a multiple of 16 columns; the MMA's N is set
-// per tile).
-//   scale factors: each CTA holds the scales of its own 128 rows of A (4 columns) and of ALL the tile's weight rows (two
-//   128-row blocks, 8 columns) in its own tensor memory; tcgen05.cp.cta_group::2, issued once, copies in both CTAs from
-//   the same shared-memory offsets.  The weight-scale blocks of a (tile, K slice) are 1024 contiguous bytes in global
-//   memory (a second copy of the scales in this tiling, written by the weight quantiser) and arrive by one tensor copy.
+// Two CTAs of a cluster share one tile of M = 256, N up to 208 (tcgen05.mma.cta_group::2): each keeps 128 of the M side's codes
+// and half of the N side's in shared memory, so a K slice of 128 costs each SM 29 KB of operand loads against 58 KB per two
+// 128 x 128 tiles of the single-CTA form, which the L2 -> SM path bounds.  208, not 256: the two accumulators (tensor-memory
+// columns 0 and 256) leave 48 columns behind each for three 16-column scale slots, one slot per ring stage.
+//   row-ragged form    M side: 256 output features of an expert's weights.  N side: its rows, in equal tiles of at most 208 rows
+//                      (a multiple of 16), so that almost no tensor work goes to padding.  The accumulator has a feature per
+//                      lane and a row per column and is transposed on its way out.
+//   weight gradients   M side: 256 rows of the output, N side: 208 columns of it (the last tile is narrower).
+// The row-ragged form had the rows on the M side before, in tiles of 256, half a tile of padding per expert: all four GEMMs
+// 18 % faster at 384 rows per expert (64 experts of 2048 x 1408: gate/up 206 -> 166, down 108 -> 88 us), 3-8 % at 1024
+// (128 of 2048 x 768: 433 -> 402, 282 -> 272 us), 3-6 % at 2048 (8 of 4096 x 14336: 1697 -> 1649, 884 -> 827 us), 10 % under
+// Dirichlet loads (128 of 2944 x 2944).
+//   scale factors: each CTA holds the scales of its own 128 of the M side (4 columns) and of ALL the tile's N side (two blocks of
+//   128, 8 columns) in its own tensor memory; tcgen05.cp.cta_group::2, issued once, copies in both CTAs from the same
+//   shared-memory offsets.  Weight-scale blocks (512 bytes per 128 features and K slice) and the weight gradients' N-side blocks
+//   (1024 bytes per 208 columns) are contiguous in global memory and arrive by one tensor copy; scales of packed rows are
+//   gathered by a warp.  (Weight scales are also stored in the 208 tiling, as their documented format has it; nothing in this
+//   file reads that copy.)
 //   warp 0      TMA producer (both CTAs; all loads complete on the first CTA's full[stage], as in the bf16 pair kernels)
 //   warp 1      first CTA: issues the MMAs and the commits for the pair
-//   warp 2      activation scales of this CTA's 128 rows
-//   warps 3..10 epilogue: 32-row slab x every other 32-column block (a 16-column remainder: plain stores)
+//   warp 2      scales of packed rows (row-ragged form: the N side's) or of the M side's 128 rows (weight gradients)
+//   warps 3..10 epilogue: a 32-lane quarter x every other 32-column block
 //   warp 11     first CTA: issues the scale copies (smem -> tensor memory) of each stage
-// What bounds it (cycle counters, throw-away builds, before the issuing roles ran on uniform values): every tcgen05
-// instruction cost its issuing thread 60-85 cycles whatever its size, so a K slice (wait, four MMAs, commit) took the MMA
-// warp ~470 cycles -- more than the ~420 the tensor pipe needs for four N = 208 MMAs.  With the three scale copies in the
-// same thread it was ~770; with two or four scale slots the chain MMA -> stage released -> copies -> MMA set the pace
-// instead (~510).  In the full kernel a slice took ~590 cycles: operand reads by the tensor core and fills by the TMA unit
-// together ask shared memory for ~140 bytes per cycle at this tile width (halving the waits and commits per slice changed
-// nothing).  Uniform issuing took 6-9 % off (see the MMA issuer); the largest shapes now run into the power cap.
-constexpr int MXP_NT = 208;                 // tile columns over the pair
-constexpr int MXP_ROWS = 2 * MX_BM;         // tile rows over the pair
+// What bounds it: a K slice takes ~590 cycles where the tensor pipe needs ~420 (four N = 208 MMAs): operand reads by the tensor
+// core and fills by the TMA unit together ask shared memory for ~140 bytes per cycle at this tile width (halving the waits and
+// commits per slice changed nothing; with scale copies in the MMA thread it took ~770, with two or four scale slots ~510 before
+// a load was issued).  The largest shapes run into the power cap.
+constexpr int MXP_NT = 208;                 // most of a tile's N over the pair
+constexpr int MXP_ROWS = 2 * MX_BM;         // a tile's M over the pair
 constexpr int MXP_STAGES = 6;
 constexpr int MXP_A_BYTES = MX_BM * MX_BK;              // 16 KB
 constexpr int MXP_B_BYTES = (MXP_NT / 2) * MX_BK;       // 13 KB
-constexpr int MXP_SFA_OFF = MXP_A_BYTES + MXP_B_BYTES;  // 512 bytes: this CTA's activation scales
-constexpr int MXP_SFB_OFF = MXP_SFA_OFF + 512;          // 1024 bytes: the tile's weight scales
+constexpr int MXP_SFA_OFF = MXP_A_BYTES + MXP_B_BYTES;  // 512 bytes: scales of this CTA's part of the M side
+constexpr int MXP_SFB_OFF = MXP_SFA_OFF + 512;          // 1024 bytes: scales of the tile's N side
 constexpr int MXP_STAGE_BYTES = 31 * 1024;              // 30.5 KB used; stages stay 1024-byte aligned
-constexpr int MXP_TX_BYTES = MXP_A_BYTES + MXP_B_BYTES + 1024;   // bytes one CTA's loads deliver per stage
+constexpr int MXP_LOW_BOX = 64;                         // rows of the smaller of the row-ragged form's two boxes of row codes
 constexpr int MXP_EPI_WARPS = 8;
 constexpr int MXP_COPY_WARP = 3 + MXP_EPI_WARPS;   // the scale-copy warp comes after the epilogue warps
 constexpr int MXP_THREADS = 32 * (4 + MXP_EPI_WARPS);
@@ -509,15 +514,15 @@ struct MxPairCtl {
     unsigned long long drain_copy;
     uint32_t tmem_base;
     int abort_flag;
-    int stage_n[MXP_STAGES];   // columns of the tile a stage belongs to (published by the first CTA's producer)
+    int stage_n[MXP_STAGES];   // N of the tile a stage belongs to (published by the first CTA's producer)
     int32_t offs[MX_MAX_E + 1];          // row-ragged form: offsets; weight gradients: slice_prefix
-    int32_t tile_prefix[MX_MAX_E + 1];   // row-ragged form: 256-row tiles of the experts before e
+    int32_t tile_prefix[MX_MAX_E + 1];   // row-ragged form: row tiles of the experts before e
 };
 constexpr int MXP_SMEM_BYTES = MXP_STAGES * MXP_STAGE_BYTES + MXP_STAGING_BYTES + 1024 + (int)sizeof(MxPairCtl);
 static_assert(MXP_SMEM_BYTES <= 232448, "exceeds the shared memory a CTA can opt in to");
 
 // The pair kernel serves two problems (template parameter WGRAD):
-//   row-ragged GEMM   out[r, :] = a[r, :] . b[e]^T for the rows r of expert e: tiles of 256 rows from `offsets`, the
+//   row-ragged GEMM   out[r, :] = a[r, :] . b[e]^T for the rows r of expert e: row tiles from `offsets`, the
 //                     contraction is k_tiles slices for every tile, b and its scale blocks are indexed by expert;
 //   weight gradient   dW[e] [M, N] = A_e^T B_e with token-quantised, transposed operands (further down): a fixed tile
 //                     list (expert x M tiles x N tiles), the contraction of expert e is the slices
@@ -526,8 +531,8 @@ struct MxPairParams {
     const int32_t* prefix;   // offsets [E + 1] / slice_prefix [E + 1]
     int E, k_tiles, n_tiles, m_tiles, n_cols, n_slices;   // k_tiles: row-ragged form; m_tiles, n_slices: weight gradients
     int M;                   // weight gradients: rows of one expert's output
-    long long sa_rows;       // rows per slice of the A-side scale words: R / M
-    const uint32_t* sa;      // scale words of the A side [slices][sa_rows]
+    long long sa_rows;       // words per slice of `sa`: R / M
+    const uint32_t* sa;      // scale words of the packed rows / of the A side [slices][sa_rows]
     bf16* out;
     long long ldo;
 };
@@ -556,28 +561,30 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t v[16]) {
 }
 
 struct MxPairTile {
-    int e, row0, row_end;   // first row of the tile and end of the valid rows, as the A operand counts them
-    int out_shift;          // output row = A row + out_shift
-    int n0, nt, width;      // first column, column-tile index, columns
+    int row0;               // weight gradients: first output row inside the expert's output; row-ragged form: first packed row
+    int rows;               // row-ragged form: packed rows
+    int out_row0;           // weight gradients: first row of the expert's output in the output tensor
+    int n0, width;          // first output column (feature); N of the MMAs
     int k0, k_tiles;        // K slices [k0, k0 + k_tiles) of both operands
-    int b_row, sfb_row0;    // first row of the tile in the B codes; row of its first scale block
+    int w_row, sf_row0;     // first row of the tile in the B codes (weight gradients) / weight codes; row of its first scale block
 };
 template <bool WGRAD>
 __device__ __forceinline__ MxPairTile mxp_decode(const MxPairParams& p, const MxPairCtl* ctl, long long t) {
     MxPairTile tl;
     if (WGRAD) {
         const int per_e = p.m_tiles * p.n_tiles;
-        tl.e = (int)(t / per_e);
-        const int local = (int)(t - (long long)tl.e * per_e);
-        tl.nt = local / p.m_tiles;   // column tile major inside an expert: the pairs running together share the B tile in L2
-        tl.row0 = (local - tl.nt * p.m_tiles) * MXP_ROWS;
-        tl.row_end = p.M;
-        tl.out_shift = tl.e * p.M;
-        tl.k0 = ctl->offs[tl.e];
-        tl.k_tiles = ctl->offs[tl.e + 1] - tl.k0;
-        tl.n0 = tl.nt * MXP_NT;
-        tl.b_row = tl.n0;
-        tl.sfb_row0 = tl.nt * p.n_slices + tl.k0;
+        const int e = (int)(t / per_e);
+        const int local = (int)(t - (long long)e * per_e);
+        const int nt = local / p.m_tiles;   // column tile major inside an expert: the pairs running together share the B tile in L2
+        tl.row0 = (local - nt * p.m_tiles) * MXP_ROWS;
+        tl.rows = 0;
+        tl.out_row0 = e * p.M;
+        tl.k0 = ctl->offs[e];
+        tl.k_tiles = ctl->offs[e + 1] - tl.k0;
+        tl.n0 = nt * MXP_NT;
+        tl.width = min(MXP_NT, p.n_cols - tl.n0);
+        tl.w_row = tl.n0;
+        tl.sf_row0 = nt * p.n_slices + tl.k0;
     } else {
         int lo = 0, hi = p.E;   // largest e with tile_prefix[e] * n_tiles <= t
         while (hi - lo > 1) {
@@ -586,18 +593,19 @@ __device__ __forceinline__ MxPairTile mxp_decode(const MxPairParams& p, const Mx
         }
         const int local = (int)(t - (long long)ctl->tile_prefix[lo] * p.n_tiles);
         const int m_tiles_e = ctl->tile_prefix[lo + 1] - ctl->tile_prefix[lo];
-        tl.e = lo;
-        tl.nt = local / m_tiles_e;   // column tile major inside an expert (the pairs running together share weight tiles in L2)
-        tl.row0 = ctl->offs[lo] + (local - tl.nt * m_tiles_e) * MXP_ROWS;
-        tl.row_end = ctl->offs[lo + 1];
-        tl.out_shift = 0;
+        const int nt = local / m_tiles_e, mt = local - nt * m_tiles_e;   // feature tile major inside an expert (the pairs running together share weight tiles in L2)
+        const int n_e = ctl->offs[lo + 1] - ctl->offs[lo];
+        const int per_tile = ((n_e + m_tiles_e - 1) / m_tiles_e + 15) & ~15;   // equal tiles, the last one takes what is left
+        tl.row0 = ctl->offs[lo] + mt * per_tile;
+        tl.rows = min(per_tile, ctl->offs[lo + 1] - tl.row0);
+        tl.out_row0 = 0;
         tl.k0 = 0;
         tl.k_tiles = p.k_tiles;
-        tl.n0 = tl.nt * MXP_NT;
-        tl.b_row = lo * p.n_cols + tl.n0;
-        tl.sfb_row0 = (lo * p.n_tiles + tl.nt) * p.k_tiles;
+        tl.n0 = nt * MXP_ROWS;
+        tl.width = (tl.rows + 15) & ~15;
+        tl.w_row = lo * p.n_cols + tl.n0;
+        tl.sf_row0 = (lo * (p.n_cols >> 7) + 2 * nt) * p.k_tiles;
     }
-    tl.width = min(MXP_NT, p.n_cols - tl.n0);
     return tl;
 }
 // K slices of tile t (the roles that do not need the rest of the tile)
@@ -611,8 +619,8 @@ __device__ __forceinline__ int mxp_k_tiles(const MxPairParams& p, const MxPairCt
 template <bool WGRAD>
 __global__ void __launch_bounds__(MXP_THREADS, 1)
 mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                    const __grid_constant__ CUtensorMap map_sfb, const __grid_constant__ CUtensorMap map_o,
-                    const MxPairParams p) {
+                    const __grid_constant__ CUtensorMap map_b_low, const __grid_constant__ CUtensorMap map_sf,
+                    const __grid_constant__ CUtensorMap map_o, const MxPairParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* tiles_ptr = smem_raw + (tiles_base - smem_u32(smem_raw));
@@ -638,14 +646,15 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tmap(&map_a);
         prefetch_tmap(&map_b);
-        prefetch_tmap(&map_sfb);
+        prefetch_tmap(&map_b_low);
+        prefetch_tmap(&map_sf);
         prefetch_tmap(&map_o);
     }
     // everything above may run while the kernel before is still finishing; the schedule is derived from its output
     grid_dependency_wait();
     for (int e = threadIdx.x; e <= p.E; e += MXP_THREADS) ctl->offs[e] = p.prefix[e];
     __syncthreads();
-    if (!WGRAD && warp == 0) exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, MXP_ROWS, lane);   // row-ragged form
+    if (!WGRAD && warp == 0) exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, MXP_NT, lane);   // row-ragged form
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                      "r"((uint32_t)MX_TMEM_COLS)
@@ -668,9 +677,13 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
                 MxPairTile tl = mxp_decode<WGRAD>(p, ctl, t);
                 auto uni = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };
-                tl.row0 = uni(tl.row0); tl.width = uni(tl.width); tl.k0 = uni(tl.k0); tl.k_tiles = uni(tl.k_tiles); tl.b_row = uni(tl.b_row);
-                const int sfb_row0 = uni(tl.sfb_row0);
-                const int b_row = tl.b_row + (int)rank * (tl.width >> 1);
+                tl.row0 = uni(tl.row0); tl.width = uni(tl.width); tl.k0 = uni(tl.k0); tl.k_tiles = uni(tl.k_tiles); tl.w_row = uni(tl.w_row);
+                // this CTA's 128 rows of the M side, its half of the N side, its scale blocks
+                const int my_n = tl.width >> 1;
+                const int a_row = (WGRAD ? tl.row0 : tl.w_row) + (int)rank * MX_BM, b_row = (WGRAD ? tl.w_row : tl.row0) + (int)rank * my_n;
+                const int sf_row0 = uni(tl.sf_row0) + (WGRAD ? 0 : (int)rank * tl.k_tiles);
+                const bool low = !WGRAD && my_n <= MXP_LOW_BOX;
+                const uint32_t bytes = WGRAD ? MXP_A_BYTES + MXP_B_BYTES + 1024 : MXP_A_BYTES + (low ? MXP_LOW_BOX * MX_BK : MXP_B_BYTES) + 512;
                 for (int kt = 0; kt < tl.k_tiles; ++kt) {
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag))) { ok = false; break; }
 #ifdef MOE_TEST_HOOKS
@@ -684,10 +697,10 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         if (rank == 0) ctl->stage_n[stage] = tl.width;   // read by the MMA thread after its wait on full[stage]
                         const uint32_t bar = full0 + stage * (uint32_t)sizeof(unsigned long long);
                         const uint32_t dst = tiles_base + stage * MXP_STAGE_BYTES;
-                        mbar_arrive_expect_tx_cluster(bar, MXP_TX_BYTES);
-                        tma_load_2d_pair(dst, &map_a, (tl.k0 + kt) * MX_BK, tl.row0 + (int)rank * MX_BM, bar);
-                        tma_load_2d_pair(dst + MXP_A_BYTES, &map_b, (tl.k0 + kt) * MX_BK, b_row, bar);
-                        tma_load_2d_pair(dst + MXP_SFB_OFF, &map_sfb, 0, sfb_row0 + kt, bar);
+                        mbar_arrive_expect_tx_cluster(bar, bytes);
+                        tma_load_2d_pair(dst, &map_a, (tl.k0 + kt) * MX_BK, a_row, bar);
+                        tma_load_2d_pair(dst + MXP_A_BYTES, low ? &map_b_low : &map_b, (tl.k0 + kt) * MX_BK, b_row, bar);
+                        tma_load_2d_pair(dst + (WGRAD ? MXP_SFB_OFF : MXP_SFA_OFF), &map_sf, 0, sf_row0 + kt, bar);
                     }
                     __syncwarp();
                     ++issued;
@@ -747,24 +760,31 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         __syncwarp();
     } else if (warp == 2) {
-        // ================= activation scales of this CTA's 128 rows =================
+        // ================= scales of the rows =================
+        // Weight gradients: the M side's, this CTA's 128 rows.  Row-ragged form: the N side's, all the tile's rows in both CTAs
+        // (at most 208: seven words per lane and slice, two blocks of 128 rows; columns past the tile's N are never read).
+        constexpr int WORDS = WGRAD ? 4 : 7;
         uint32_t stage = 0, phase = 0;
         bool ok = true;
         for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
             const MxPairTile tl = mxp_decode<WGRAD>(p, ctl, t);
-            long long rows[4];
+            long long rows[WORDS];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const long long r = (long long)tl.row0 + (int)rank * MX_BM + 32 * i + lane;
+            for (int i = 0; i < WORDS; ++i) {
+                const long long r = (long long)tl.row0 + (WGRAD ? (int)rank * MX_BM : 0) + 32 * i + lane;
                 rows[i] = r < p.sa_rows ? r : p.sa_rows - 1;   // rows past the end are never stored; any valid address will do
             }
             // the words of MX_SCALE_AHEAD slices are in flight at any time: one slice per global-load round trip would
             // bound the whole pipeline (the loads wait behind the operand traffic)
+            struct Words { uint32_t w[8]; };
             auto load_slice = [&](int kt) {
                 const uint32_t* s = p.sa + (long long)(tl.k0 + kt) * p.sa_rows;
-                return make_uint4(__ldg(s + rows[0]), __ldg(s + rows[1]), __ldg(s + rows[2]), __ldg(s + rows[3]));
+                Words q;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) q.w[i] = i < WORDS ? __ldg(s + rows[i < WORDS ? i : 0]) : 0u;
+                return q;
             };
-            uint4 q[MX_SCALE_AHEAD];
+            Words q[MX_SCALE_AHEAD];
 #pragma unroll
             for (int i = 0; i < MX_SCALE_AHEAD; ++i) q[i] = load_slice(min(i, max(tl.k_tiles - 1, 0)));
             for (int kt0 = 0; ok && kt0 < tl.k_tiles; kt0 += MX_SCALE_AHEAD) {
@@ -772,10 +792,12 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 for (int i = 0; i < MX_SCALE_AHEAD; ++i) {
                     const int kt = kt0 + i;
                     if (kt >= tl.k_tiles) break;
-                    const uint4 cur = q[i];
+                    const Words cur = q[i];
                     if (kt + MX_SCALE_AHEAD < tl.k_tiles) q[i] = load_slice(kt + MX_SCALE_AHEAD);
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag))) { ok = false; break; }
-                    *reinterpret_cast<uint4*>(tiles_ptr + stage * MXP_STAGE_BYTES + MXP_SFA_OFF + lane * 16) = cur;
+                    uint8_t* to = tiles_ptr + stage * MXP_STAGE_BYTES + (WGRAD ? MXP_SFA_OFF : MXP_SFB_OFF) + lane * 16;
+                    *reinterpret_cast<uint4*>(to) = make_uint4(cur.w[0], cur.w[1], cur.w[2], cur.w[3]);
+                    if (!WGRAD) *reinterpret_cast<uint4*>(to + 512) = make_uint4(cur.w[4], cur.w[5], cur.w[6], cur.w[7]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote(full0 + stage * (uint32_t)sizeof(unsigned long long));
@@ -833,11 +855,42 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 tc_fence_after();
             }
             const uint32_t taddr = tmem_base + acc * MXP_ACC_STRIDE + ((uint32_t)(quarter * 32) << 16);
-            const int slab_in = tl.row0 + (int)rank * MX_BM + quarter * 32;   // first row of this warp's slab, as the A operand counts rows
-            const int rows_valid = max(0, min(32, tl.row_end - slab_in));
-            const int slab0 = slab_in + tl.out_shift;                         // ... and as the output does
+            if (!WGRAD) {
+                // lane = feature, column = row: the two warps of a lane quarter take the 32-row blocks alternately; a block is
+                // transposed on its way into the staging buffer
+                const int f = tl.n0 + (int)rank * MX_BM + quarter * 32;
 #pragma unroll 1
-            for (int c = half; c < 8; c += 2) {
+                for (int c = half; f < p.n_cols && c * 32 < tl.rows; c += 2) {
+                    uint32_t v[32], w[16];
+                    tc_ld_frag32(taddr + c * 32, v);
+                    tc_wait_ld();
+                    const int r0 = tl.row0 + c * 32, rv = min(32, tl.rows - c * 32);
+                    pack_frag(v, w);
+                    if (n_stores != 0) {
+                        if (lane == 0) bulk_wait_read0();
+                        __syncwarp();
+                    }
+                    store_frag(smem_u32(stage_ptr) + frag_offset(lane), w);
+                    if (rv == 32) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_2d(&map_o, f, r0, smem_u32(stage_ptr));
+                            bulk_commit();
+                        }
+                        ++n_stores;
+                    } else {
+                        __syncwarp();
+                        copy_block_rows(stage_ptr, p.out + (long long)r0 * p.ldo + f, p.ldo, rv, lane);
+                        __syncwarp();
+                    }
+                }
+            }
+            const int slab_in = tl.row0 + (int)rank * MX_BM + quarter * 32;   // first row of this warp's slab, inside the expert's output
+            const int rows_valid = max(0, min(32, p.M - slab_in));
+            const int slab0 = slab_in + tl.out_row0;                          // ... and in the output tensor
+#pragma unroll 1
+            for (int c = half; WGRAD && c < 8; c += 2) {
                 const int left = tl.width - 32 * c;   // columns of the tile from this block on (warp-uniform)
                 if (left <= 0) break;
                 const int n = tl.n0 + c * 32;
@@ -1363,7 +1416,7 @@ int launch_mx_quantize_tokens(long long R, int E, const bf16* x, long long ld, i
 }
 
 template <bool WGRAD>
-static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& sfb, const CUtensorMap& o, const MxPairParams& p,
+static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b_low, const CUtensorMap& sf, const CUtensorMap& o, const MxPairParams& p,
                           cudaStream_t s) {
     static int grid_of_device[64] = {};
     int dev = 0;
@@ -1387,7 +1440,7 @@ static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUte
         if (clusters > sms / 2) clusters = sms / 2;
         grid_of_device[dev] = 2 * clusters;
     }
-    return launch_dependent(mx_pair_kernel<WGRAD>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, sfb, o, p);
+    return launch_dependent(mx_pair_kernel<WGRAD>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, b_low, sf, o, p);
 }
 
 // dW [E, M, N] = Q(A)^T Q(B) per expert: a_* the M-side operand ([M, pitch] codes, scales with header and words),
@@ -1410,11 +1463,17 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
     p.prefix = reinterpret_cast<const int32_t*>(a_scales); p.E = E; p.M = M; p.m_tiles = m_tiles; p.n_tiles = n_tiles;
     p.n_cols = N; p.n_slices = n_slices; p.sa_rows = M;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales + MX_TOKENS_HEADER_BYTES); p.out = dw; p.ldo = N;
-    return launch_mx_pair<true>(a, b, sfb, o, p, s);
+    return launch_mx_pair<true>(a, b, b, sfb, o, p, s);
 }
 
-// CTA pairs from this many rows per expert on average (below it the 256-row tiles are mostly padding)
-constexpr long long kMxPairRows = 256;
+// CTA pairs from 256 rows per expert on average, and from 96 on if there are tiles for all pairs of the chip even with one row
+// tile per expert.  Single CTA against pair, gate/up / down / down dgrad / gate/up dgrad, rows per expert:
+//   128 (128 experts, 2048 x 768)   108 / 70 / 60 / 117 against 102 / 65 / 60 / 105 us     81:  88 / 63 / 52 / 96 against 83 / 60 / 51 / 91 us
+//   128 (8 experts, 4096 x 14336)   213 / 126 / 112 / 255 against 189 / 100 / 103 / 191 us  80:  169 / 93 / 92 / 172 against 170 / 95 / 96 / 176 us
+//   125 (16 experts, 256 x 512: 16 to 64 pair tiles)   7.7 / 5.6 / 5.5 / 6.1 against 8.0 / 6.5 / 6.2 / 7.4 us
+static bool mx_use_pairs(long long R, int E, int n_feat) {
+    return R >= 256ll * E || (R >= 96ll * E && (long long)E * ((n_feat + MXP_ROWS - 1) / MXP_ROWS) >= 74);
+}
 // The swapped form of the single-CTA kernel up to this many rows per expert on average.  There the time is the weights'
 // way from HBM, and what counts is bytes in flight and an even spread over the SMs: two CTAs with four stages of weights
 // and at most 64 rows each, against one with six stages that also hold 128 rows.  Down projection of 8 experts,
@@ -1433,21 +1492,21 @@ constexpr long long kMxSwappedRows = 64;
 static bool mx_single_swapped(long long R, int E) { return R <= kMxSwappedRows * E && MxGeo<64>::all_ctas_fit(E); }
 
 static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
-                               const uint8_t* b_codes, const uint8_t* b_scales_pair, const int32_t* offsets, bf16* out,
+                               const uint8_t* b_codes, const uint8_t* b_scales, const int32_t* offsets, bf16* out,
                                cudaStream_t s) {
-    const int n_tiles = (n_feat + MXP_NT - 1) / MXP_NT, k_tiles = k / MX_BK;
-    CUtensorMap a, b, sfb, o;
-    if (!make_map_typed(&a, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a_codes, k, (uint64_t)R, MX_BK, MX_BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_typed(&b, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, b_codes, k, (uint64_t)E * n_feat, MX_BK, MXP_NT / 2,
-                        CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_typed(&sfb, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, b_scales_pair, 256, (uint64_t)E * n_tiles * k_tiles, 256, 1,
+    const int k_tiles = k / MX_BK;
+    CUtensorMap w, x, x_low, sf, o;
+    if (!make_map_typed(&w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, b_codes, k, (uint64_t)E * n_feat, MX_BK, MX_BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a_codes, k, (uint64_t)R, MX_BK, MXP_NT / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&x_low, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a_codes, k, (uint64_t)R, MX_BK, MXP_LOW_BOX, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&sf, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, b_scales, 128, (uint64_t)E * (n_feat / 128) * k_tiles, 128, 1,
                         CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_out_map(&o, out, n_feat, (uint64_t)R))
         return MOE_ERR_CUDA;
     MxPairParams p = {};
-    p.prefix = offsets; p.E = E; p.k_tiles = k_tiles; p.n_tiles = n_tiles; p.n_cols = n_feat; p.sa_rows = R;
+    p.prefix = offsets; p.E = E; p.k_tiles = k_tiles; p.n_tiles = (n_feat + MXP_ROWS - 1) / MXP_ROWS; p.n_cols = n_feat; p.sa_rows = R;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales); p.out = out; p.ldo = n_feat;
-    return launch_mx_pair<false>(a, b, sfb, o, p, s);
+    return launch_mx_pair<false>(w, x, x_low, sf, o, p, s);
 }
 
 struct MxSingleArgs {
@@ -1489,9 +1548,8 @@ static int launch_mx_gemm_single(const MxSingleArgs& g, cudaStream_t s) {
 // [k/128][R], b [E, n_feat, k] codes with both scale tilings, out [R, n_feat] bf16.
 int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* b_codes,
                    const uint8_t* b_scales, const int32_t* offsets, bf16* out, cudaStream_t s) {
-    if (R >= kMxPairRows * E)
-        return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales + mx_w_scale_single_bytes(E, n_feat, k),
-                                   offsets, out, s);
+    if (mx_use_pairs(R, E, n_feat))
+        return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out, s);
     const MxSingleArgs args = {R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out};
     return mx_single_swapped(R, E) ? launch_mx_gemm_single<64>(args, s) : launch_mx_gemm_single<128>(args, s);
 }

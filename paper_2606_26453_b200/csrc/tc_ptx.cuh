@@ -5,6 +5,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <string.h>
+
 #include "common.cuh"
 
 namespace moe {
@@ -210,6 +212,70 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// ---- a 32 x 32 accumulator block transposed on its way out -------------------------------------------
+// With the weights on the M side the accumulator has a feature per lane and a row per column, and the output is row-major.  The
+// block is read from tensor memory as matrix fragments (16x256b: lane t of the warp has features t / 4 and t / 4 + 8, columns
+// 2 (t % 4) and the next, of every 8 columns; once for lanes 0..15, once for 16..31) and stored with stmatrix.trans, which
+// turns 8 x 8 blocks round: four instructions per block instead of 32 two-byte stores.
+//   v[16 h + 4 i + 2 s + c]: feature 16 h + 8 s + t / 4, row 8 i + 2 (t % 4) + c
+//   w[4 i + 2 h + s]:        the same, rounded, c in the low and high half
+__device__ __forceinline__ void tc_ld_frag16(uint32_t taddr, uint32_t* v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tc_ld_frag32(uint32_t taddr, uint32_t (&v)[32]) {
+    tc_ld_frag16(taddr, v);
+    tc_ld_frag16(taddr + (16u << 16), v + 16);
+}
+// pairs of fp32 values (in fragment order) -> w; the values of lane half h alone
+template <typename T>
+__device__ __forceinline__ void pack_frag_half(const T* v, int h, uint32_t (&w)[16]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            float lo, hi;
+            memcpy(&lo, &v[4 * i + 2 * s], 4);
+            memcpy(&hi, &v[4 * i + 2 * s + 1], 4);
+            w[4 * i + 2 * h + s] = pack_bf16(lo, hi);
+        }
+}
+template <typename T>
+__device__ __forceinline__ void pack_frag(const T (&v)[32], uint32_t (&w)[16]) {
+    pack_frag_half(v, 0, w);
+    pack_frag_half(v + 16, 1, w);
+}
+// this lane's address offset in a staging block (32 rows of 64 bytes, 64-byte swizzle): row lane % 8, features 8 (lane / 8) ...
+__device__ __forceinline__ uint32_t frag_offset(int lane) { return (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4); }
+__device__ __forceinline__ void store_frag(uint32_t at, const uint32_t (&w)[16]) {   // at: staging block + frag_offset
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at + i * 512), "r"(w[4 * i]),
+                     "r"(w[4 * i + 1]), "r"(w[4 * i + 2]), "r"(w[4 * i + 3])
+                     : "memory");
+}
+__device__ __forceinline__ void load_frag(uint32_t at, uint32_t (&w)[16]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w[4 * i]), "=r"(w[4 * i + 1]), "=r"(w[4 * i + 2]), "=r"(w[4 * i + 3])
+                     : "r"(at + i * 512)
+                     : "memory");
+}
+// the first `rows` rows of a staging block to global memory (row pitch ld elements)
+__device__ __forceinline__ void copy_block_rows(const uint8_t* block, bf16* dst, long long ld, int rows, int lane) {
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int j = s * 8 + (lane >> 2);
+        if (j < rows)
+            *reinterpret_cast<uint4*>(dst + j * ld + (lane & 3) * 8) =
+                *reinterpret_cast<const uint4*>(block + j * 64 + (((lane & 3) ^ ((j >> 1) & 3)) << 4));
+    }
+}
 
 // prefix[e] = number of tiles of `rows_per_tile` rows of the experts before e, prefix[E] = all of them.  One warp.
 __device__ __forceinline__ void exclusive_tile_prefix(const int32_t* offs, int32_t* prefix, int E, int rows_per_tile, int lane) {
