@@ -33,7 +33,7 @@
 //   row-ragged (forward, dgrad): output rows are the packed rows of an expert.  A tile starts at
 //     offsets[e] + TILE_M*i; loading past the expert's last row is harmless, stores are clipped.
 //     With small experts the padding of the fixed-height tiles is a sizeable share of the tensor
-//     work; two pair variants avoid it: the swapped kinds (FWD_PLAIN_T, DGRAD_T: weights on the M
+//     work; two pair variants avoid it: the swapped kinds (FWD_PLAIN_T, DGRAD_T, FWD_SWIGLU_T: weights on the M
 //     side of the MMA, the expert's rows on the N side, any tile height that is a multiple of 16)
 //     and, for the SwiGLU forward, half-height last tiles (FWD_SWIGLU_H: M = 128 over the pair).
 //   contraction-ragged (wgrad; the paper's dW1_e = X_e^T G_e): the expert's rows are the
@@ -87,16 +87,17 @@ constexpr int TMEM_COLS = 512;
 // any height that is a multiple of 16 (up to 256) instead of a fixed 128 / 256: an expert's rows are split into
 // equal tiles and almost no tensor work goes to padding.  The accumulator comes out transposed (lane = feature,
 // column = row); the epilogue transposes it back through its shared-memory staging blocks.
+// FWD_SWIGLU_T is the SwiGLU forward in that form, with 64 gate and 64 up features per CTA in one accumulator.
 // FWD_SWIGLU_H is FWD_SWIGLU in pair mode with half-height last tiles (small experts); a kind of its own so that the
 // kernel for large experts carries none of its bookkeeping.
 // DGRAD_SB / DGRAD_T_SB are DGRAD / DGRAD_T of the down projection with the SwiGLU backward fused into the epilogue:
 // the accumulator (dHact, fp32, never rounded) meets the saved pre-activations [g | u], which the epilogue warps fetch
 // as 32 x 32 blocks with bulk tensor loads, and the kernel writes dGU = [dg | du] instead of dHact.
 enum Kind { FWD_SWIGLU = 0, FWD_PLAIN = 1, DGRAD = 2, WGRAD = 3, FWD_PLAIN_T = 4, DGRAD_T = 5, FWD_SWIGLU_H = 6,
-            DGRAD_SB = 7, DGRAD_T_SB = 8 };
+            DGRAD_SB = 7, DGRAD_T_SB = 8, FWD_SWIGLU_T = 9 };
 __host__ __device__ constexpr bool wgrad(int kind) { return kind == WGRAD; }
 __host__ __device__ constexpr bool swiglu(int kind) { return kind == FWD_SWIGLU || kind == FWD_SWIGLU_H; }
-__host__ __device__ constexpr bool swapped(int kind) { return kind == FWD_PLAIN_T || kind == DGRAD_T || kind == DGRAD_T_SB; }
+__host__ __device__ constexpr bool swapped(int kind) { return kind == FWD_PLAIN_T || kind == DGRAD_T || kind == DGRAD_T_SB || kind == FWD_SWIGLU_T; }
 __host__ __device__ constexpr bool fused_sb(int kind) { return kind == DGRAD_SB || kind == DGRAD_T_SB; }
 // the kind whose operand loads and MMAs a kind shares
 __host__ __device__ constexpr int load_kind(int kind) { return kind == DGRAD_SB ? DGRAD : (kind == DGRAD_T_SB ? DGRAD_T : kind); }
@@ -270,7 +271,7 @@ __device__ __forceinline__ Tile decode_tile(const Params& p, const SharedCtl* ct
             const int per_tile = ((n_e + m_tiles_e - 1) / m_tiles_e + 15) & ~15;
             tl.row0 = ctl->offs[lo] + mt * per_tile;
             tl.rows = min(per_tile, tl.row_end - tl.row0);
-            tl.n0 = nt * TILE_M;   // output features per tile: 128, or 256 over a CTA pair
+            tl.n0 = nt * (KIND == FWD_SWIGLU_T ? SWAP_FEATS : TILE_M);   // a pair's tile: 256 features; SwiGLU: gate and up of 128
         } else {
             tl.row0 = ctl->offs[lo] + mt * TILE_M;
             tl.n0 = nt * BN;
@@ -317,7 +318,12 @@ __device__ __forceinline__ void stage_loads(const Tile& tl, int kb, const Params
         // In pair mode each CTA loads its own 128 features and half of the tile's rows (N/2 of the MMA's N,
         // N = rows rounded up to 16), in boxes of 32 rows; a single CTA loads all rows in boxes of 64.
         const int feat0 = tl.n0 + (PAIR ? (int)rank * SWAP_FEATS : 0);
-        if (KIND == FWD_PLAIN_T) {
+        if (KIND == FWD_SWIGLU_T) {
+            // 64 gate features, then the same 64 up features: gate and up of a feature land 64 tensor-memory lanes apart
+            const int ky = tl.e * p.b_rows_per_e + kb * BK, c = (tl.n0 >> 6) + (int)rank;
+            tma_load_3d(a_dst, map_b0, 0, ky, c, full);
+            tma_load_3d(a_dst + CHUNK_BYTES, map_b1, 0, ky, c, full);
+        } else if (KIND == FWD_PLAIN_T) {
             tma_load_3d(a_dst, map_b0, 0, tl.e * p.b_rows_per_e + kb * BK, feat0 >> 6, full);
         } else {
             const bool second = kb >= p.k_split;
@@ -391,8 +397,8 @@ template <int KIND, bool PAIR>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
                     const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_o0,
-                    const __grid_constant__ CUtensorMap map_o1, const __grid_constant__ CUtensorMap map_x,
-                    const Params p) {
+                    const __grid_constant__ CUtensorMap map_o1, const __grid_constant__ CUtensorMap map_r2,
+                    const __grid_constant__ CUtensorMap map_r1, const Params p) {
     using G = Geo<PAIR, fused_sb(KIND)>;
     constexpr int STAGES = G::STAGES;
     constexpr int STAGE_BYTES = G::STAGE_BYTES;
@@ -403,7 +409,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     static_assert(!HALF_TILES || PAIR, "half-height tiles exist in pair mode only");
     constexpr int ROW_TILE = SWAP ? SWAP_ROWS : G::TILE_M;   // rows an expert's tile count is computed from
     // operand major-ness of the MMA's M side (A) and N side (B); for the swapped kinds A is the weight tile
-    constexpr bool A_MN = (wgrad(KIND) || KIND == FWD_PLAIN_T);
+    constexpr bool A_MN = (wgrad(KIND) || KIND == FWD_PLAIN_T || KIND == FWD_SWIGLU_T);
     constexpr bool B_MN = (swiglu(KIND) || KIND == FWD_PLAIN || wgrad(KIND));
     constexpr uint32_t IDESC = make_idesc(G::TILE_M, BN, A_MN, B_MN);
     constexpr uint32_t IDESC_HALF = make_idesc(BM, BN, A_MN, B_MN);   // 128 x 256 over the CTA pair
@@ -444,7 +450,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         prefetch_tmap(&map_b1);
         prefetch_tmap(&map_o0);
         prefetch_tmap(&map_o1);
-        prefetch_tmap(&map_x);
+        prefetch_tmap(&map_r2);
+        prefetch_tmap(&map_r1);
     }
     // everything above may run while the kernel before is still finishing; the schedule is derived from its output
     grid_dependency_wait();
@@ -548,12 +555,12 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                         if (fix) {
                             const uint32_t land = smem_u32(&ctl->landed[stage]);
                             mbar_arrive_expect_tx(land, bytes);
-                            stage_loads<KIND, PAIR, false>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst,
+                            stage_loads<KIND, PAIR, false>(tl, kb, p, &map_a, &map_r2, &map_r1, &map_b0, &map_b1, a_dst,
                                                            a_dst + G::A_BYTES, land, rank, my_rows);
                         } else {
                             const uint32_t land = full0 + stage * (uint32_t)sizeof(unsigned long long);
                             if (PAIR) mbar_arrive_expect_tx_cluster(land, bytes); else mbar_arrive_expect_tx(land, bytes);
-                            stage_loads<KIND, PAIR, PAIR>(tl, kb, p, &map_a, &map_o1, &map_x, &map_b0, &map_b1, a_dst,
+                            stage_loads<KIND, PAIR, PAIR>(tl, kb, p, &map_a, &map_r2, &map_r1, &map_b0, &map_b1, a_dst,
                                                           a_dst + G::A_BYTES, land, rank, my_rows);
                         }
                     }
@@ -766,6 +773,16 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
         };
+        // FWD_SWIGLU_T: the two warps that hold gate and up of the same features (named barriers 1..4)
+        auto pair_sync = [](int id) { asm volatile("barrier.sync %0, 64;" ::"r"(id) : "memory"); };
+        auto pair_all = [](int id, bool mine) {
+            uint32_t all;
+            asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %2, 0; barrier.red.and.pred q, %1, 64, p; selp.u32 %0, 1, 0, q; }"
+                         : "=r"(all)
+                         : "r"(id), "r"((uint32_t)mine)
+                         : "memory");
+            return all != 0;
+        };
         // dg = dh*u*s*(1+g*(1-s)), du = dh*g*s with s = 1/(1+exp(-g))
         auto swiglu_grad = [](float dh, float g, float u, float& dg, float& du) {
             const float sg = __fdividef(1.f, 1.f + __expf(-g));
@@ -840,7 +857,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const long long t = tile_of<KIND>(it, first_tile, tile_stride, n_tiles_total);
             if (t < 0) break;
             const Tile tl = decode_tile<KIND, G::TILE_M>(p, ctl, t);
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag))) break;
+            bool ready = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag));
+            // (a gate and an up warp go through all barriers of theirs or neither does: the verdict is taken together)
+            if (KIND == FWD_SWIGLU_T) ready = pair_all(1 + (quarter & 1) + 2 * half, ready);
+            if (!ready) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16);
             // first row of this warp's slab.  Half-height pair tile (FWD_SWIGLU, M = 128 over two CTAs): this CTA holds
@@ -852,7 +872,56 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int rows_valid = wgrad(KIND) ? (slab0 < p.m_rows ? 32 : 0) : max(0, min(32, tl.row_end - slab0));
             const int slab_y = wgrad(KIND) ? tl.e * p.m_rows + slab0 : slab0;
             const long long row = (long long)slab0 + lane;
-            if (SWAP) {
+            if (KIND == FWD_SWIGLU_T) {
+                // Lanes 0..63 hold the gate values of this CTA's 64 features, lanes 64..127 their up values (columns: rows of
+                // the tile, as in the other swapped kinds).  The warp of a gate quarter and that of its up quarter (two further
+                // on, two warps earlier) take the same 32-row blocks: the up warp hands its block over in fp32 through the two
+                // warps' staging blocks, then writes U while the gate warp forms and writes H and G.
+                const bool up = quarter >= 2;
+                const int bar_id = 1 + (quarter & 1) + 2 * half;
+                uint8_t* up_stage = up ? stage_ptr : stage_ptr - 2 * STAGING_BLOCK_BYTES;
+                uint8_t* gate_stage = up ? stage_ptr + 2 * STAGING_BLOCK_BYTES : stage_ptr;
+                const int feat0 = tl.n0 + (int)rank * 64 + (quarter & 1) * 32;
+                const int n_row_blocks = feat0 < p.n_cols ? (tl.rows + 31) >> 5 : 0;
+#pragma unroll 1
+                for (int i = half; i < n_row_blocks; i += 2) {
+                    uint32_t v[32], w[16];
+                    tc_ld_frag32(taddr + i * 32, v);
+                    staging_free();
+                    tc_wait_ld();
+                    const int r0 = tl.row0 + i * 32, rv = min(32, tl.rows - i * 32);
+                    pair_sync(bar_id);
+                    if (up) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            *reinterpret_cast<uint4*>((j < 4 ? up_stage : gate_stage) + (j & 3) * 512 + lane * 16) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                        pair_sync(bar_id);
+                        if (p.gu) pack_frag(v, w);
+                        pair_sync(bar_id);
+                        if (p.gu) put_block(w, p.gu, &map_o1, 2ll * p.I, p.I + feat0, r0, rv);
+                    } else {
+                        float h[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float g = __uint_as_float(v[j]);
+                            h[j] = __fdividef(g, 1.f + __expf(-g));
+                        }
+                        pair_sync(bar_id);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float4 u = *reinterpret_cast<const float4*>((j < 4 ? up_stage : gate_stage) + (j & 3) * 512 + lane * 16);
+                            h[4 * j] *= u.x; h[4 * j + 1] *= u.y; h[4 * j + 2] *= u.z; h[4 * j + 3] *= u.w;
+                        }
+                        pack_frag(h, w);
+                        pair_sync(bar_id);
+                        put_block(w, p.out0, &map_o0, p.I, feat0, r0, rv);
+                        if (p.gu) {
+                            pack_frag(v, w);
+                            put_block(w, p.gu, &map_o1, 2ll * p.I, feat0, r0, rv);
+                        }
+                    }
+                }
+            } else if (SWAP) {
                 // lane = output feature, tensor-memory column = row of the tile; the two warps of a lane quarter
                 // take the 32-row blocks alternately
                 const int feat0 = tl.n0 + (PAIR ? (int)rank * SWAP_FEATS : 0) + quarter * 32;
@@ -1052,11 +1121,11 @@ bool make_map_mn(CUtensorMap* map, const void* base, uint64_t cols, uint64_t row
 // Grid of a launch: one CTA per SM (single), or as many CTA pairs as can be resident at once (pair).
 // A pair that could not be co-scheduled would run after the others and double the kernel's duration,
 // so the pair grid is sized from the occupancy query, per device and kernel.
-// Swapped kinds: `a`, `o1` and `x` are the row operand's maps with boxes of 4, 2 and 1 times the smallest box
-// (32 rows in pair mode, 64 otherwise); the other kinds pass `a` for `x`.
+// Swapped kinds: `a`, `r2` and `r1` are the row operand's maps with boxes of 4, 2 and 1 times the smallest box
+// (32 rows in pair mode, 64 otherwise); FWD_SWIGLU_H: `r1` has boxes of half a tile's rows; the other kinds pass `a`.
 template <int KIND, bool PAIR>
 int launch(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& o0,
-           const CUtensorMap& o1, const CUtensorMap& x, const Params& p, cudaStream_t s) {
+           const CUtensorMap& o1, const CUtensorMap& r2, const CUtensorMap& r1, const Params& p, cudaStream_t s) {
     static int grid_of_device[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
@@ -1082,7 +1151,7 @@ int launch(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, c
         }
     }
     return launch_dependent(kernel, grid_of_device[dev], NUM_THREADS, Geo<PAIR, fused_sb(KIND)>::SMEM_BYTES, PAIR ? 2 : 1, s, a, b0, b1, o0,
-                            o1, x, p);
+                            o1, r2, r1, p);
 }
 
 bool rows_per_expert_below(const moe_dims_t& d, long long rows) { return (long long)d.T * d.K < rows * d.E; }
@@ -1094,7 +1163,10 @@ bool rows_per_expert_below(const moe_dims_t& d, long long rows) { return (long l
 //   1024  (16 experts, 4096 x 4096)   385 / 386 / 810 against 358 / 357 / 759 us
 //   1536  (64 experts, 2048 x 1408)   384 / 418 / 780 against 374 / 403 / 751 us
 //   2048  (8 experts, 4096 x 14336)  1332 / 1250 / 2731 against 1328 / 1226 / 2956 us
-// With larger experts the padding is small and the fixed-height tiles have fewer MMAs to issue.  The line holds for Zipf and
+// With larger experts the padding is small and the fixed-height tiles have fewer MMAs to issue.  (Measured with each form alone for
+// half a second: in short bursts in turn, which share one power state, the swapped form looks 1-3 % faster at 2048 rows and
+// more, but its tiles of unlike heights drift apart along the contraction and fetch more from HBM -- gate/up dgrad of 8 experts of
+// 4096 x 14336 14.2 against 10.3 GB -- and under the power cap it is 7 to 22 % slower.)  The line holds for Zipf and
 // Dirichlet loads with the same averages: at 768 of them (64 experts, 2048 x 1408) 285 / 308 / 552 against 269 / 290 / 521 us
 // under the first, 1500 (16 experts, 4096 x 4096) 697 / 692 / 1515 against 689 / 694 / 1437 us under the second.
 // A contraction of fewer than 512 elements is over before the swapped form's transposed epilogue, and the line lies at 512
@@ -1109,10 +1181,27 @@ bool use_swapped(const moe_dims_t& d, int contraction) { return rows_per_expert_
 //   8 experts, 4096 x 14336   588 / 794 / 946 / 1099 against 502 / 712 / 885 / 1074 us
 // (a contraction of 4096 would bear a higher line).
 bool use_swapped_fused(const moe_dims_t& d) { return rows_per_expert_below(d, 512); }
+// The SwiGLU forward swapped (gate and up of 128 features x up to 256 rows per tile), below 1600 rows like the other swapped forms.
+// Its epilogue passes 4 KB per block of 32 x 32 values through shared memory, beside the operands' traffic, and that outlasts short
+// contractions; below 96 rows per expert the weights' bytes count and not the tiles.  At fewer than about eight tiles per CTA pair
+// the last tile's epilogue shows (only against the pair forms: single-CTA tiles lose more to padding).  Gate/up forward, other
+// forms against this one (* each alone for half a second, the rest in turn in short bursts):
+//   384 rows (64 experts of 1408)   contraction 2048: 365 -> 314 us *, 1536: 242 -> 222, 1280: 204 -> 192, 1024: 158 -> 160
+//   1024 rows (128 experts, 2048 x 768) 784 -> 761 us *; (16 experts of 2048) contraction 4096: 929 -> 866 us (of 4096), 1536: 181 -> 178,
+//        1280: 151 -> 159, 1024: 123 -> 143, 768: 100 -> 130
+//   Dirichlet loads, 451 rows on average (128 experts, 2880 x 2880)   2044 -> 1896 us *
+//   Zipf loads, 4096 rows on average (64 experts, 4096 x 1536)   5200 -> 5870 us *, 2048 rows (8 experts, 4096 x 14336) 2985 -> 3108 us *
+//   few tiles: 1000 rows (8 experts, 2048 x 192) 17.5 -> 19.5 us
+//   fewer rows: 250 (8 experts, 4096 x 14336) 528 -> 469 us, 96 (64 experts, 2048 x 1408) 150 -> 136, 69 (32 experts, 2048 x 1024) 51 -> 54,
+//        56 (128 experts, 2880 x 2880) 527 -> 527, 2 (128 experts, 2048 x 768) 89 -> 94
+bool use_swapped_swiglu(const moe_dims_t& d) {
+    if (rows_per_expert_below(d, 96) || !rows_per_expert_below(d, 1600) || d.H < 1536) return false;
+    return rows_per_expert_below(d, 320) || (long long)d.T * d.K * d.I >= 8ll * 74 * 256 * 128;
+}
 // Half-height last tiles of the SwiGLU forward, see launch_gateup_fwd.
 bool use_half_tiles(const moe_dims_t& d) { return rows_per_expert_below(d, 1600); }
-// The SwiGLU forward has no swapped form (measured slower: two accumulators per tile).  Its pair kernel runs an
-// expert's last <= 128 rows as a half-height tile, which makes pairs worthwhile from 320 rows per expert on average.
+// Where it does not run swapped, the SwiGLU forward has pair tiles of 256 rows, an expert's last <= 128 rows as a half-height
+// tile, which makes pairs worthwhile from 320 rows per expert on average; below it single-CTA tiles of 128 rows.
 constexpr long long kSwigluPairRows = 320;
 bool use_pairs_for_swiglu(const moe_dims_t& d) { return (long long)d.T * d.K >= kSwigluPairRows * d.E; }
 // Weight gradients have no row padding to lose, so pairs already win from 256 rows per expert.
@@ -1132,6 +1221,20 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
     // were 2-4 % faster (at 768 / 1024 / 1536 rows the half-height tiles are 3 / 3 / 1 %
     // faster under even loads; under Zipf and Dirichlet loads with averages of 512 to 1500 rows 0-4 % slower: 16 experts,
     // 4096 x 4096, 768 rows 795 -> 820 us).
+    if (use_swapped_swiglu(d)) {
+        const uint32_t box = 32;            // row boxes of 32 / 64 / 128 rows per CTA
+        CUtensorMap a, a2, a1, b0, b1, o0, o1;
+        if (!make_map(&a, x_perm, d.H, R, BK, 4 * box) || !make_map(&a2, x_perm, d.H, R, BK, 2 * box) ||
+            !make_map(&a1, x_perm, d.H, R, BK, box) || !make_map_mn(&b0, w_gate, d.I, (uint64_t)d.E * d.H, 1) ||
+            !make_map_mn(&b1, w_up, d.I, (uint64_t)d.E * d.H, 1) || !make_out_map(&o0, h_act, d.I, R) ||
+            !make_out_map(&o1, gu ? gu : h_act, gu ? 2ull * d.I : d.I, R))
+            return MOE_ERR_CUDA;
+        Params p = {};
+        p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
+        p.n_tiles = (d.I + SWAP_FEATS - 1) / SWAP_FEATS; p.n_cols = d.I; p.b_rows_per_e = d.H;
+        p.out0 = h_act; p.gu = gu; p.I = d.I; p.ldo = d.I; p.n_split = d.I;
+        return launch<FWD_SWIGLU_T, true>(a, b0, b1, o0, o1, a2, a1, p, s);
+    }
     const bool half_tiles = pair && use_half_tiles(d);
     CUtensorMap a, ah, b0, b1, o0, o1;
     if (!make_map(&a, x_perm, d.H, R, BK, BM) || !make_map(&ah, x_perm, d.H, R, BK, BM / 2) ||
@@ -1143,8 +1246,8 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
     p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
     p.n_tiles = (d.I + 127) / 128; p.n_cols = 2 * d.I; p.b_rows_per_e = d.H;
     p.out0 = h_act; p.gu = gu; p.I = d.I; p.ldo = d.I; p.n_split = 2 * d.I;
-    if (half_tiles) return launch<FWD_SWIGLU_H, true>(a, b0, b1, o0, o1, ah, p, s);
-    return pair ? launch<FWD_SWIGLU, true>(a, b0, b1, o0, o1, a, p, s) : launch<FWD_SWIGLU, false>(a, b0, b1, o0, o1, a, p, s);
+    if (half_tiles) return launch<FWD_SWIGLU_H, true>(a, b0, b1, o0, o1, a, ah, p, s);
+    return pair ? launch<FWD_SWIGLU, true>(a, b0, b1, o0, o1, a, a, p, s) : launch<FWD_SWIGLU, false>(a, b0, b1, o0, o1, a, a, p, s);
 }
 
 // Down forward: A = h_act [R,I]; B = w_down viewed as [E*I, H].
@@ -1164,7 +1267,7 @@ int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, 
         p.offsets = offsets; p.E = d.E; p.k_blocks = d.I / BK; p.k_split = p.k_blocks;
         p.n_tiles = (d.H + feats - 1) / feats; p.n_cols = d.H; p.b_rows_per_e = d.I;
         p.out0 = y_perm; p.ldo = d.H; p.n_split = d.H;
-        return launch<FWD_PLAIN_T, true>(a, b0, b0, o0, a2, a1, p, s);
+        return launch<FWD_PLAIN_T, true>(a, b0, b0, o0, o0, a2, a1, p, s);
     }
     // larger experts: 256-row pair tiles (each CTA loads half of B's columns)
     CUtensorMap a, b0, o0;
@@ -1175,7 +1278,7 @@ int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, 
     p.offsets = offsets; p.E = d.E; p.k_blocks = d.I / BK; p.k_split = p.k_blocks;
     p.n_tiles = (d.H + BN - 1) / BN; p.n_cols = d.H; p.b_rows_per_e = d.I;
     p.out0 = y_perm; p.ldo = d.H; p.n_split = d.H;
-    return launch<FWD_PLAIN, true>(a, b0, b0, o0, o0, a, p, s);
+    return launch<FWD_PLAIN, true>(a, b0, b0, o0, o0, a, a, p, s);
 }
 
 // Down dgrad: dh_act = dy_perm . w_down[e]^T.  A = dy_perm [R,H]; B = w_down viewed as [E*I, H] (rows are
@@ -1196,7 +1299,7 @@ int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_do
         p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
         p.n_tiles = (d.I + feats - 1) / feats; p.n_cols = d.I; p.b_rows_per_e = d.I;
         p.out0 = dh_act; p.ldo = d.I; p.n_split = d.I;
-        return launch<DGRAD_T, true>(a, b0, b0, o0, a2, a1, p, s);
+        return launch<DGRAD_T, true>(a, b0, b0, o0, o0, a2, a1, p, s);
     }
     CUtensorMap a, b0, o0;
     if (!make_map(&a, dy_perm, d.H, R, BK, BM) || !make_map(&b0, w_down, d.H, (uint64_t)d.E * d.I, BK, BN / 2) ||
@@ -1206,7 +1309,7 @@ int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_do
     p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
     p.n_tiles = (d.I + BN - 1) / BN; p.n_cols = d.I; p.b_rows_per_e = d.I;
     p.out0 = dh_act; p.ldo = d.I; p.n_split = d.I;
-    return launch<DGRAD, true>(a, b0, b0, o0, o0, a, p, s);
+    return launch<DGRAD, true>(a, b0, b0, o0, o0, a, a, p, s);
 }
 
 // Down dgrad with the SwiGLU backward in its epilogue: dgu = [dg | du] from dh = dy_perm . w_down[e]^T (kept in fp32)
@@ -1228,13 +1331,13 @@ int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const
             !make_map(&a1, dy_perm, d.H, R, BK, box) || !make_map(&b0, w_down, d.H, (uint64_t)d.E * d.I, BK, SWAP_FEATS))
             return MOE_ERR_CUDA;
         p.n_tiles = (d.I + feats - 1) / feats;
-        return launch<DGRAD_T_SB, true>(a, b0, g, o0, a2, a1, p, s);
+        return launch<DGRAD_T_SB, true>(a, b0, g, o0, o0, a2, a1, p, s);
     }
     CUtensorMap a, b0;
     if (!make_map(&a, dy_perm, d.H, R, BK, BM) || !make_map(&b0, w_down, d.H, (uint64_t)d.E * d.I, BK, BN / 2))
         return MOE_ERR_CUDA;
     p.n_tiles = (d.I + BN - 1) / BN;
-    return launch<DGRAD_SB, true>(a, b0, g, o0, o0, a, p, s);
+    return launch<DGRAD_SB, true>(a, b0, g, o0, o0, a, a, p, s);
 }
 
 // Gate/up dgrad: dx_perm = dg . w_gate[e]^T + du . w_up[e]^T.  A = dgu [R,2I]; the contraction runs over the
@@ -1255,7 +1358,7 @@ int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate
         p.offsets = offsets; p.E = d.E; p.k_blocks = 2 * d.I / BK; p.k_split = d.I / BK;
         p.n_tiles = (d.H + feats - 1) / feats; p.n_cols = d.H; p.b_rows_per_e = d.H;
         p.out0 = dx_perm; p.ldo = d.H; p.n_split = d.H;
-        return launch<DGRAD_T, true>(a, b0, b1, o0, a2, a1, p, s);
+        return launch<DGRAD_T, true>(a, b0, b1, o0, o0, a2, a1, p, s);
     }
     const uint32_t bn = BN / 2;
     CUtensorMap a, b0, b1, o0;
@@ -1266,7 +1369,7 @@ int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate
     p.offsets = offsets; p.E = d.E; p.k_blocks = 2 * d.I / BK; p.k_split = d.I / BK;
     p.n_tiles = (d.H + BN - 1) / BN; p.n_cols = d.H; p.b_rows_per_e = d.H;
     p.out0 = dx_perm; p.ldo = d.H; p.n_split = d.H;
-    return launch<DGRAD, true>(a, b0, b1, o0, o0, a, p, s);
+    return launch<DGRAD, true>(a, b0, b1, o0, o0, a, a, p, s);
 }
 
 // Weight gradients: the tile grid is static (M x N per expert).  Pairs (256 x 256 tiles) pay off once an
@@ -1286,7 +1389,7 @@ int launch_down_wgrad(const moe_dims_t& d, const bf16* h_act, const bf16* dy_per
     p.offsets = offsets; p.E = d.E; p.m_rows = d.I; p.m_tiles = (d.I + tile_m - 1) / tile_m;
     p.n_tiles = (d.H + BN - 1) / BN; p.n_cols = d.H; p.n_split = d.H; p.ldo = d.H;
     p.out0 = dw_down; p.out1 = nullptr;
-    return pair ? launch<WGRAD, true>(a, b0, b0, o0, o0, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o0, a, p, s);
+    return pair ? launch<WGRAD, true>(a, b0, b0, o0, o0, a, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o0, a, a, p, s);
 }
 
 // Gate/up wgrad (the paper's dW1): [dw_gate[e] | dw_up[e]] = x_perm_e^T . dgu_e.  A = x_perm [R,H] (M = H),
@@ -1304,7 +1407,7 @@ int launch_gateup_wgrad(const moe_dims_t& d, const bf16* x_perm, const bf16* dgu
     p.offsets = offsets; p.E = d.E; p.m_rows = d.H; p.m_tiles = (d.H + tile_m - 1) / tile_m;
     p.n_tiles = (2 * d.I + BN - 1) / BN; p.n_cols = 2 * d.I; p.n_split = d.I; p.ldo = d.I;
     p.out0 = dw_gate; p.out1 = dw_up;
-    return pair ? launch<WGRAD, true>(a, b0, b0, o0, o1, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o1, a, p, s);
+    return pair ? launch<WGRAD, true>(a, b0, b0, o0, o1, a, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o1, a, a, p, s);
 }
 
 }  // namespace moe

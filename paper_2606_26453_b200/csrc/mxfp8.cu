@@ -1467,12 +1467,13 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
 }
 
 // CTA pairs from 256 rows per expert on average, and from 96 on if there are tiles for all pairs of the chip even with one row
-// tile per expert.  Single CTA against pair, gate/up / down / down dgrad / gate/up dgrad, rows per expert:
+// tile per expert and the contraction is at least 512.  Single CTA against pair, gate/up / down / down dgrad / gate/up dgrad, rows per expert:
 //   128 (128 experts, 2048 x 768)   108 / 70 / 60 / 117 against 102 / 65 / 60 / 105 us     81:  88 / 63 / 52 / 96 against 83 / 60 / 51 / 91 us
 //   128 (8 experts, 4096 x 14336)   213 / 126 / 112 / 255 against 189 / 100 / 103 / 191 us  80:  169 / 93 / 92 / 172 against 170 / 95 / 96 / 176 us
 //   125 (16 experts, 256 x 512: 16 to 64 pair tiles)   7.7 / 5.6 / 5.5 / 6.1 against 8.0 / 6.5 / 6.2 / 7.4 us
-static bool mx_use_pairs(long long R, int E, int n_feat) {
-    return R >= 256ll * E || (R >= 96ll * E && (long long)E * ((n_feat + MXP_ROWS - 1) / MXP_ROWS) >= 74);
+//   229 (2 experts, gate/up of 6272 features each, contraction 128)   6.5 against 7.4 us
+static bool mx_use_pairs(long long R, int E, int n_feat, int k) {
+    return R >= 256ll * E || (R >= 96ll * E && k >= 512 && (long long)E * ((n_feat + MXP_ROWS - 1) / MXP_ROWS) >= 74);
 }
 // The swapped form of the single-CTA kernel up to this many rows per expert on average.  There the time is the weights'
 // way from HBM, and what counts is bytes in flight and an even spread over the SMs: two CTAs with four stages of weights
@@ -1548,7 +1549,7 @@ static int launch_mx_gemm_single(const MxSingleArgs& g, cudaStream_t s) {
 // [k/128][R], b [E, n_feat, k] codes with both scale tilings, out [R, n_feat] bf16.
 int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* b_codes,
                    const uint8_t* b_scales, const int32_t* offsets, bf16* out, cudaStream_t s) {
-    if (mx_use_pairs(R, E, n_feat))
+    if (mx_use_pairs(R, E, n_feat, k))
         return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out, s);
     const MxSingleArgs args = {R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out};
     return mx_single_swapped(R, E) ? launch_mx_gemm_single<64>(args, s) : launch_mx_gemm_single<128>(args, s);

@@ -17,9 +17,10 @@ CASES = {   # output features, contraction, rows of each expert
     "low_box_edges": (256, 640, [128, 129, 1, 16, 17, 1040, 624]), # 64 rows per CTA and more; five tiles of 208
     "empty_and_last": (640, 384, [0, 900, 0, 33, 0]),
     "many_slices": (256, 1152, [300, 250]),                        # more slices than scale words in flight
-    "96_rows": (256, 128, [96] * 74),                              # the first sizes of the pair form with few rows ...
-    "96_rows_too_few_tiles": (256, 128, [96] * 73),                # ... and the last of the other
-    "96_rows_uneven": (384, 128, [1, 0, 31, 33, 352] + [99] * 42),
+    "96_rows": (256, 512, [96] * 74),                              # the first sizes of the pair form with few rows ...
+    "96_rows_too_few_tiles": (256, 512, [96] * 73),                # ... and the last of the other:
+    "96_rows_short": (256, 384, [96] * 74),                        # too few tiles, too short a contraction
+    "96_rows_uneven": (384, 512, [1, 0, 31, 33, 352] + [99] * 42),
 }
 
 
