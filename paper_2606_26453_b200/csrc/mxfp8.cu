@@ -1009,6 +1009,27 @@ __device__ __forceinline__ int mx_block_exp(const uint4& v) {
     m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 2));
     return mx_scale_exp(fmaxf(mx_lo(m), mx_hi(m)));
 }
+// 32 bytes (16 bf16 values) with one load if the operand is 32-byte aligned, as two halves if only 16 (what callers owe).
+__device__ __forceinline__ void mx_load32(const uint4* p, bool whole, uint4& lo, uint4& hi) {
+    if (whole) {
+        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
+                     : "l"(p));
+    } else {
+        lo = __ldg(p);
+        hi = __ldg(p + 1);
+    }
+}
+// Scale exponent of a block of 32 values held by 2 consecutive lanes, 16 each.
+__device__ __forceinline__ int mx_block_exp2(const uint4& lo, const uint4& hi) {
+    uint32_t m = mx_abs_max(mx_abs_max4(lo), mx_abs_max4(hi));
+    m = mx_abs_max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    return mx_scale_exp(fmaxf(mx_lo(m), mx_hi(m)));
+}
+__device__ __forceinline__ uint4 mx_codes16(const uint4& lo, const uint4& hi, int se) {   // 16 consecutive values -> 16 code bytes
+    const uint2 a = mx_codes8(lo, se), b = mx_codes8(hi, se);
+    return make_uint4(a.x, a.y, b.x, b.y);
+}
 // Where the scale word of feature `f` (4 scale bytes of one K slice) sits inside a 128-feature block of 512 bytes, in words.
 __device__ __forceinline__ int mx_sf_word(int f) { return (f % 32) * 4 + (f % 128) / 32; }
 // The scale words of 128 features f0 .. f0 + 127 (f0 a multiple of 128) of one K slice, in shared memory, into both
@@ -1021,9 +1042,9 @@ __device__ __forceinline__ void mx_store_weight_scales(const uint32_t* words, in
     *reinterpret_cast<uint32_t*>(pair + nt * pair_stride + (c >> 7) * 512 + mx_sf_word(c) * 4) = words[i];
 }
 
-// rows x n bf16 -> codes (same layout) and scales.  A block takes 128 rows x one 128-wide slice; a half-warp holds a row
-// (8 elements per lane, one 16-byte load), eight rows one after the other with their loads all in flight; the 4 lanes of a
-// block of 32 agree on its scale through two shuffles.  The scale bytes meet in shared memory and leave as one 32-bit word
+// rows x n bf16 -> codes (same layout) and scales.  A block takes 128 rows x one 128-wide slice; eight lanes hold a row (16
+// elements per lane, one 32-byte load), four rows one after the other with their loads all in flight; the 2 lanes of a
+// block of 32 agree on its scale through one shuffle.  The scale bytes meet in shared memory and leave as one 32-bit word
 // per (row, slice):
 //   WEIGHTS = false (activations): word [slice][row], 512 contiguous bytes per block of threads;
 //   WEIGHTS = true  (weights whose contraction axis is contiguous, rows = E * n_feat, e.g. W_down read as [I, H] for the
@@ -1031,13 +1052,13 @@ __device__ __forceinline__ void mx_store_weight_scales(const uint32_t* words, in
 //                    column range of a wider operand (out_k_tiles slices per row, this input filling slices
 //                    out_kt0 .. out_kt0 + n/128): W_gate and W_up side by side along the contraction of the gate/up
 //                    data gradient.
-// 3 bytes of HBM traffic per element, so bound by HBM only if few instructions and few partial sectors go into one.  Inside
-// an FP8 step, 201 M weights (128 x 2048 x 768): 242 -> 122 us (4.9 TB/s); activations 131072 x 2048: 184 -> 119 us
-// (6.8 TB/s).  Before, a warp walked along a row: every (row, slice) took a 64-bit division, eight shuffles and, for
-// weights, two 4-byte stores into a sector each.
+// 3 bytes of HBM traffic per element, so bound by HBM only if few instructions and few partial sectors go into one.  201 M weights
+// (128 x 768 x 2048) 115 -> 95 us (6.4 TB/s), two of them side by side 238 -> 194 us, activations 131072 x 2048 125 -> 122 us
+// (6.6 TB/s), each against a half-warp per row with 16-byte loads and 8-byte stores.  (With a warp walking along a row, every
+// (row, slice) took a 64-bit division, eight shuffles and, for weights, two 4-byte stores into a sector each: 242 and 184 us.)
 template <bool WEIGHTS>
 __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n, int n_feat,
-                                                               int out_k_tiles, int out_kt0, uint2* __restrict__ codes,
+                                                               int out_k_tiles, int out_kt0, uint4* __restrict__ codes,
                                                                uint8_t* __restrict__ scales, uint8_t* __restrict__ scales_pair) {
     __shared__ __align__(16) uint8_t sf[128 * 4];
     if (!grid_dependency_wait_tested()) return;
@@ -1045,19 +1066,23 @@ __global__ void __launch_bounds__(256) mx_quantize_rows_kernel(const uint4* __re
     const int k_tiles = n >> 7;
     const int row_tile = (int)(blockIdx.x / (unsigned)k_tiles), kt = (int)(blockIdx.x - (unsigned)row_tile * (unsigned)k_tiles);
     const long long row0 = 128ll * row_tile;
-    const int sub = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+    const int sub = threadIdx.x >> 3, l8 = threadIdx.x & 7;
     const int n_rows = (int)min(128ll, rows - row0);
-    const uint4* src = x + (row0 + sub) * (n >> 3) + kt * 16 + l16;
-    uint2* dst = codes + ((row0 + sub) * out_k_tiles + out_kt0 + kt) * 16 + l16;
-    const long long src_step = 16ll * (n >> 3), dst_step = 16ll * out_k_tiles * 16;
-    uint4 v[8];
+    const bool whole = (reinterpret_cast<uintptr_t>(x) & 31) == 0;
+    const uint4* src = x + (row0 + sub) * (n >> 3) + kt * 16 + l8 * 2;
+    uint4* dst = codes + ((row0 + sub) * out_k_tiles + out_kt0 + kt) * 8 + l8;
+    const long long src_step = 32ll * (n >> 3), dst_step = 32ll * out_k_tiles * 8;
+    uint4 lo[4], hi[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = sub + 16 * i < n_rows ? __ldg(src + i * src_step) : make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < 4; ++i) {
+        lo[i] = hi[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (sub + 32 * i < n_rows) mx_load32(src + i * src_step, whole, lo[i], hi[i]);
+    }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int se = mx_block_exp(v[i]);
-        if (sub + 16 * i < n_rows) dst[i * dst_step] = mx_codes8(v[i], se);
-        if ((l16 & 3) == 0) sf[(sub + 16 * i) * 4 + (l16 >> 2)] = (uint8_t)(se + 127);
+    for (int i = 0; i < 4; ++i) {
+        const int se = mx_block_exp2(lo[i], hi[i]);
+        if (sub + 32 * i < n_rows) dst[i * dst_step] = mx_codes16(lo[i], hi[i], se);
+        if ((l8 & 1) == 0) sf[(sub + 32 * i) * 4 + (l8 >> 1)] = (uint8_t)(se + 127);
     }
     __syncthreads();
     const int i = threadIdx.x;
@@ -1358,7 +1383,7 @@ size_t mx_w_scale_bytes(int E, int n_feat, int k) {
 static unsigned mx_row_quantiser_blocks(long long rows, int k) { return (unsigned)((rows + 127) / 128 * (k / 128)); }
 
 int launch_mx_quantize_rows(long long rows, int n, const bf16* x, uint8_t* codes, uint8_t* scales, cudaStream_t s) {
-    return launch_streaming(mx_quantize_rows_kernel<false>, mx_row_quantiser_blocks(rows, n), s, reinterpret_cast<const uint4*>(x), rows, n, 0, n / 128, 0, reinterpret_cast<uint2*>(codes), scales,
+    return launch_streaming(mx_quantize_rows_kernel<false>, mx_row_quantiser_blocks(rows, n), s, reinterpret_cast<const uint4*>(x), rows, n, 0, n / 128, 0, reinterpret_cast<uint4*>(codes), scales,
                             static_cast<uint8_t*>(nullptr));
 }
 
@@ -1389,7 +1414,7 @@ int launch_mx_quantize_w_rows(int E, int n_feat, int k, int k_total, int k_off, 
                               cudaStream_t s) {
     const long long rows = (long long)E * n_feat;
     return launch_streaming(mx_quantize_rows_kernel<true>, mx_row_quantiser_blocks(rows, k), s, reinterpret_cast<const uint4*>(w), rows, k, n_feat,
-                            k_total / 128, k_off / 128, reinterpret_cast<uint2*>(codes), scales,
+                            k_total / 128, k_off / 128, reinterpret_cast<uint4*>(codes), scales,
                             scales + mx_w_scale_single_bytes(E, n_feat, k_total));
 }
 

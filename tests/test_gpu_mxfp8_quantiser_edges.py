@@ -95,3 +95,27 @@ def test_transposing_quantisers_take_any_16_byte_alignment(shift):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     want = np.stack([O.mxfp8_quantize(w[e].T)[0] for e in range(E)])               # [E, H, I]
     assert np.array_equal(out[0][0].cpu().numpy().reshape(E, H, I), want)
+
+
+@pytest.mark.parametrize("rows", [1, 33, 130])
+def test_row_quantisers_take_any_16_byte_alignment(rows):
+    from paper_2606_26453_b200 import binding as B
+    n, E = 384, 2
+    rng = np.random.default_rng(rows)
+    x = W.round_to_bf16(rng.standard_normal((rows, n)).astype(np.float32))
+    w = W.round_to_bf16(rng.standard_normal((E, n, 128)).astype(np.float32))      # W_down [E, I, H]
+    d = B.dims(rows, 128, n, E, 1)
+    for shift in (8, 16):                                                         # elements: 16 and 32 bytes into the buffer
+        def shifted(a):
+            room = torch.zeros(a.size + 32, dtype=torch.bfloat16, device="cuda")
+            room[shift:shift + a.size] = Hh.to_dev_bf16(a).flatten()
+            return room[shift:shift + a.size].view(a.shape)
+        c, s = _u8(rows * n + 16)[16:], _u8(B.moe_mxfp8_act_scale_bytes(d))
+        B.moe_mxfp8_quantize_h_act(d, shifted(x), c, s)
+        wc, ws = _u8(E * n * 128 + 16)[16:], _u8(B.moe_mxfp8_w_down_dgrad_scale_bytes(d))
+        B.moe_mxfp8_quantize_w_down_dgrad(d, shifted(w), wc, ws)
+        torch.cuda.synchronize()
+        codes, scales, _ = O.mxfp8_quantize(x)
+        assert np.array_equal(c.cpu().numpy().reshape(rows, n), codes)
+        assert np.array_equal(_act_scales_from_layout(s.cpu().numpy(), rows, n), scales)
+        assert np.array_equal(wc.cpu().numpy().reshape(E, n, 128), O.mxfp8_quantize(w)[0])
