@@ -29,6 +29,9 @@ int sm_count();
 //     histogram kernel, lets it start only after its own wait.)
 //   - grid_launch_dependents() comes after grid_dependency_wait(), so no more than one kernel is ever ahead of its turn and a
 //     kernel that has started knows everything before its immediate predecessor to be complete.
+//   - A weight gradient that a call launches right behind a data gradient on the same inputs does not depend on it.  Behind a
+//     short one it runs beside it: no wait at its start (that it has started means that all before the data gradient is complete), the wait before
+//     it lets ITS successor start, so that a kernel which has waited for it has waited for both.
 //   - The GEMMs call it at the end of each warp's role.  One thread's call counts for its CTA, so the row-ragged bf16 kinds,
 //     where one warp has no role, trigger right after set-up, and the CTAs of a GEMM that follows take each SM as it comes
 //     free.  With the call behind the last barrier of the teardown steps of long GEMMs take longer, chip idle between steps:
@@ -116,13 +119,13 @@ int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, 
 int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const int32_t* offsets,
                       bf16* dh_act, cudaStream_t s);
 int launch_down_wgrad(const moe_dims_t& d, const bf16* h_act, const bf16* dy_perm, const int32_t* offsets,
-                      bf16* dw_down, cudaStream_t s);
+                      bf16* dw_down, bool beside, cudaStream_t s);   // beside: right behind launch_down_dgrad, see above
 int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const bf16* gu,
                                  const int32_t* offsets, bf16* dgu, cudaStream_t s);
 int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate, const bf16* w_up,
                         const int32_t* offsets, bf16* dx_perm, cudaStream_t s);
 int launch_gateup_wgrad(const moe_dims_t& d, const bf16* x_perm, const bf16* dgu, const int32_t* offsets,
-                        bf16* dw_gate, bf16* dw_up, cudaStream_t s);
+                        bf16* dw_gate, bf16* dw_up, bool beside, cudaStream_t s);
 
 // ---- block-scaled FP8 down projection (mxfp8.cu) -------------------------------------------------
 size_t mx_w_scale_single_bytes(int E, int n_feat, int k);   // weight scales in the single-CTA tiling

@@ -120,6 +120,7 @@ struct Params {
     bf16* out1;
     bf16* gu;            // FWD_SWIGLU: [R, 2I] or null
     int I;               // FWD_SWIGLU
+    int beside;          // WGRAD: nothing here depends on the kernel right before, a data gradient of the same call (see common.cuh)
 };
 
 struct SharedCtl {
@@ -454,7 +455,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         prefetch_tmap(&map_r1);
     }
     // everything above may run while the kernel before is still finishing; the schedule is derived from its output
-    grid_dependency_wait();
+    if (!wgrad(KIND) || !p.beside) grid_dependency_wait();
     for (int e = threadIdx.x; e <= p.E; e += NUM_THREADS) ctl->offs[e] = p.offsets[e];
     __syncthreads();
     if (wgrad(KIND)) {
@@ -1084,6 +1085,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
 
     // ---- teardown ----
+    if (wgrad(KIND) && p.beside) grid_dependency_wait();   // what follows this kernel takes both to be complete
     grid_launch_dependents();   // as late as this: see common.cuh
     tc_fence_before();
     __syncthreads();
@@ -1377,7 +1379,7 @@ int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate
 // the independent 128 x 256 tiles are faster.
 // Down wgrad: dw_down[e] [I,H] = h_act_e^T . dy_perm_e.  A = h_act [R,I] (M = I), B = dy_perm [R,H] (N = H).
 int launch_down_wgrad(const moe_dims_t& d, const bf16* h_act, const bf16* dy_perm, const int32_t* offsets,
-                      bf16* dw_down, cudaStream_t s) {
+                      bf16* dw_down, bool beside, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     const bool pair = use_pairs_for_wgrad(d);
     const int tile_m = pair ? 2 * BM : BM;
@@ -1388,14 +1390,14 @@ int launch_down_wgrad(const moe_dims_t& d, const bf16* h_act, const bf16* dy_per
     Params p = {};
     p.offsets = offsets; p.E = d.E; p.m_rows = d.I; p.m_tiles = (d.I + tile_m - 1) / tile_m;
     p.n_tiles = (d.H + BN - 1) / BN; p.n_cols = d.H; p.n_split = d.H; p.ldo = d.H;
-    p.out0 = dw_down; p.out1 = nullptr;
+    p.out0 = dw_down; p.out1 = nullptr; p.beside = beside;
     return pair ? launch<WGRAD, true>(a, b0, b0, o0, o0, a, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o0, a, a, p, s);
 }
 
 // Gate/up wgrad (the paper's dW1): [dw_gate[e] | dw_up[e]] = x_perm_e^T . dgu_e.  A = x_perm [R,H] (M = H),
 // B = dgu [R,2I] (N = 2I); output columns below I go to dw_gate, the rest to dw_up.
 int launch_gateup_wgrad(const moe_dims_t& d, const bf16* x_perm, const bf16* dgu, const int32_t* offsets,
-                        bf16* dw_gate, bf16* dw_up, cudaStream_t s) {
+                        bf16* dw_gate, bf16* dw_up, bool beside, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     const bool pair = use_pairs_for_wgrad(d);
     const int tile_m = pair ? 2 * BM : BM;
@@ -1406,7 +1408,7 @@ int launch_gateup_wgrad(const moe_dims_t& d, const bf16* x_perm, const bf16* dgu
     Params p = {};
     p.offsets = offsets; p.E = d.E; p.m_rows = d.H; p.m_tiles = (d.H + tile_m - 1) / tile_m;
     p.n_tiles = (2 * d.I + BN - 1) / BN; p.n_cols = 2 * d.I; p.n_split = d.I; p.ldo = d.I;
-    p.out0 = dw_gate; p.out1 = dw_up;
+    p.out0 = dw_gate; p.out1 = dw_up; p.beside = beside;
     return pair ? launch<WGRAD, true>(a, b0, b0, o0, o1, a, a, p, s) : launch<WGRAD, false>(a, b0, b0, o0, o1, a, a, p, s);
 }
 
