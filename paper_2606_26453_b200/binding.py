@@ -116,6 +116,12 @@ def load_library() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = ctypes.c_int
             fn.argtypes = argtypes
+        lib.addresses = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in sigs}
+        try:
+            from . import _pycall
+        except ImportError as e:
+            raise ImportError("the binding's helper _pycall is missing: build it with `python -m paper_2606_26453_b200.build`") from e
+        lib.native_call = _pycall.call
         _lib = lib
     return _lib
 
@@ -124,26 +130,26 @@ def status_string(status: int) -> str:
     return load_library().moe_status_string(int(status)).decode()
 
 
-# A call of the smallest layers takes the device a few microseconds, so what the binding adds counts: pointers and stream
-# travel as plain integers (the declared argument types convert them), and the stream handle is asked for directly -- building
-# torch's Stream object took 3.2 of the 12 us that such a call cost the host, the wrapping of the pointers another 2.
-def _ptr(t):
-    if t is None or isinstance(t, int):
-        return t
-    if not t.is_contiguous():
-        raise ValueError("tensor must be contiguous")
-    return t.data_ptr()
+# A call of the smallest layers takes the device a few microseconds, so what the binding adds counts: the arguments are marshalled in
+# C (csrc/pycall.c: tensors must be contiguous; integers pass as addresses, None as NULL), and the stream handle is asked for
+# directly -- building torch's Stream object took 3.2 of the 12 us that such a call once cost the host.
+_cuda_is_initialized = torch.cuda.is_initialized
+_cuda_device = getattr(torch._C, "_cuda_getDevice", None)
+_cuda_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream() -> int:
     """Handle of the current torch stream of the current device."""
-    if not torch.cuda.is_initialized():
+    if not _cuda_is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _cuda_raw_stream(_cuda_device())
 
 
-def _call(name: str, *args) -> None:
-    rc = getattr(_lib or load_library(), name)(*args)
+def _call(name: str, d: MoeDims, *args) -> None:
+    if not isinstance(d, MoeDims):
+        raise TypeError(f"{name}: the first argument must be a MoeDims")
+    lib = _lib or load_library()
+    rc = lib.native_call(lib.addresses[name], d, *args, _stream())
     if rc != 0:
         raise MoeError(name, rc, status_string(rc))
 
@@ -169,85 +175,75 @@ def moe_device_status() -> int:
 
 
 def moe_permute(d, x, topk_idx, x_perm, counts, offsets, row_to_pair, pair_to_row, workspace):
-    _call("moe_permute", ctypes.byref(d), _ptr(x), _ptr(topk_idx), _ptr(x_perm), _ptr(counts), _ptr(offsets),
-          _ptr(row_to_pair), _ptr(pair_to_row), _ptr(workspace), ctypes.c_size_t(workspace.numel() * workspace.element_size()),
-          _stream())
+    _call("moe_permute", d, x, topk_idx, x_perm, counts, offsets, row_to_pair, pair_to_row, workspace,
+          workspace.numel() * workspace.element_size())
 
 
 def moe_permute_static_scratch(d, x, topk_idx, x_perm, counts, offsets, row_to_pair, pair_to_row):
     """moe_permute for callers that may not allocate: the scratch is a fixed array inside the library
     (shared by all calls on a device; see the header for the size limit and the no-overlap rule)."""
-    _call("moe_permute_static_scratch", ctypes.byref(d), _ptr(x), _ptr(topk_idx), _ptr(x_perm), _ptr(counts),
-          _ptr(offsets), _ptr(row_to_pair), _ptr(pair_to_row), _stream())
+    _call("moe_permute_static_scratch", d, x, topk_idx, x_perm, counts, offsets, row_to_pair, pair_to_row)
 
 
 def moe_permute_bwd(d, dx_perm, pair_to_row, dx):
-    _call("moe_permute_bwd", ctypes.byref(d), _ptr(dx_perm), _ptr(pair_to_row), _ptr(dx), _stream())
+    _call("moe_permute_bwd", d, dx_perm, pair_to_row, dx)
 
 
 def moe_grouped_gemm_gateup_swiglu(d, x_perm, w_gate, w_up, offsets, h_act, gu_saved):
-    _call("moe_grouped_gemm_gateup_swiglu", ctypes.byref(d), _ptr(x_perm), _ptr(w_gate), _ptr(w_up), _ptr(offsets),
-          _ptr(h_act), _ptr(gu_saved), _stream())
+    _call("moe_grouped_gemm_gateup_swiglu", d, x_perm, w_gate, w_up, offsets, h_act, gu_saved)
 
 
 def moe_grouped_gemm_down(d, h_act, w_down, offsets, y_perm):
-    _call("moe_grouped_gemm_down", ctypes.byref(d), _ptr(h_act), _ptr(w_down), _ptr(offsets), _ptr(y_perm), _stream())
+    _call("moe_grouped_gemm_down", d, h_act, w_down, offsets, y_perm)
 
 
 def moe_unpermute_combine(d, y_perm, topk_w, pair_to_row, y):
-    _call("moe_unpermute_combine", ctypes.byref(d), _ptr(y_perm), _ptr(topk_w), _ptr(pair_to_row), _ptr(y), _stream())
+    _call("moe_unpermute_combine", d, y_perm, topk_w, pair_to_row, y)
 
 
 def moe_unpermute_combine_bwd(d, dy, y_perm, topk_w, pair_to_row, dy_perm, dtopk_w):
-    _call("moe_unpermute_combine_bwd", ctypes.byref(d), _ptr(dy), _ptr(y_perm), _ptr(topk_w), _ptr(pair_to_row),
-          _ptr(dy_perm), _ptr(dtopk_w), _stream())
+    _call("moe_unpermute_combine_bwd", d, dy, y_perm, topk_w, pair_to_row, dy_perm, dtopk_w)
 
 
 def moe_grouped_gemm_down_dgrad(d, dy_perm, w_down, offsets, dh_act):
-    _call("moe_grouped_gemm_down_dgrad", ctypes.byref(d), _ptr(dy_perm), _ptr(w_down), _ptr(offsets), _ptr(dh_act),
-          _stream())
+    _call("moe_grouped_gemm_down_dgrad", d, dy_perm, w_down, offsets, dh_act)
 
 
 def moe_grouped_gemm_down_wgrad(d, h_act, dy_perm, offsets, dw_down):
-    _call("moe_grouped_gemm_down_wgrad", ctypes.byref(d), _ptr(h_act), _ptr(dy_perm), _ptr(offsets), _ptr(dw_down),
-          _stream())
+    _call("moe_grouped_gemm_down_wgrad", d, h_act, dy_perm, offsets, dw_down)
 
 
 def moe_grouped_gemm_down_bwd(d, dy_perm, h_act, w_down, offsets, dh_act, dw_down):
-    _call("moe_grouped_gemm_down_bwd", ctypes.byref(d), _ptr(dy_perm), _ptr(h_act), _ptr(w_down), _ptr(offsets),
-          _ptr(dh_act), _ptr(dw_down), _stream())
+    _call("moe_grouped_gemm_down_bwd", d, dy_perm, h_act, w_down, offsets, dh_act, dw_down)
 
 
 def moe_router_topk(d, logits, topk_idx, topk_w):
-    _call("moe_router_topk", ctypes.byref(d), _ptr(logits), _ptr(topk_idx), _ptr(topk_w), _stream())
+    _call("moe_router_topk", d, logits, topk_idx, topk_w)
 
 
 def moe_router_topk_bwd(d, topk_idx, topk_w, dtopk_w, dlogits):
-    _call("moe_router_topk_bwd", ctypes.byref(d), _ptr(topk_idx), _ptr(topk_w), _ptr(dtopk_w), _ptr(dlogits), _stream())
+    _call("moe_router_topk_bwd", d, topk_idx, topk_w, dtopk_w, dlogits)
 
 
 def moe_swiglu_bwd(d, dh_act, gu_saved, dgu):
-    _call("moe_swiglu_bwd", ctypes.byref(d), _ptr(dh_act), _ptr(gu_saved), _ptr(dgu), _stream())
+    _call("moe_swiglu_bwd", d, dh_act, gu_saved, dgu)
 
 
 def moe_grouped_gemm_down_dgrad_swiglu_bwd(d, dy_perm, w_down, gu_saved, offsets, dgu):
-    _call("moe_grouped_gemm_down_dgrad_swiglu_bwd", ctypes.byref(d), _ptr(dy_perm), _ptr(w_down), _ptr(gu_saved),
-          _ptr(offsets), _ptr(dgu), _stream())
+    _call("moe_grouped_gemm_down_dgrad_swiglu_bwd", d, dy_perm, w_down, gu_saved, offsets, dgu)
 
 
 def moe_grouped_gemm_gateup_dgrad(d, dgu, w_gate, w_up, offsets, dx_perm):
-    _call("moe_grouped_gemm_gateup_dgrad", ctypes.byref(d), _ptr(dgu), _ptr(w_gate), _ptr(w_up), _ptr(offsets),
-          _ptr(dx_perm), _stream())
+    _call("moe_grouped_gemm_gateup_dgrad", d, dgu, w_gate, w_up, offsets, dx_perm)
 
 
 def moe_grouped_gemm_gateup_wgrad(d, x_perm, dgu, offsets, dw_gate, dw_up):
-    _call("moe_grouped_gemm_gateup_wgrad", ctypes.byref(d), _ptr(x_perm), _ptr(dgu), _ptr(offsets), _ptr(dw_gate),
-          _ptr(dw_up), _stream())
+    _call("moe_grouped_gemm_gateup_wgrad", d, x_perm, dgu, offsets, dw_gate, dw_up)
 
 
 def moe_grouped_gemm_gateup_swiglu_bwd(d, dh_act, gu_saved, x_perm, w_gate, w_up, offsets, dgu, dx_perm, dw_gate, dw_up):
-    _call("moe_grouped_gemm_gateup_swiglu_bwd", ctypes.byref(d), _ptr(dh_act), _ptr(gu_saved), _ptr(x_perm),
-          _ptr(w_gate), _ptr(w_up), _ptr(offsets), _ptr(dgu), _ptr(dx_perm), _ptr(dw_gate), _ptr(dw_up), _stream())
+    _call("moe_grouped_gemm_gateup_swiglu_bwd", d, dh_act, gu_saved, x_perm, w_gate, w_up, offsets, dgu, dx_perm,
+          dw_gate, dw_up)
 
 
 def moe_mxfp8_act_scale_bytes(d: MoeDims) -> int:
@@ -259,16 +255,15 @@ def moe_mxfp8_w_down_scale_bytes(d: MoeDims) -> int:
 
 
 def moe_mxfp8_quantize_h_act(d, h_act, codes, scales):
-    _call("moe_mxfp8_quantize_h_act", ctypes.byref(d), _ptr(h_act), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_h_act", d, h_act, codes, scales)
 
 
 def moe_mxfp8_quantize_w_down(d, w_down, codes_t, scales):
-    _call("moe_mxfp8_quantize_w_down", ctypes.byref(d), _ptr(w_down), _ptr(codes_t), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_w_down", d, w_down, codes_t, scales)
 
 
 def moe_grouped_gemm_down_mxfp8(d, h_codes, h_scales, w_codes_t, w_scales, offsets, y_perm):
-    _call("moe_grouped_gemm_down_mxfp8", ctypes.byref(d), _ptr(h_codes), _ptr(h_scales), _ptr(w_codes_t), _ptr(w_scales),
-          _ptr(offsets), _ptr(y_perm), _stream())
+    _call("moe_grouped_gemm_down_mxfp8", d, h_codes, h_scales, w_codes_t, w_scales, offsets, y_perm)
 
 
 def moe_mxfp8_dy_scale_bytes(d: MoeDims) -> int:
@@ -280,16 +275,15 @@ def moe_mxfp8_w_down_dgrad_scale_bytes(d: MoeDims) -> int:
 
 
 def moe_mxfp8_quantize_dy_perm(d, dy_perm, codes, scales):
-    _call("moe_mxfp8_quantize_dy_perm", ctypes.byref(d), _ptr(dy_perm), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_dy_perm", d, dy_perm, codes, scales)
 
 
 def moe_mxfp8_quantize_w_down_dgrad(d, w_down, codes, scales):
-    _call("moe_mxfp8_quantize_w_down_dgrad", ctypes.byref(d), _ptr(w_down), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_w_down_dgrad", d, w_down, codes, scales)
 
 
 def moe_grouped_gemm_down_dgrad_mxfp8(d, dy_codes, dy_scales, w_codes, w_scales, offsets, dh_act):
-    _call("moe_grouped_gemm_down_dgrad_mxfp8", ctypes.byref(d), _ptr(dy_codes), _ptr(dy_scales), _ptr(w_codes), _ptr(w_scales),
-          _ptr(offsets), _ptr(dh_act), _stream())
+    _call("moe_grouped_gemm_down_dgrad_mxfp8", d, dy_codes, dy_scales, w_codes, w_scales, offsets, dh_act)
 
 
 def moe_mxfp8_dgu_scale_bytes(d: MoeDims) -> int:
@@ -301,16 +295,15 @@ def moe_mxfp8_w_gateup_dgrad_scale_bytes(d: MoeDims) -> int:
 
 
 def moe_mxfp8_quantize_dgu(d, dgu, codes, scales):
-    _call("moe_mxfp8_quantize_dgu", ctypes.byref(d), _ptr(dgu), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_dgu", d, dgu, codes, scales)
 
 
 def moe_mxfp8_quantize_w_gateup_dgrad(d, w_gate, w_up, codes, scales):
-    _call("moe_mxfp8_quantize_w_gateup_dgrad", ctypes.byref(d), _ptr(w_gate), _ptr(w_up), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_w_gateup_dgrad", d, w_gate, w_up, codes, scales)
 
 
 def moe_grouped_gemm_gateup_dgrad_mxfp8(d, dgu_codes, dgu_scales, w_codes, w_scales, offsets, dx_perm):
-    _call("moe_grouped_gemm_gateup_dgrad_mxfp8", ctypes.byref(d), _ptr(dgu_codes), _ptr(dgu_scales), _ptr(w_codes),
-          _ptr(w_scales), _ptr(offsets), _ptr(dx_perm), _stream())
+    _call("moe_grouped_gemm_gateup_dgrad_mxfp8", d, dgu_codes, dgu_scales, w_codes, w_scales, offsets, dx_perm)
 
 
 def moe_mxfp8_x_scale_bytes(d: MoeDims) -> int:
@@ -322,20 +315,19 @@ def moe_mxfp8_w_gateup_scale_bytes(d: MoeDims) -> int:
 
 
 def moe_mxfp8_quantize_x_perm(d, x_perm, codes, scales):
-    _call("moe_mxfp8_quantize_x_perm", ctypes.byref(d), _ptr(x_perm), _ptr(codes), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_x_perm", d, x_perm, codes, scales)
 
 
 def moe_mxfp8_quantize_w_gateup(d, w_gate, w_up, codes_t, scales):
-    _call("moe_mxfp8_quantize_w_gateup", ctypes.byref(d), _ptr(w_gate), _ptr(w_up), _ptr(codes_t), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_w_gateup", d, w_gate, w_up, codes_t, scales)
 
 
 def moe_grouped_gemm_gateup_mxfp8(d, x_codes, x_scales, w_codes_t, w_scales, offsets, gu):
-    _call("moe_grouped_gemm_gateup_mxfp8", ctypes.byref(d), _ptr(x_codes), _ptr(x_scales), _ptr(w_codes_t), _ptr(w_scales),
-          _ptr(offsets), _ptr(gu), _stream())
+    _call("moe_grouped_gemm_gateup_mxfp8", d, x_codes, x_scales, w_codes_t, w_scales, offsets, gu)
 
 
 def moe_swiglu_mxfp8(d, gu, h_act, h_codes, h_scales):
-    _call("moe_swiglu_mxfp8", ctypes.byref(d), _ptr(gu), _ptr(h_act), _ptr(h_codes), _ptr(h_scales), _stream())
+    _call("moe_swiglu_mxfp8", d, gu, h_act, h_codes, h_scales)
 
 
 def moe_mxfp8_tokens_codes_bytes(d: MoeDims, n_features: int) -> int:
@@ -347,33 +339,28 @@ def moe_mxfp8_tokens_scale_bytes(d: MoeDims, n_features: int) -> int:
 
 
 def moe_mxfp8_quantize_tokens(d, x, ld, col0, n_features, offsets, codes_t, scales):
-    _call("moe_mxfp8_quantize_tokens", ctypes.byref(d), _ptr(x), int(ld), int(col0), int(n_features), _ptr(offsets),
-          _ptr(codes_t), _ptr(scales), _stream())
+    _call("moe_mxfp8_quantize_tokens", d, x, int(ld), int(col0), int(n_features), offsets, codes_t, scales)
 
 
 def moe_grouped_gemm_down_wgrad_mxfp8(d, h_codes_t, h_scales, dy_codes_t, dy_scales, dw_down):
-    _call("moe_grouped_gemm_down_wgrad_mxfp8", ctypes.byref(d), _ptr(h_codes_t), _ptr(h_scales), _ptr(dy_codes_t),
-          _ptr(dy_scales), _ptr(dw_down), _stream())
+    _call("moe_grouped_gemm_down_wgrad_mxfp8", d, h_codes_t, h_scales, dy_codes_t, dy_scales, dw_down)
 
 
 def moe_grouped_gemm_gateup_wgrad_mxfp8(d, x_codes_t, x_scales, dg_codes_t, dg_scales, du_codes_t, du_scales, dw_gate, dw_up):
-    _call("moe_grouped_gemm_gateup_wgrad_mxfp8", ctypes.byref(d), _ptr(x_codes_t), _ptr(x_scales), _ptr(dg_codes_t),
-          _ptr(dg_scales), _ptr(du_codes_t), _ptr(du_scales), _ptr(dw_gate), _ptr(dw_up), _stream())
+    _call("moe_grouped_gemm_gateup_wgrad_mxfp8", d, x_codes_t, x_scales, dg_codes_t, dg_scales, du_codes_t, du_scales,
+          dw_gate, dw_up)
 
 
 def moe_swiglu_bwd_mxfp8(d, dh_act, gu_saved, dgu, dgu_codes, dgu_scales):
-    _call("moe_swiglu_bwd_mxfp8", ctypes.byref(d), _ptr(dh_act), _ptr(gu_saved), _ptr(dgu), _ptr(dgu_codes), _ptr(dgu_scales),
-          _stream())
+    _call("moe_swiglu_bwd_mxfp8", d, dh_act, gu_saved, dgu, dgu_codes, dgu_scales)
 
 
 def moe_layer_fwd_bwd_host(d, x_host, topk_idx_host, topk_w_host, dy_host, w_gate, w_up, w_down, y_host, dx_host,
                            dtopk_w_host, dw_gate, dw_up, dw_down, arena):
     """x_host, topk_idx_host, topk_w_host, dy_host, y_host, dx_host, dtopk_w_host are CPU tensors
     (pinned for asynchronous copies); the rest are CUDA tensors."""
-    _call("moe_layer_fwd_bwd_host", ctypes.byref(d), _ptr(x_host), _ptr(topk_idx_host), _ptr(topk_w_host),
-          _ptr(dy_host), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(y_host), _ptr(dx_host), _ptr(dtopk_w_host),
-          _ptr(dw_gate), _ptr(dw_up), _ptr(dw_down), _ptr(arena),
-          ctypes.c_size_t(arena.numel() * arena.element_size()), _stream())
+    _call("moe_layer_fwd_bwd_host", d, x_host, topk_idx_host, topk_w_host, dy_host, w_gate, w_up, w_down, y_host,
+          dx_host, dtopk_w_host, dw_gate, dw_up, dw_down, arena, arena.numel() * arena.element_size())
 
 
 # ---------------------------------------------------------------------------------------------

@@ -1,9 +1,10 @@
-"""Builds libmoe_b200.so (sm_100a only) in-tree with nvcc.  `python -m paper_2606_26453_b200.build`."""
+"""Builds libmoe_b200.so (sm_100a only) and the binding's CPython helper in-tree.  `python -m paper_2606_26453_b200.build`."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
@@ -31,7 +32,22 @@ def needs_build(path: str = LIB_PATH) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+PYCALL_PATH = os.path.join(PKG_DIR, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+PYCALL_SOURCE = os.path.join(CSRC, "pycall.c")
+
+
+def build_pycall(force: bool = False) -> str:
+    """The module that marshals the binding's arguments (plain C, no CUDA)."""
+    if force or not os.path.exists(PYCALL_PATH) or os.path.getmtime(PYCALL_SOURCE) > os.path.getmtime(PYCALL_PATH):
+        cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_path("include"), "-o", PYCALL_PATH, PYCALL_SOURCE]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("gcc failed:\n" + res.stdout + res.stderr)
+    return PYCALL_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False, waittest: bool = False) -> str:
+    build_pycall(force)
     path = WAITTEST_LIB_PATH if waittest else LIB_PATH
     if not force and not needs_build(path):
         return path

@@ -1,0 +1,54 @@
+"""The binding's argument marshalling (csrc/pycall.c), without a device: every entry point rejects these arguments before it launches
+anything."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2606_26453_b200 import build
+
+
+@pytest.fixture(scope="module")
+def B():
+    build.build_library()
+    from paper_2606_26453_b200 import binding
+    binding.load_library()
+    return binding
+
+
+def test_arguments_arrive_in_their_places(B):
+    lib, d = B.load_library(), B.dims(256, 256, 512, 8, 2)
+    call = lambda name, *a: lib.native_call(lib.addresses[name], d, *a)
+    assert call("moe_permute_bwd", None, 256, 256, 0) == 1                      # NULL
+    assert call("moe_permute_bwd", 256, 264, 256, 0) == 4                       # misaligned
+    t = torch.zeros(64, dtype=torch.uint8)
+    start = -t.data_ptr() % 16
+    assert call("moe_permute_bwd", 256, 256, t[start + 8:], None) == 4          # a tensor's address
+    assert call("moe_permute", *[256] * 8, 8, 0) == 5                           # on the stack: workspace bytes ...
+    assert call("moe_layer_fwd_bwd_host", *[256] * 14, 8, 0) != 0               # ... and the last argument but one of the longest call
+    assert call("moe_mxfp8_quantize_tokens", 256, 512, 0, -1, 256, 256, 256, 0) != 0   # ints
+    d2 = B.MoeDims(256, 200, 512, 8, 2)
+    assert lib.native_call(lib.addresses["moe_permute_bwd"], d2, 256, 256, 256, 0) == 3
+
+
+def test_refused_arguments(B):
+    lib, d = B.load_library(), B.dims(256, 256, 512, 8, 2)
+    address = lib.addresses["moe_permute_bwd"]
+    with pytest.raises(ValueError, match="contiguous"):
+        lib.native_call(address, d, torch.zeros(4, 4).t(), 256, 256, 0)
+    for bad in (1.5, "x", object()):
+        with pytest.raises((TypeError, AttributeError)):
+            lib.native_call(address, d, bad, 256, 256, 0)
+    with pytest.raises(TypeError):
+        lib.native_call(address, b"short", 256, 256, 256, 0)
+    with pytest.raises(TypeError):
+        lib.native_call(address, d, *[256] * 18)
+    with pytest.raises(TypeError):
+        B._call("moe_permute_bwd", ctypes.byref(d), 256, 256, 256)
+    with pytest.raises(ValueError):
+        lib.native_call(0, d, 256)
+
+
+def test_every_entry_point_fits(B):
+    lib = B.load_library()
+    assert all(len(getattr(lib, name).argtypes) - 1 <= 17 for name in lib.addresses)
