@@ -399,9 +399,9 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
 }
 
 // ------------------------------------------------------------------------------------------------
-// a5: one block per token, one thread per 16-byte piece of the row.
+// a5: LANES threads per token (a whole block, or several tokens to a block), one thread per 16-byte piece of the row.
 // dy_perm[row_k, :] = w_k * dy[t, :]; dtopk_w[t,k] = <dy[t,:], y_perm[row_k,:]> (warp shuffles, then a
-// fixed-order sum over the block's warps: deterministic).  y_perm pieces are fetched four slots at a time
+// fixed-order sum over the token's warps: deterministic).  y_perm pieces are fetched four slots at a time
 // (three blocks per SM: with the 80 registers that allows nothing spills; at five blocks per SM the K = 8 kernel
 // spilled and ran 16 % slower inside a step; the instance for a run-time K keeps 32 accumulators and takes two blocks).
 // TRIGGER (grid_launch_dependents) only in small grids and blocks of some length: 40000 tokens of 256 from one expert each
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kThreads) gather_sum_kernel(const uint4* __res
 // lets a GEMM in early.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTriggerPieces = 1024;   // 16-byte pieces that a block moves, 3 ns of the chip's bandwidth
-template <int KT, bool WITH_DW, bool TRIGGER>
+template <int KT, bool WITH_DW, bool TRIGGER, int LANES>
 __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(const uint4* __restrict__ dy,
                                                                   const uint4* __restrict__ y_perm,
                                                                   const float* __restrict__ topk_w,
@@ -417,9 +417,11 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
                                                                   uint4* __restrict__ dy_perm,
                                                                   float* __restrict__ dtopk_w, int T, int hv, int K) {
     constexpr int KA = KT > 0 ? KT : 32;
+    constexpr int WARPS = LANES / 32;   // per token
     __shared__ float partial[kWarpsPerBlock][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x;
+    const int c0 = threadIdx.x % LANES;
+    const int t = blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES;
     const int kk = KT > 0 ? KT : K;
     const int32_t* rows = pair_to_row + (long long)t * K;
     const float* wt = topk_w + (long long)t * K;
@@ -428,7 +430,8 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
     for (int k = 0; k < KA; ++k) dot[k] = 0.f;
     if (!grid_dependency_wait_tested()) return;
     if (TRIGGER) grid_launch_dependents();
-    for (int c = threadIdx.x; c < hv; c += kThreads) {
+    const int n_c = t < T ? hv : 0;
+    for (int c = c0; c < n_c; c += LANES) {
         const uint4 dv = ldg16(dy + (long long)t * hv + c);
         float d[8];
         unpack8(dv, d);
@@ -471,12 +474,13 @@ __global__ void __launch_bounds__(kThreads, KT > 0 ? 3 : 2) combine_bwd_kernel(c
                 if (lane == 0) partial[warp][k] = v;
             }
         }
-        __syncthreads();
-        if (threadIdx.x < kk) {
+        if (WARPS > 1) __syncthreads(); else __syncwarp();
+        if (c0 < kk && t < T) {
+            const int first = warp / WARPS * WARPS;   // of the token's warps
             float v = 0.f;
 #pragma unroll
-            for (int wq = 0; wq < kWarpsPerBlock; ++wq) v += partial[wq][threadIdx.x];
-            dtopk_w[(long long)t * K + threadIdx.x] = v;
+            for (int wq = 0; wq < WARPS; ++wq) v += partial[first + wq][c0];
+            dtopk_w[(long long)t * K + c0] = v;
         }
     }
 }
@@ -608,20 +612,40 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
                    : gather_sum_dispatch<false, false>(d, src, nullptr, pair_to_row, out, s);
 }
 
-template <bool WITH_DW, bool TRIGGER>
+// Threads per token: the most that leave every thread two pieces of the row or more and the fewest places empty (32 for narrow rows).
+// A block per token, as before, against this (T x H, K; us): 20000 x 256, 2 25.3 -> 8.2; 20000 x 512, 2 45.1 -> 16.7, K = 8 120 -> 59;
+// 20000 x 832, 4 90 -> 55; 20000 x 1024, 3 70 -> 47; 10000 x 1280, 8 86 -> 73; 8192 x 1536, 4 47 -> 39; 16384 x 2048, 8 181 -> 174;
+// 14442 x 2880, 4 137 -> 121; 8192 x 4096, 2 54.7 (a block per token stays: 128 threads 55.4).
+static int combine_bwd_lanes_of(int hv) {
+    int best = 32;
+    for (int lanes = 64; lanes <= kThreads && 2 * lanes <= hv; lanes *= 2)
+        if ((hv + lanes - 1) / lanes * lanes <= (hv + best - 1) / best * best) best = lanes;
+    return best;
+}
+template <bool WITH_DW, bool TRIGGER, int LANES>
 static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w,
                                  const int32_t* p2r, uint4* dyp, float* dw, cudaStream_t s) {
     const int hv = d.H / 8;
-    const unsigned blocks = (unsigned)d.T;
+    constexpr int TOKENS = kThreads / LANES;
+    const unsigned blocks = (unsigned)((d.T + TOKENS - 1) / TOKENS);
 #define MOE_CB_CASE(KT) \
-    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW, TRIGGER>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW, TRIGGER, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     switch (d.K) {
         MOE_CB_CASE(1) MOE_CB_CASE(2) MOE_CB_CASE(3) MOE_CB_CASE(4) MOE_CB_CASE(5) MOE_CB_CASE(6) MOE_CB_CASE(7)
         MOE_CB_CASE(8)
         default:
-            return launch_streaming(combine_bwd_kernel<0, WITH_DW, TRIGGER>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+            return launch_streaming(combine_bwd_kernel<0, WITH_DW, TRIGGER, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     }
 #undef MOE_CB_CASE
+}
+template <bool WITH_DW, bool TRIGGER>
+static int combine_bwd_lanes(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w, const int32_t* p2r, uint4* dyp,
+                             float* dw, cudaStream_t s) {
+    const int lanes = combine_bwd_lanes_of(d.H / 8);
+    if (lanes == 32) return combine_bwd_dispatch<WITH_DW, TRIGGER, 32>(d, dy, yp, w, p2r, dyp, dw, s);
+    if (lanes == 64) return combine_bwd_dispatch<WITH_DW, TRIGGER, 64>(d, dy, yp, w, p2r, dyp, dw, s);
+    if (lanes == 128) return combine_bwd_dispatch<WITH_DW, TRIGGER, 128>(d, dy, yp, w, p2r, dyp, dw, s);
+    return combine_bwd_dispatch<WITH_DW, TRIGGER, 256>(d, dy, yp, w, p2r, dyp, dw, s);
 }
 
 int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, const float* topk_w,
@@ -629,12 +653,13 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    const bool trigger = d.T <= (int)kSmallGrid || (2ll * d.K + 1) * (d.H / 8) >= kTriggerPieces;
+    const int tokens = kThreads / combine_bwd_lanes_of(d.H / 8);   // per block
+    const bool trigger = d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
     if (dtopk_w != nullptr)
-        return trigger ? combine_bwd_dispatch<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
-                       : combine_bwd_dispatch<true, false>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s);
-    return trigger ? combine_bwd_dispatch<false, true>(d, a, b, topk_w, pair_to_row, o, nullptr, s)
-                   : combine_bwd_dispatch<false, false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
+        return trigger ? combine_bwd_lanes<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
+                       : combine_bwd_lanes<true, false>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s);
+    return trigger ? combine_bwd_lanes<false, true>(d, a, b, topk_w, pair_to_row, o, nullptr, s)
+                   : combine_bwd_lanes<false, false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
 }
 
 // ------------------------------------------------------------------------------------------------
