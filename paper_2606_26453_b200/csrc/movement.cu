@@ -5,6 +5,8 @@
 // (16-byte loads) K times, so the bytes moved are the algorithmic minimum.  The permutation indices
 // never depend on the order in which atomics land: ranks come from warp-level match/ballot
 // scans over pairs taken in ascending pair id, which makes the result the unique stable sort.
+#include <initializer_list>
+
 #include "common.cuh"
 
 namespace moe {
@@ -37,7 +39,7 @@ __device__ __forceinline__ uint4 pack8(const float f[8]) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// a1 in two launches, or one with few pairs (kDirectPairs).
+// a1 in two launches, one with few pairs (kDirectPairs), three with many (kScanEntries).
 //   hist      : one block per `chunk` consecutive pairs (a multiple of 256): the number of pairs of each
 //               expert in the chunk (shared-memory atomics: counts are order-free)          -> ws[chunk][e]
 //   rank_rows : one block per kTokPerBlock consecutive tokens.  The block
@@ -137,8 +139,43 @@ struct RankRowsSmem {
     }
 };
 
-// DIRECT: few pairs, no histogram kernel before: every block counts all of them by itself (ws, chunk and n_chunks unused).
-template <bool DIRECT>
+// Many chunks: instead of every block of rank_rows summing all histogram rows, the rows become running sums in place (what came
+// before a chunk) and the totals go to `counts`.  One warp per expert, one lane per chunk.
+__global__ void __launch_bounds__(kThreads) permute_scan_kernel(int32_t* __restrict__ ws, int E, int n_chunks, int32_t* __restrict__ counts) {
+    const int e = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (!grid_dependency_wait_tested()) return;
+    grid_launch_dependents();
+    if (e >= E) return;
+    int run = 0;
+    for (int a0 = 0; a0 < n_chunks; a0 += 32 * kIdxGroup) {
+        int v[kIdxGroup];
+#pragma unroll
+        for (int g = 0; g < kIdxGroup; ++g) {
+            const int a = a0 + 32 * g + lane;
+            v[g] = a < n_chunks ? ws[(size_t)a * E + e] : 0;
+        }
+#pragma unroll
+        for (int g = 0; g < kIdxGroup; ++g) {
+            const int a = a0 + 32 * g + lane;
+            int incl = v[g];
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += t;
+            }
+            if (a < n_chunks) ws[(size_t)a * E + e] = run + incl - v[g];
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    if (lane == 0) counts[e] = run;
+}
+
+// How a block of rank_rows learns what came before it and how many pairs there are (SUMS):
+//   kSumRows  it sums the histogram rows
+//   kCountAll few pairs, no histogram kernel before: it counts all of them by itself (ws, chunk and n_chunks unused)
+//   kScanned  many pairs: permute_scan_kernel has run, the row of its chunk and `counts` say it
+enum PermuteSums { kSumRows = 0, kCountAll = 1, kScanned = 2 };
+template <int SUMS>
 __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     const int32_t* __restrict__ topk_idx, int R, int E, int K, int T, int chunk, int n_chunks,
     const int32_t* __restrict__ ws, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
@@ -159,12 +196,12 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     const int t0 = blockIdx.x * kTokPerBlock, t1 = min(T, t0 + kTokPerBlock);
     const long long p_begin = (long long)t0 * K, p_end = (long long)t1 * K;
     const int n_own = (int)(p_end - p_begin);
-    const int my_chunk = DIRECT ? 0 : (int)(p_begin / chunk);        // histogram rows wholly before this block: a < my_chunk
+    const int my_chunk = SUMS == kCountAll ? 0 : (int)(p_begin / chunk);        // histogram rows wholly before this block: a < my_chunk
     const long long chunk_begin = (long long)my_chunk * chunk;
     const int n_units = rows ? (t1 - t0) * n_seg : 0;                // row segments this block copies
     const int n_pre = min(kRowLookahead, n_units);
 
-    if (DIRECT) {   // the routing indices and the rows may come from the kernel before
+    if (SUMS == kCountAll) {   // the routing indices and the rows may come from the kernel before
         if (!grid_dependency_wait_tested()) return;
         grid_launch_dependents();
     }
@@ -224,7 +261,7 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     // pass 1: this warp's histogram over its own pairs
     int32_t* mine = whist + warp * E;
     if (own >= 0) atomicAdd(&mine[own], 1);   // counts only: order-free
-    if (DIRECT) {
+    if (SUMS == kCountAll) {
         // the pairs from this block's first on: with those before, in `base`, they make the totals
         const int n_after = R - n_before;
         for (int i0 = threadIdx.x; i0 < n_after; i0 += kPermThreads * kIdxGroup) {
@@ -244,7 +281,12 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
         // ---- (2) the chunk histograms are complete and visible from here on ----
         if (!grid_dependency_wait_tested()) return;
         grid_launch_dependents();
-        for (int i = threadIdx.x; i < n_chunks * E; i += kPermThreads) {
+        if (SUMS == kScanned)
+            for (int e = threadIdx.x; e < E; e += kPermThreads) {
+                total[e] = counts[e];
+                atomicAdd(&base[e], ws[(size_t)my_chunk * E + e]);
+            }
+        for (int i = threadIdx.x; SUMS == kSumRows && i < n_chunks * E; i += kPermThreads) {
             const int v = ws[i];
             if (v != 0) {
                 const int a = i / E, e = i - a * E;
@@ -276,7 +318,7 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     __syncthreads();
     if (blockIdx.x == 0) {
         for (int e = threadIdx.x; e <= E; e += kPermThreads) offsets[e] = offs[e];
-        for (int e = threadIdx.x; e < E; e += kPermThreads) counts[e] = total[e];
+        for (int e = threadIdx.x; SUMS != kScanned && e < E; e += kPermThreads) counts[e] = total[e];
     }
     // per-warp counts -> first row of each (warp, expert)
     for (int e = threadIdx.x; e < E; e += kPermThreads) {
@@ -547,18 +589,31 @@ int movement_read_and_clear_status(int* status_out) {
 // is no histogram launch: the call takes 6.3 us instead of 8.3 (256 tokens of 256 to 2 of 8 experts, 32 of 2048 to 8 of 128, 2000 of 256 to
 // one each 8.5 instead of 11.0).  At 4096 pairs 9.0 against 8.2 us (512 tokens of 2048 to 8 of 128 experts).
 constexpr int kDirectPairs = 2048;
+// From this many histogram entries (chunks of 2048 pairs times experts) on a launch in between turns them into running sums: with
+// 16384 entries every block of rank_rows summed them all, and that outlasted the rows unless they were long.  32768 tokens of 256 and of
+// 1024 to 8 of 128 experts 240 -> 52 and 241 -> 105 us, 4000 of 1024 to 8 of 1024 56 -> 34, 20000 of 640 to 3 of 40 (1200 entries)
+// 37.8 -> 31.0, 16384 of 2048 to 8 of 128 110 -> 107, 32768 of 4096 to 8 of 64 391 -> 389 us.  With fewer the launch costs more: 4096 of 2048 to 6
+// of 64 (768 entries) 25.9 -> 26.7, 1777 of 2880 to 4 of 128 (512) 12.8 -> 13.7 us.  Chunks of 1024 pairs: 512 were 0-5 % slower, 256 5-30 %.
+constexpr long long kScanEntries = 1024;
+static int permute_scan_chunk(long long R) {
+    const long long need = (R + 4095) / 4096;
+    return (int)(need > 1024 ? (need + kThreads - 1) / kThreads * kThreads : 1024);
+}
 int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, bf16* x_perm, int32_t* counts,
                    int32_t* offsets, int32_t* row_to_pair, int32_t* pair_to_row, void* workspace,
                    cudaStream_t s) {
     const int R = d.T * d.K, E = d.E;
-    const int chunk = permute_chunk(R);
+    const bool direct = R <= kDirectPairs;
+    const bool scanned = !direct && (long long)((R + 2047) / 2048) * E >= kScanEntries;
+    const int chunk = scanned ? permute_scan_chunk(R) : permute_chunk(R);
     const int n_chunks = (R + chunk - 1) / chunk;
     int32_t* ws = static_cast<int32_t*>(workspace);
-    const bool direct = R <= kDirectPairs;
-    if (!direct) {
-        const int st_ = launch_dependent(permute_hist_kernel, n_chunks, kThreads, E * sizeof(int32_t), 1, s, topk_idx, R, E, chunk, ws);
-        if (st_ != MOE_OK) return st_;
-    }
+    int st_ = MOE_OK;
+    if (!direct) st_ = launch_dependent(permute_hist_kernel, n_chunks, kThreads, E * sizeof(int32_t), 1, s, topk_idx, R, E, chunk, ws);
+    if (st_ == MOE_OK && scanned)
+        st_ = launch_dependent(permute_scan_kernel, (E + kWarpsPerBlock - 1) / kWarpsPerBlock, kThreads, 0, 1, s, ws, E, n_chunks, counts);
+    if (st_ != MOE_OK) return st_;
+    auto kernel = direct ? permute_rank_rows_kernel<kCountAll> : scanned ? permute_rank_rows_kernel<kScanned> : permute_rank_rows_kernel<kSumRows>;
 
     const bool rows = x_perm != nullptr;
     const int row_bytes = d.H * 2;
@@ -570,16 +625,13 @@ int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, 
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MOE_ERR_CUDA;
     if (!attr_set[dev]) {
         const RankRowsSmem largest(1024, kRowMaxSeg, true);
-        if (cudaFuncSetAttribute(permute_rank_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 largest.total_bytes) != cudaSuccess ||
-            cudaFuncSetAttribute(permute_rank_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 largest.total_bytes) != cudaSuccess)
-            return MOE_ERR_CUDA;
+        for (auto k : {permute_rank_rows_kernel<kSumRows>, permute_rank_rows_kernel<kCountAll>, permute_rank_rows_kernel<kScanned>})
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, largest.total_bytes) != cudaSuccess) return MOE_ERR_CUDA;
         attr_set[dev] = true;
     }
     const unsigned grid = (unsigned)((d.T + kTokPerBlock - 1) / kTokPerBlock);
     // its blocks start, prefetch rows and count from the routing indices while the histogram kernel is still running
-    return launch_dependent(direct ? permute_rank_rows_kernel<true> : permute_rank_rows_kernel<false>, grid, kPermThreads, lay.total_bytes, 1, s, topk_idx, R, E, d.K, d.T, chunk,
+    return launch_dependent(kernel, grid, kPermThreads, lay.total_bytes, 1, s, topk_idx, R, E, d.K, d.T, chunk,
                             n_chunks, ws, counts, offsets, row_to_pair, pair_to_row, reinterpret_cast<const uint8_t*>(x),
                             reinterpret_cast<uint8_t*>(x_perm), row_bytes, seg_bytes, n_seg);
 }
