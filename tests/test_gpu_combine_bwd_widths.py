@@ -23,7 +23,7 @@ def test_widths(H, T, K):
     w = rng.random((T, K), dtype=np.float32)
     d = B.dims(T, H, 64, E, K)
     dyp = torch.full((R + 1, H), float("nan"), dtype=torch.bfloat16, device="cuda")
-    dw = torch.full((T + 1, K), float("nan"), device="cuda")
+    dw = torch.full((T + 1, K), float("nan"), dtype=torch.float32, device="cuda")
     B.moe_unpermute_combine_bwd(d, Hh.to_dev_bf16(dy), Hh.to_dev_bf16(yp), torch.from_numpy(w).cuda(), torch.from_numpy(p2r).cuda(), dyp[:R], dw[:T])
     only = torch.full((R, H), float("nan"), dtype=torch.bfloat16, device="cuda")
     B.moe_unpermute_combine_bwd(d, Hh.to_dev_bf16(dy), None, torch.from_numpy(w).cuda(), torch.from_numpy(p2r).cuda(), only, None)
