@@ -31,7 +31,11 @@ int sm_count();
 //     kernel that has started knows everything before its immediate predecessor to be complete.
 //   - A weight gradient that a call launches right behind a data gradient on the same inputs does not depend on it.  Behind a
 //     short one it runs beside it: no wait at its start (that it has started means that all before the data gradient is complete), the wait before
-//     it lets ITS successor start, so that a kernel which has waited for it has waited for both.
+//     it lets ITS successor start, so that a kernel which has waited for it has waited for both.  Only a wait is documented to make
+//     earlier kernels' writes visible, and this form reads without one.  What it reads was written before the data gradient; that
+//     kernel's threads have waited for those writes and fence (release_to_dependents) before any of them can trigger, so the writes
+//     are performed at the scope of the device before the weight gradient can start, and its threads fence (acquire_unwaited) before they
+//     read: nothing older comes out of an L1, by loads or by bulk copies.
 //   - The GEMMs call it at the end of each warp's role.  One thread's call counts for its CTA, so the row-ragged bf16 kinds,
 //     where one warp has no role, trigger right after set-up, and the CTAs of a GEMM that follows take each SM as it comes
 //     free.  With the call behind the last barrier of the teardown steps of long GEMMs take longer, chip idle between steps:
@@ -52,6 +56,12 @@ __device__ __forceinline__ bool grid_dependency_wait_tested() {
     uint32_t done;
     asm volatile("griddepcontrol.wait; mov.u32 %0, 1;" : "=r"(done) : : "memory");
     return done != 0;
+}
+// The two sides of a dependent that reads without waiting (see above).
+__device__ __forceinline__ void release_to_dependents() { __threadfence(); }
+__device__ __forceinline__ void acquire_unwaited() {
+    __threadfence();
+    asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -455,8 +455,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         prefetch_tmap(&map_r1);
     }
     // everything above may run while the kernel before is still finishing; the schedule is derived from its output
-    if (!wgrad(KIND) || !p.beside) grid_dependency_wait();
+    if (!wgrad(KIND) || !p.beside) grid_dependency_wait(); else acquire_unwaited();
     for (int e = threadIdx.x; e <= p.E; e += NUM_THREADS) ctl->offs[e] = p.offsets[e];
+    if (KIND == DGRAD || KIND == DGRAD_T) release_to_dependents();   // a weight gradient may run beside this kernel
     __syncthreads();
     if (wgrad(KIND)) {
         // experts by row count, largest first (ties: lower id first): rank by counting, O(E^2 / threads)

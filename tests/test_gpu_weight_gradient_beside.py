@@ -37,3 +37,39 @@ def test_combined_calls(counts, H, I, in_place):
         for k, c in zip(outs, copies):
             assert torch.equal(c, want[k]), k
     assert B.moe_device_status() == 0
+
+
+def test_inputs_that_change_from_call_to_call():
+    """Steps of two workloads by turns through the same buffers, nothing waited for in between: the routing, the packed rows and the
+    gradients that a weight gradient reads without waiting for the kernel before it are those of its own step."""
+    from paper_2606_26453_b200 import binding as B
+    H, I = 256, 512
+    hosts = [Hh.ragged_workload(c, K=1, H=H, I=I, seed=s) for c, s in (([64] * 8, 41), ([130, 0, 3, 200, 64, 17, 97, 1], 43))]
+    (cfg, _), E = hosts[0], 8
+    devs = [Hh.device_workload(h) for _, h in hosts]
+    outs = ("y", "dx", "dtopk_w", "dw_gate", "dw_up", "dw_down")
+    b = B.alloc_layer_buffers(cfg.T, H, I, E, 1)
+
+    def step(w):
+        B.layer_forward(b, w["X"], w["topk_idx"], w["topk_w"], w["W_gate"], w["W_up"], w["W_down"])
+        B.layer_backward(b, w["dY"], w["topk_w"], w["W_gate"], w["W_up"], w["W_down"])
+        return {k: getattr(b, k).clone() for k in outs}
+
+    want = []
+    for w in devs:
+        Hb = Hh.run_cuda_layer(w, E)      # buffers of its own
+        B.moe_grouped_gemm_down_wgrad(Hb.d, Hb.h_act, Hb.dy_perm, Hb.offsets, Hb.dw_down)
+        B.moe_grouped_gemm_gateup_wgrad(Hb.d, Hb.x_perm, Hb.dgu, Hb.offsets, Hb.dw_gate, Hb.dw_up)
+        torch.cuda.synchronize()
+        want.append({k: getattr(Hb, k).clone() for k in outs})
+    live = {k: torch.empty_like(v) for k, v in devs[0].items()}
+    got = []
+    for i in range(40):
+        for k, v in live.items():
+            v.copy_(devs[i % 2][k])
+        got.append(step(live))
+    torch.cuda.synchronize()
+    assert B.moe_device_status() == 0
+    for i, g in enumerate(got):
+        for k in outs:
+            assert torch.equal(g[k], want[i % 2][k]), (i, k)
