@@ -20,6 +20,9 @@ int mx_read_and_clear_status(int* status_out);         // the block-scaled FP8 k
 // Number of SMs of the current device (cached per device ordinal).
 int sm_count();
 
+// CTA pairs the chip takes at once, one CTA per SM: what the rules of the dispatch count tiles against.  (The launches ask the device.)
+constexpr int kChipPairs = 148 / 2;
+
 // ---- programmatic dependent launch --------------------------------------------------------------
 // The library's kernels are launched as programmatic dependents of whatever precedes them on the stream: their blocks may be
 // placed, and may set up barriers, while the last blocks of the kernel before are still running.

@@ -462,23 +462,23 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // and half of the N side's in shared memory, so a K slice of 128 costs each SM 29 KB of operand loads against 58 KB per two
 // 128 x 128 tiles of the single-CTA form, which the L2 -> SM path bounds.  208, not 256: the two accumulators (tensor-memory
 // columns 0 and 256) leave 48 columns behind each for three 16-column scale slots, one slot per ring stage.
-//   row-ragged form    M side: 256 output features of an expert's weights.  N side: its rows, in equal tiles of at most 208 rows
+//   weights on M       M side: 256 output features of an expert's weights.  N side: its rows, in equal tiles of at most 208 rows
 //                      (a multiple of 16), so that almost no tensor work goes to padding.  The accumulator has a feature per
 //                      lane and a row per column and is transposed on its way out.
+//   rows on M          M side: 256 rows of an expert, half a tile of padding on average.  N side: 208 features (the last tile is narrower).
 //   weight gradients   M side: 256 rows of the output, N side: 208 columns of it (the last tile is narrower).
-// The row-ragged form had the rows on the M side before, in tiles of 256, half a tile of padding per expert: all four GEMMs
+// Rows on M against weights on M: all four GEMMs
 // 18 % faster at 384 rows per expert (64 experts of 2048 x 1408: gate/up 206 -> 166, down 108 -> 88 us), 3-8 % at 1024
 // (128 of 2048 x 768: 433 -> 402, 282 -> 272 us), 3-6 % at 2048 (8 of 4096 x 14336: 1697 -> 1649, 884 -> 827 us), 10 % under
-// Dirichlet loads (128 of 2944 x 2944).
+// Dirichlet loads (128 of 2944 x 2944).  Not where it has the more tiles: mx_form.
 //   scale factors: each CTA holds the scales of its own 128 of the M side (4 columns) and of ALL the tile's N side (two blocks of
 //   128, 8 columns) in its own tensor memory; tcgen05.cp.cta_group::2, issued once, copies in both CTAs from the same
-//   shared-memory offsets.  Weight-scale blocks (512 bytes per 128 features and K slice) and the weight gradients' N-side blocks
-//   (1024 bytes per 208 columns) are contiguous in global memory and arrive by one tensor copy; scales of packed rows are
-//   gathered by a warp.  (Weight scales are also stored in the 208 tiling, as their documented format has it; nothing in this
-//   file reads that copy.)
+//   shared-memory offsets.  Weight-scale blocks (on M: 512 bytes per 128 features and K slice, on N: 1024 bytes per 208) and the
+//   weight gradients' N-side blocks (1024 bytes per 208 columns) are contiguous in global memory and arrive by one tensor copy;
+//   scales of packed rows are gathered by a warp.
 //   warp 0      TMA producer (both CTAs; all loads complete on the first CTA's full[stage], as in the bf16 pair kernels)
 //   warp 1      first CTA: issues the MMAs and the commits for the pair
-//   warp 2      scales of packed rows (row-ragged form: the N side's) or of the M side's 128 rows (weight gradients)
+//   warp 2      scales of packed rows (weights on M: the N side's) or of the M side's 128 rows
 //   warps 3..10 epilogue: a 32-lane quarter x every other 32-column block
 //   warp 11     first CTA: issues the scale copies (smem -> tensor memory) of each stage
 // What bounds it: a K slice takes ~590 cycles where the tensor pipe needs ~420 (four N = 208 MMAs): operand reads by the tensor
@@ -493,7 +493,7 @@ constexpr int MXP_B_BYTES = (MXP_NT / 2) * MX_BK;       // 13 KB
 constexpr int MXP_SFA_OFF = MXP_A_BYTES + MXP_B_BYTES;  // 512 bytes: scales of this CTA's part of the M side
 constexpr int MXP_SFB_OFF = MXP_SFA_OFF + 512;          // 1024 bytes: scales of the tile's N side
 constexpr int MXP_STAGE_BYTES = 31 * 1024;              // 30.5 KB used; stages stay 1024-byte aligned
-constexpr int MXP_LOW_BOX = 64;                         // rows of the smaller of the row-ragged form's two boxes of row codes
+constexpr int MXP_LOW_BOX = 64;                         // weights on M: rows of the smaller of the two boxes of row codes
 constexpr int MXP_EPI_WARPS = 8;
 constexpr int MXP_COPY_WARP = 3 + MXP_EPI_WARPS;   // the scale-copy warp comes after the epilogue warps
 constexpr int MXP_THREADS = 32 * (4 + MXP_EPI_WARPS);
@@ -515,13 +515,13 @@ struct MxPairCtl {
     uint32_t tmem_base;
     int abort_flag;
     int stage_n[MXP_STAGES];   // N of the tile a stage belongs to (published by the first CTA's producer)
-    int32_t offs[MX_MAX_E + 1];          // row-ragged form: offsets; weight gradients: slice_prefix
-    int32_t tile_prefix[MX_MAX_E + 1];   // row-ragged form: row tiles of the experts before e
+    int32_t offs[MX_MAX_E + 1];          // row-ragged forms: offsets; weight gradients: slice_prefix
+    int32_t tile_prefix[MX_MAX_E + 1];   // row-ragged forms: row tiles of the experts before e
 };
 constexpr int MXP_SMEM_BYTES = MXP_STAGES * MXP_STAGE_BYTES + MXP_STAGING_BYTES + 1024 + (int)sizeof(MxPairCtl);
 static_assert(MXP_SMEM_BYTES <= 232448, "exceeds the shared memory a CTA can opt in to");
 
-// The pair kernel serves two problems (template parameter WGRAD):
+// The pair kernel serves two problems, the first in two forms (template parameter FORM):
 //   row-ragged GEMM   out[r, :] = a[r, :] . b[e]^T for the rows r of expert e: row tiles from `offsets`, the
 //                     contraction is k_tiles slices for every tile, b and its scale blocks are indexed by expert;
 //   weight gradient   dW[e] [M, N] = A_e^T B_e with token-quantised, transposed operands (further down): a fixed tile
@@ -529,7 +529,7 @@ static_assert(MXP_SMEM_BYTES <= 232448, "exceeds the shared memory a CTA can opt
 //                     [slice_prefix[e], slice_prefix[e + 1]) of both operands, nothing is indexed by expert but the output.
 struct MxPairParams {
     const int32_t* prefix;   // offsets [E + 1] / slice_prefix [E + 1]
-    int E, k_tiles, n_tiles, m_tiles, n_cols, n_slices;   // k_tiles: row-ragged form; m_tiles, n_slices: weight gradients
+    int E, k_tiles, n_tiles, m_tiles, n_cols, n_slices;   // k_tiles: row-ragged forms; m_tiles, n_slices: weight gradients
     int M;                   // weight gradients: rows of one expert's output
     long long sa_rows;       // words per slice of `sa`: R / M
     const uint32_t* sa;      // scale words of the packed rows / of the A side [slices][sa_rows]
@@ -560,24 +560,25 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t v[16]) {
         : "memory");
 }
 
+enum MxPairForm { MXP_WEIGHTS_M = 0, MXP_ROWS_M = 1, MXP_WGRAD = 2 };
 struct MxPairTile {
-    int row0;               // weight gradients: first output row inside the expert's output; row-ragged form: first packed row
-    int rows;               // row-ragged form: packed rows
+    int row0;               // weight gradients: first output row inside the expert's output; row-ragged forms: first packed row
+    int rows;               // rows from there to the end of the expert's output; row-ragged forms: of the expert, at most a tile's
     int out_row0;           // weight gradients: first row of the expert's output in the output tensor
     int n0, width;          // first output column (feature); N of the MMAs
     int k0, k_tiles;        // K slices [k0, k0 + k_tiles) of both operands
     int w_row, sf_row0;     // first row of the tile in the B codes (weight gradients) / weight codes; row of its first scale block
 };
-template <bool WGRAD>
+template <int FORM>
 __device__ __forceinline__ MxPairTile mxp_decode(const MxPairParams& p, const MxPairCtl* ctl, long long t) {
     MxPairTile tl;
-    if (WGRAD) {
+    if (FORM == MXP_WGRAD) {
         const int per_e = p.m_tiles * p.n_tiles;
         const int e = (int)(t / per_e);
         const int local = (int)(t - (long long)e * per_e);
         const int nt = local / p.m_tiles;   // column tile major inside an expert: the pairs running together share the B tile in L2
         tl.row0 = (local - nt * p.m_tiles) * MXP_ROWS;
-        tl.rows = 0;
+        tl.rows = p.M - tl.row0;
         tl.out_row0 = e * p.M;
         tl.k0 = ctl->offs[e];
         tl.k_tiles = ctl->offs[e + 1] - tl.k0;
@@ -595,32 +596,34 @@ __device__ __forceinline__ MxPairTile mxp_decode(const MxPairParams& p, const Mx
         const int m_tiles_e = ctl->tile_prefix[lo + 1] - ctl->tile_prefix[lo];
         const int nt = local / m_tiles_e, mt = local - nt * m_tiles_e;   // feature tile major inside an expert (the pairs running together share weight tiles in L2)
         const int n_e = ctl->offs[lo + 1] - ctl->offs[lo];
-        const int per_tile = ((n_e + m_tiles_e - 1) / m_tiles_e + 15) & ~15;   // equal tiles, the last one takes what is left
+        // rows on the N side: equal tiles, the last one takes what is left
+        const int per_tile = FORM == MXP_ROWS_M ? MXP_ROWS : ((n_e + m_tiles_e - 1) / m_tiles_e + 15) & ~15;
         tl.row0 = ctl->offs[lo] + mt * per_tile;
         tl.rows = min(per_tile, ctl->offs[lo + 1] - tl.row0);
         tl.out_row0 = 0;
         tl.k0 = 0;
         tl.k_tiles = p.k_tiles;
-        tl.n0 = nt * MXP_ROWS;
-        tl.width = (tl.rows + 15) & ~15;
+        tl.n0 = nt * (FORM == MXP_ROWS_M ? MXP_NT : MXP_ROWS);
+        tl.width = FORM == MXP_ROWS_M ? min(MXP_NT, p.n_cols - tl.n0) : (tl.rows + 15) & ~15;
         tl.w_row = lo * p.n_cols + tl.n0;
-        tl.sf_row0 = (lo * (p.n_cols >> 7) + 2 * nt) * p.k_tiles;
+        tl.sf_row0 = (FORM == MXP_ROWS_M ? lo * p.n_tiles + nt : lo * (p.n_cols >> 7) + 2 * nt) * p.k_tiles;
     }
     return tl;
 }
 // K slices of tile t (the roles that do not need the rest of the tile)
-template <bool WGRAD>
+template <int FORM>
 __device__ __forceinline__ int mxp_k_tiles(const MxPairParams& p, const MxPairCtl* ctl, long long t) {
-    if (!WGRAD) return p.k_tiles;
+    if (FORM != MXP_WGRAD) return p.k_tiles;
     const int e = (int)(t / ((long long)p.m_tiles * p.n_tiles));
     return ctl->offs[e + 1] - ctl->offs[e];
 }
 
-template <bool WGRAD>
+template <int FORM>
 __global__ void __launch_bounds__(MXP_THREADS, 1)
 mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                     const __grid_constant__ CUtensorMap map_b_low, const __grid_constant__ CUtensorMap map_sf,
                     const __grid_constant__ CUtensorMap map_o, const MxPairParams p) {
+    constexpr bool ROWS_N = FORM == MXP_WEIGHTS_M;   // the packed rows are the N side
     extern __shared__ uint8_t smem_raw[];
     const uint32_t tiles_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* tiles_ptr = smem_raw + (tiles_base - smem_u32(smem_raw));
@@ -654,7 +657,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     grid_dependency_wait();
     for (int e = threadIdx.x; e <= p.E; e += MXP_THREADS) ctl->offs[e] = p.prefix[e];
     __syncthreads();
-    if (!WGRAD && warp == 0) exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, MXP_NT, lane);   // row-ragged form
+    if (FORM != MXP_WGRAD && warp == 0) exclusive_tile_prefix(ctl->offs, ctl->tile_prefix, p.E, ROWS_N ? MXP_NT : MXP_ROWS, lane);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                      "r"((uint32_t)MX_TMEM_COLS)
@@ -666,7 +669,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     cluster_sync_all();   // the other CTA's barriers and tensor memory exist from here on
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, ctl->tmem_base, 0);
-    const long long n_tiles_total = WGRAD ? (long long)p.E * p.m_tiles * p.n_tiles : (long long)__shfl_sync(0xffffffffu, ctl->tile_prefix[p.E], 0) * p.n_tiles;
+    const long long n_tiles_total = FORM == MXP_WGRAD ? (long long)p.E * p.m_tiles * p.n_tiles : (long long)__shfl_sync(0xffffffffu, ctl->tile_prefix[p.E], 0) * p.n_tiles;
     const uint32_t full0 = map_to_cta(smem_u32(&ctl->full[0]), 0);   // full[] of the MMA-issuing CTA
 
     if (warp == 0) {
@@ -675,15 +678,15 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             uint32_t stage = 0, phase = 0, issued = 0;
             bool ok = true;
             for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
-                MxPairTile tl = mxp_decode<WGRAD>(p, ctl, t);
+                MxPairTile tl = mxp_decode<FORM>(p, ctl, t);
                 auto uni = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };
                 tl.row0 = uni(tl.row0); tl.width = uni(tl.width); tl.k0 = uni(tl.k0); tl.k_tiles = uni(tl.k_tiles); tl.w_row = uni(tl.w_row);
                 // this CTA's 128 rows of the M side, its half of the N side, its scale blocks
                 const int my_n = tl.width >> 1;
-                const int a_row = (WGRAD ? tl.row0 : tl.w_row) + (int)rank * MX_BM, b_row = (WGRAD ? tl.w_row : tl.row0) + (int)rank * my_n;
-                const int sf_row0 = uni(tl.sf_row0) + (WGRAD ? 0 : (int)rank * tl.k_tiles);
-                const bool low = !WGRAD && my_n <= MXP_LOW_BOX;
-                const uint32_t bytes = WGRAD ? MXP_A_BYTES + MXP_B_BYTES + 1024 : MXP_A_BYTES + (low ? MXP_LOW_BOX * MX_BK : MXP_B_BYTES) + 512;
+                const int a_row = (ROWS_N ? tl.w_row : tl.row0) + (int)rank * MX_BM, b_row = (ROWS_N ? tl.row0 : tl.w_row) + (int)rank * my_n;
+                const int sf_row0 = uni(tl.sf_row0) + (ROWS_N ? (int)rank * tl.k_tiles : 0);
+                const bool low = ROWS_N && my_n <= MXP_LOW_BOX;
+                const uint32_t bytes = ROWS_N ? MXP_A_BYTES + (low ? MXP_LOW_BOX * MX_BK : MXP_B_BYTES) + 512 : MXP_A_BYTES + MXP_B_BYTES + 1024;
                 for (int kt = 0; kt < tl.k_tiles; ++kt) {
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag))) { ok = false; break; }
 #ifdef MOE_TEST_HOOKS
@@ -700,7 +703,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         mbar_arrive_expect_tx_cluster(bar, bytes);
                         tma_load_2d_pair(dst, &map_a, (tl.k0 + kt) * MX_BK, a_row, bar);
                         tma_load_2d_pair(dst + MXP_A_BYTES, low ? &map_b_low : &map_b, (tl.k0 + kt) * MX_BK, b_row, bar);
-                        tma_load_2d_pair(dst + (WGRAD ? MXP_SFB_OFF : MXP_SFA_OFF), &map_sf, 0, sf_row0 + kt, bar);
+                        tma_load_2d_pair(dst + (ROWS_N ? MXP_SFA_OFF : MXP_SFB_OFF), &map_sf, 0, sf_row0 + kt, bar);
                     }
                     __syncwarp();
                     ++issued;
@@ -724,7 +727,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0, n = MXP_NT;
             bool ok = true;
             for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
-                const int k_tiles_t = __shfl_sync(0xffffffffu, mxp_k_tiles<WGRAD>(p, ctl, t), 0);
+                const int k_tiles_t = __shfl_sync(0xffffffffu, mxp_k_tiles<FORM>(p, ctl, t), 0);
                 if (k_tiles_t == 0) continue;   // (weight gradients) an expert without rows: the epilogue writes zeros on its own
                 if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag))) break;
                 tc_fence_after();
@@ -761,17 +764,17 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         __syncwarp();
     } else if (warp == 2) {
         // ================= scales of the rows =================
-        // Weight gradients: the M side's, this CTA's 128 rows.  Row-ragged form: the N side's, all the tile's rows in both CTAs
+        // On the M side: this CTA's 128 rows.  On the N side: all the tile's rows in both CTAs
         // (at most 208: seven words per lane and slice, two blocks of 128 rows; columns past the tile's N are never read).
-        constexpr int WORDS = WGRAD ? 4 : 7;
+        constexpr int WORDS = ROWS_N ? 7 : 4;
         uint32_t stage = 0, phase = 0;
         bool ok = true;
         for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
-            const MxPairTile tl = mxp_decode<WGRAD>(p, ctl, t);
+            const MxPairTile tl = mxp_decode<FORM>(p, ctl, t);
             long long rows[WORDS];
 #pragma unroll
             for (int i = 0; i < WORDS; ++i) {
-                const long long r = (long long)tl.row0 + (WGRAD ? (int)rank * MX_BM : 0) + 32 * i + lane;
+                const long long r = (long long)tl.row0 + (ROWS_N ? 0 : (int)rank * MX_BM) + 32 * i + lane;
                 rows[i] = r < p.sa_rows ? r : p.sa_rows - 1;   // rows past the end are never stored; any valid address will do
             }
             // the words of MX_SCALE_AHEAD slices are in flight at any time: one slice per global-load round trip would
@@ -795,9 +798,9 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     const Words cur = q[i];
                     if (kt + MX_SCALE_AHEAD < tl.k_tiles) q[i] = load_slice(kt + MX_SCALE_AHEAD);
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag))) { ok = false; break; }
-                    uint8_t* to = tiles_ptr + stage * MXP_STAGE_BYTES + (WGRAD ? MXP_SFA_OFF : MXP_SFB_OFF) + lane * 16;
+                    uint8_t* to = tiles_ptr + stage * MXP_STAGE_BYTES + (ROWS_N ? MXP_SFB_OFF : MXP_SFA_OFF) + lane * 16;
                     *reinterpret_cast<uint4*>(to) = make_uint4(cur.w[0], cur.w[1], cur.w[2], cur.w[3]);
-                    if (!WGRAD) *reinterpret_cast<uint4*>(to + 512) = make_uint4(cur.w[4], cur.w[5], cur.w[6], cur.w[7]);
+                    if (ROWS_N) *reinterpret_cast<uint4*>(to + 512) = make_uint4(cur.w[4], cur.w[5], cur.w[6], cur.w[7]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote(full0 + stage * (uint32_t)sizeof(unsigned long long));
@@ -815,7 +818,7 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             for (long long t = first_tile; ok && t < n_tiles_total; t += tile_stride) {
-                const int k_tiles_t = __shfl_sync(0xffffffffu, mxp_k_tiles<WGRAD>(p, ctl, t), 0);
+                const int k_tiles_t = __shfl_sync(0xffffffffu, mxp_k_tiles<FORM>(p, ctl, t), 0);
                 for (int kt = 0; kt < k_tiles_t; ++kt) {
                     if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->full[stage]), phase, abort_flag))) { ok = false; break; }
                     tc_fence_after();
@@ -848,14 +851,14 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t empty0 = map_to_cta(smem_u32(&ctl->tmem_empty[0]), 0);
         uint32_t n_stores = 0, acc = 0, acc_phase = 0;
         for (long long t = first_tile; t < n_tiles_total; t += tile_stride) {
-            const MxPairTile tl = mxp_decode<WGRAD>(p, ctl, t);
+            const MxPairTile tl = mxp_decode<FORM>(p, ctl, t);
             const bool have_acc = tl.k_tiles != 0;
             if (have_acc) {
                 if (!__all_sync(0xffffffffu, mx_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag))) break;
                 tc_fence_after();
             }
             const uint32_t taddr = tmem_base + acc * MXP_ACC_STRIDE + ((uint32_t)(quarter * 32) << 16);
-            if (!WGRAD) {
+            if (ROWS_N) {
                 // lane = feature, column = row: the two warps of a lane quarter take the 32-row blocks alternately; a block is
                 // transposed on its way into the staging buffer
                 const int f = tl.n0 + (int)rank * MX_BM + quarter * 32;
@@ -886,11 +889,11 @@ mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     }
                 }
             }
-            const int slab_in = tl.row0 + (int)rank * MX_BM + quarter * 32;   // first row of this warp's slab, inside the expert's output
-            const int rows_valid = max(0, min(32, p.M - slab_in));
-            const int slab0 = slab_in + tl.out_row0;                          // ... and in the output tensor
+            const int slab_in = (int)rank * MX_BM + quarter * 32;   // first row of this warp's slab, inside the tile
+            const int rows_valid = max(0, min(32, tl.rows - slab_in));
+            const int slab0 = tl.out_row0 + tl.row0 + slab_in;      // ... and in the output tensor
 #pragma unroll 1
-            for (int c = half; WGRAD && c < 8; c += 2) {
+            for (int c = half; !ROWS_N && c < 8; c += 2) {
                 const int left = tl.width - 32 * c;   // columns of the tile from this block on (warp-uniform)
                 if (left <= 0) break;
                 const int n = tl.n0 + c * 32;
@@ -1440,7 +1443,7 @@ int launch_mx_quantize_tokens(long long R, int E, const bf16* x, long long ld, i
                             pitch, codes_t, reinterpret_cast<uint32_t*>(sa), sb);
 }
 
-template <bool WGRAD>
+template <int FORM>
 static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b_low, const CUtensorMap& sf, const CUtensorMap& o, const MxPairParams& p,
                           cudaStream_t s) {
     static int grid_of_device[64] = {};
@@ -1454,18 +1457,18 @@ static int launch_mx_pair(const CUtensorMap& a, const CUtensorMap& b, const CUte
     cfg.dynamicSmemBytes = MXP_SMEM_BYTES;
     cfg.attrs = attr; cfg.numAttrs = 1;
     if (grid_of_device[dev] == 0) {
-        if (cudaFuncSetAttribute(mx_pair_kernel<WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MXP_SMEM_BYTES) != cudaSuccess)
+        if (cudaFuncSetAttribute(mx_pair_kernel<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, MXP_SMEM_BYTES) != cudaSuccess)
             return MOE_ERR_CUDA;
         const int sms = sm_count();
         if (sms <= 0) return MOE_ERR_CUDA;
         // as many pairs as can be resident at once: a pair that had to wait for a free SM pair would double the duration
         cfg.gridDim = dim3(2 * (sms / 2));
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, mx_pair_kernel<WGRAD>, &cfg) != cudaSuccess || clusters <= 0) return MOE_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&clusters, mx_pair_kernel<FORM>, &cfg) != cudaSuccess || clusters <= 0) return MOE_ERR_CUDA;
         if (clusters > sms / 2) clusters = sms / 2;
         grid_of_device[dev] = 2 * clusters;
     }
-    return launch_dependent(mx_pair_kernel<WGRAD>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, b_low, sf, o, p);
+    return launch_dependent(mx_pair_kernel<FORM>, grid_of_device[dev], MXP_THREADS, MXP_SMEM_BYTES, 2, s, a, b, b_low, sf, o, p);
 }
 
 // dW [E, M, N] = Q(A)^T Q(B) per expert: a_* the M-side operand ([M, pitch] codes, scales with header and words),
@@ -1488,17 +1491,41 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
     p.prefix = reinterpret_cast<const int32_t*>(a_scales); p.E = E; p.M = M; p.m_tiles = m_tiles; p.n_tiles = n_tiles;
     p.n_cols = N; p.n_slices = n_slices; p.sa_rows = M;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales + MX_TOKENS_HEADER_BYTES); p.out = dw; p.ldo = N;
-    return launch_mx_pair<true>(a, b, b, sfb, o, p, s);
+    return launch_mx_pair<MXP_WGRAD>(a, b, b, sfb, o, p, s);
 }
 
-// CTA pairs from 256 rows per expert on average, and from 96 on if there are tiles for all pairs of the chip even with one row
-// tile per expert and the contraction is at least 512.  Single CTA against pair, gate/up / down / down dgrad / gate/up dgrad, rows per expert:
+// Which kernel for R rows of E experts, n_feat output features, a contraction of k.
+// CTA pairs, weights on M, from 256 rows per expert on average, and from 96 on if there are tiles for all pairs of the chip even with
+// one row tile per expert and the contraction is at least 512.  Single CTA against pair, gate/up / down / down dgrad / gate/up dgrad, rows per expert:
 //   128 (128 experts, 2048 x 768)   108 / 70 / 60 / 117 against 102 / 65 / 60 / 105 us     81:  88 / 63 / 52 / 96 against 83 / 60 / 51 / 91 us
 //   128 (8 experts, 4096 x 14336)   213 / 126 / 112 / 255 against 189 / 100 / 103 / 191 us  80:  169 / 93 / 92 / 172 against 170 / 95 / 96 / 176 us
 //   125 (16 experts, 256 x 512: 16 to 64 pair tiles)   7.7 / 5.6 / 5.5 / 6.1 against 8.0 / 6.5 / 6.2 / 7.4 us
 //   229 (2 experts, gate/up of 6272 features each, contraction 128)   6.5 against 7.4 us
-static bool mx_use_pairs(long long R, int E, int n_feat, int k) {
-    return R >= 256ll * E || (R >= 96ll * E && k >= 512 && (long long)E * ((n_feat + MXP_ROWS - 1) / MXP_ROWS) >= 74);
+// Not where 256 features per tile leave half (128 features) or a quarter (384) of them empty: of 128 features single CTAs, whatever the
+// rows (weights on M / rows on M / single CTA: 893 rows, 110 experts, k 2688 76 / 62 / 64 us, 3794, 4, k 1024 13.0 / 9.4 / 8.1, 98, 170, k 768 13.2 /
+// 12.7 / 9.6), of 384 rows on M, below 256 rows single CTAs (5263, 9, k 8064 176 / 144 / 169, 733, 10, k 2432 16.5 / 11.7 / 13.4, 110, 129, k 1024
+// 22.5 / 22.3 / 19.9).
+// And not where it takes more rounds of tiles over the chip's CTA pairs, each round at its price (a tile of w rows on N 0.76 + 0.24 w / 208 of
+// a full one's time, a single CTA's tile 0.81).  Tiles per expert: the mean of those of an even load and those of one whose experts end
+// anywhere in a tile.  Weights on M / rows on M: 481 rows, 85 experts, 1664 features, k 768 76 / 65 us, 419, 152, 3328, k 640 234 / 199 us.  Weights
+// on M / single CTA: 106 rows, 15 experts, 2432 features, k 896 12.9 / 10.6 us, 96, 130, 640, k 3456 69 / 61 us.
+// 2340 drawn shapes from 96 rows on: this rule 3.2 % above the best form of each on average, weights on M from 256 rows throughout 6.3 %,
+// rows on M 9.0 %; slower than rows on M by more than a tenth 18 of them, with weights on M throughout 265.
+enum MxGemmForm { MX_SINGLE, MX_PAIR_WEIGHTS_M, MX_PAIR_ROWS_M };
+static MxGemmForm mx_form(long long R, int E, int n_feat, int k) {
+    const int on_m = (n_feat + MXP_ROWS - 1) / MXP_ROWS, on_n = (n_feat + MXP_NT - 1) / MXP_NT;   // tiles of features
+    const bool mostly_full = 5 * n_feat >= 4 * MXP_ROWS * on_m, small = R < 256ll * E;
+    if (R < 96ll * E || n_feat <= 128) return MX_SINGLE;
+    if (small && !(mostly_full && k >= 512 && (long long)E * on_m >= kChipPairs)) return MX_SINGLE;
+    if (!mostly_full) return MX_PAIR_ROWS_M;
+    const double rows = (double)R / E;
+    const auto rounds = [&](double tile_rows, double feature_tiles, int at_once) {
+        return ceil(E * (ceil(rows / tile_rows) + rows / tile_rows + 0.5) / 2 * feature_tiles / at_once);
+    };
+    const double tile_n = ceil(rows / ceil(rows / MXP_NT) / 16) * 16;
+    const double weights_m = rounds(MXP_NT, on_m, kChipPairs) * (0.76 + 0.24 * (tile_n / MXP_NT + 1) / 2);
+    if (small) return 0.95 * weights_m < 0.81 * rounds(MX_BM, n_feat / MX_BN, 2 * kChipPairs) ? MX_PAIR_WEIGHTS_M : MX_SINGLE;
+    return 1.03 * rounds(MXP_ROWS, on_n, kChipPairs) < weights_m ? MX_PAIR_ROWS_M : MX_PAIR_WEIGHTS_M;
 }
 // The swapped form of the single-CTA kernel up to this many rows per expert on average.  There the time is the weights'
 // way from HBM, and what counts is bytes in flight and an even spread over the SMs: two CTAs with four stages of weights
@@ -1517,7 +1544,7 @@ static bool mx_use_pairs(long long R, int E, int n_feat, int k) {
 constexpr long long kMxSwappedRows = 64;
 static bool mx_single_swapped(long long R, int E) { return R <= kMxSwappedRows * E && MxGeo<64>::all_ctas_fit(E); }
 
-static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
+static int launch_mx_gemm_pair_weights_m(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
                                const uint8_t* b_codes, const uint8_t* b_scales, const int32_t* offsets, bf16* out,
                                cudaStream_t s) {
     const int k_tiles = k / MX_BK;
@@ -1532,7 +1559,23 @@ static int launch_mx_gemm_pair(long long R, int E, int n_feat, int k, const uint
     MxPairParams p = {};
     p.prefix = offsets; p.E = E; p.k_tiles = k_tiles; p.n_tiles = (n_feat + MXP_ROWS - 1) / MXP_ROWS; p.n_cols = n_feat; p.sa_rows = R;
     p.sa = reinterpret_cast<const uint32_t*>(a_scales); p.out = out; p.ldo = n_feat;
-    return launch_mx_pair<false>(w, x, x_low, sf, o, p, s);
+    return launch_mx_pair<MXP_WEIGHTS_M>(w, x, x_low, sf, o, p, s);
+}
+static int launch_mx_gemm_pair_rows_m(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales,
+                                      const uint8_t* b_codes, const uint8_t* b_scales, const int32_t* offsets, bf16* out,
+                                      cudaStream_t s) {
+    const int k_tiles = k / MX_BK, n_tiles = (n_feat + MXP_NT - 1) / MXP_NT;
+    CUtensorMap x, w, sf, o;
+    if (!make_map_typed(&x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a_codes, k, (uint64_t)R, MX_BK, MX_BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, b_codes, k, (uint64_t)E * n_feat, MX_BK, MXP_NT / 2, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_typed(&sf, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, b_scales + mx_w_scale_single_bytes(E, n_feat, k), 256,
+                        (uint64_t)E * n_tiles * k_tiles, 256, 1, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_out_map(&o, out, n_feat, (uint64_t)R))
+        return MOE_ERR_CUDA;
+    MxPairParams p = {};
+    p.prefix = offsets; p.E = E; p.k_tiles = k_tiles; p.n_tiles = n_tiles; p.n_cols = n_feat; p.sa_rows = R;
+    p.sa = reinterpret_cast<const uint32_t*>(a_scales); p.out = out; p.ldo = n_feat;
+    return launch_mx_pair<MXP_ROWS_M>(x, w, w, sf, o, p, s);
 }
 
 struct MxSingleArgs {
@@ -1574,8 +1617,9 @@ static int launch_mx_gemm_single(const MxSingleArgs& g, cudaStream_t s) {
 // [k/128][R], b [E, n_feat, k] codes with both scale tilings, out [R, n_feat] bf16.
 int launch_mx_gemm(long long R, int E, int n_feat, int k, const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* b_codes,
                    const uint8_t* b_scales, const int32_t* offsets, bf16* out, cudaStream_t s) {
-    if (mx_use_pairs(R, E, n_feat, k))
-        return launch_mx_gemm_pair(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out, s);
+    const MxGemmForm form = mx_form(R, E, n_feat, k);
+    if (form == MX_PAIR_WEIGHTS_M) return launch_mx_gemm_pair_weights_m(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out, s);
+    if (form == MX_PAIR_ROWS_M) return launch_mx_gemm_pair_rows_m(R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out, s);
     const MxSingleArgs args = {R, E, n_feat, k, a_codes, a_scales, b_codes, b_scales, offsets, out};
     return mx_single_swapped(R, E) ? launch_mx_gemm_single<64>(args, s) : launch_mx_gemm_single<128>(args, s);
 }
@@ -1588,6 +1632,8 @@ extern "C" void moe_test_mx_single_ctas(int R, int E, int* ctas, int* smem) {
     *ctas = swapped ? MxGeo<64>::CTAS : MxGeo<128>::CTAS;
     *smem = swapped ? MxGeo<64>::smem_bytes(E) : MxGeo<128>::smem_bytes(E);
 }
+// ... and the kernel that R rows of E experts, n_feat features and a contraction of k go to (MxGemmForm).
+extern "C" int moe_test_mx_form(long long R, int E, int n_feat, int k) { return mx_form(R, E, n_feat, k); }
 #endif
 
 }  // namespace moe

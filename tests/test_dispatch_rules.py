@@ -1,0 +1,20 @@
+"""The rules that choose between the forms of a kernel, by the library's test-only build, without a device."""
+import ctypes
+
+from paper_2606_26453_b200 import build
+from tests.test_gpu_mxfp8_pair_tiles import CASES
+
+
+def test_mxfp8_gemm():
+    """Which kernel a shape goes to: single CTAs, pairs with the weights on the M side, pairs with the rows there."""
+    lib = ctypes.CDLL(build.build_library(waittest=True))
+    lib.moe_test_mx_form.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 3
+    forms = {name: lib.moe_test_mx_form(sum(c), len(c), H, I) for name, (H, I, c) in CASES.items()}
+    assert forms == {"one_feature_block": 0, "last_tile_half_wide": 1, "low_box_edges": 1, "empty_and_last": 0, "many_slices": 1,
+                     "rows_m_edges": 2, "rows_m_halves": 2, "rows_m_empty": 2, "rows_m_many_slices": 2, "rows_m_narrow_last": 2, "96_rows": 1,
+                     "96_rows_too_few_tiles": 0, "96_rows_short": 0, "96_rows_uneven": 0}
+    # sizes at which each was found the better one: many rows of 128 and of 384 features, row tiles of 208 that are just exceeded, few rows
+    for R, E, n, k, form in ((893 * 110, 110, 128, 2688, 0), (5263 * 9, 9, 384, 8064, 2), (733 * 10, 10, 384, 2432, 2), (481 * 85, 85, 1664, 768, 2),
+                             (419 * 152, 152, 3328, 640, 2), (110 * 129, 129, 384, 1024, 0), (106 * 15, 15, 2432, 896, 0), (96 * 130, 130, 640, 3456, 0), (128 * 128, 128, 1536, 2048, 1), (384 * 64, 64, 2816, 2048, 1),
+                             (1024 * 128, 128, 2048, 768, 1), (2048 * 8, 8, 28672, 4096, 1), (2048 * 8, 8, 4096, 14336, 1), (25 * 8, 8, 4096, 14336, 0)):
+        assert lib.moe_test_mx_form(R, E, n, k) == form, (R, E, n, k)

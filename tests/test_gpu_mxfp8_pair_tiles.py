@@ -1,5 +1,5 @@
-"""The CTA-pair block-scaled FP8 GEMM at the edges of its tiles (256 output features, equal tiles of at most 208 rows) and at the
-lines where it takes over from the single-CTA kernel, through the down projection, against the exact products of the dequantised
+"""The CTA-pair block-scaled FP8 GEMM at the edges of its tiles (256 output features and equal tiles of at most 208 rows, or 256 rows
+and 208 features) and at the lines where it takes over from the single-CTA kernel, through the down projection, against the exact products of the dequantised
 operands with the tolerance of the other FP8 GEMM tests."""
 import numpy as np
 import pytest
@@ -12,11 +12,18 @@ from tests import helpers as Hh
 pytestmark = pytest.mark.gpu
 
 CASES = {   # output features, contraction, rows of each expert
-    "one_tile_half_wide": (128, 128, [256]),                       # the second CTA has no features; 256 rows: two tiles of 128
-    "row_edges": (384, 256, [207, 208, 209, 415, 416, 417]),       # a tile and half a one wide; one, two and three row tiles
+    "one_feature_block": (128, 128, [256]),                        # a single CTA's
+    # 256 features a tile:
+    "last_tile_half_wide": (640, 256, [207, 208, 209, 415, 416, 417]),   # the second CTA has no features; one, two and three row tiles
     "low_box_edges": (256, 640, [128, 129, 1, 16, 17, 1040, 624]), # 64 rows per CTA and more; five tiles of 208
     "empty_and_last": (640, 384, [0, 900, 0, 33, 0]),
     "many_slices": (256, 1152, [300, 250]),                        # more slices than scale words in flight
+    # 256 rows a tile:
+    "rows_m_edges": (384, 256, [255, 256, 257, 511, 512, 513]),    # columns 208 and 176; one, two and three row tiles
+    "rows_m_halves": (384, 640, [127, 128, 129, 1, 33, 1040, 624]),  # the second CTA's rows: none, one; five tiles
+    "rows_m_empty": (384, 128, [0, 900, 0, 33, 0, 700]),
+    "rows_m_many_slices": (384, 1152, [300, 250]),
+    "rows_m_narrow_last": (1664, 128, [431] * 8),                  # eight tiles of 208 against six and a half of 256
     "96_rows": (256, 512, [96] * 74),                              # the first sizes of the pair form with few rows ...
     "96_rows_too_few_tiles": (256, 512, [96] * 73),                # ... and the last of the other:
     "96_rows_short": (256, 384, [96] * 74),                        # too few tiles, too short a contraction
