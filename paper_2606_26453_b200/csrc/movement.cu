@@ -665,12 +665,19 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
 }
 
 // Threads per token: the most that leave every thread two pieces of the row or more and the fewest places empty (32 for narrow rows).
-// A block per token, as before, against this (T x H, K; us): 20000 x 256, 2 25.3 -> 8.2; 20000 x 512, 2 45.1 -> 16.7, K = 8 120 -> 59;
+// A block per token against this (T x H, K; us): 20000 x 256, 2 25.3 -> 8.2; 20000 x 512, 2 45.1 -> 16.7, K = 8 120 -> 59;
 // 20000 x 832, 4 90 -> 55; 20000 x 1024, 3 70 -> 47; 10000 x 1280, 8 86 -> 73; 8192 x 1536, 4 47 -> 39; 16384 x 2048, 8 181 -> 174;
 // 14442 x 2880, 4 137 -> 121; 8192 x 4096, 2 54.7 (a block per token stays: 128 threads 55.4).
-static int combine_bwd_lanes_of(int hv) {
+// Of few tokens no fewer threads than give every SM two blocks of them: one thread's pieces come one after the other, and with fewer
+// the chip waits for them (32 / 256 threads: 12 x 7744, 7 24.7 / 6.9 us, 515 x 3776, 6 11.6 / 7.1, 41 x 2624, 7 9.9 / 6.8).
+// Rows of 3584 and more fill a block well enough whatever their width, and it keeps more loads in flight (32 / 256 threads: 3593 x
+// 5696, 6 112 / 93 us, without dtopk_w 63 / 53; 11279 x 3648, 5 168 / 160 and 98 / 88).
+constexpr int kLongRowPieces = 3584 / 8;
+static int combine_bwd_lanes_of(int T, int hv) {
+    if (hv >= kLongRowPieces) return kThreads;
     int best = 32;
-    for (int lanes = 64; lanes <= kThreads && 2 * lanes <= hv; lanes *= 2)
+    while (best < kThreads && 2 * best <= hv && (long long)T * best < 2ll * 2 * kChipPairs * kThreads) best *= 2;
+    for (int lanes = 2 * best; lanes <= kThreads && 2 * lanes <= hv; lanes *= 2)
         if ((hv + lanes - 1) / lanes * lanes <= (hv + best - 1) / best * best) best = lanes;
     return best;
 }
@@ -693,7 +700,7 @@ static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint
 template <bool WITH_DW, bool TRIGGER>
 static int combine_bwd_lanes(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w, const int32_t* p2r, uint4* dyp,
                              float* dw, cudaStream_t s) {
-    const int lanes = combine_bwd_lanes_of(d.H / 8);
+    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8);
     if (lanes == 32) return combine_bwd_dispatch<WITH_DW, TRIGGER, 32>(d, dy, yp, w, p2r, dyp, dw, s);
     if (lanes == 64) return combine_bwd_dispatch<WITH_DW, TRIGGER, 64>(d, dy, yp, w, p2r, dyp, dw, s);
     if (lanes == 128) return combine_bwd_dispatch<WITH_DW, TRIGGER, 128>(d, dy, yp, w, p2r, dyp, dw, s);
@@ -705,7 +712,7 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    const int tokens = kThreads / combine_bwd_lanes_of(d.H / 8);   // per block
+    const int tokens = kThreads / combine_bwd_lanes_of(d.T, d.H / 8);   // per block
     const bool trigger = d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
     if (dtopk_w != nullptr)
         return trigger ? combine_bwd_lanes<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
@@ -713,6 +720,11 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     return trigger ? combine_bwd_lanes<false, true>(d, a, b, topk_w, pair_to_row, o, nullptr, s)
                    : combine_bwd_lanes<false, false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
 }
+
+#ifdef MOE_TEST_HOOKS
+// Test-only build: threads per token of a combine backward.
+extern "C" int moe_test_combine_bwd_lanes(int T, int H) { return combine_bwd_lanes_of(T, H / 8); }
+#endif
 
 // ------------------------------------------------------------------------------------------------
 // Route-permute without a caller-provided workspace.  The chunk-histogram table lives in a

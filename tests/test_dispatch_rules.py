@@ -18,3 +18,12 @@ def test_mxfp8_gemm():
                              (419 * 152, 152, 3328, 640, 2), (110 * 129, 129, 384, 1024, 0), (106 * 15, 15, 2432, 896, 0), (96 * 130, 130, 640, 3456, 0), (128 * 128, 128, 1536, 2048, 1), (384 * 64, 64, 2816, 2048, 1),
                              (1024 * 128, 128, 2048, 768, 1), (2048 * 8, 8, 28672, 4096, 1), (2048 * 8, 8, 4096, 14336, 1), (25 * 8, 8, 4096, 14336, 0)):
         assert lib.moe_test_mx_form(R, E, n, k) == form, (R, E, n, k)
+
+
+def test_threads_per_token_of_the_combine_backward():
+    """Narrow rows share a block; not so few tokens that the chip is not full, nor long rows."""
+    lanes = ctypes.CDLL(build.build_library(waittest=True)).moe_test_combine_bwd_lanes
+    for T, H, want in ((20000, 256, 32), (20000, 512, 32), (20000, 832, 32), (20000, 1024, 64), (10000, 1280, 32), (16384, 2048, 128), (8192, 4096, 256),
+                       (14442, 2880, 128), (27, 2304, 256), (12, 7744, 256), (515, 3776, 256), (41, 2624, 256), (3593, 5696, 256), (4736, 1152, 32),
+                       (2367, 1152, 64), (1, 64, 32), (1, 512, 64), (2368, 3072, 128), (2368, 3328, 32), (2367, 3328, 64), (2368, 3584, 256)):
+        assert lanes(T, H) == want, (T, H, lanes(T, H))

@@ -11,8 +11,8 @@ from tests import helpers as Hh
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H", [64, 256, 320, 1024, 1280, 2048, 2880, 4096, 4160])
-@pytest.mark.parametrize("T,K", [(1, 1), (7, 3), (13, 8), (5, 20)])
+@pytest.mark.parametrize("H", [64, 256, 320, 1024, 1280, 2048, 2880, 3520, 4096, 4160])
+@pytest.mark.parametrize("T,K", [(1, 1), (7, 3), (13, 8), (5, 20), (2373, 2)])   # the last: enough tokens for 32 threads each
 def test_widths(H, T, K):
     from paper_2606_26453_b200 import binding as B
     E, R = max(K, 4), T * K
