@@ -156,7 +156,7 @@ def permute_launches(cfg):
     """Kernels of one route-permute: ranking alone, histogram and ranking, or a scan in between (csrc/movement.cu)."""
     if cfg.R <= 2048:
         return 1
-    return 3 if (cfg.R + 2047) // 2048 * cfg.E >= 1024 else 2
+    return 3 if (cfg.T + 3) // 4 * ((cfg.R + 2047) // 2048 * cfg.E) >= 1500000 else 2
 
 
 GEMM_CALLS = ["gateup_swiglu", "down", "down_dgrad", "down_wgrad", "gateup_dgrad", "gateup_wgrad"]

@@ -39,7 +39,7 @@ __device__ __forceinline__ uint4 pack8(const float f[8]) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// a1 in two launches, one with few pairs (kDirectPairs), three with many (kScanEntries).
+// a1 in two launches, one with few pairs (kDirectPairs), three with many (kScanSums).
 //   hist      : one block per `chunk` consecutive pairs (a multiple of 256): the number of pairs of each
 //               expert in the chunk (shared-memory atomics: counts are order-free)          -> ws[chunk][e]
 //   rank_rows : one block per kTokPerBlock consecutive tokens.  The block
@@ -589,22 +589,36 @@ int movement_read_and_clear_status(int* status_out) {
 // is no histogram launch: the call takes 6.3 us instead of 8.3 (256 tokens of 256 to 2 of 8 experts, 32 of 2048 to 8 of 128, 2000 of 256 to
 // one each 8.5 instead of 11.0).  At 4096 pairs 9.0 against 8.2 us (512 tokens of 2048 to 8 of 128 experts).
 constexpr int kDirectPairs = 2048;
-// From this many histogram entries (chunks of 2048 pairs times experts) on a launch in between turns them into running sums: with
-// 16384 entries every block of rank_rows summed them all, and that outlasted the rows unless they were long.  32768 tokens of 256 and of
-// 1024 to 8 of 128 experts 240 -> 52 and 241 -> 105 us, 4000 of 1024 to 8 of 1024 56 -> 34, 20000 of 640 to 3 of 40 (1200 entries)
-// 37.8 -> 31.0, 16384 of 2048 to 8 of 128 110 -> 107, 32768 of 4096 to 8 of 64 391 -> 389 us.  With fewer the launch costs more: 4096 of 2048 to 6
-// of 64 (768 entries) 25.9 -> 26.7, 1777 of 2880 to 4 of 128 (512) 12.8 -> 13.7 us.  Chunks of 1024 pairs: 512 were 0-5 % slower, 256 5-30 %.
-constexpr long long kScanEntries = 1024;
+// Every block of rank_rows sums all histogram entries (chunks of 2048 pairs times experts), unless a launch in between turns them into
+// running sums.  That launch costs about 2 us and is worth it from this many sums over all blocks on:
+//   tokens x width to K of E experts   entries     sums   each block sums  / scan in between, us
+//   32768 x 256, 8 of 128                16384   134 M    240 / 52
+//   13004 x 640, 7 of 274                12330    40 M     86 / 34
+//   31938 x 64, 1 of 115                  1840    15 M     68 / 46
+//   36485 x 128, 7 of 8                   1000   9.1 M     64 / 50
+//    9678 x 128, 6 of 34                   986   2.4 M     22 / 19
+//    5118 x 2496, 5 of 95                 1235   1.6 M     32 / 32
+//    2976 x 2624, 5 of 264                2112   1.6 M     21 / 22
+//    2354 x 448, 3 of 552                 2208   1.3 M     12.0 / 13.5
+//     536 x 3008, 5 of 999                1998   0.27 M    14 / 21
+//    4096 x 2048, 6 of 64                  768   0.79 M    25.9 / 26.7
+// Its chunks are of 1024 pairs: 512 were 0-5 % slower, 256 5-30 %.
+constexpr long long kScanSums = 1500000;
 static int permute_scan_chunk(long long R) {
     const long long need = (R + 4095) / 4096;
     return (int)(need > 1024 ? (need + kThreads - 1) / kThreads * kThreads : 1024);
+}
+static PermuteSums permute_sums(const moe_dims_t& d) {
+    const long long R = (long long)d.T * d.K, blocks = (d.T + kTokPerBlock - 1) / kTokPerBlock;
+    if (R <= kDirectPairs) return kCountAll;
+    return blocks * ((R + 2047) / 2048 * d.E) >= kScanSums ? kScanned : kSumRows;
 }
 int launch_permute(const moe_dims_t& d, const bf16* x, const int32_t* topk_idx, bf16* x_perm, int32_t* counts,
                    int32_t* offsets, int32_t* row_to_pair, int32_t* pair_to_row, void* workspace,
                    cudaStream_t s) {
     const int R = d.T * d.K, E = d.E;
-    const bool direct = R <= kDirectPairs;
-    const bool scanned = !direct && (long long)((R + 2047) / 2048) * E >= kScanEntries;
+    const PermuteSums sums = permute_sums(d);
+    const bool direct = sums == kCountAll, scanned = sums == kScanned;
     const int chunk = scanned ? permute_scan_chunk(R) : permute_chunk(R);
     const int n_chunks = (R + chunk - 1) / chunk;
     int32_t* ws = static_cast<int32_t*>(workspace);
@@ -724,6 +738,11 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
 #ifdef MOE_TEST_HOOKS
 // Test-only build: threads per token of a combine backward.
 extern "C" int moe_test_combine_bwd_lanes(int T, int H) { return combine_bwd_lanes_of(T, H / 8); }
+// ... and the kernels that a route-permute launches.
+extern "C" int moe_test_permute_launches(int T, int K, int E) {
+    const PermuteSums sums = permute_sums({T, 64, 64, E, K});
+    return sums == kCountAll ? 1 : sums == kScanned ? 3 : 2;
+}
 #endif
 
 // ------------------------------------------------------------------------------------------------

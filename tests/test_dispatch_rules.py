@@ -27,3 +27,16 @@ def test_threads_per_token_of_the_combine_backward():
                        (14442, 2880, 128), (27, 2304, 256), (12, 7744, 256), (515, 3776, 256), (41, 2624, 256), (3593, 5696, 256), (4736, 1152, 32),
                        (2367, 1152, 64), (1, 64, 32), (1, 512, 64), (2368, 3072, 128), (2368, 3328, 32), (2367, 3328, 64), (2368, 3584, 256)):
         assert lanes(T, H) == want, (T, H, lanes(T, H))
+
+
+def test_launches_of_a_permute():
+    """A scan goes in between where the blocks' sums are worth a launch; the benchmark's count of launches follows the library's."""
+    import bench
+    from paper_2606_26453_b200 import workloads as W
+    launches = ctypes.CDLL(build.build_library(waittest=True)).moe_test_permute_launches
+    for T, K, E, want in ((2048, 1, 128, 1), (2049, 1, 128, 2), (32768, 8, 128, 3), (36485, 7, 8, 3), (5118, 5, 95, 3), (2354, 3, 552, 2), (536, 5, 999, 2),
+                          (4096, 6, 64, 2), (1420, 7, 236, 2), (14336, 1, 128, 3), (6250, 4, 73, 2), (6250, 4, 74, 3),
+                          (8192, 1, 183, 2), (8192, 1, 184, 3)):
+        assert launches(T, K, E) == want, (T, K, E)
+    for T, K, E in [(c.T, c.K, c.E) for c in W.CONFIGS.values()] + [(T, K, E) for T in (1, 2047, 2048, 3000, 8192, 60000) for K in (1, 2, 8) for E in (8, 183, 184, 1000)]:
+        assert bench.permute_launches(W.MoeConfig("x", T=T, H=64, I=64, E=E, K=K, cfg_id=0)) == launches(T, K, E), (T, K, E)

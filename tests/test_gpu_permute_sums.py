@@ -1,5 +1,5 @@
 """Route-permute on both sides of the number of pairs (2048) from which a histogram launch goes before the ranking, and of the number of
-histogram entries (1024) from which a scan launch goes in between: indices, offsets, counts and rows against the oracle, bit for
+sums over all blocks (1.5 million) from which a scan launch goes in between: indices, offsets, counts and rows against the oracle, bit for
 bit, with expert ids outside [0, E) among them."""
 import numpy as np
 import pytest
@@ -13,9 +13,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,K,E", [(1, 1, 1), (5, 3, 1024), (2047, 1, 3), (2048, 1, 128), (2049, 1, 128), (64, 32, 40), (65, 32, 40), (682, 3, 7),
-                                   (683, 3, 7), (14336, 1, 128), (14337, 1, 128), (4099, 8, 1000), (1024, 10, 300), (33000, 1, 64)])
+                                   (683, 3, 7), (14336, 1, 128), (14337, 1, 128), (4099, 8, 1000), (1024, 10, 300), (33000, 1, 64), (8192, 1, 183), (8192, 1, 184), (36485, 7, 8)])
 @pytest.mark.parametrize("invalid", [False, True])
-def test_few_pairs(T, K, E, invalid):
+def test_both_sides_of_the_lines(T, K, E, invalid):
     from paper_2606_26453_b200 import binding as B
     H, R, guard = 192, T * K, 16
     rng = np.random.default_rng(R + E)
