@@ -60,7 +60,9 @@ inline bool apart(const void* a, size_t na, const void* b, size_t nb) {
 // A data gradient of at most about two tiles per CTA pair, beside which a weight gradient finds SMs without work.  256 tokens of 256
 // to 2 of 8 experts of 512: a training step 50.4 -> 47.1 us on the device.  Behind a long one there is next to nothing to gain (steps of 64 and 128
 // experts 0.1-0.3 %), and 128 experts of 2880 x 2880 lose 1 % of the call: the weight gradient's largest tiles no longer start together.
-inline bool leaves_sms_free(size_t rows, int E, int n) { return (rows / 256 + E) * (n / 256 + 1) <= 2 * 74; }
+// Nor where hardly an expert has a row: then the weight gradient is a stream of zeros, and the data gradient is slow beside it (10 rows,
+// 67 experts of 256 x 1856: gate/up and SwiGLU backward 43.9 alone, 54.1 us beside; 10, 69 of 3008 x 320, down backward 39.2 / 45.3).
+inline bool leaves_sms_free(size_t rows, int E, int n) { return 4 * rows > (size_t)E && (rows / 256 + E) * (n / 256 + 1) <= 2 * kChipPairs; }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -684,5 +686,10 @@ int moe_layer_fwd_bwd_host(const moe_dims_t* dims, const void* x_host, const int
     if (cudaStreamWaitEvent(s, lane->down_done, 0) != cudaSuccess) return MOE_ERR_CUDA;
     return MOE_OK;
 }
+
+#ifdef MOE_TEST_HOOKS
+// Test-only build: whether a combined backward call lets its weight gradient run beside a data gradient of `rows` rows and n features.
+int moe_test_weight_gradient_beside(int rows, int E, int n) { return leaves_sms_free((size_t)rows, E, n); }
+#endif
 
 }  // extern "C"

@@ -40,3 +40,11 @@ def test_launches_of_a_permute():
         assert launches(T, K, E) == want, (T, K, E)
     for T, K, E in [(c.T, c.K, c.E) for c in W.CONFIGS.values()] + [(T, K, E) for T in (1, 2047, 2048, 3000, 8192, 60000) for K in (1, 2, 8) for E in (8, 183, 184, 1000)]:
         assert bench.permute_launches(W.MoeConfig("x", T=T, H=64, I=64, E=E, K=K, cfg_id=0)) == launches(T, K, E), (T, K, E)
+
+
+def test_weight_gradient_beside_a_data_gradient():
+    """Beside a short data gradient, not one that fills the chip, nor where hardly an expert has a row."""
+    beside = ctypes.CDLL(build.build_library(waittest=True)).moe_test_weight_gradient_beside
+    for rows, E, n, want in ((512, 8, 512, 1), (512, 8, 256, 1), (10500, 2, 512, 1), (16384, 64, 2048, 0), (10, 67, 256, 0), (10, 69, 320, 0), (8, 32, 256, 0),
+                             (9, 32, 256, 1), (1, 1, 64, 1), (18944 - 256, 1, 255, 1), (147 * 256 + 255, 1, 64, 1), (148 * 256, 1, 64, 0)):
+        assert beside(rows, E, n) == want, (rows, E, n)
