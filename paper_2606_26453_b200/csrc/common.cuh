@@ -22,6 +22,12 @@ int sm_count();
 
 // CTA pairs the chip takes at once, one CTA per SM: what the rules of the dispatch count tiles against.  (The launches ask the device.)
 constexpr int kChipPairs = 148 / 2;
+// Rounds of tiles of `tile_rows` rows, times `feature_tiles`, for R rows of E experts, `at_once` of them at a time.  The host does not know
+// the load: per expert the mean of the tiles of an even one and of one whose experts end anywhere in a tile.
+inline double tile_rounds(long long R, int E, int tile_rows, long long feature_tiles, int at_once) {
+    const double tiles = (double)R / E / tile_rows;
+    return ceil(E * (ceil(tiles) + tiles + 0.5) / 2 * (double)feature_tiles / at_once);
+}
 
 // ---- programmatic dependent launch --------------------------------------------------------------
 // The library's kernels are launched as programmatic dependents of whatever precedes them on the stream: their blocks may be

@@ -1187,7 +1187,7 @@ bool use_swapped_fused(const moe_dims_t& d) { return rows_per_expert_below(d, 51
 // The SwiGLU forward swapped (gate and up of 128 features x up to 256 rows per tile), below 1600 rows like the other swapped forms.
 // Its epilogue passes 4 KB per block of 32 x 32 values through shared memory, beside the operands' traffic, and that outlasts short
 // contractions; below 96 rows per expert the weights' bytes count and not the tiles.  At fewer than about eight tiles per CTA pair
-// the last tile's epilogue shows (only against the pair forms: single-CTA tiles lose more to padding).  Gate/up forward, other
+// the last tile's epilogue shows (against the pair forms).  Gate/up forward, other
 // forms against this one (* each alone for half a second, the rest in turn in short bursts):
 //   384 rows (64 experts of 1408)   contraction 2048: 365 -> 314 us *, 1536: 242 -> 222, 1280: 204 -> 192, 1024: 158 -> 160
 //   1024 rows (128 experts, 2048 x 768) 784 -> 761 us *; (16 experts of 2048) contraction 4096: 929 -> 866 us (of 4096), 1536: 181 -> 178,
@@ -1197,9 +1197,17 @@ bool use_swapped_fused(const moe_dims_t& d) { return rows_per_expert_below(d, 51
 //   few tiles: 1000 rows (8 experts, 2048 x 192) 17.5 -> 19.5 us
 //   fewer rows: 250 (8 experts, 4096 x 14336) 528 -> 469 us, 96 (64 experts, 2048 x 1408) 150 -> 136, 69 (32 experts, 2048 x 1024) 51 -> 54,
 //        56 (128 experts, 2880 x 2880) 527 -> 527, 2 (128 experts, 2048 x 768) 89 -> 94
+// Below 320 rows not while the single CTAs' tiles of 128 rows all run at once, unless the swapped ones do too and are not much higher:
+// a longer tile then only lengthens the call.  Single CTAs / swapped: 315 rows (4 experts, 2560 x 1216) 22.4 / 29.6 us, 294 (22, 1920 x
+// 256) 22.7 / 28.1, Dirichlet 236 (5, 3840 x 1408) 32.9 / 43.2, 162 (19, 3584 x 512) 38.7 / 57.2, but 107 (5, 2944 x 896) 0.74 of the time.  264
+// drawn shapes: 1.7 % above the better form on average, swapped throughout 2.8 %, 3.5 % without saved pre-activations (2.0 % now).
 bool use_swapped_swiglu(const moe_dims_t& d) {
     if (rows_per_expert_below(d, 96) || !rows_per_expert_below(d, 1600) || d.H < 1536) return false;
-    return rows_per_expert_below(d, 320) || (long long)d.T * d.K * d.I >= 8ll * 74 * 256 * 128;
+    const long long R = (long long)d.T * d.K, feature_tiles = (d.I + SWAP_FEATS - 1) / SWAP_FEATS;
+    if (!rows_per_expert_below(d, 320)) return R * d.I >= 8ll * kChipPairs * SWAP_ROWS * SWAP_FEATS;
+    if (tile_rounds(R, d.E, BM, feature_tiles, 2 * kChipPairs) > 1) return true;
+    const double rows = (double)R / d.E, tile = rows / ceil(rows / SWAP_ROWS);
+    return tile_rounds(R, d.E, SWAP_ROWS, feature_tiles, kChipPairs) <= 1 && tile <= 176;
 }
 // Half-height last tiles of the SwiGLU forward, see launch_gateup_fwd.
 bool use_half_tiles(const moe_dims_t& d) { return rows_per_expert_below(d, 1600); }
@@ -1211,6 +1219,11 @@ bool use_pairs_for_swiglu(const moe_dims_t& d) { return (long long)d.T * d.K >= 
 bool use_pairs_for_wgrad(const moe_dims_t& d) { return (long long)d.T * d.K >= 256ll * d.E; }
 
 }  // namespace
+
+#ifdef MOE_TEST_HOOKS
+// Test-only build: whether the SwiGLU forward of these sizes runs swapped.
+extern "C" int moe_test_use_swapped_swiglu(int T, int H, int I, int E, int K) { return use_swapped_swiglu({T, H, I, E, K}); }
+#endif
 
 // Gate/up forward: A = x_perm [R,H]; B = w_gate, w_up viewed as [E*H, I]; fused width 2I in tiles of
 // 128 gate + 128 up columns.

@@ -1506,8 +1506,7 @@ int launch_mx_wgrad(long long R, int E, int M, int N, const uint8_t* a_codes_t, 
 // 12.7 / 9.6), of 384 rows on M, below 256 rows single CTAs (5263, 9, k 8064 176 / 144 / 169, 733, 10, k 2432 16.5 / 11.7 / 13.4, 110, 129, k 1024
 // 22.5 / 22.3 / 19.9).
 // And not where it takes more rounds of tiles over the chip's CTA pairs, each round at its price (a tile of w rows on N 0.76 + 0.24 w / 208 of
-// a full one's time, a single CTA's tile 0.81).  Tiles per expert: the mean of those of an even load and those of one whose experts end
-// anywhere in a tile.  Weights on M / rows on M: 481 rows, 85 experts, 1664 features, k 768 76 / 65 us, 419, 152, 3328, k 640 234 / 199 us.  Weights
+// a full one's time, a single CTA's tile 0.81).  Weights on M / rows on M: 481 rows, 85 experts, 1664 features, k 768 76 / 65 us, 419, 152, 3328, k 640 234 / 199 us.  Weights
 // on M / single CTA: 106 rows, 15 experts, 2432 features, k 896 12.9 / 10.6 us, 96, 130, 640, k 3456 69 / 61 us.
 // 2340 drawn shapes from 96 rows on: this rule 3.2 % above the best form of each on average, weights on M from 256 rows throughout 6.3 %,
 // rows on M 9.0 %; slower than rows on M by more than a tenth 18 of them, with weights on M throughout 265.
@@ -1518,14 +1517,10 @@ static MxGemmForm mx_form(long long R, int E, int n_feat, int k) {
     if (R < 96ll * E || n_feat <= 128) return MX_SINGLE;
     if (small && !(mostly_full && k >= 512 && (long long)E * on_m >= kChipPairs)) return MX_SINGLE;
     if (!mostly_full) return MX_PAIR_ROWS_M;
-    const double rows = (double)R / E;
-    const auto rounds = [&](double tile_rows, double feature_tiles, int at_once) {
-        return ceil(E * (ceil(rows / tile_rows) + rows / tile_rows + 0.5) / 2 * feature_tiles / at_once);
-    };
-    const double tile_n = ceil(rows / ceil(rows / MXP_NT) / 16) * 16;
-    const double weights_m = rounds(MXP_NT, on_m, kChipPairs) * (0.76 + 0.24 * (tile_n / MXP_NT + 1) / 2);
-    if (small) return 0.95 * weights_m < 0.81 * rounds(MX_BM, n_feat / MX_BN, 2 * kChipPairs) ? MX_PAIR_WEIGHTS_M : MX_SINGLE;
-    return 1.03 * rounds(MXP_ROWS, on_n, kChipPairs) < weights_m ? MX_PAIR_ROWS_M : MX_PAIR_WEIGHTS_M;
+    const double rows = (double)R / E, tile_n = ceil(rows / ceil(rows / MXP_NT) / 16) * 16;
+    const double weights_m = tile_rounds(R, E, MXP_NT, on_m, kChipPairs) * (0.76 + 0.24 * (tile_n / MXP_NT + 1) / 2);
+    if (small) return 0.95 * weights_m < 0.81 * tile_rounds(R, E, MX_BM, n_feat / MX_BN, 2 * kChipPairs) ? MX_PAIR_WEIGHTS_M : MX_SINGLE;
+    return 1.03 * tile_rounds(R, E, MXP_ROWS, on_n, kChipPairs) < weights_m ? MX_PAIR_ROWS_M : MX_PAIR_WEIGHTS_M;
 }
 // The swapped form of the single-CTA kernel up to this many rows per expert on average.  There the time is the weights'
 // way from HBM, and what counts is bytes in flight and an even spread over the SMs: two CTAs with four stages of weights

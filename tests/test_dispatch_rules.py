@@ -3,6 +3,7 @@ import ctypes
 
 from paper_2606_26453_b200 import build
 from tests.test_gpu_mxfp8_pair_tiles import CASES
+from tests.test_gpu_tile_edges import SWAPPED_SWIGLU
 
 
 def test_mxfp8_gemm():
@@ -48,3 +49,16 @@ def test_weight_gradient_beside_a_data_gradient():
     for rows, E, n, want in ((512, 8, 512, 1), (512, 8, 256, 1), (10500, 2, 512, 1), (16384, 64, 2048, 0), (10, 67, 256, 0), (10, 69, 320, 0), (8, 32, 256, 0),
                              (9, 32, 256, 1), (1, 1, 64, 1), (18944 - 256, 1, 255, 1), (147 * 256 + 255, 1, 64, 1), (148 * 256, 1, 64, 0)):
         assert beside(rows, E, n) == want, (rows, E, n)
+
+
+def test_swapped_swiglu_forward():
+    """From 96 rows per expert and widths of 1536 on, but below 320 rows not where single CTAs take one round; from 320 rows on with eight
+    tiles and more per pair; not from 1600 on."""
+    swapped = ctypes.CDLL(build.build_library(waittest=True)).moe_test_use_swapped_swiglu
+    for H, I, counts in SWAPPED_SWIGLU:
+        assert swapped(sum(counts), H, I, len(counts), 1), (H, I, counts)
+    for R, E, H, I, want in ((95, 1, 1536, 128, 0), (96, 1, 1472, 128, 0), (177, 1, 1536, 128, 0), (315 * 4, 4, 2560, 1216, 0), (294 * 22, 22, 1920, 256, 0),
+                             (236 * 5, 5, 3840, 1408, 0), (162 * 19, 19, 3584, 512, 0), (107 * 5, 5, 2944, 896, 1), (107 * 43, 43, 1792, 640, 1),
+                             (250 * 8, 8, 4096, 14336, 1), (320 * 80, 80, 1536, 64, 0), (384 * 64, 64, 2048, 1408, 1), (1024 * 128, 128, 2048, 768, 1),
+                             (1599 * 8, 8, 4096, 14336, 1), (1600 * 8, 8, 4096, 14336, 0), (1000 * 8, 8, 2048, 192, 0)):
+        assert swapped(R, H, I, E, 1) == want, (R, E, H, I)

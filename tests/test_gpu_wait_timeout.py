@@ -115,3 +115,41 @@ def test_block_scaled_kernels_give_up_the_same_way(counts):
     assert status() == 0
     Hh.assert_close(Hh.to_np64(yp), O.down_mxfp8(h, host["W_down"], ref["offsets"]), "Y_perm (MXFP8) after a timed-out call",
                     rel_fro=Hh.PER_CALL_FROBENIUS)
+
+
+def test_swapped_swiglu_forward_gives_up_the_same_way():
+    """The same for the swapped SwiGLU forward, whose epilogue warps meet in pairs at named barriers: they leave together."""
+    lib = ctypes.CDLL(build.build_library(waittest=True))
+    p = ctypes.c_void_p
+    lib.moe_grouped_gemm_gateup_swiglu.argtypes = [ctypes.POINTER(Dims), p, p, p, p, p, p, p]
+    lib.moe_device_status.argtypes = [ctypes.POINTER(ctypes.c_int)]
+    lib.moe_test_withhold_first_stage.argtypes = [ctypes.c_int]
+
+    def status():
+        out = ctypes.c_int(0)
+        assert lib.moe_device_status(ctypes.byref(out)) == 0
+        return out.value
+
+    cfg, host = Hh.ragged_workload([150, 0, 257, 40], K=1, H=1536, I=192, seed=37)
+    assert lib.moe_test_use_swapped_swiglu(cfg.T, cfg.H, cfg.I, cfg.E, cfg.K)
+    ref = O.layer_fwd(host["X"], host["topk_idx"], host["topk_w"], host["W_gate"], host["W_up"], host["W_down"])
+    x, wg, wu = (Hh.to_dev_bf16(a) for a in (host["X"][np.argsort(host["topk_idx"][:, 0], kind="stable")], host["W_gate"], host["W_up"]))
+    off = torch.from_numpy(ref["offsets"]).cuda()
+    h = torch.zeros((cfg.R, cfg.I), dtype=torch.bfloat16, device="cuda")
+    gu = torch.zeros((cfg.R, 2 * cfg.I), dtype=torch.bfloat16, device="cuda")
+    d = Dims(cfg.T, cfg.H, cfg.I, cfg.E, cfg.K)
+    stream = p(torch.cuda.current_stream().cuda_stream)
+
+    def forward():
+        return lib.moe_grouped_gemm_gateup_swiglu(ctypes.byref(d), *(p(t.data_ptr()) for t in (x, wg, wu, off, h, gu)), stream)
+
+    assert status() == 0
+    assert lib.moe_test_withhold_first_stage(1) == 0
+    assert forward() == 0
+    torch.cuda.synchronize()                            # the kernel returns by itself
+    assert status() == MOE_ERR_TIMEOUT
+    assert lib.moe_test_withhold_first_stage(0) == 0
+    assert forward() == 0
+    torch.cuda.synchronize()
+    assert status() == 0
+    Hh.assert_close(Hh.to_np64(h), ref["H_act"], "H_act after a timed-out call", rel_fro=Hh.PER_CALL_FROBENIUS)
