@@ -117,6 +117,7 @@ def load_library() -> ctypes.CDLL:
             fn.restype = ctypes.c_int
             fn.argtypes = argtypes
         lib.addresses = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in sigs}
+        lib.entries = {name: (address, len(sigs[name]) - 1) for name, address in lib.addresses.items()}
         try:
             from . import _pycall
         except ImportError as e:
@@ -149,7 +150,7 @@ def _call(name: str, d: MoeDims, *args) -> None:
     if not isinstance(d, MoeDims):
         raise TypeError(f"{name}: the first argument must be a MoeDims")
     lib = _lib or load_library()
-    rc = lib.native_call(lib.addresses[name], d, *args, _stream())
+    rc = lib.native_call(lib.entries[name], d, *args, _stream())
     if rc != 0:
         raise MoeError(name, rc, status_string(rc))
 

@@ -31,12 +31,21 @@ static int argument(PyObject *o, uint64_t *out) {
     return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
 }
 
-/* call(address, dims, argument, ...) -> status.  Every parameter of the entry points after `dims` is a pointer, a size_t or an int:
+/* call(entry, dims, argument, ...) -> status.  `entry` is a function's address, or (address, number of parameters after `dims`), which
+ * the arguments are then counted against.  Every parameter of the entry points after `dims` is a pointer, a size_t or an int:
  * an integer register or an eight-byte stack slot each, so a caller of 64-bit integers fits them all (x86-64 and AArch64 ABIs). */
 static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n) {
     (void)self;
-    if (n < 2 || n - 2 > MAX_ARGS) { PyErr_SetString(PyExc_TypeError, "call(address, dims, up to 17 arguments)"); return NULL; }
-    void *fn = PyLong_AsVoidPtr(args[0]);
+    if (n < 2 || n - 2 > MAX_ARGS) { PyErr_SetString(PyExc_TypeError, "call(entry, dims, up to 17 arguments)"); return NULL; }
+    PyObject *address = args[0];
+    if (PyTuple_Check(address)) {
+        if (PyTuple_GET_SIZE(address) != 2) { PyErr_SetString(PyExc_TypeError, "entry must be an address or (address, parameters)"); return NULL; }
+        const Py_ssize_t want = PyLong_AsSsize_t(PyTuple_GET_ITEM(address, 1));
+        if (want == -1 && PyErr_Occurred()) return NULL;
+        if (want != n - 2) { PyErr_Format(PyExc_TypeError, "%zd arguments after dims, the function takes %zd", n - 2, want); return NULL; }
+        address = PyTuple_GET_ITEM(address, 0);
+    }
+    void *fn = PyLong_AsVoidPtr(address);
     if (fn == NULL) {
         if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "null address");
         return NULL;
@@ -77,7 +86,7 @@ static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n) {
     return PyLong_FromLong(rc);
 }
 
-static PyMethodDef methods[] = {{"call", (PyCFunction)(void (*)(void))call, METH_FASTCALL, "call(address, dims, *arguments) -> status"},
+static PyMethodDef methods[] = {{"call", (PyCFunction)(void (*)(void))call, METH_FASTCALL, "call(entry, dims, *arguments) -> status"},
                                 {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", NULL, -1, methods, NULL, NULL, NULL, NULL};
 

@@ -25,8 +25,11 @@ def test_arguments_arrive_in_their_places(B):
     start = -t.data_ptr() % 16
     assert call("moe_permute_bwd", 256, 256, t[start + 8:], None) == 4          # a tensor's address
     assert call("moe_permute", *[256] * 8, 8, 0) == 5                           # on the stack: workspace bytes ...
-    assert call("moe_layer_fwd_bwd_host", *[256] * 14, 8, 0) != 0               # ... and the last argument but one of the longest call
-    assert call("moe_mxfp8_quantize_tokens", 256, 512, 0, -1, 256, 256, 256, 0) != 0   # ints
+    assert call("moe_layer_fwd_bwd_host", *[256] * 14, 8, 0) == 5               # ... and the last argument but one of the longest call
+    # ints, one at a time: row pitch, first column, features (a multiple of 128 that ends inside the pitch)
+    for ints, status in (((512, 0, -1), 3), ((512, 0, 0), 3), ((512, 0, 64), 3), ((512, -8, 256), 2), ((512, 4, 256), 2), ((512, 264, 256), 2),
+                         ((255, 0, 256), 2), ((256, 8, 256), 2), ((-512, 0, 256), 2)):
+        assert call("moe_mxfp8_quantize_tokens", 256, *ints, 256, 256, 256, 0) == status, ints
     d2 = B.MoeDims(256, 200, 512, 8, 2)
     assert lib.native_call(lib.addresses["moe_permute_bwd"], d2, 256, 256, 256, 0) == 3
 
@@ -47,6 +50,20 @@ def test_refused_arguments(B):
         B._call("moe_permute_bwd", ctypes.byref(d), 256, 256, 256)
     with pytest.raises(ValueError):
         lib.native_call(0, d, 256)
+    with pytest.raises(TypeError):
+        lib.native_call((address,), d, 256, 256, 256, 0)
+
+
+def test_arguments_are_counted(B):
+    """A missing or surplus argument would have the callee read what happens to be in a register or on the stack as a pointer."""
+    lib, d = B.load_library(), B.dims(256, 256, 512, 8, 2)
+    for name in lib.addresses:
+        n = len(getattr(lib, name).argtypes) - 1
+        assert lib.entries[name] == (lib.addresses[name], n)
+        for wrong in {0, n - 1, n + 1}:
+            with pytest.raises(TypeError):
+                lib.native_call(lib.entries[name], d, *[None] * wrong)
+        assert lib.native_call(lib.entries[name], d, *[None] * n) != 0, name
 
 
 def test_every_entry_point_fits(B):
