@@ -120,11 +120,35 @@ def load_library() -> ctypes.CDLL:
         lib.entries = {name: (address, len(sigs[name]) - 1) for name, address in lib.addresses.items()}
         try:
             from . import _pycall
-        except ImportError as e:
-            raise ImportError("the binding's helper _pycall is missing: build it with `python -m paper_2606_26453_b200.build`") from e
-        lib.native_call = _pycall.call
+            lib.native_call = _pycall.call
+        except ImportError:   # built for another Python, or without a C compiler
+            lib.native_call = _ctypes_caller(lib)
         _lib = lib
     return _lib
+
+
+def _ctypes_caller(lib):
+    """What csrc/pycall.c does, through ctypes: the same calls and refusals, 2 us more of the host's time each."""
+    functions = {address: getattr(lib, name) for name, address in lib.addresses.items()}
+
+    def argument(o):
+        if o is None or isinstance(o, int):
+            return o or 0
+        if not o.is_contiguous():
+            raise ValueError("tensor must be contiguous")
+        return o.data_ptr()
+
+    def call(entry, d, *args):
+        address, n = entry if isinstance(entry, tuple) and len(entry) == 2 else (entry, None)
+        if address == 0:
+            raise ValueError("null address")
+        fn = functions.get(address) if isinstance(address, int) else None
+        if fn is None or not isinstance(d, MoeDims):
+            raise TypeError("call(entry, dims, arguments)")
+        if len(args) != len(fn.argtypes) - 1 or n not in (None, len(args)):
+            raise TypeError(f"{len(args)} arguments after dims, the function takes {len(fn.argtypes) - 1}")
+        return fn(ctypes.byref(d), *map(argument, args))
+    return call
 
 
 def status_string(status: int) -> str:
@@ -132,7 +156,7 @@ def status_string(status: int) -> str:
 
 
 # A call of the smallest layers takes the device a few microseconds, so what the binding adds counts: the arguments are marshalled in
-# C (csrc/pycall.c: tensors must be contiguous; integers pass as addresses, None as NULL), and the stream handle is asked for
+# C where its helper is built (csrc/pycall.c: tensors must be contiguous; integers pass as addresses, None as NULL), and the stream handle is asked for
 # directly -- building torch's Stream object took 3.2 of the 12 us that such a call once cost the host.
 _cuda_is_initialized = torch.cuda.is_initialized
 _cuda_device = getattr(torch._C, "_cuda_getDevice", None)

@@ -1,6 +1,9 @@
-"""The binding's argument marshalling (csrc/pycall.c), without a device: every entry point rejects these arguments before it launches
-anything."""
+"""The binding's argument marshalling, by csrc/pycall.c and by ctypes where that is not built, without a device: every entry point rejects
+these arguments before it launches anything."""
 import ctypes
+import os
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -8,11 +11,15 @@ import torch
 from paper_2606_26453_b200 import build
 
 
-@pytest.fixture(scope="module")
-def B():
+@pytest.fixture(params=["C", "ctypes"])
+def B(request, monkeypatch):
     build.build_library()
     from paper_2606_26453_b200 import binding
-    binding.load_library()
+    lib = binding.load_library()
+    from paper_2606_26453_b200 import _pycall
+    assert lib.native_call is _pycall.call
+    if request.param == "ctypes":
+        monkeypatch.setattr(lib, "native_call", binding._ctypes_caller(lib))
     return binding
 
 
@@ -69,3 +76,28 @@ def test_arguments_are_counted(B):
 def test_every_entry_point_fits(B):
     lib = B.load_library()
     assert all(len(getattr(lib, name).argtypes) - 1 <= 17 for name in lib.addresses)
+
+
+def test_without_the_helper():
+    """A build for another Python, or none at all: the binding still loads and calls."""
+    code = """
+import sys
+sys.modules["paper_2606_26453_b200._pycall"] = None      # importing it raises ImportError
+from paper_2606_26453_b200 import binding as B
+lib = B.load_library()
+assert lib.native_call.__module__ == B.__name__
+assert lib.native_call(lib.entries["moe_permute_bwd"], B.dims(256, 256, 512, 8, 2), 256, 264, 256, 0) == 4
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=os.path.dirname(build.PKG_DIR))
+
+
+@pytest.mark.parametrize("compiler", ["/nonexistent/cc", "false"])
+def test_library_is_built_without_a_c_compiler(monkeypatch, tmp_path, compiler):
+    monkeypatch.setenv("CC", compiler)
+    monkeypatch.setattr(build, "PYCALL_PATH", str(tmp_path / "_pycall.so"))
+    monkeypatch.setattr(build, "LIB_PATH", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(build, "_compile", lambda path, verbose, waittest: open(path, "w").close())
+    with pytest.warns(RuntimeWarning, match="was not built"):
+        assert os.path.exists(build.build_library())
+    with pytest.raises((OSError, RuntimeError)):
+        build.build_pycall()
