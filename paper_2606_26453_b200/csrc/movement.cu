@@ -686,11 +686,14 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
 // the chip waits for them (32 / 256 threads: 12 x 7744, 7 24.7 / 6.9 us, 515 x 3776, 6 11.6 / 7.1, 41 x 2624, 7 9.9 / 6.8).
 // Rows of 3584 and more fill a block well enough whatever their width, and it keeps more loads in flight (32 / 256 threads: 3593 x
 // 5696, 6 112 / 93 us, without dtopk_w 63 / 53; 11279 x 3648, 5 168 / 160 and 98 / 88).
-constexpr int kLongRowPieces = 3584 / 8;
-static int combine_bwd_lanes_of(int T, int hv) {
+// Without dtopk_w there is no y_perm to read, and from 1600 wide on fewer than 128 threads a token keep too little in flight (2433 x 3200, 7 26 / 33 us with
+// 256 / 32 threads, 4279 x 2304, 3 16.5 / 21.6).
+constexpr int kLongRowPieces = 3584 / 8, kWideRowPieces = 1600 / 8;
+static int combine_bwd_lanes_of(int T, int hv, bool with_dw) {
     if (hv >= kLongRowPieces) return kThreads;
     int best = 32;
     while (best < kThreads && 2 * best <= hv && (long long)T * best < 2ll * 2 * kChipPairs * kThreads) best *= 2;
+    if (best == 32 && !with_dw && hv >= kWideRowPieces) best = 128;
     for (int lanes = 2 * best; lanes <= kThreads && 2 * lanes <= hv; lanes *= 2)
         if ((hv + lanes - 1) / lanes * lanes <= (hv + best - 1) / best * best) best = lanes;
     return best;
@@ -714,7 +717,7 @@ static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint
 template <bool WITH_DW, bool TRIGGER>
 static int combine_bwd_lanes(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w, const int32_t* p2r, uint4* dyp,
                              float* dw, cudaStream_t s) {
-    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8);
+    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8, WITH_DW);
     if (lanes == 32) return combine_bwd_dispatch<WITH_DW, TRIGGER, 32>(d, dy, yp, w, p2r, dyp, dw, s);
     if (lanes == 64) return combine_bwd_dispatch<WITH_DW, TRIGGER, 64>(d, dy, yp, w, p2r, dyp, dw, s);
     if (lanes == 128) return combine_bwd_dispatch<WITH_DW, TRIGGER, 128>(d, dy, yp, w, p2r, dyp, dw, s);
@@ -726,7 +729,7 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    const int tokens = kThreads / combine_bwd_lanes_of(d.T, d.H / 8);   // per block
+    const int tokens = kThreads / combine_bwd_lanes_of(d.T, d.H / 8, dtopk_w != nullptr);   // per block
     const bool trigger = d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
     if (dtopk_w != nullptr)
         return trigger ? combine_bwd_lanes<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
@@ -737,7 +740,7 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
 
 #ifdef MOE_TEST_HOOKS
 // Test-only build: threads per token of a combine backward.
-extern "C" int moe_test_combine_bwd_lanes(int T, int H) { return combine_bwd_lanes_of(T, H / 8); }
+extern "C" int moe_test_combine_bwd_lanes(int T, int H, int with_dw) { return combine_bwd_lanes_of(T, H / 8, with_dw != 0); }
 // ... and the kernels that a route-permute launches.
 extern "C" int moe_test_permute_launches(int T, int K, int E) {
     const PermuteSums sums = permute_sums({T, 64, 64, E, K});

@@ -27,7 +27,9 @@ def test_threads_per_token_of_the_combine_backward():
     for T, H, want in ((20000, 256, 32), (20000, 512, 32), (20000, 832, 32), (20000, 1024, 64), (10000, 1280, 32), (16384, 2048, 128), (8192, 4096, 256),
                        (14442, 2880, 128), (27, 2304, 256), (12, 7744, 256), (515, 3776, 256), (41, 2624, 256), (3593, 5696, 256), (4736, 1152, 32),
                        (2367, 1152, 64), (1, 64, 32), (1, 512, 64), (2368, 3072, 128), (2368, 3328, 32), (2367, 3328, 64), (2368, 3584, 256)):
-        assert lanes(T, H) == want, (T, H, lanes(T, H))
+        assert lanes(T, H, 1) == want, (T, H, lanes(T, H, 1))
+    for T, H, want in ((20000, 1024, 64), (20000, 1536, 64), (20000, 1600, 128), (4279, 2304, 128), (2433, 3200, 128), (27, 2304, 256), (8192, 4096, 256)):
+        assert lanes(T, H, 0) == want, (T, H, lanes(T, H, 0))   # without dtopk_w
 
 
 def test_launches_of_a_permute():
