@@ -704,24 +704,28 @@ static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint
     const int hv = d.H / 8;
     constexpr int TOKENS = kThreads / LANES;
     const unsigned blocks = (unsigned)((d.T + TOKENS - 1) / TOKENS);
+    // (narrowest rows: 8 pieces; from K = 8 on a block of them moves kTriggerPieces, and the form without a trigger is never asked for)
 #define MOE_CB_CASE(KT) \
-    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW, TRIGGER, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+    case KT: return launch_streaming(combine_bwd_kernel<KT, WITH_DW, TRIGGER || (2 * KT + 1) * 8 * TOKENS >= kTriggerPieces, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     switch (d.K) {
         MOE_CB_CASE(1) MOE_CB_CASE(2) MOE_CB_CASE(3) MOE_CB_CASE(4) MOE_CB_CASE(5) MOE_CB_CASE(6) MOE_CB_CASE(7)
         MOE_CB_CASE(8)
         default:
-            return launch_streaming(combine_bwd_kernel<0, WITH_DW, TRIGGER, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
+            return launch_streaming(combine_bwd_kernel<0, WITH_DW, true, LANES>, blocks, s, dy, yp, w, p2r, dyp, dw, d.T, hv, d.K);
     }
 #undef MOE_CB_CASE
 }
-template <bool WITH_DW, bool TRIGGER>
+template <bool WITH_DW>
 static int combine_bwd_lanes(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w, const int32_t* p2r, uint4* dyp,
                              float* dw, cudaStream_t s) {
-    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8, WITH_DW);
-    if (lanes == 32) return combine_bwd_dispatch<WITH_DW, TRIGGER, 32>(d, dy, yp, w, p2r, dyp, dw, s);
-    if (lanes == 64) return combine_bwd_dispatch<WITH_DW, TRIGGER, 64>(d, dy, yp, w, p2r, dyp, dw, s);
-    if (lanes == 128) return combine_bwd_dispatch<WITH_DW, TRIGGER, 128>(d, dy, yp, w, p2r, dyp, dw, s);
-    return combine_bwd_dispatch<WITH_DW, TRIGGER, 256>(d, dy, yp, w, p2r, dyp, dw, s);
+    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8, WITH_DW), tokens = kThreads / lanes;   // per block
+    // (with more than 32 threads per token the grid is small or the rows are long, always)
+    const bool trigger = lanes > 32 || d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
+    if (!trigger) return combine_bwd_dispatch<WITH_DW, false, 32>(d, dy, yp, w, p2r, dyp, dw, s);
+    if (lanes == 32) return combine_bwd_dispatch<WITH_DW, true, 32>(d, dy, yp, w, p2r, dyp, dw, s);
+    if (lanes == 64) return combine_bwd_dispatch<WITH_DW, true, 64>(d, dy, yp, w, p2r, dyp, dw, s);
+    if (lanes == 128) return combine_bwd_dispatch<WITH_DW, true, 128>(d, dy, yp, w, p2r, dyp, dw, s);
+    return combine_bwd_dispatch<WITH_DW, true, 256>(d, dy, yp, w, p2r, dyp, dw, s);
 }
 
 int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, const float* topk_w,
@@ -729,13 +733,8 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
     const uint4* a = reinterpret_cast<const uint4*>(dy);
     const uint4* b = reinterpret_cast<const uint4*>(y_perm);
     uint4* o = reinterpret_cast<uint4*>(dy_perm);
-    const int tokens = kThreads / combine_bwd_lanes_of(d.T, d.H / 8, dtopk_w != nullptr);   // per block
-    const bool trigger = d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
-    if (dtopk_w != nullptr)
-        return trigger ? combine_bwd_lanes<true, true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
-                       : combine_bwd_lanes<true, false>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s);
-    return trigger ? combine_bwd_lanes<false, true>(d, a, b, topk_w, pair_to_row, o, nullptr, s)
-                   : combine_bwd_lanes<false, false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
+    return dtopk_w != nullptr ? combine_bwd_lanes<true>(d, a, b, topk_w, pair_to_row, o, dtopk_w, s)
+                              : combine_bwd_lanes<false>(d, a, b, topk_w, pair_to_row, o, nullptr, s);
 }
 
 #ifdef MOE_TEST_HOOKS

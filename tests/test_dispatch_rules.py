@@ -30,6 +30,12 @@ def test_threads_per_token_of_the_combine_backward():
         assert lanes(T, H, 1) == want, (T, H, lanes(T, H, 1))
     for T, H, want in ((20000, 1024, 64), (20000, 1536, 64), (20000, 1600, 128), (4279, 2304, 128), (2433, 3200, 128), (27, 2304, 256), (8192, 4096, 256)):
         assert lanes(T, H, 0) == want, (T, H, lanes(T, H, 0))   # without dtopk_w
+    # the form that leaves its successor to the end exists for 32 threads per token only: others are small grids or blocks of 1024 pieces and more
+    for T in (*range(1, 3000, 61), 592, 593, 1184, 1185, 2367, 2368, 4735, 4736, 100000):
+        for H in range(64, 8192, 64):
+            for with_dw in (0, 1):
+                n = lanes(T, H, with_dw)
+                assert n == 32 or T <= 592 * (256 // n) or 3 * (H // 8) * (256 // n) >= 1024, (T, H, with_dw, n)
 
 
 def test_launches_of_a_permute():
