@@ -11,7 +11,7 @@ def test_mxfp8_gemm():
     lib = ctypes.CDLL(build.build_library(waittest=True))
     lib.moe_test_mx_form.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 3
     forms = {name: lib.moe_test_mx_form(sum(c), len(c), H, I) for name, (H, I, c) in CASES.items()}
-    assert forms == {"one_feature_block": 0, "last_tile_half_wide": 1, "low_box_edges": 1, "empty_and_last": 0, "many_slices": 1,
+    assert forms == {"one_tile_half_wide": 0, "row_edges": 2, "last_tile_half_wide": 1, "low_box_edges": 1, "empty_and_last": 0, "many_slices": 1,
                      "rows_m_edges": 2, "rows_m_halves": 2, "rows_m_empty": 2, "rows_m_many_slices": 2, "rows_m_narrow_last": 2, "96_rows": 1,
                      "96_rows_too_few_tiles": 0, "96_rows_short": 0, "96_rows_uneven": 0}
     # sizes at which each was found the better one: many rows of 128 and of 384 features, row tiles of 208 that are just exceeded, few rows

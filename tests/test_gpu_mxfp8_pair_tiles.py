@@ -12,7 +12,8 @@ from tests import helpers as Hh
 pytestmark = pytest.mark.gpu
 
 CASES = {   # output features, contraction, rows of each expert
-    "one_feature_block": (128, 128, [256]),                        # a single CTA's
+    "one_tile_half_wide": (128, 128, [256]),                       # one block of features: a single CTA's
+    "row_edges": (384, 256, [207, 208, 209, 415, 416, 417]),       # 256 rows a tile; one and two row tiles
     # 256 features a tile:
     "last_tile_half_wide": (640, 256, [207, 208, 209, 415, 416, 417]),   # the second CTA has no features; one, two and three row tiles
     "low_box_edges": (256, 640, [128, 129, 1, 16, 17, 1040, 624]), # 64 rows per CTA and more; five tiles of 208

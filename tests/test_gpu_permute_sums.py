@@ -13,9 +13,19 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,K,E", [(1, 1, 1), (5, 3, 1024), (2047, 1, 3), (2048, 1, 128), (2049, 1, 128), (64, 32, 40), (65, 32, 40), (682, 3, 7),
-                                   (683, 3, 7), (14336, 1, 128), (14337, 1, 128), (4099, 8, 1000), (1024, 10, 300), (33000, 1, 64), (8192, 1, 183), (8192, 1, 184), (36485, 7, 8)])
+                                   (683, 3, 7), (14336, 1, 128), (14337, 1, 128), (4099, 8, 1000), (1024, 10, 300), (33000, 1, 64)])
 @pytest.mark.parametrize("invalid", [False, True])
-def test_both_sides_of_the_lines(T, K, E, invalid):
+def test_few_pairs(T, K, E, invalid):
+    check(T, K, E, invalid)
+
+
+@pytest.mark.parametrize("T,K,E", [(8192, 1, 183), (8192, 1, 184), (36485, 7, 8)])
+@pytest.mark.parametrize("invalid", [False, True])
+def test_many_pairs(T, K, E, invalid):
+    check(T, K, E, invalid)
+
+
+def check(T, K, E, invalid):
     from paper_2606_26453_b200 import binding as B
     H, R, guard = 192, T * K, 16
     rng = np.random.default_rng(R + E)
