@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kThreads) permute_hist_kernel(const int32_t* _
     int32_t* hist = smem_i;   // [E]
     if (!grid_dependency_wait_tested()) return;
     // rank_rows reads the routing indices and token rows before its own wait: it may start from here on, not earlier
+    release_to_dependents();
     grid_launch_dependents();
     for (int e = threadIdx.x; e < E; e += kThreads) hist[e] = 0;
     __syncthreads();
@@ -144,6 +145,7 @@ struct RankRowsSmem {
 __global__ void __launch_bounds__(kThreads) permute_scan_kernel(int32_t* __restrict__ ws, int E, int n_chunks, int32_t* __restrict__ counts) {
     const int e = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (!grid_dependency_wait_tested()) return;
+    release_to_dependents();   // (as the histogram kernel)
     grid_launch_dependents();
     if (e >= E) return;
     int run = 0;
@@ -204,6 +206,8 @@ __global__ void __launch_bounds__(kPermThreads) permute_rank_rows_kernel(
     if (SUMS == kCountAll) {   // the routing indices and the rows may come from the kernel before
         if (!grid_dependency_wait_tested()) return;
         grid_launch_dependents();
+    } else if (!acquire_unwaited()) {   // they come from before the histogram kernel, which has waited for them and fenced
+        return;
     }
     // ---- (1) nothing here needs the histogram kernel's output ----
     auto issue_load = [&](int u) {   // lane 0 of warp 0

@@ -25,6 +25,33 @@ def test_many_pairs(T, K, E, invalid):
     check(T, K, E, invalid)
 
 
+@pytest.mark.parametrize("T,K,E", [(3000, 2, 40), (32768, 8, 128)])   # two launches, three
+def test_inputs_that_change_from_call_to_call(T, K, E):
+    """Two routings and inputs by turns through the same buffers, nothing waited for in between: the ranking kernel, which reads both
+    before it waits for the kernel before it, sees those of its own call."""
+    from paper_2606_26453_b200 import binding as B
+    H, rng = 64, np.random.default_rng(T)
+    idx = [torch.from_numpy(rng.integers(0, n, size=(T, K)).astype(np.int32)).cuda() for n in (E, E // 2)]
+    X = [Hh.to_dev_bf16(W.round_to_bf16(rng.standard_normal((T, H), dtype=np.float32))) for _ in idx]
+    d, i32 = B.dims(T, H, 64, E, K), dict(dtype=torch.int32, device="cuda")
+    ws = torch.empty(B.moe_permute_workspace_bytes(d), dtype=torch.uint8, device="cuda")
+    xp, counts, offsets, r2p, p2r = torch.empty((T * K, H), dtype=torch.bfloat16, device="cuda"), *(torch.empty(n, **i32) for n in (E, E + 1, T * K, T * K))
+    live_x, live_idx, got = torch.empty_like(X[0]), torch.empty_like(idx[0]), []
+    for i in range(40):
+        live_x.copy_(X[i % 2])
+        live_idx.copy_(idx[i % 2])
+        B.moe_permute(d, live_x, live_idx, xp, counts, offsets, r2p, p2r, ws)
+        got.append([t.clone() for t in (xp, r2p, offsets)])
+    torch.cuda.synchronize()
+    assert B.moe_device_status() == 0
+    for i, (xp_i, r2p_i, offsets_i) in enumerate(got):
+        flat = idx[i % 2].flatten().long()
+        order = torch.argsort(flat, stable=True)
+        assert torch.equal(r2p_i.long(), order), i
+        assert torch.equal(offsets_i[1:].long(), torch.bincount(flat, minlength=E).cumsum(0)), i
+        assert torch.equal(xp_i, X[i % 2][order // K]), i
+
+
 def check(T, K, E, invalid):
     from paper_2606_26453_b200 import binding as B
     H, R, guard = 192, T * K, 16
