@@ -236,7 +236,7 @@ int moe_router_topk_bwd(const moe_dims_t* dims, const int32_t* topk_idx, const f
  *                              slice kt of row r are bytes scales[(kt*R + r)*4 + 0..3].
  *   moe_mxfp8_quantize_w_down  w_down [E,I,H] bf16 -> codes_t [E,H,I] bytes (transposed: contraction contiguous);
  *                              scales: moe_mxfp8_w_down_scale_bytes(dims) bytes holding every scale twice, in
- *                              groups of 128 features (what the GEMMs read) and in groups of 208:
+ *                              groups of 128 features and of 208 (a GEMM reads one of them):
  *                              first [E][H/128][I/128][512]: the scale of feature h, block b of 32 along I, is
  *                              byte (h%32)*16 + ((h%128)/32)*4 + b%4 of the 512-byte group (e, h/128, b/4);
  *                              then [E][ceil(H/208)][I/128][1024]: with h' = h%208 the same scale is byte

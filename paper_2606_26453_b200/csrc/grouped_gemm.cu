@@ -1172,17 +1172,23 @@ bool rows_per_expert_below(const moe_dims_t& d, long long rows) { return (long l
 // 4096 x 14336 14.2 against 10.3 GB -- and under the power cap it is 7 to 22 % slower.)  The line holds for Zipf and
 // Dirichlet loads with the same averages: at 768 of them (64 experts, 2048 x 1408) 285 / 308 / 552 against 269 / 290 / 521 us
 // under the first, 1500 (16 experts, 4096 x 4096) 697 / 692 / 1515 against 689 / 694 / 1437 us under the second.
-// A contraction of fewer than 512 elements is over before the swapped form's transposed epilogue, and the line lies at 512
-// rows: down dgrad of 16 experts to 8192 features, fixed against swapped, contraction 256 at 768 / 1100 / 1500 rows
-// 75 / 104 / 130 against 85 / 115 / 143 us, 384 at 768 / 1500 rows 98 / 162 against 106 / 174 us; 512 at 768 / 1100 rows
-// 113 / 157 against 120 / 153 us and, of 32 experts to 2048 features, 60 / 83 against 62 / 84 us.
+// For contractions of fewer than 512 elements the line lies at 512 rows: drawn when the swapped form stored its blocks two bytes at a time,
+// which outlasted them (contraction 256 at 768 / 1100 / 1500 rows 75 / 104 / 130 against 85 / 115 / 143 us).  With the fragment epilogue it
+// would lie higher: down dgrad of 16 experts to 8192 features, even loads, each form alone, fixed against swapped, contraction 256 at 512 /
+// 768 / 1100 / 1500 rows 57 / 78 / 110 / 136 against 53 / 75 / 102 / 132 us, 384 73 / 99 / 137 / 170 against 66 / 93 / 127 / 165 us.
+// And the present figures above it: 32 experts of 2048 x 1408 at 768 / 1024 / 1536 / 2048 rows 0.95-0.99 of the fixed form's time in all
+// three, 16 of 4096 x 4096 0.96-1.00 at 768 and 1024, 1.01 at 1536 and 2048 (gate/up dgrad 1.04 and 1.07); 8 of 4096 x 14336 down
+// 1.01 / 0.97 / 1.00 / 1.10, down dgrad 0.95 / 0.94 / 0.98 / 1.00, but gate/up dgrad, a contraction of 28672, 1.16 / 1.07 / 1.18 / 1.25:
+// so long a contraction would bear a lower line.
 bool use_swapped(const moe_dims_t& d, int contraction) { return rows_per_expert_below(d, contraction < 512 ? 512 : 1600); }
-// The down dgrad with the SwiGLU backward in its epilogue: there the swapped form also transposes the two blocks it fetches,
-// and that outlasts contractions of 2048, so the line lies at 512 rows.  Fixed against swapped at 512 / 768 / 1024 / 1536 rows:
-//   64 experts, 2048 x 1408   249 / 312 / 443 /  621 against 240 / 343 / 450 /  639 us
-//   16 experts, 4096 x 4096   324 / 456 / 564 /  776 against 304 / 411 / 520 /  756 us
-//   8 experts, 4096 x 14336   588 / 794 / 946 / 1099 against 502 / 712 / 885 / 1074 us
-// (a contraction of 4096 would bear a higher line).
+// The down dgrad with the SwiGLU backward in its epilogue: there the swapped form also transposes the two blocks it fetches.  The line
+// at 512 rows was drawn when that took two bytes at a time and outlasted contractions of 2048 (64 experts of 2048 x 1408 at 768 / 1536
+// rows 312 / 621 against 343 / 639 us).  With fragments the swapped form is the faster one above it as well, even loads, each alone,
+// fixed against swapped at 512 / 768 / 1024 / 1536 / 2048 rows:
+//   64 experts, 2048 x 1408   261 / 359 / 457 /  633 /  823 against 247 / 340 / 445 /  623 /  816 us
+//   16 experts, 4096 x 4096   312 / 429 / 530 /  757 /  985 against 286 / 396 / 508 /  729 /  967 us
+//   8 experts, 4096 x 14336   526 / 726 / 920 / 1312 / 1682 against 487 / 681 / 869 / 1253 / 1649 us
+// so a line at 1600 as above would gain 1-8 % between (not taken up here).
 bool use_swapped_fused(const moe_dims_t& d) { return rows_per_expert_below(d, 512); }
 // The SwiGLU forward swapped (gate and up of 128 features x up to 256 rows per tile), below 1600 rows like the other swapped forms.
 // Its epilogue passes 4 KB per block of 32 x 32 values through shared memory, beside the operands' traffic, and that outlasts short
