@@ -35,7 +35,7 @@ inline double tile_rounds(long long R, int E, int tile_rows, long long feature_t
 // The rules that keep this equivalent to plain stream order:
 //   - grid_dependency_wait() comes before a kernel's first access to global memory.  It returns once the kernels before have
 //     completed and their writes are visible.  (rank_rows of the route-permute reads its INPUTS earlier: its predecessor, the
-//     histogram or the scan kernel, lets it start only after its own wait, with the fences of the next rule but one.)
+//     histogram or the scan kernel, lets it start only after its own wait and a fence, and it reads them past the L1; see the next rule but one.)
 //   - grid_launch_dependents() comes after grid_dependency_wait(), so no more than one kernel is ever ahead of its turn and a
 //     kernel that has started knows everything before its immediate predecessor to be complete.
 //   - A weight gradient that a call launches right behind a data gradient on the same inputs does not depend on it.  Behind a
@@ -68,11 +68,9 @@ __device__ __forceinline__ bool grid_dependency_wait_tested() {
 }
 // The two sides of a dependent that reads without waiting (see above).
 __device__ __forceinline__ void release_to_dependents() { __threadfence(); }
-__device__ __forceinline__ bool acquire_unwaited() {   // (a result to test, for read-only loads: see above)
-    uint32_t done;
+__device__ __forceinline__ void acquire_unwaited() {
     __threadfence();
-    asm volatile("fence.proxy.async.global; mov.u32 %0, 1;" : "=r"(done) : : "memory");
-    return done != 0;
+    asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
