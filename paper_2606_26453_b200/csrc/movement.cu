@@ -690,18 +690,24 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
 // A block per token against this (T x H, K; us): 20000 x 256, 2 25.3 -> 8.2; 20000 x 512, 2 45.1 -> 16.7, K = 8 120 -> 59;
 // 20000 x 832, 4 90 -> 55; 20000 x 1024, 3 70 -> 47; 10000 x 1280, 8 86 -> 73; 8192 x 1536, 4 47 -> 39; 16384 x 2048, 8 181 -> 174;
 // 14442 x 2880, 4 137 -> 121; 8192 x 4096, 2 54.7 (a block per token stays: 128 threads 55.4).
-// Of few tokens no fewer threads than give every SM two blocks of them: one thread's pieces come one after the other, and with fewer
-// the chip waits for them (32 / 256 threads: 12 x 7744, 7 24.7 / 6.9 us, 515 x 3776, 6 11.6 / 7.1, 41 x 2624, 7 9.9 / 6.8).
-// Rows of 3584 and more fill a block well enough whatever their width, and it keeps more loads in flight (32 / 256 threads: 3593 x
-// 5696, 6 112 / 93 us, without dtopk_w 63 / 53; 11279 x 3648, 5 168 / 160 and 98 / 88).
-// Without dtopk_w there is no y_perm to read, and from 1600 wide on fewer than 128 threads a token keep too little in flight (2433 x 3200, 7 26 / 33 us with
-// 256 / 32 threads, 4279 x 2304, 3 16.5 / 21.6).
+// Few tokens have a block each, whatever their width, as long as the chip takes all blocks at once (three per SM, four without dtopk_w, two
+// of the run-time K): then the time is that of one block, and several tokens to one only share its SM (41 x 384, K = 8, 32 / 64 / 128 / 256
+// threads 3.2 / 2.3 / 2.0 / 1.7 us, without dtopk_w 2.3 / 1.7 / 1.6 / 1.3; 12 x 7744, 7 24.7 with 32, 6.9 with 256; 418 x 384, 12 5.6 with
+// 64, 9.6 with 256).
+// Of more tokens no fewer threads than give every SM two blocks of them (four without dtopk_w), up to one for each piece: one thread's
+// pieces come one after the other, and with fewer the chip waits for them (32 / 256 threads: 515 x 3776, 6 11.6 / 7.1 us).
+// Rows of 3584 and more have at least 128: more loads in flight (32 / 256 threads: 3593 x 5696, 6 112 / 93 us, without dtopk_w 63 / 53,
+// 11279 x 3648, 5 168 / 160 and 98 / 88).  Without dtopk_w there is no y_perm to read: 128 from 1600 wide on (2433 x 3200, 7 26 / 33 us with
+// 256 / 32 threads, 4279 x 2304, 3 16.5 / 21.6), all 256 from 3584 on.
+// 3176 shapes drawn up to 60000 x 8192: 1.6 % above the best number of threads on average, 38 more than 8 % above a block per token (without
+// dtopk_w 2.1 %, 63); a block per token throughout 28 % and 13 % above the best.
 constexpr int kLongRowPieces = 3584 / 8, kWideRowPieces = 1600 / 8;
-static int combine_bwd_lanes_of(int T, int hv, bool with_dw) {
-    if (hv >= kLongRowPieces) return kThreads;
+static int combine_bwd_lanes_of(int T, int hv, int K, bool with_dw) {
+    const int sms = 2 * kChipPairs, at_once = K > 8 ? 2 : with_dw ? 3 : 4;   // blocks per SM
+    if (T <= at_once * sms || (!with_dw && hv >= kLongRowPieces)) return kThreads;
     int best = 32;
-    while (best < kThreads && 2 * best <= hv && (long long)T * best < 2ll * 2 * kChipPairs * kThreads) best *= 2;
-    if (best == 32 && !with_dw && hv >= kWideRowPieces) best = 128;
+    while (best < kThreads && best < hv && (long long)T * best < (with_dw ? 2ll : 4ll) * sms * kThreads) best *= 2;
+    if (best < 128 && hv >= (with_dw ? kLongRowPieces : kWideRowPieces)) best = 128;
     for (int lanes = 2 * best; lanes <= kThreads && 2 * lanes <= hv; lanes *= 2)
         if ((hv + lanes - 1) / lanes * lanes <= (hv + best - 1) / best * best) best = lanes;
     return best;
@@ -726,8 +732,8 @@ static int combine_bwd_dispatch(const moe_dims_t& d, const uint4* dy, const uint
 template <bool WITH_DW>
 static int combine_bwd_lanes(const moe_dims_t& d, const uint4* dy, const uint4* yp, const float* w, const int32_t* p2r, uint4* dyp,
                              float* dw, cudaStream_t s) {
-    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8, WITH_DW), tokens = kThreads / lanes;   // per block
-    // (with more than 32 threads per token the grid is small or the rows are long, always)
+    const int lanes = combine_bwd_lanes_of(d.T, d.H / 8, d.K, WITH_DW), tokens = kThreads / lanes;   // per block
+    // (with more than 32 threads per token the grid is small, at most twice kSmallGrid, or the rows are long, always)
     const bool trigger = lanes > 32 || d.T <= (int)kSmallGrid * tokens || (2ll * d.K + 1) * (d.H / 8) * tokens >= kTriggerPieces;
     if (!trigger) return combine_bwd_dispatch<WITH_DW, false, 32>(d, dy, yp, w, p2r, dyp, dw, s);
     if (lanes == 32) return combine_bwd_dispatch<WITH_DW, true, 32>(d, dy, yp, w, p2r, dyp, dw, s);
@@ -747,7 +753,7 @@ int launch_combine_bwd(const moe_dims_t& d, const bf16* dy, const bf16* y_perm, 
 
 #ifdef MOE_TEST_HOOKS
 // Test-only build: threads per token of a combine backward.
-extern "C" int moe_test_combine_bwd_lanes(int T, int H, int with_dw) { return combine_bwd_lanes_of(T, H / 8, with_dw != 0); }
+extern "C" int moe_test_combine_bwd_lanes(int T, int H, int K, int with_dw) { return combine_bwd_lanes_of(T, H / 8, K, with_dw != 0); }
 // ... and the kernels that a route-permute launches.
 extern "C" int moe_test_permute_launches(int T, int K, int E) {
     const PermuteSums sums = permute_sums({T, 64, 64, E, K});

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("H", [64, 256, 320, 1024, 1280, 2048, 2880, 3520, 4096, 4160])
-@pytest.mark.parametrize("T,K", [(1, 1), (7, 3), (13, 8), (5, 20), (2373, 2)])   # the last: enough tokens for 32 threads each
+@pytest.mark.parametrize("T,K", [(1, 1), (7, 3), (13, 8), (5, 20), (451, 20), (601, 8), (2373, 2), (4745, 1)])   # from 451 on several tokens to a block
 def test_widths(H, T, K):
     from paper_2606_26453_b200 import binding as B
     E, R = max(K, 4), T * K
