@@ -171,7 +171,7 @@ int moe_grouped_gemm_down_dgrad(const moe_dims_t* dims, const void* dy_perm, con
     const void* const req[] = {dy_perm, w_down, offsets, dh_act};
     const void* const opt[] = {nullptr};
     MOE_VALIDATE(dims, req, opt);
-    return launch_down_dgrad(*dims, cb(dy_perm), cb(w_down), offsets, mb(dh_act), st(stream));
+    return launch_down_dgrad(*dims, cb(dy_perm), cb(w_down), offsets, mb(dh_act), false, st(stream));
 }
 
 int moe_grouped_gemm_down_dgrad_swiglu_bwd(const moe_dims_t* dims, const void* dy_perm, const void* w_down,
@@ -193,13 +193,13 @@ int moe_grouped_gemm_down_wgrad(const moe_dims_t* dims, const void* h_act, const
 
 int moe_grouped_gemm_down_bwd(const moe_dims_t* dims, const void* dy_perm, const void* h_act, const void* w_down,
                               const int32_t* offsets, void* dh_act, void* dw_down, moe_stream_t stream) {
-    int s = moe_grouped_gemm_down_dgrad(dims, dy_perm, w_down, offsets, dh_act, stream);
-    if (s != MOE_OK) return s;
-    const void* const req[] = {h_act, dy_perm, offsets, dw_down};
+    const void* const req[] = {dy_perm, w_down, offsets, dh_act, h_act, dw_down};
     const void* const opt[] = {nullptr};
     MOE_VALIDATE(dims, req, opt);
     const size_t rows = (size_t)dims->T * dims->K, ri = rows * dims->I * 2, rh = rows * dims->H * 2, w = (size_t)dims->E * dims->H * dims->I * 2;
     const bool beside = leaves_sms_free(rows, dims->E, dims->I) && apart(dw_down, w, w_down, w) && apart(dw_down, w, dy_perm, rh) && apart(dw_down, w, dh_act, ri) && apart(dh_act, ri, h_act, ri);
+    const int s = launch_down_dgrad(*dims, cb(dy_perm), cb(w_down), offsets, mb(dh_act), beside, st(stream));
+    if (s != MOE_OK) return s;
     return launch_down_wgrad(*dims, cb(h_act), cb(dy_perm), offsets, mb(dw_down), beside, st(stream));
 }
 
@@ -216,7 +216,7 @@ int moe_grouped_gemm_gateup_dgrad(const moe_dims_t* dims, const void* dgu, const
     const void* const req[] = {dgu, w_gate, w_up, offsets, dx_perm};
     const void* const opt[] = {nullptr};
     MOE_VALIDATE(dims, req, opt);
-    return launch_gateup_dgrad(*dims, cb(dgu), cb(w_gate), cb(w_up), offsets, mb(dx_perm), st(stream));
+    return launch_gateup_dgrad(*dims, cb(dgu), cb(w_gate), cb(w_up), offsets, mb(dx_perm), false, st(stream));
 }
 
 int moe_grouped_gemm_gateup_wgrad(const moe_dims_t* dims, const void* x_perm, const void* dgu,
@@ -231,17 +231,17 @@ int moe_grouped_gemm_gateup_swiglu_bwd(const moe_dims_t* dims, const void* dh_ac
                                        const void* x_perm, const void* w_gate, const void* w_up,
                                        const int32_t* offsets, void* dgu, void* dx_perm, void* dw_gate,
                                        void* dw_up, moe_stream_t stream) {
-    int s = moe_swiglu_bwd(dims, dh_act, gu_saved, dgu, stream);
-    if (s != MOE_OK) return s;
-    s = moe_grouped_gemm_gateup_dgrad(dims, dgu, w_gate, w_up, offsets, dx_perm, stream);
-    if (s != MOE_OK) return s;
-    const void* const req[] = {x_perm, dgu, offsets, dw_gate, dw_up};
+    const void* const req[] = {dh_act, gu_saved, dgu, w_gate, w_up, offsets, dx_perm, x_perm, dw_gate, dw_up};
     const void* const opt[] = {nullptr};
     MOE_VALIDATE(dims, req, opt);
     const size_t rows = (size_t)dims->T * dims->K, ri2 = rows * dims->I * 4, rh = rows * dims->H * 2, w = (size_t)dims->E * dims->H * dims->I * 2;
     bool beside = leaves_sms_free(rows, dims->E, dims->H) && apart(dx_perm, rh, x_perm, rh);
     for (const void* dw : {dw_gate, dw_up})
         beside = beside && apart(dw, w, w_gate, w) && apart(dw, w, w_up, w) && apart(dw, w, dgu, ri2) && apart(dw, w, dx_perm, rh);
+    int s = moe_swiglu_bwd(dims, dh_act, gu_saved, dgu, stream);
+    if (s != MOE_OK) return s;
+    s = launch_gateup_dgrad(*dims, cb(dgu), cb(w_gate), cb(w_up), offsets, mb(dx_perm), beside, st(stream));
+    if (s != MOE_OK) return s;
     return launch_gateup_wgrad(*dims, cb(x_perm), cb(dgu), offsets, mb(dw_gate), mb(dw_up), beside, st(stream));
 }
 

@@ -42,7 +42,7 @@ inline double tile_rounds(long long R, int E, int tile_rows, long long feature_t
 //     short one it runs beside it: no wait at its start (that it has started means that all before the data gradient is complete), the wait before
 //     it lets ITS successor start, so that a kernel which has waited for it has waited for both.  Only a wait is documented to make
 //     earlier kernels' writes visible, and this form reads without one.  What it reads was written before the data gradient; that
-//     kernel's threads have waited for those writes and fence (release_to_dependents) before any of them can trigger, so the writes
+//     kernel's threads (it is told) have waited for those writes and fence (release_to_dependents) before any of them can trigger, so the writes
 //     are performed at the scope of the device before the weight gradient can start, and its threads fence (acquire_unwaited) before they
 //     read: nothing older comes out of an L1, by loads or by bulk copies.
 //   - The GEMMs call it at the end of each warp's role.  One thread's call counts for its CTA, so the row-ragged bf16 kinds,
@@ -136,13 +136,13 @@ int launch_gateup_fwd(const moe_dims_t& d, const bf16* x_perm, const bf16* w_gat
 int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, const int32_t* offsets,
                     bf16* y_perm, cudaStream_t s);
 int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const int32_t* offsets,
-                      bf16* dh_act, cudaStream_t s);
+                      bf16* dh_act, bool beside, cudaStream_t s);
 int launch_down_wgrad(const moe_dims_t& d, const bf16* h_act, const bf16* dy_perm, const int32_t* offsets,
-                      bf16* dw_down, bool beside, cudaStream_t s);   // beside: right behind launch_down_dgrad, see above
+                      bf16* dw_down, bool beside, cudaStream_t s);   // beside: this right behind launch_down_dgrad, both with the same value; see above
 int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const bf16* gu,
                                  const int32_t* offsets, bf16* dgu, cudaStream_t s);
 int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate, const bf16* w_up,
-                        const int32_t* offsets, bf16* dx_perm, cudaStream_t s);
+                        const int32_t* offsets, bf16* dx_perm, bool beside, cudaStream_t s);
 int launch_gateup_wgrad(const moe_dims_t& d, const bf16* x_perm, const bf16* dgu, const int32_t* offsets,
                         bf16* dw_gate, bf16* dw_up, bool beside, cudaStream_t s);
 

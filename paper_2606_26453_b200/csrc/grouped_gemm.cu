@@ -120,7 +120,8 @@ struct Params {
     bf16* out1;
     bf16* gu;            // FWD_SWIGLU: [R, 2I] or null
     int I;               // FWD_SWIGLU
-    int beside;          // WGRAD: nothing here depends on the kernel right before, a data gradient of the same call (see common.cuh)
+    int beside;          // WGRAD: nothing here depends on the kernel right before, a data gradient of the same call (see common.cuh);
+                         // DGRAD, DGRAD_T: such a weight gradient comes next
 };
 
 struct SharedCtl {
@@ -457,7 +458,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // everything above may run while the kernel before is still finishing; the schedule is derived from its output
     if (!wgrad(KIND) || !p.beside) grid_dependency_wait(); else acquire_unwaited();
     for (int e = threadIdx.x; e <= p.E; e += NUM_THREADS) ctl->offs[e] = p.offsets[e];
-    if (KIND == DGRAD || KIND == DGRAD_T) release_to_dependents();   // a weight gradient may run beside this kernel
+    if ((KIND == DGRAD || KIND == DGRAD_T) && p.beside) release_to_dependents();   // a weight gradient will run beside this kernel
     __syncthreads();
     if (wgrad(KIND)) {
         // experts by row count, largest first (ties: lower id first): rank by counting, O(E^2 / threads)
@@ -1309,7 +1310,7 @@ int launch_down_fwd(const moe_dims_t& d, const bf16* h_act, const bf16* w_down, 
 // Down dgrad: dh_act = dy_perm . w_down[e]^T.  A = dy_perm [R,H]; B = w_down viewed as [E*I, H] (rows are
 // output columns, K = H contiguous).
 int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_down, const int32_t* offsets,
-                      bf16* dh_act, cudaStream_t s) {
+                      bf16* dh_act, bool beside, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     if (use_swapped(d, d.H)) {
         // swapped roles: M side = w_down tile (128 features of I, K-major), N side = rows of dy_perm
@@ -1320,7 +1321,7 @@ int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_do
             !make_map(&a1, dy_perm, d.H, R, BK, box) ||
             !make_map(&b0, w_down, d.H, (uint64_t)d.E * d.I, BK, SWAP_FEATS) || !make_out_map(&o0, dh_act, d.I, R))
             return MOE_ERR_CUDA;
-        Params p = {};
+        Params p = {}; p.beside = beside;
         p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
         p.n_tiles = (d.I + feats - 1) / feats; p.n_cols = d.I; p.b_rows_per_e = d.I;
         p.out0 = dh_act; p.ldo = d.I; p.n_split = d.I;
@@ -1330,7 +1331,7 @@ int launch_down_dgrad(const moe_dims_t& d, const bf16* dy_perm, const bf16* w_do
     if (!make_map(&a, dy_perm, d.H, R, BK, BM) || !make_map(&b0, w_down, d.H, (uint64_t)d.E * d.I, BK, BN / 2) ||
         !make_out_map(&o0, dh_act, d.I, R))
         return MOE_ERR_CUDA;
-    Params p = {};
+    Params p = {}; p.beside = beside;
     p.offsets = offsets; p.E = d.E; p.k_blocks = d.H / BK; p.k_split = p.k_blocks;
     p.n_tiles = (d.I + BN - 1) / BN; p.n_cols = d.I; p.b_rows_per_e = d.I;
     p.out0 = dh_act; p.ldo = d.I; p.n_split = d.I;
@@ -1368,7 +1369,7 @@ int launch_down_dgrad_swiglu_bwd(const moe_dims_t& d, const bf16* dy_perm, const
 // Gate/up dgrad: dx_perm = dg . w_gate[e]^T + du . w_up[e]^T.  A = dgu [R,2I]; the contraction runs over the
 // gate half against w_gate viewed as [E*H, I], then over the up half against w_up.
 int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate, const bf16* w_up,
-                        const int32_t* offsets, bf16* dx_perm, cudaStream_t s) {
+                        const int32_t* offsets, bf16* dx_perm, bool beside, cudaStream_t s) {
     const uint64_t R = (uint64_t)d.T * d.K;
     if (use_swapped(d, 2 * d.I)) {
         const int feats = 2 * SWAP_FEATS;   // a CTA pair's tile
@@ -1379,7 +1380,7 @@ int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate
             !make_map(&b0, w_gate, d.I, (uint64_t)d.E * d.H, BK, SWAP_FEATS) ||
             !make_map(&b1, w_up, d.I, (uint64_t)d.E * d.H, BK, SWAP_FEATS) || !make_out_map(&o0, dx_perm, d.H, R))
             return MOE_ERR_CUDA;
-        Params p = {};
+        Params p = {}; p.beside = beside;
         p.offsets = offsets; p.E = d.E; p.k_blocks = 2 * d.I / BK; p.k_split = d.I / BK;
         p.n_tiles = (d.H + feats - 1) / feats; p.n_cols = d.H; p.b_rows_per_e = d.H;
         p.out0 = dx_perm; p.ldo = d.H; p.n_split = d.H;
@@ -1390,7 +1391,7 @@ int launch_gateup_dgrad(const moe_dims_t& d, const bf16* dgu, const bf16* w_gate
     if (!make_map(&a, dgu, 2ull * d.I, R, BK, BM) || !make_map(&b0, w_gate, d.I, (uint64_t)d.E * d.H, BK, bn) ||
         !make_map(&b1, w_up, d.I, (uint64_t)d.E * d.H, BK, bn) || !make_out_map(&o0, dx_perm, d.H, R))
         return MOE_ERR_CUDA;
-    Params p = {};
+    Params p = {}; p.beside = beside;
     p.offsets = offsets; p.E = d.E; p.k_blocks = 2 * d.I / BK; p.k_split = d.I / BK;
     p.n_tiles = (d.H + BN - 1) / BN; p.n_cols = d.H; p.b_rows_per_e = d.H;
     p.out0 = dx_perm; p.ldo = d.H; p.n_split = d.H;

@@ -101,3 +101,12 @@ def test_library_is_built_without_a_c_compiler(monkeypatch, tmp_path, compiler):
         assert os.path.exists(build.build_library())
     with pytest.raises((OSError, RuntimeError)):
         build.build_pycall()
+
+
+@pytest.mark.parametrize("name", ["moe_grouped_gemm_down_bwd", "moe_grouped_gemm_gateup_swiglu_bwd"])
+def test_combined_calls_look_at_all_arguments_before_the_first_launch(B, name):
+    lib, d = B.load_library(), B.dims(256, 256, 512, 8, 2)
+    n = lib.entries[name][1] - 1
+    for i in range(n):
+        for bad, status in ((0, 1), (264, 4)):
+            assert lib.native_call(lib.entries[name], d, *[bad if j == i else 256 for j in range(n)], 0) == status, (i, bad)
