@@ -693,7 +693,8 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
 // Few tokens have a block each, whatever their width, as long as the chip takes all blocks at once (three per SM, four without dtopk_w, two
 // of the run-time K): then the time is that of one block, and several tokens to one only share its SM (41 x 384, K = 8, 32 / 64 / 128 / 256
 // threads 3.2 / 2.3 / 2.0 / 1.7 us, without dtopk_w 2.3 / 1.7 / 1.6 / 1.3; 12 x 7744, 7 24.7 with 32, 6.9 with 256; 418 x 384, 12 5.6 with
-// 64, 9.6 with 256).
+// 64, 9.6 with 256).  Rows of one warp's width gain 0.1 us by it, and more than a block per SM costs their successor as much again (a step
+// of 256 x 256, 2 45.3 us on the device, 45.1 with eight tokens to a block).
 // Of more tokens no fewer threads than give every SM two blocks of them (four without dtopk_w), up to one for each piece: one thread's
 // pieces come one after the other, and with fewer the chip waits for them (32 / 256 threads: 515 x 3776, 6 11.6 / 7.1 us).
 // Rows of 3584 and more have at least 128: more loads in flight (32 / 256 threads: 3593 x 5696, 6 112 / 93 us, without dtopk_w 63 / 53,
@@ -704,7 +705,7 @@ int launch_gather_sum(const moe_dims_t& d, const bf16* src_perm, const float* to
 constexpr int kLongRowPieces = 3584 / 8, kWideRowPieces = 1600 / 8;
 static int combine_bwd_lanes_of(int T, int hv, int K, bool with_dw) {
     const int sms = 2 * kChipPairs, at_once = K > 8 ? 2 : with_dw ? 3 : 4;   // blocks per SM
-    if (T <= at_once * sms || (!with_dw && hv >= kLongRowPieces)) return kThreads;
+    if (T <= (hv > 32 ? at_once : 1) * sms || (!with_dw && hv >= kLongRowPieces)) return kThreads;
     int best = 32;
     while (best < kThreads && best < hv && (long long)T * best < (with_dw ? 2ll : 4ll) * sms * kThreads) best *= 2;
     if (best < 128 && hv >= (with_dw ? kLongRowPieces : kWideRowPieces)) best = 128;

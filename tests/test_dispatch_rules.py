@@ -26,11 +26,11 @@ def test_threads_per_token_of_the_combine_backward():
     lanes = ctypes.CDLL(build.build_library(waittest=True)).moe_test_combine_bwd_lanes
     for T, H, want in ((20000, 256, 32), (20000, 512, 32), (20000, 832, 32), (20000, 1024, 64), (10000, 1280, 32), (16384, 2048, 128), (8192, 4096, 256),
                        (14442, 2880, 128), (27, 2304, 256), (12, 7744, 256), (515, 3776, 256), (41, 2624, 256), (3593, 5696, 256), (4736, 1152, 32),
-                       (2367, 1152, 64), (1, 64, 256), (444, 64, 256), (445, 64, 32), (445, 512, 64), (445, 1088, 256), (2368, 3072, 128), (2368, 3328, 32), (2367, 3328, 64), (2368, 3584, 128), (6681, 4352, 128), (9000, 3520, 64)):
+                       (2367, 1152, 64), (1, 64, 256), (148, 256, 256), (149, 256, 32), (444, 320, 256), (445, 320, 64), (445, 512, 64), (445, 1088, 256), (2368, 3072, 128), (2368, 3328, 32), (2367, 3328, 64), (2368, 3584, 128), (6681, 4352, 128), (9000, 3520, 64)):
         assert lanes(T, H, 2, 1) == want, (T, H, lanes(T, H, 2, 1))
-    for T, H, want in ((592, 64, 256), (593, 256, 32), (593, 1088, 256), (4735, 1152, 64), (4736, 1152, 32), (20000, 1024, 64), (20000, 1536, 64), (20000, 1600, 128), (4279, 2304, 128), (2433, 3200, 128), (27, 2304, 256), (8192, 4096, 256)):
+    for T, H, want in ((148, 256, 256), (149, 256, 32), (592, 320, 256), (593, 320, 64), (593, 1088, 256), (4735, 1152, 64), (4736, 1152, 32), (20000, 1024, 64), (20000, 1536, 64), (20000, 1600, 128), (4279, 2304, 128), (2433, 3200, 128), (27, 2304, 256), (8192, 4096, 256)):
         assert lanes(T, H, 2, 0) == want, (T, H, lanes(T, H, 2, 0))   # without dtopk_w
-    assert lanes(296, 64, 9, 1) == lanes(296, 64, 9, 0) == 256 and lanes(297, 64, 9, 1) == 32   # fewer blocks at once of the run-time K
+    assert lanes(296, 320, 9, 1) == lanes(296, 320, 9, 0) == 256 and lanes(297, 320, 9, 1) == 64   # fewer blocks at once of the run-time K
     # the form that leaves its successor to the end exists for 32 threads per token only: others are small grids or blocks of 1024 pieces and more
     for T in (*range(1, 3000, 61), 592, 593, 1184, 1185, 2367, 2368, 4735, 4736, 100000):
         for H in range(64, 8192, 64):
